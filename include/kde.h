@@ -77,7 +77,8 @@ typedef enum {
 
 /* ---- evaluation paths --------------------------------------------------- */
 typedef enum {
-  KDE_PATH_AUTO = 0,       /* Gaussian -> TC_SPLIT16, compact -> CUTOFF       */
+  KDE_PATH_AUTO = 0,       /* Gaussian -> TC_SPLIT16 (with KDE_FLAG_SKIP_ZERO */
+                           /* where that is the faster), compact -> CUTOFF    */
   KDE_PATH_SIMT_FP32 = 1,  /* FP32 direct sum on the CUDA cores (Table 1)    */
   KDE_PATH_TC_FP16 = 2,    /* Gaussian as F = A B^T on tcgen05, FP16 operands */
   KDE_PATH_TC_SPLIT16 = 3, /* same, hi/lo FP16 operands, three products       */
@@ -86,7 +87,7 @@ typedef enum {
 
 #define KDE_FLAG_SYNC 1u         /* wait for completion and check device flags */
 #define KDE_FLAG_SKIP_ZERO 2u    /* TC paths: block-sparse skipping. Points are */
-                                 /* sorted into 32x32-cell bins and each 256x256*/
+                                 /* sorted into small bins and each 256x256    */
                                  /* tile reads only the bins within 6.45        */
                                  /* h sqrt(2 ln 2) (~7.6 h) of it; beyond that  */
                                  /* every FP16 operand is exactly zero, so no   */

@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
         for (int cb = 0; cb < 8; ++cb) {
           uint32_t d[16];
-          tmem_ld16_async(acc + cb * 16, d);
+          tmem_ld_async(acc + cb * 16, d);
           tmem_wait_ld();
           if (cb == 7) {  // every column is in registers: release the accumulator
             tc_fence_before();

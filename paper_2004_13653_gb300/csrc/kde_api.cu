@@ -205,8 +205,10 @@ struct InstPlan {
   int splits;
   int64_t n_pad, prep_begin;
   size_t off_gxt, off_gyt, off_part, off_run;  // off_run: SIMT running sums
-  // tensor-core path: the instance's tile family and accumulator chunk
+  // tensor-core path: the instance's tile family and accumulator chunk;
+  // sparse: block-sparse skipping (asked for, or AUTO's choice)
   int fam, k_chunk, split_req;
+  bool sparse;
   int tiles_m, tiles_n, items;
   int64_t per_split;
   // cutoff path, and the bin sort of block-sparse tensor-core instances
@@ -222,6 +224,61 @@ struct InstPlan {
 // (hi and lo alike); the margin over the exact bound sqrt(41) = 6.403 covers
 // the FP32 rounding of the offsets and of ex2.approx.
 constexpr double kSparseReach = 6.45;
+
+// Reach of a Gaussian operand in cells of the grid, and the 256-cell tiles of
+// one axis (n cells, `tiles` tiles) whose reach a point lies in, its sort bin
+// with it: at most (256 + 2 reach + bin) / 256 of them, as for a point in the
+// middle of a wide grid; fewer on average over the grid, where the reach of a
+// point near an edge falls outside.
+double sparse_reach_cells(const kde_args* a) {
+  return kSparseReach / (a->cell * kernel_sigma(KDE_GAUSSIAN, a->h));
+}
+double sparse_tiles_per_point(double reach_cells, int bin, int tiles) {
+  return std::min((double)tiles, (256.0 + 2.0 * reach_cells + bin) / 256.0);
+}
+double sparse_tiles_average(double reach_cells, int bin, int n, int tiles) {
+  double cells = 0.0;  // of the axis that lie within each tile's reach
+  for (int t = 0; t < tiles; ++t) {
+    const double lo = std::max(0.0, 256.0 * t - reach_cells - bin);
+    const double hi = std::min((double)n, 256.0 * (t + 1) + reach_cells);
+    cells += std::max(0.0, hi - lo);
+  }
+  return cells / n;
+}
+
+// AUTO's choice between the dense and the block-sparse contraction of a
+// Gaussian instance, from the time each takes on this GPU: dense about 1.92e9
+// FLOP per microsecond, block-sparse 1.8e9 on the (tile, point) pairs within
+// reach and about 80 us + 60 us per million points of sort, work list and
+// reduce.  The pairs are taken halfway between points spread evenly and points
+// all in the middle (tracks lie somewhere between).  The block-sparse
+// contraction skips only products that are exactly zero, so the choice never
+// changes what is summed.  It is taken where it should be 10% ahead; near the
+// line either costs about the same (300,007 points x 777 x 1111, reach 421
+// cells: dense 1.27 ms, block-sparse 1.18 ms), far from it the block-sparse
+// one wins by the ratio of the pairs (20M x 4096^2, reach 31 cells: 1030 ms
+// against 8.7 ms).
+bool auto_sparse(const kde_args* a, int bin) {
+  const int tm = (a->nx + 255) / 256, tn = (a->ny + 255) / 256;
+  const double rc = sparse_reach_cells(a);
+  const double per_tile = (double)a->n * 65536.0 * 6.0;
+  const double dense = per_tile * tm * tn / 1.92e9;
+  const double most = sparse_tiles_per_point(rc, bin, tm) * sparse_tiles_per_point(rc, bin, tn);
+  const double even = sparse_tiles_average(rc, bin, a->nx, tm) *
+                      sparse_tiles_average(rc, bin, a->ny, tn);
+  const double sparse = per_tile * 0.5 * (most + even) / 1.8e9 + 80.0 + 60e-6 * (double)a->n;
+  return 1.1 * sparse < dense;
+}
+
+// Side of the block-sparse sort bins, in cells: a tile reads every point of
+// the bins within its reach, (256 + 2 reach + bin)^2 cells' worth, so finer
+// bins mean fewer products; the bins of one call stay within the 2^16 that
+// two radix passes sort (kSparseBin = 32 where even those are more).
+int sparse_sort_bin(int nx, int ny, int instances) {
+  for (int bin = 4; bin < kSparseBin; bin *= 2)
+    if (((int64_t)(nx + bin - 1) / bin) * ((ny + bin - 1) / bin) * instances <= 65536) return bin;
+  return kSparseBin;
+}
 
 // The adjoint takes the tensor-core contractions when the window kernel's
 // cells per point exceed this fraction of the grid padded to 256-cell tiles
@@ -282,7 +339,9 @@ struct BatchPlan {
   int n_tc = 0, n_cut = 0, n_simt = 0, n_reduce = 0, tc_items = 0, max_side = 1;
   int64_t total_pad = 0, cut_m = 0, total_bins = 0, reduce_cells = 0, cut_bins = 0;
   int64_t cut_slice_bins = 0;  // output blocks of cutoff instances that split heavy blocks
-  bool sparse = false;  // block-sparse tensor-core instances
+  bool sparse = false;  // some tensor-core instances are block-sparse
+  bool auto_sparse = false;  // ... by AUTO's choice: the dense plan does as well
+  int n_sparse = 0, sparse_fam = -1;
   int tiles_total = 0, piece_len = 0, max_pieces = 0;
   size_t off_sp_total = 0, off_sp_np = 0, off_sp_pb = 0, off_sp_nf = 0, off_sp_fb = 0,
          off_sp_tail = 0, off_sp_temp = 0, off_sp_part = 0;
@@ -295,8 +354,10 @@ struct BatchPlan {
       off_hout, total;
 };
 
+// allow_sparse: whether AUTO may choose the block-sparse contraction (false
+// when its workspace cannot be had).
 int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling* tiles,
-              bool probe_memory, BatchPlan* P) {
+              bool probe_memory, bool allow_sparse, BatchPlan* P) {
   P->count = count;
   P->in.assign(count, InstPlan());
   const int sms = sm_count();
@@ -365,7 +426,14 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   if (want_pair && !pair_ok)
     return fail(KDE_EINVAL, "CTA-pair tiles need tile_n 256, 64-point stages and two CTAs");
   t.pair = want_pair || (!no_pair && pair_ok) ? 1 : 0;
-  P->sparse = want_sparse;
+  // AUTO may pick the block-sparse contraction per instance; a caller who
+  // names a path or any part of the tiling gets the contraction that he asked for
+  const bool may_sparse =
+      allow_sparse && ctas >= 2 && (!o || (o->path == KDE_PATH_AUTO && !o->tile_n && !o->k_chunk &&
+                                           !o->split_k && !o->stage_points &&
+                                           !(o->flags & (KDE_FLAG_CTA_PAIR | KDE_FLAG_ONE_CTA))));
+  int n_tc_all = 0;
+  for (int k = 0; k < count; ++k) n_tc_all += is_tc(P->in[k].path);
 
   if (tc_split16 >= 0 && (t.k_chunk % t.stage_points || t.k_chunk < 2 * t.stage_points))
     return fail(KDE_EINVAL, "k_chunk %d must be a multiple of, and at least twice, the %d-point stage",
@@ -377,9 +445,27 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     InstPlan& I = P->in[k];
     I.fam = -1;
     I.split_req = o ? o->split_k : 0;
+    I.sparse = false;
     if (!is_tc(I.path)) continue;
     TcPlan f = t;
     int kc = t.k_chunk;
+    const bool own_tiling =
+        tiles && (tiles[k].tile_n || tiles[k].k_chunk || tiles[k].split_k ||
+                  tiles[k].stage_points || tiles[k].flags);
+    I.sparse = want_sparse ||
+               (may_sparse && !own_tiling &&
+                auto_sparse(&A[k], sparse_sort_bin(A[k].nx, A[k].ny, n_tc_all)));
+    if (I.sparse) {
+      f.pair = 1;
+      f.tile_n = 256;
+      f.stage_points = 64;
+      f.skip_zero = 1;
+      // sorted points put a whole chunk's mass on the same cells, so the
+      // accumulators are drained every 64 points: the tensor core's FP32
+      // accumulation then loses no more than the dense contraction's does
+      if (!(o && o->k_chunk) && f.split16) kc = 64;
+      P->auto_sparse = P->auto_sparse || !want_sparse;
+    }
     if (tiles) {
       const kde_tiling& ti = tiles[k];
       if ((ti.tile_n != 0 && ti.tile_n != 128 && ti.tile_n != 256) ||
@@ -388,7 +474,7 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
           (ti.flags & ~(KDE_FLAG_CTA_PAIR | KDE_FLAG_ONE_CTA)) ||
           ((ti.flags & KDE_FLAG_CTA_PAIR) && (ti.flags & KDE_FLAG_ONE_CTA)))
         return fail(KDE_EINVAL, "instance %d: invalid tiling", k);
-      if (P->sparse) {
+      if (I.sparse) {
         if ((ti.flags & KDE_FLAG_ONE_CTA) || (ti.tile_n && ti.tile_n != 256) ||
             (ti.stage_points && ti.stage_points != 64))
           return fail(KDE_ENOTSUP, "instance %d: block-sparse skipping runs on 256 x 256 CTA-pair "
@@ -410,19 +496,26 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       }
       if (ti.k_chunk) kc = ti.k_chunk;
       if (ti.split_k) I.split_req = ti.split_k;
-      if (kc % f.stage_points || kc < 2 * f.stage_points)
+      if (kc % f.stage_points || (ti.k_chunk && kc < 2 * f.stage_points))
         return fail(KDE_EINVAL, "instance %d: k_chunk %d must be a multiple of, and at least "
                     "twice, the %d-point stage", k, kc, f.stage_points);
     }
     I.k_chunk = kc;
     for (int q = 0; q < (int)P->fam.size() && I.fam < 0; ++q) {
       const TcPlan& g = P->fam[q].plan;
-      if (g.pair == f.pair && g.tile_n == f.tile_n && g.stage_points == f.stage_points) I.fam = q;
+      if (g.pair == f.pair && g.tile_n == f.tile_n && g.stage_points == f.stage_points &&
+          g.skip_zero == f.skip_zero)
+        I.fam = q;
     }
     if (I.fam < 0) {
       I.fam = (int)P->fam.size();
       P->fam.push_back(TcFamily());
       P->fam.back().plan = f;
+    }
+    if (I.sparse) {
+      P->sparse = true;
+      P->sparse_fam = I.fam;
+      ++P->n_sparse;
     }
   }
 
@@ -451,7 +544,7 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
         splits = (int)std::max<int64_t>(1, std::min<int64_t>({want, maxs, 64}));
       }
       ++P->n_simt;
-    } else if (is_tc(I.path) && P->sparse) {
+    } else if (is_tc(I.path) && I.sparse) {
       // block-sparse: the work list is built on the device; no point splits
       splits = 1;
       I.per_split = I.n_pad;
@@ -514,34 +607,46 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     // bins of the block-sparse instances follow the cutoff bins in the sort
     double est = 0.0;
     int64_t bound = 0;
-    for (int k : P->tc_order) {
+    const TcFamily& sf = P->fam[P->sparse_fam];
+    for (int k : sf.order) {
       const kde_args* a = &A[k];
       InstPlan& I = P->in[k];
       const double cs = a->cell * kernel_sigma(KDE_GAUSSIAN, a->h);
-      I.geo = cutoff_geometry(a->nx, a->ny, cs, kSparseReach, kSparseBin);
+      I.geo = cutoff_geometry(a->nx, a->ny, cs, kSparseReach,
+                              sparse_sort_bin(a->nx, a->ny, P->n_sparse));
       I.bin_begin = (int)P->total_bins;
       P->total_bins += I.geo.nbins;
       I.cut_begin = P->cut_m;
       P->cut_m += I.n_pad;
       I.tile_begin = P->tiles_total;
       P->tiles_total += I.tiles_m * I.tiles_n;
-      est += 1.5 * (double)I.n_pad;
+      const double rc = sparse_reach_cells(a);
+      est += (double)I.n_pad * sparse_tiles_per_point(rc, I.geo.bin, I.tiles_m) *
+             sparse_tiles_per_point(rc, I.geo.bin, I.tiles_n);
     }
     // pieces of about an eighth of each CTA pair's share, in whole drain chunks
     const int clusters = std::max(1, ctas / 2);
     int64_t L = (int64_t)(est / (8.0 * clusters));
     L = std::max<int64_t>(2048, std::min<int64_t>(kSparseMaxPiece, L));
-    L = (L + t.k_chunk - 1) / t.k_chunk * t.k_chunk;
+    for (int k : sf.order) {  // whole accumulator chunks of every instance
+      const int64_t kc = std::max(P->in[k].k_chunk, sf.plan.stage_points);
+      L = (L + kc - 1) / kc * kc;
+    }
     P->piece_len = (int)L;
-    for (int k : P->tc_order) {
+    for (int k : sf.order) {
       const kde_args* a = &A[k];
       const InstPlan& I = P->in[k];
-      // a bin lies within reach of at most `per_axis` tiles along each axis
-      const double rc = kSparseReach / (a->cell * kernel_sigma(KDE_GAUSSIAN, a->h));
-      const int64_t per_axis = (int64_t)std::ceil((288.0 + 2.0 * rc) / 256.0) + 1;
-      const int64_t tiles = (int64_t)I.tiles_m * I.tiles_n;
-      const int64_t reach_tiles = std::min(per_axis * per_axis, tiles);
-      bound += (I.n_pad * reach_tiles + L - 1) / L + tiles;
+      // a bin of b cells lies within the reach r of the tiles t with
+      // 256 t in (x - 255.5 - r, x + b - 0.5 + r), x its first cell: at most
+      // floor((b + 255 + 2 r) / 256) + 1 of them along an axis (the hundredth
+      // of a cell covers the rounding of the ranges' FP64)
+      const double rc = range_reach(kSparseReach, I.geo) /
+                        (a->cell * kernel_sigma(KDE_GAUSSIAN, a->h));
+      const int64_t per_axis = (int64_t)std::min(
+          1e6, std::floor((I.geo.bin + 255.0 + 2.0 * rc + 0.01) / 256.0) + 1.0);
+      const int64_t reach_tiles = std::min<int64_t>(per_axis, I.tiles_m) *
+                                  std::min<int64_t>(per_axis, I.tiles_n);
+      bound += (I.n_pad * reach_tiles + L - 1) / L + (int64_t)I.tiles_m * I.tiles_n;
     }
     if (bound > (1 << 24) || P->tiles_total > (1 << 26))
       return fail(KDE_EINVAL, "block-sparse work list too large (%lld pieces)", (long long)bound);
@@ -554,9 +659,9 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   // batches on CTA pairs: balance the pairs' work with a host-side schedule
   // (items of different instances differ in length; round robin left the last
   // pair finishing 7% after the mean on the 256-instance batch)
-  if (count > 1 && !P->sparse) {
+  if (count > 1) {
     for (TcFamily& f : P->fam) {
-      if (!f.plan.pair || f.items < 2) continue;
+      if (!f.plan.pair || f.plan.skip_zero || f.items < 2) continue;
       std::vector<int64_t> cost;
       cost.reserve(f.items);
       for (int k : f.order) {
@@ -571,7 +676,6 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       f.sched = lpt_schedule(cost, pair_clusters(f.plan, f.items));
     }
   }
-  if (P->sparse && P->fam.size() > 1) return fail(KDE_EINVAL, "block-sparse batch with two tilings");
   P->cz = cutoff_sizes(P->cut_m, P->total_bins);
 
   size_t off = 0;
@@ -581,7 +685,7 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   P->off_wts = take(sizeof(float) * (size_t)P->total_pad);
   P->off_tab_prep = take(sizeof(PrepInst) * (size_t)count);
   P->off_tab_tc = take(sizeof(TcInst) * (size_t)std::max(P->n_tc, 1));
-  P->off_tab_cut = take(sizeof(CutInst) * (size_t)std::max(P->n_cut + (P->sparse ? P->n_tc : 0), 1));
+  P->off_tab_cut = take(sizeof(CutInst) * (size_t)std::max(P->n_cut + P->n_sparse, 1));
   P->off_tab_red = take(sizeof(ReduceInst) * (size_t)std::max(P->n_reduce, 1));
   for (TcFamily& f : P->fam)
     if (!f.sched.empty()) f.off_sched = take(sizeof(uint32_t) * f.sched.size());
@@ -669,7 +773,13 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     if (rc) return rc;
   }
   BatchPlan P;
-  int rc = make_plan(A, count, o, tiles, true, &P);
+  int rc = make_plan(A, count, o, tiles, true, true, &P);
+  // AUTO's block-sparse plan is a choice: where its work list or workspace is
+  // out of reach, the call runs dense as an explicit TC_SPLIT16 call does
+  if (rc && P.auto_sparse) {
+    P = BatchPlan();
+    rc = make_plan(A, count, o, tiles, true, false, &P);
+  }
   if (rc) return rc;
   cudaStream_t s = stream_of(o);
   // host output makes the call wait for its copy back, unless the caller
@@ -678,6 +788,12 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   const bool sync = force_sync || (o && (o->flags & KDE_FLAG_SYNC)) || (P.host_out && !host_async);
   void* wsv = nullptr;
   rc = acquire_workspace(o, P.total, s, &wsv);
+  if (rc == KDE_ENOMEM && P.auto_sparse) {
+    P = BatchPlan();
+    rc = make_plan(A, count, o, tiles, true, false, &P);
+    if (rc) return rc;
+    rc = acquire_workspace(o, P.total, s, &wsv);
+  }
   if (rc) return rc;
   char* base = static_cast<char*>(wsv);
   CallScalars* scal = reinterpret_cast<CallScalars*>(base + P.off_scal);
@@ -771,7 +887,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     q.start = nullptr;
     q.cs = q.reach = q.inv_binw = q.range_reach = 0.0;
     q.nbx = q.nby = q.bin_begin = q.tile_begin = 0;
-    if (P.sparse) {  // points in bin order; the sparse reduce writes the output
+    if (I.sparse) {  // points in bin order; the sparse reduce writes the output
       q.pts = reinterpret_cast<const float4*>(base + P.off_co_spts);
       q.wts = reinterpret_cast<const float*>(base + P.off_co_sw);
       q.part = out_dev[k];
@@ -831,7 +947,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   }
   const int n_cut_only = (int)cut.size();
   if (P.sparse) {  // bin-sort entries of the block-sparse instances, after the cutoff ones
-    for (int k : P.tc_order) {
+    for (int k : P.fam[P.sparse_fam].order) {
       const InstPlan& I = P.in[k];
       CutInst q = {};
       q.gxt = prep[k].gxt;
@@ -897,12 +1013,14 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     cs.ocount = reinterpret_cast<uint32_t*>(base + P.off_co_ocount);
     cs.err = batch_scal;
   }
-  // The compact instances (sort and gather) overlap the tensor-core
-  // contraction on the side stream when no block-sparse instance needs the
-  // sort first: the contraction is enqueued first, its CTAs take every SM,
-  // the small sort kernels fit beside them and the gather fills the SMs its
-  // tail frees.  They write disjoint buffers, so results do not change.
-  const bool overlap = P.n_cut && P.n_tc && !P.sparse;
+  // The compact instances' gather overlaps the tensor-core contractions on the
+  // side stream: the contractions are enqueued first and their CTAs take every
+  // SM, and the gather fills the SMs their tails free.  Without block-sparse
+  // instances, whose contraction needs the sort first, the small sort kernels
+  // move there as well (they fit beside the contraction's CTAs).  The two
+  // sides write disjoint buffers, so results do not change.
+  const bool overlap = P.n_cut && P.n_tc;
+  const bool sort_aside = overlap && !P.sparse;
   cudaStream_t s2 = s;
   cudaEvent_t fork = nullptr, join = nullptr;
   struct EventGuard {
@@ -912,17 +1030,19 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
         if (*x) cudaEventDestroy(*x);
     }
   } guard{{&fork, &join}};
+  if ((P.n_cut || P.sparse) && !sort_aside)
+    KDE_CUDA(launch_bin_sort(d_cut, (int)cut.size(), P.cut_m, P.total_bins, pts, wts, P.cz, cs, s),
+             "bin sort");
   if (overlap) {
     if (int rc = side_stream(&s2)) return rc;
     KDE_CUDA(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming), "create event");
     KDE_CUDA(cudaEventCreateWithFlags(&join, cudaEventDisableTiming), "create event");
     KDE_CUDA(cudaEventRecord(fork, s), "fork to the side stream");
   }
-  if ((P.n_cut || P.sparse) && !overlap)
-    KDE_CUDA(launch_bin_sort(d_cut, (int)cut.size(), P.cut_m, P.total_bins, pts, wts, P.cz, cs, s),
-             "bin sort");
-  if (P.n_tc && P.sparse) {
-    SparseCtl sp;
+  SparseCtl sp;
+  const TcInst* d_sp = nullptr;  // the block-sparse family's instances
+  if (P.sparse) {
+    d_sp = d_tc + P.fam[P.sparse_fam].tab_begin;
     sp.piece_begin = reinterpret_cast<const uint32_t*>(base + P.off_sp_pb);
     sp.full_begin = reinterpret_cast<const uint32_t*>(base + P.off_sp_fb);
     sp.tail_tile = reinterpret_cast<const uint32_t*>(base + P.off_sp_tail);
@@ -931,25 +1051,29 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     sp.tiles_total = P.tiles_total;
     sp.piece_len = P.piece_len;
     sp.max_pieces = P.max_pieces;
-    KDE_CUDA(launch_sparse_plan(d_tc, P.n_tc, sp, reinterpret_cast<uint32_t*>(base + P.off_sp_np),
+    KDE_CUDA(launch_sparse_plan(d_sp, P.n_sparse, sp,
+                                reinterpret_cast<uint32_t*>(base + P.off_sp_np),
                                 reinterpret_cast<uint32_t*>(base + P.off_sp_nf),
                                 reinterpret_cast<uint32_t*>(base + P.off_sp_temp), batch_scal, s),
              "block-sparse work list");
-    KDE_CUDA(launch_tc_pair(P.fam[0].plan, d_tc, P.n_tc, 0, &sp, nullptr, batch_scal, s),
-             "block-sparse tensor-core contraction");
-    KDE_CUDA(launch_sparse_reduce(d_tc, P.n_tc, sp, s), "block-sparse reduce");
-  } else if (P.n_tc) {
-    for (const TcFamily& f : P.fam) {  // one persistent launch per tile family
-      if (f.items < 1) continue;
-      const int nf = (int)f.order.size();
-      const uint32_t* sched =
-          f.sched.empty() ? nullptr : reinterpret_cast<const uint32_t*>(base + f.off_sched);
-      KDE_CUDA(f.plan.pair ? launch_tc_pair(f.plan, d_tc + f.tab_begin, nf, f.items, nullptr, sched,
-                                            batch_scal, s)
-                           : launch_tc(f.plan, d_tc + f.tab_begin, nf, f.items, batch_scal, s),
-               "tensor-core contraction");
-    }
   }
+  for (const TcFamily& f : P.fam) {  // one persistent launch per tile family
+    const int nf = (int)f.order.size();
+    if (f.plan.skip_zero) {
+      KDE_CUDA(launch_tc_pair(f.plan, d_sp, nf, 0, &sp, nullptr, batch_scal, s),
+               "block-sparse tensor-core contraction");
+      continue;
+    }
+    if (f.items < 1) continue;
+    const uint32_t* sched =
+        f.sched.empty() ? nullptr : reinterpret_cast<const uint32_t*>(base + f.off_sched);
+    KDE_CUDA(f.plan.pair ? launch_tc_pair(f.plan, d_tc + f.tab_begin, nf, f.items, nullptr, sched,
+                                          batch_scal, s)
+                         : launch_tc(f.plan, d_tc + f.tab_begin, nf, f.items, batch_scal, s),
+             "tensor-core contraction");
+  }
+  if (P.sparse)
+    KDE_CUDA(launch_sparse_reduce(d_sp, P.n_sparse, sp, s), "block-sparse reduce");
   for (int k = 0; k < count; ++k) {
     const InstPlan& I = P.in[k];
     if (I.path != KDE_PATH_SIMT_FP32) continue;
@@ -960,8 +1084,10 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   }
   if (overlap) {
     KDE_CUDA(cudaStreamWaitEvent(s2, fork, 0), "side stream waits for the prepared points");
-    KDE_CUDA(launch_bin_sort(d_cut, (int)cut.size(), P.cut_m, P.total_bins, pts, wts, P.cz, cs, s2),
-             "bin sort");
+    if (sort_aside)
+      KDE_CUDA(launch_bin_sort(d_cut, (int)cut.size(), P.cut_m, P.total_bins, pts, wts, P.cz, cs,
+                               s2),
+               "bin sort");
     KDE_CUDA(launch_cutoff_eval(d_cut, n_cut_only, P.cut_bins, P.cut_slice_bins, cs, s2),
              "cutoff evaluation");
     KDE_CUDA(cudaEventRecord(join, s2), "join from the side stream");
@@ -1044,7 +1170,11 @@ int kde_workspace_size(const kde_args* a, const kde_opts* opts, size_t* bytes) {
   int rc = validate(a, opts);
   if (rc) return rc;
   BatchPlan pl;
-  rc = make_plan(a, 1, opts, nullptr, true, &pl);
+  rc = make_plan(a, 1, opts, nullptr, true, true, &pl);
+  if (rc && pl.auto_sparse) {
+    pl = BatchPlan();
+    rc = make_plan(a, 1, opts, nullptr, true, false, &pl);
+  }
   if (rc) return rc;
   *bytes = pl.total;
   return KDE_OK;

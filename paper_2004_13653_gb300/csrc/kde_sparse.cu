@@ -9,8 +9,8 @@
 // from it along x or along y.  Skipping those (tile, point) pairs therefore
 // changes no product, only which zeros are added.
 //
-// The points are sorted into 32 x 32-cell bins (the cutoff path's stable
-// radix sort, with that reach); a 256 x 256 tile then needs only the bins
+// The points are sorted into bins of 4 to 32 cells a side (the cutoff path's
+// stable radix sort, with that reach); a 256 x 256 tile then needs only the bins
 // within reach, i.e. one contiguous run of sorted points per bin row.  This
 // file builds the work list (points per tile, cut into pieces of a fixed
 // length, and the exclusive scan of the pieces per tile) and sums each
@@ -32,31 +32,37 @@ __device__ __forceinline__ int inst_of_tile(const TcInst* __restrict__ tab, int 
   return a;
 }
 
-// One thread per tile: the points its bin rows hold, its piece count and its
-// count of full pieces.  npieces and nfull have tiles_total + 1 entries; the
-// last are zero so that the exclusive scans end with the totals.
-__global__ void k_sparse_totals(const TcInst* __restrict__ tab, int ninst, SparseCtl sp,
-                                uint32_t* __restrict__ tile_total, uint32_t* __restrict__ npieces,
-                                uint32_t* __restrict__ nfull) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t > sp.tiles_total) return;
-  if (t == sp.tiles_total) {
-    npieces[t] = 0;
-    nfull[t] = 0;
-    return;
-  }
+// The points of a tile's bin rows, one warp per tile, the rows over its lanes
+// (one thread per tile was a chain of a hundred dependent reads: 27 us for the
+// 16 tiles of 1024^2).
+__device__ __forceinline__ uint32_t tile_points(const TcInst* __restrict__ tab, int ninst, int t) {
   const TcInst& I = tab[inst_of_tile(tab, ninst, t)];
   const int local = t - I.tile_begin;
   const int tm = local % I.tiles_m, tn = local / I.tiles_m;
   const BinRange br = tile_bins(I.cs, I.range_reach, I.inv_binw, I.nbx, I.nby, tm, tn);
-  uint64_t total = 0;
-  for (int by = br.lo_by; br.lo_bx <= br.hi_bx && by <= br.hi_by; ++by) {
-    const int row = I.bin_begin + by * I.nbx;
-    total += I.start[row + br.hi_bx + 1] - I.start[row + br.lo_bx];
-  }
-  tile_total[t] = (uint32_t)total;
-  npieces[t] = (uint32_t)((total + sp.piece_len - 1) / sp.piece_len);
-  nfull[t] = (uint32_t)(total / sp.piece_len);
+  uint32_t total = 0;  // the sort holds fewer than 2^32 points
+  if (br.lo_bx <= br.hi_bx)
+    for (int by = br.lo_by + (threadIdx.x & 31); by <= br.hi_by; by += 32) {
+      const int row = I.bin_begin + by * I.nbx;
+      total += __ldg(I.start + row + br.hi_bx + 1) - __ldg(I.start + row + br.lo_bx);
+    }
+  return __reduce_add_sync(0xffffffffu, total);
+}
+
+// The tiles' points, piece counts and counts of full pieces.  npieces and
+// nfull have tiles_total + 1 entries; the last are zero so that the exclusive
+// scans end with the totals.
+__global__ void k_sparse_totals(const TcInst* __restrict__ tab, int ninst, SparseCtl sp,
+                                uint32_t* __restrict__ tile_total, uint32_t* __restrict__ npieces,
+                                uint32_t* __restrict__ nfull) {
+  const int t = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (t > sp.tiles_total) return;
+  uint32_t total = 0;
+  if (t < sp.tiles_total) total = tile_points(tab, ninst, t);
+  if ((threadIdx.x & 31) != 0) return;
+  if (t < sp.tiles_total) tile_total[t] = total;
+  npieces[t] = (uint32_t)(((uint64_t)total + sp.piece_len - 1) / sp.piece_len);
+  nfull[t] = total / (uint32_t)sp.piece_len;
 }
 
 // Lists the tiles whose last piece is short, longest first: a counting sort
@@ -73,15 +79,14 @@ __device__ __forceinline__ int tail_key(uint32_t rem, uint32_t L) {
   return 1 + (int)(((uint64_t)(rem - 1) * kTailClasses) / L);
 }
 
-__global__ void __launch_bounds__(kTailThreads) k_sparse_tails(SparseCtl sp) {
-  __shared__ uint32_t cnt[kTailKeys];
-  __shared__ uint32_t warp_sum[kTailThreads / 32];
+__device__ __forceinline__ void list_tails(const SparseCtl& sp, uint32_t (&cnt)[kTailKeys],
+                                           uint32_t (&warp_sum)[kTailThreads / 32]) {
   const int tid = threadIdx.x;
   const uint32_t L = (uint32_t)sp.piece_len;
   if (tid < kTailKeys) cnt[tid] = 0;
   __syncthreads();
   for (int t = tid; t < sp.tiles_total; t += kTailThreads) {
-    const uint32_t rem = __ldg(sp.tile_total + t) % L;
+    const uint32_t rem = sp.tile_total[t] % L;
     if (rem) atomicAdd(&cnt[tail_key(rem, L)], 1u);
   }
   __syncthreads();
@@ -112,30 +117,103 @@ __global__ void __launch_bounds__(kTailThreads) k_sparse_tails(SparseCtl sp) {
   __syncthreads();
   uint32_t* tail = const_cast<uint32_t*>(sp.tail_tile);
   for (int t = tid; t < sp.tiles_total; t += kTailThreads) {
-    const uint32_t rem = __ldg(sp.tile_total + t) % L;
+    const uint32_t rem = sp.tile_total[t] % L;
     if (rem) tail[atomicAdd(&cnt[tail_key(rem, L)], 1u)] = t;
   }
 }
 
+__global__ void __launch_bounds__(kTailThreads) k_sparse_tails(SparseCtl sp) {
+  __shared__ uint32_t cnt[kTailKeys];
+  __shared__ uint32_t warp_sum[kTailThreads / 32];
+  list_tails(sp, cnt, warp_sum);
+}
+
+// The whole work list of at most kTailThreads tiles in one CTA: totals (a warp
+// per tile), both exclusive scans (a tile per thread) and the tails.  Five
+// launches of a few microseconds each become one (1024^2: 35 us -> 7 us with
+// the totals' rows over the lanes).
+__global__ void __launch_bounds__(kTailThreads)
+    k_sparse_plan(const TcInst* __restrict__ tab, int ninst, SparseCtl sp,
+                  uint32_t* __restrict__ tile_total, uint32_t* __restrict__ piece_begin,
+                  uint32_t* __restrict__ full_begin) {
+  __shared__ uint32_t cnt[kTailKeys];
+  __shared__ uint32_t warp_sum[kTailThreads / 32];
+  __shared__ uint32_t totals[kTailThreads];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int t = warp; t < sp.tiles_total; t += kTailThreads / 32) {
+    const uint32_t total = tile_points(tab, ninst, t);
+    if (lane == 0) totals[t] = total;
+  }
+  __syncthreads();
+  const uint32_t L = (uint32_t)sp.piece_len;
+  const uint32_t total = tid < sp.tiles_total ? totals[tid] : 0u;
+  if (tid < sp.tiles_total) tile_total[tid] = total;
+  const uint32_t full = total / L, pieces = full + (total % L ? 1u : 0u);
+#pragma unroll
+  for (int which = 0; which < 2; ++which) {
+    const uint32_t c = which ? full : pieces;
+    uint32_t v = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t n = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += n;
+    }
+    if (lane == 31) warp_sum[warp] = v;
+    __syncthreads();
+    uint32_t before = 0, all = 0;
+    for (int w = 0; w < kTailThreads / 32; ++w) {
+      if (w < warp) before += warp_sum[w];
+      all += warp_sum[w];
+    }
+    uint32_t* out = which ? full_begin : piece_begin;
+    if (tid < sp.tiles_total) out[tid] = before + v - c;
+    if (tid == 0) out[sp.tiles_total] = all;
+    __syncthreads();
+  }
+  list_tails(sp, cnt, warp_sum);  // reads tile_total, written before the barriers above
+}
+
 // out cell (i, j) of tile t = sum over the tile's pieces, in order.  Grid:
-// (tiles, 16); thread = local column i, 16 local rows per block.
-__global__ void __launch_bounds__(256)
+// (tiles, 256 / kRedRows); a thread sums four adjacent columns of one row,
+// eight pieces' loads in flight at a time (the adds stay in piece order).
+// Bound by HBM (256 KB per piece); a dense cluster's tile holds most of the
+// pieces, so its rows are spread over 128 blocks and each thread keeps enough
+// bytes in flight: 1.47M points x 1024^2, 16 tiles: 323 us with one column per
+// thread, 16 rows per block and one load at a time.
+constexpr int kRedRows = 2;
+__global__ void __launch_bounds__(64 * kRedRows)
     k_sparse_reduce(const TcInst* __restrict__ tab, int ninst, SparseCtl sp) {
   const int t = blockIdx.x;
   const TcInst& I = tab[inst_of_tile(tab, ninst, t)];
   const int local = t - I.tile_begin;
   const int tm = local % I.tiles_m, tn = local / I.tiles_m;
-  const int il = threadIdx.x, i = tm * 256 + il;
-  if (i >= I.nx) return;
+  const int il = 4 * (threadIdx.x & 63), i = tm * 256 + il;
+  const int jl = blockIdx.y * kRedRows + (threadIdx.x >> 6), j = tn * 256 + jl;
+  if (i >= I.nx || j >= I.ny) return;
   const int p0 = min((int)sp.piece_begin[t], sp.max_pieces);
   const int p1 = min((int)sp.piece_begin[t + 1], sp.max_pieces);
-  for (int jl = blockIdx.y * 16; jl < blockIdx.y * 16 + 16; ++jl) {
-    const int j = tn * 256 + jl;
-    if (j >= I.ny) break;
-    float acc = 0.f;
-    for (int p = p0; p < p1; ++p) acc += sp.part[(int64_t)p * 65536 + jl * 256 + il];
-    I.part[(int64_t)j * I.nx + i] = acc;
+  const float* src = sp.part + jl * 256 + il;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  constexpr int kAhead = 8;
+  for (int p = p0; p < p1; p += kAhead) {
+    float4 v[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (p + u < p1) v[u] = __ldcs(reinterpret_cast<const float4*>(src + (int64_t)(p + u) * 65536));
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (p + u < p1) {
+        acc.x += v[u].x;
+        acc.y += v[u].y;
+        acc.z += v[u].z;
+        acc.w += v[u].w;
+      }
   }
+  float* out = I.part + (int64_t)j * I.nx + i;
+  const float r[4] = {acc.x, acc.y, acc.z, acc.w};
+#pragma unroll
+  for (int c = 0; c < 4; ++c)  // out is 4-byte aligned only, and nx any number
+    if (i + c < I.nx) out[c] = r[c];
 }
 
 }  // namespace
@@ -149,8 +227,15 @@ cudaError_t launch_sparse_plan(const TcInst* tab, int ninst, const SparseCtl& sp
                                CallScalars* err, cudaStream_t s) {
   (void)err;
   if (sp.piece_len <= 0) return cudaErrorInvalidValue;
+  if (sp.tiles_total <= kTailThreads) {
+    k_sparse_plan<<<1, kTailThreads, 0, s>>>(tab, ninst, sp, const_cast<uint32_t*>(sp.tile_total),
+                                             const_cast<uint32_t*>(sp.piece_begin),
+                                             const_cast<uint32_t*>(sp.full_begin));
+    note_launches(1);
+    return cudaGetLastError();
+  }
   const int m = sp.tiles_total + 1;
-  k_sparse_totals<<<(m + 255) / 256, 256, 0, s>>>(
+  k_sparse_totals<<<(m + 7) / 8, 256, 0, s>>>(
       tab, ninst, sp, const_cast<uint32_t*>(sp.tile_total), npieces, nfull);
   note_launches(1);
   cudaError_t e = cudaGetLastError();
@@ -166,7 +251,7 @@ cudaError_t launch_sparse_plan(const TcInst* tab, int ninst, const SparseCtl& sp
 
 cudaError_t launch_sparse_reduce(const TcInst* tab, int ninst, const SparseCtl& sp,
                                  cudaStream_t s) {
-  k_sparse_reduce<<<dim3(sp.tiles_total, 16), 256, 0, s>>>(tab, ninst, sp);
+  k_sparse_reduce<<<dim3(sp.tiles_total, 256 / kRedRows), 64 * kRedRows, 0, s>>>(tab, ninst, sp);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -344,8 +344,8 @@ __global__ void __launch_bounds__(Cfg<BN, SPLIT, KS>::kThreads, 1)
 #pragma unroll 1
         for (int cb = 0; cb < HN / 32; ++cb) {
           uint32_t ra[32], rr[32];
-          tmem_ld32_async(acc_col + cb * 32, ra);
-          if (!first) tmem_ld32_async(run_col + cb * 32, rr);
+          tmem_ld_async(acc_col + cb * 32, ra);
+          if (!first) tmem_ld_async(run_col + cb * 32, rr);
           tmem_wait_ld();
           if (cb == HN / 32 - 1) {
             tc_fence_before();

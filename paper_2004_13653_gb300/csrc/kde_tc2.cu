@@ -10,10 +10,10 @@
 // CTA with a 128 x 256 tile, and each SM's shared memory serves half of B.
 //
 // Roles, by warpgroup (setmaxnreg divides the registers per warpgroup):
-//   WG0   warp 0: MMA issue (leader CTA, one thread); warp 1: loads and
-//         re-centres the points of each stage; warp 2: signals each finished
-//         stage to the leader (one cluster arrive per CTA and stage); warp 3
-//         idles.  48 registers.
+//   WG0   warp 0: MMA issue (leader CTA, one thread); warp 1 (block-sparse:
+//         and warp 3, in turn): loads and re-centres the points of each
+//         stage; warp 2: signals each finished stage to the leader (one
+//         cluster arrive per CTA and stage).  48 registers.
 //   WG1-2 warps 4-11: epilogue.  Each thread owns one TMEM lane (an x cell)
 //         and 128 of the tile's 256 y cells, and keeps their running sums in
 //         its registers (168 registers).
@@ -63,7 +63,7 @@ constexpr int kPrmFloats = 3 * kKS + kKS / 2;
 // warp roles and register budgets (see the file comment)
 constexpr int kWarps = 20;
 constexpr int kThreads = 32 * kWarps;
-constexpr int kWarpMma = 0, kWarpLoader = 1, kWarpSignal = 2;
+constexpr int kWarpMma = 0, kWarpLoader = 1, kWarpSignal = 2, kWarpLoader2 = 3;
 constexpr int kFirstEpiWarp = 4, kEpiWarps = 8;
 constexpr int kFirstProducerWarp = 12, kProducerWarps = 8;
 constexpr int kRowsPerThread = kRows / 32;  // operand rows per producer thread
@@ -294,15 +294,23 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t b0 = smem_base + s * C::kStageBytes + C::kOffB;
             const uint64_t ahi = desc_swz(a0, 2u, 1024u), alo = desc_swz(a0 + C::kABytes, 2u, 1024u);
             const uint64_t bhi = desc_swz(b0, 2u, 1024u), blo = desc_swz(b0 + C::kBBytes, 2u, 1024u);
+            // split: the small products first.  Every MMA step truncates its
+            // sum at the accumulator's magnitude; on a fresh accumulator the
+            // 2 kKS/16 small steps then lose next to nothing, and only the
+            // kKS/16 large ones count
+            if (SPLIT) {
 #pragma unroll
-            for (int k = 0; k < kKS / 16; ++k) {
-              const uint32_t acc = (fresh && k == 0) ? 0u : 1u;
-              const uint64_t dk = (uint64_t)(2 * k);
-              mma_f16_pair(acc_addr, ahi + dk, bhi + dk, C::kIdesc, acc);
-              if (SPLIT) {
-                mma_f16_pair(acc_addr, ahi + dk, blo + dk, C::kIdesc, 1u);
+              for (int k = 0; k < kKS / 16; ++k) {
+                const uint64_t dk = (uint64_t)(2 * k);
+                mma_f16_pair(acc_addr, ahi + dk, blo + dk, C::kIdesc, fresh && k == 0 ? 0u : 1u);
                 mma_f16_pair(acc_addr, alo + dk, bhi + dk, C::kIdesc, 1u);
               }
+            }
+#pragma unroll
+            for (int k = 0; k < kKS / 16; ++k) {
+              const uint64_t dk = (uint64_t)(2 * k);
+              mma_f16_pair(acc_addr, ahi + dk, bhi + dk, C::kIdesc,
+                           !SPLIT && fresh && k == 0 ? 0u : 1u);
             }
             mma_commit_pair(&empty[s]);
             if (st + 1 == itm.nst || (st + 1) % CS == 0) {
@@ -316,8 +324,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_wait(mmadone, 0, abort_flag, scal, kRoleMma, /*honour_abort=*/false);
       }
       __syncwarp();
-    } else if (warp == kWarpLoader) {
+    } else if (warp == kWarpLoader || (SPARSE && warp == kWarpLoader2)) {
       // ------------------------------------------------------- point loader
+      // Block-sparse: two warps take the stages in turn.  A stage there is a
+      // chain of dependent reads (bin starts, then points), about as long as
+      // the stage's MMAs, and one warp would set the pace of the contraction
+      // (20M x 4096^2, 256-point chunks: 9.4 ms per density with one, 8.2 with
+      // two).
+      const uint32_t mine = warp == kWarpLoader ? 0u : 1u;
       uint32_t g = 0;
       bool ok = true;
       for (int rd = 0, it = item_at(0); ok && it >= 0; it = item_at(++rd)) {
@@ -332,6 +346,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           cur.init(I.start, I.bin_begin, I.nbx,
                    tile_bins(I.cs, I.range_reach, I.inv_binw, I.nbx, I.nby, itm.tm, itm.tn));
         for (int st = 0; ok && st < itm.nst; st += kGroup) {
+          if (SPARSE && (g & 1u) != mine) {  // the other loader's stage
+            ++g;
+            continue;
+          }
           const int ng = min(kGroup, itm.nst - st);
           float4 P[kGroup][2];
           float W[kGroup][2];
@@ -442,17 +460,26 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!(ok = mbar_wait(&accfull[b], (dc >> 1) & 1u, abort_flag, scal, kRoleEpilogue))) break;
         tc_fence_after();
         const uint32_t acc_col = tmem_base + b * 256u + lane_off + colh * 128;
+        // Block-sparse chunks are one stage long, so the drain has to keep up
+        // with the MMAs: 32 columns per wait and packed adds (20M x 4096^2:
+        // 8.82 ms per density, 9.52 with 8 columns and scalar adds).  Dense
+        // chunks leave time enough, and the narrow drain spills nothing there.
+        constexpr int kDrain = SPARSE ? 32 : 8;
 #pragma unroll
-        for (int cb = 0; cb < 16; ++cb) {
-          uint32_t ra[8];
-          tmem_ld8_async(acc_col + cb * 8, ra);
+        for (int cb = 0; cb < 128 / kDrain; ++cb) {
+          uint32_t ra[kDrain];
+          tmem_ld_async(acc_col + cb * kDrain, ra);
           tmem_wait_ld();
           if (ch == 0) {
 #pragma unroll
-            for (int c = 0; c < 8; ++c) run[cb * 8 + c] = __uint_as_float(ra[c]);
+            for (int c = 0; c < kDrain; ++c) run[cb * kDrain + c] = __uint_as_float(ra[c]);
+          } else if (SPARSE) {
+#pragma unroll
+            for (int c = 0; c < kDrain; c += 2)
+              add2_rn(run[cb * kDrain + c], run[cb * kDrain + c + 1], ra[c], ra[c + 1]);
           } else {
 #pragma unroll
-            for (int c = 0; c < 8; ++c) run[cb * 8 + c] += __uint_as_float(ra[c]);
+            for (int c = 0; c < kDrain; ++c) run[cb * kDrain + c] += __uint_as_float(ra[c]);
           }
         }
         // the accumulator is read: the MMAs of chunk dc + 2 may overwrite it
