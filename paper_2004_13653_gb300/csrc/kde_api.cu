@@ -1545,15 +1545,13 @@ int kde_dp_simplify(const double* points, const int64_t* traj_offsets, int64_t n
   CallScalars* scal = static_cast<CallScalars*>(wsv);
   KDE_CUDA(cudaMemsetAsync(scal, 0, sizeof(CallScalars), s), "clear scalars");
   int64_t kept = 0;
-  int its = 0;
+  int its = 0, err = 0;
   KDE_CUDA(launch_dp(points, n, traj_offsets, ntraj, eps, keep, out_points, out_offsets,
-                     static_cast<char*>(wsv) + align256(sizeof(CallScalars)), scal, &kept, &its, s),
+                     static_cast<char*>(wsv) + align256(sizeof(CallScalars)), scal, &kept, &its,
+                     &err, s),
            "Douglas-Peucker");
-  CallScalars hs;
-  KDE_CUDA(cudaMemcpyAsync(&hs, scal, sizeof(hs), cudaMemcpyDeviceToHost, s), "read status");
-  KDE_CUDA(cudaStreamSynchronize(s), "synchronize");
-  if (hs.err & kErrNonFinite) return fail(KDE_EDATA, "non-finite coordinate");
-  if (hs.err & kErrBadArg) return fail(KDE_EINVAL, "traj_offsets must rise from 0 to n");
+  if (err & kErrNonFinite) return fail(KDE_EDATA, "non-finite coordinate");
+  if (err & kErrBadArg) return fail(KDE_EINVAL, "traj_offsets must rise from 0 to n");
   if (n_kept) *n_kept = kept;
   if (iterations) *iterations = its;
   g_err[0] = 0;

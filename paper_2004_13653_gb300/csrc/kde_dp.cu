@@ -28,12 +28,17 @@
 // cooperative launch: the three steps are phases of a persistent kernel
 // separated by grid-wide barriers, and the count of points kept in an
 // iteration is read on the device, so no level costs a host round trip.
+// Trajectories that fit in shared memory (the usual case) skip all of that:
+// k_dp_local gives each a CTA, which runs the same levels on it alone (see the
+// kernel).
 // The VED is evaluated with
 // explicitly rounded FP64 operations in the order of Eq. 9, so every
 // comparison -- and therefore the kept set -- is identical to a sequential
-// FP64 evaluation.  The kept points are then compacted with the Sec. IV-A
-// exclusive scan.
+// FP64 evaluation.  The kept points are then compacted: counts per block of
+// points, the Sec. IV-A exclusive scan over the blocks, and each point's place
+// in its block from ballots.
 #include <cooperative_groups.h>
+#include <float.h>
 
 #include "kde_internal.cuh"
 
@@ -81,12 +86,64 @@ __device__ __forceinline__ void traj_bounds(const int64_t* __restrict__ off, int
   b = min(max(off[lo + 1], a), n);
 }
 
+// What the planning kernel decides; lives in the workspace, zeroed per call.
+struct DpCtl {
+  uint32_t n_local[2];  // trajectories on the work lists of k_dp_local: short, long ones
+  uint32_t next[2];     // the next of them to take
+  uint32_t n_long;      // trajectories left to the level kernel
+  uint32_t irregular;   // the offsets do not rise: every point goes to the level kernel
+};
+
+// One thread per trajectory: those of 3..short_max points go on the first work
+// list (two points or fewer have nothing to split), those of up to local_max
+// on the second, filled from its end; longer ones are counted.  Trajectories
+// of one or two points are finished here.
+__global__ void k_dp_plan(const double2* __restrict__ xy, const int64_t* __restrict__ off,
+                          int64_t ntraj, int64_t n, uint8_t* __restrict__ flag,
+                          CallScalars* __restrict__ scal, int short_max, int local_max, DpCtl* __restrict__ ctl,
+                          uint32_t* __restrict__ list,
+                          uint32_t list_cap, int* __restrict__ iterations) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k == 0) atomicMax(iterations, 1);
+  int64_t a = 0, b = 0;
+  if (k < ntraj) {
+    a = off ? off[k] : 0;
+    b = off ? off[k + 1] : n;
+    if (a < 0 || b < a || b > n || (k == 0 && a != 0) || (k == ntraj - 1 && b != n))
+      atomicOr(&ctl->irregular, 1u);
+  }
+  const int64_t len = b - a;
+  if ((len == 1 || len == 2) && a >= 0 && b <= n)
+    for (int64_t p = a; p < b; ++p) {
+      const double2 q = xy[p];
+      flag[p] = kKept;
+      if (!(isfinite(q.x) && isfinite(q.y))) atomicOr(&scal->err, kErrNonFinite);
+    }
+  if (len > local_max) atomicAdd(&ctl->n_long, 1u);
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const bool mine = len >= 3 && len <= local_max && (len > short_max) == (c == 1);
+    const unsigned m = __ballot_sync(0xffffffffu, mine);
+    uint32_t at = 0;
+    if (lane == 0 && m) at = atomicAdd(&ctl->n_local[c], (uint32_t)__popc(m));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+    if (mine && at < list_cap) list[c ? list_cap - 1 - at : at] = (uint32_t)k;
+  }
+}
+
+// The level kernel's per-point and per-segment state, for the points it will
+// process, and every point's flag; nothing to do when that kernel has no
+// trajectory (k_dp_plan and k_dp_local then cover every point).
 __global__ void k_dp_init(const double2* __restrict__ xy, int64_t n,
                           const int64_t* __restrict__ off, int64_t ntraj, int32_t* __restrict__ s,
                           int32_t* __restrict__ e, uint8_t* __restrict__ flag,
                           unsigned long long* __restrict__ segmax, uint32_t* __restrict__ segarg,
-                          double* __restrict__ seglen, CallScalars* __restrict__ scal) {
+                          double* __restrict__ seglen, int local_max,
+                          const DpCtl* __restrict__ ctl, CallScalars* __restrict__ scal) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const bool all = __ldg(&ctl->irregular) != 0u;
+  if (!all && __ldg(&ctl->n_long) == 0u) return;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += stride) {
     int64_t a, b;
     traj_bounds(off, ntraj, n, p, a, b);
@@ -97,18 +154,317 @@ __global__ void k_dp_init(const double2* __restrict__ xy, int64_t n,
       a = p;
       b = p + 1;
     }
+    flag[p] = (p == a || p == b - 1 || bad) ? kKept : 0;
+    if (bad) atomicOr(&scal->err, kErrNonFinite);
+    if (!all && b - a <= local_max) continue;
     s[p] = (int32_t)a;
     e[p] = (int32_t)(b - 1);
-    flag[p] = (p == a || p == b - 1 || bad) ? kKept : 0;
     if (p == a) seglen[p] = seg_len(q, xy[b - 1]);
     segmax[p] = 0ull;
     segmax[n + p] = 0ull;
     segarg[p] = kNoArg;
     segarg[n + p] = kNoArg;
-    if (bad) atomicOr(&scal->err, kErrNonFinite);
   }
   if (off && blockIdx.x == 0 && threadIdx.x == 0 && (off[0] != 0 || off[ntraj] != n))
     atomicOr(&scal->err, kErrBadArg);
+}
+
+// ------------------------------------------- whole trajectories in one CTA
+//
+// A trajectory in shared memory: its segments are worked off level by level,
+// each by one warp (no grid-wide barriers, and a trajectory that is finished
+// costs nothing while others go on); short trajectories have a CTA of one
+// warp, so not even CTA-wide ones.  GB300 does 2
+// FP64 operations per SM and clock, so the cross product of every open point
+// at every level would still take most of the time; it is bracketed in FP32
+// instead.  On coordinates relative to the trajectory's first point, as sums
+// of two FP32 numbers (within u^2 R of the exact ones, |x| <= R, u = 2^-24),
+// each difference is within 2 u |v| + 6 u^2 R of the exact one, and
+// c = |vx dy - vy dx| within
+//   E = 6 u (|vx dy| + |vy dx|) + 6 u^2 R (|vx| + |vy| + |dx| + |dy|) + 36 u^4 R^2
+// of the FP64 evaluation (whose own roundings are far smaller); a third is
+// added for the rounding of E itself and 1e-37 for underflow.  Only the points
+// whose upper bound c + E reaches the segment's largest lower bound
+// c - E, and eps times a lower bound of the segment's length, can be the split
+// or tie with it.  Where that leaves one point and its lower bound exceeds eps
+// times an upper bound of the length, it is the split; otherwise (about one
+// segment in a hundred) the points left are evaluated in FP64, from the
+// original coordinates and by the same steps as in the level kernel.  Either
+// way the split is the one that kernel finds.
+//
+// Segments of at most kSmall points leave the levels: one thread finishes each
+// (dp_finish), a warp's 32 at a time.
+// Bound by instruction issue (per point and level about 50 instructions).
+// 4000 tracks of 500 fixes at 10 m: 3.51 ms in the level kernel; here 2.08 ms
+// with FP64 for every point left by the brackets, 0.38 ms with FP64 for the
+// undecided segments only but a thread per point and CTA-wide phases, 0.20 ms
+// with a warp per segment.
+__device__ __forceinline__ float sqrt_approx(float v) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+constexpr int kSmall = 16;       // interior points of a segment that one thread finishes
+constexpr int kLocalMax = 9728;  // points of a trajectory: 21.5 bytes each, 209 KB
+// Shared memory for trajectories of up to m points (m a multiple of 128): the
+// coordinates, two lists of at most m / 16 longer segments (each has more than
+// kSmall interior points of its own), one of at most m / 2 small ones, the
+// points' levels and states.
+constexpr size_t dp_local_smem(int m) { return (size_t)m * 21 + (size_t)m / 2; }
+
+// The FP32 bracket of a point's cross product with its segment, and of the
+// segment's length.
+struct DpBracket {
+  float lo, hi;          // of c; lo = 0, hi = inf: to be evaluated in FP64
+  float len_lo, len_hi;
+};
+// v0, A, B: (x hi, y hi, x lo, y lo); uR = 8 u^2 R
+__device__ __forceinline__ DpBracket dp_bracket(float4 v0, float4 A, float4 B, float uR,
+                                                float tiny) {
+  constexpr float u = 0x1p-24f;
+  const float vx = (v0.x - A.x) + (v0.z - A.z), vy = (v0.y - A.y) + (v0.w - A.w);
+  const float dx = (B.x - A.x) + (B.z - A.z), dy = (B.y - A.y) + (B.w - A.w);
+  const float t0 = vx * dy, t1 = vy * dx;
+  const float c = fabsf(t0 - t1);
+  const float E = fmaf(uR, (fabsf(vx) + fabsf(vy)) + (fabsf(dx) + fabsf(dy)),
+                       fmaf(8.f * u, fabsf(t0) + fabsf(t1), tiny));
+  DpBracket r;
+  const float len = sqrt_approx(fmaf(dx, dx, dy * dy));
+  r.len_lo = fmaf(len, 1.f - 1e-6f, -6.f * uR);
+  r.len_hi = fmaf(len, 1.f + 1e-6f, fmaf(6.f, uR, 1e-18f));
+  r.hi = (c + E) * (1.f + 1e-6f);
+  // a segment that may have zero length is measured by distances, not by cross
+  // products: all its points are evaluated, as where the bounds overflow
+  const bool exact = !(r.len_lo > 0.f) || !(r.hi < FLT_MAX);
+  r.lo = exact || !(c > E) ? 0.f : (c - E) * (1.f - 1e-6f);
+  if (exact) r.hi = INFINITY;  // below no bound, an overflown one included
+  return r;
+}
+
+// The split of segment (s, e) by FP64 alone, by one thread; -1: nothing above
+// eps.
+__device__ __noinline__ int dp_split_exact(const double2* __restrict__ P, int s, int e,
+                                           double eps) {
+  const double2 A = P[s], B = P[e];
+  const double len = seg_len(A, B);
+  double cmax = 0.0;
+  for (int i = s + 1; i < e; ++i) {
+    const double c = ved_num(P[i], A, B, len);
+    if (c > cmax) cmax = c;
+  }
+  const double dmax = cmax == 0.0 ? 0.0 : ved_of(cmax, len);
+  if (!(dmax > eps)) return -1;
+  for (int i = s + 1; i < e; ++i) {
+    const double c = ved_num(P[i], A, B, len);
+    if (c >= __dmul_rn(cmax, 1.0 - 1e-15) && (c == cmax || ved_of(c, len) == dmax)) return i;
+  }
+  return -1;
+}
+
+// Finishes the segment (s0, e0) by one thread: from left to right, splitting
+// the leftmost open segment until nothing in it is above eps.  lvl[k] is one
+// more than the level at which point k was kept; a segment's level is the
+// larger one of its ends'.  Returns the largest level + 2 of a split (what the
+// level loop would have counted).
+__device__ __forceinline__ int dp_finish(const double2* __restrict__ P,
+                                         const float4* __restrict__ q, uint8_t* st, uint16_t* lvl,
+                                         int s0, int e0, float uR, float tiny, float eps_lo,
+                                         float eps_hi, double eps) {
+  int s = s0, e = e0, most = 0;
+  while (s < e0) {
+    const float4 A = q[s], B = q[e];
+    float best_lo = 0.f, top = -1.f, second = -1.f, len_lo = 0.f, len_hi = 0.f;
+    int at = -1;
+    for (int i = s + 1; i < e; ++i) {
+      const DpBracket b = dp_bracket(q[i], A, B, uR, tiny);
+      best_lo = fmaxf(best_lo, b.lo);
+      if (b.hi > top) {
+        second = top;
+        top = b.hi;
+        at = i;
+      } else {
+        second = fmaxf(second, b.hi);
+      }
+      len_lo = b.len_lo;
+      len_hi = b.len_hi;
+    }
+    int k = -1;
+    if (at >= 0 && !(top < eps_lo * len_lo))
+      k = second < best_lo && best_lo > eps_hi * len_hi ? at : dp_split_exact(P, s, e, eps);
+    if (k >= 0) {
+      const int level = max((int)lvl[s], (int)lvl[e]);
+      st[k] = kKept;
+      lvl[k] = (uint16_t)(level + 1);
+      most = max(most, level + 2);
+      e = k;
+    } else {
+      for (int i = s + 1; i < e; ++i) st[i] = kDone;
+      s = e;
+      if (s < e0) {
+        ++e;
+        while (e < e0 && st[e] != kKept) ++e;
+      }
+    }
+  }
+  return most;
+}
+
+// The split of segment (s, e) by one warp, every lane alike; -1: nothing in it
+// is above eps.
+__device__ __forceinline__ int dp_split_warp(const double2* __restrict__ P,
+                                             const float4* __restrict__ q, int s, int e, float uR,
+                                             float tiny, float eps_lo, float eps_hi, double eps) {
+  const int lane = threadIdx.x & 31;
+  const float4 A = q[s], B = q[e];
+  float best_lo = 0.f, top = 0.f, second = 0.f;
+  int at = -1;
+  DpBracket b = dp_bracket(A, A, B, uR, tiny);  // the length's bounds
+  for (int i = s + 1 + lane; i < e; i += 32) {
+    const DpBracket c = dp_bracket(q[i], A, B, uR, tiny);
+    best_lo = fmaxf(best_lo, c.lo);
+    if (c.hi > top) {
+      second = top;
+      top = c.hi;
+      at = i;
+    } else {
+      second = fmaxf(second, c.hi);
+    }
+  }
+  const float low = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(best_lo)));
+  const float high = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(top)));
+  if (high < eps_lo * b.len_lo) return -1;
+  // the points whose upper bound reaches the largest lower bound
+  const unsigned one = __ballot_sync(0xffffffffu, at >= 0 && top >= low);
+  const unsigned more = __ballot_sync(0xffffffffu, at >= 0 && second >= low && second > 0.f);
+  if (!more && __popc(one) == 1 && low > eps_hi * b.len_hi)
+    return __shfl_sync(0xffffffffu, at, __ffs(one) - 1);
+  // undecided: those points in FP64 (every point of a segment whose bounds say
+  // nothing: low is 0 there)
+  const double2 Ad = P[s], Bd = P[e];
+  const double len = seg_len(Ad, Bd);
+  double cmax = 0.0;
+  for (int i = s + 1 + lane; i < e; i += 32)
+    if (dp_bracket(q[i], A, B, uR, tiny).hi >= low) {
+      const double c = ved_num(P[i], Ad, Bd, len);
+      if (c > cmax) cmax = c;
+    }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double c = __shfl_xor_sync(0xffffffffu, cmax, o);
+    if (c > cmax) cmax = c;
+  }
+  const double dmax = cmax == 0.0 ? 0.0 : ved_of(cmax, len);
+  if (!(dmax > eps)) return -1;
+  uint32_t first = kNoArg;
+  for (int i = s + 1 + lane; i < e; i += 32)
+    if (first == kNoArg && dp_bracket(q[i], A, B, uR, tiny).hi >= low) {
+      const double c = ved_num(P[i], Ad, Bd, len);
+      if (c >= __dmul_rn(cmax, 1.0 - 1e-15) && (c == cmax || ved_of(c, len) == dmax))
+        first = (uint32_t)i;
+    }
+  return (int)__reduce_min_sync(0xffffffffu, first);  // kNoArg = -1
+}
+
+// list: the trajectories of class cls (0: from the list's start, 1: from its
+// end), each of at most m points.
+__global__ void __launch_bounds__(512)
+    k_dp_local(const double2* __restrict__ xy, const int64_t* __restrict__ off, int64_t n,
+               double eps, int m, int cls, DpCtl* __restrict__ ctl,
+               const uint32_t* __restrict__ list, uint32_t list_cap, uint8_t* __restrict__ flag,
+               CallScalars* __restrict__ scal, int* __restrict__ iterations) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  float4* q = reinterpret_cast<float4*>(smem);
+  uint32_t* longs = reinterpret_cast<uint32_t*>(q + m);  // [2][m / 16]: start | end << 16
+  uint32_t* small = longs + 2 * (m / 16);                // [m / 2]
+  uint16_t* lvl = reinterpret_cast<uint16_t*>(small + m / 2);  // kept points: level + 1
+  uint8_t* st = reinterpret_cast<uint8_t*>(lvl + m);
+  __shared__ uint32_t s_item, s_r, s_small, s_count[2];
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const int warp = tid >> 5, warps = nt >> 5;
+  if (__ldg(&ctl->irregular)) return;
+  const uint32_t n_local = __ldg(&ctl->n_local[cls]);
+  constexpr float u = 0x1p-24f;
+  const float eps_lo = (float)(eps * (1.0 - 1e-6)), eps_hi = (float)(eps * (1.0 + 1e-6));
+  int most = 1;
+  bool worked = false;
+  auto list_segment = [&](int s, int e, uint32_t* next, uint32_t* n_next) {
+    const uint32_t w = (uint32_t)s | ((uint32_t)e << 16);
+    if (e - s < 2) return;
+    if (e - s - 1 <= kSmall) small[atomicAdd(&s_small, 1u)] = w;
+    else next[atomicAdd(n_next, 1u)] = w;
+  };
+  for (;;) {
+    __syncthreads();  // the previous trajectory's state is no longer read
+    if (tid == 0) {
+      s_item = atomicAdd(&ctl->next[cls], 1u);
+      s_r = s_small = s_count[0] = s_count[1] = 0u;
+    }
+    __syncthreads();
+    const uint32_t item = s_item;
+    if (item >= n_local) break;
+    worked = true;
+    const uint32_t k = list[cls ? list_cap - 1 - item : item];
+    const int64_t a = off ? off[k] : 0;
+    const int len = (int)((off ? off[k + 1] : n) - a);
+    const double2* P = xy + a;
+    const double2 o = P[0];
+    float r = 0.f;
+    bool bad = false;
+    for (int i = tid; i < len; i += nt) {
+      const double2 p = P[i];
+      const float2 x = split_bits(p.x - o.x), y = split_bits(p.y - o.y);
+      // an infinite or undefined coordinate: the high word's exponent is full
+      bad |= ((unsigned)__double2hiint(p.x) & 0x7ff00000u) == 0x7ff00000u ||
+             ((unsigned)__double2hiint(p.y) & 0x7ff00000u) == 0x7ff00000u;
+      q[i] = make_float4(x.x, y.x, x.y, y.y);
+      r = fmaxf(r, fmaxf(fabsf(x.x), fabsf(y.x)));
+      st[i] = i == 0 || i == len - 1 ? kKept : 0;
+      lvl[i] = 0;
+    }
+    if (tid == 0) list_segment(0, len - 1, longs, &s_count[0]);
+    if (bad) atomicOr(&scal->err, kErrNonFinite);
+    const uint32_t rb = __reduce_max_sync(0xffffffffu, __float_as_uint(r));
+    if (lane == 0) atomicMax(&s_r, rb);
+    __syncthreads();
+    // (hi is cut, not rounded: 2^-23 above it, inside the margins)
+    const float R = __uint_as_float(s_r);
+    const float uR = 8.f * u * u * R, tiny = fmaf(uR, uR, 1e-37f);
+    for (int it = 0; it < len; ++it) {
+      const uint32_t count = s_count[it & 1];
+      if (!count) break;
+      const uint32_t* cur = longs + (it & 1) * (m / 16);
+      uint32_t* next = longs + ((it & 1) ^ 1) * (m / 16);
+      for (uint32_t j = warp; j < count; j += warps) {
+        const int s = (int)(cur[j] & 0xffffu), e = (int)(cur[j] >> 16);
+        const int at = dp_split_warp(P, q, s, e, uR, tiny, eps_lo, eps_hi, eps);
+        if (at < 0) {
+          for (int i = s + 1 + lane; i < e; i += 32) st[i] = kDone;
+        } else {
+          most = max(most, it + 2);
+          if (lane == 0) {
+            st[at] = kKept;
+            lvl[at] = (uint16_t)(it + 1);
+            list_segment(s, at, next, &s_count[(it & 1) ^ 1]);
+            list_segment(at, e, next, &s_count[(it & 1) ^ 1]);
+          }
+        }
+      }
+      __syncthreads();
+      if (tid == 0) s_count[it & 1] = 0u;  // the list after next
+      __syncthreads();
+    }
+    const uint32_t ns = s_small;
+    for (uint32_t j = tid; j < ns; j += nt) {
+      const uint32_t w = small[j];
+      most = max(most, dp_finish(P, q, st, lvl, (int)(w & 0xffffu), (int)(w >> 16), uR, tiny,
+                                 eps_lo, eps_hi, eps));
+    }
+    __syncthreads();
+    for (int i = tid; i < len; i += nt) flag[a + i] = st[i];
+  }
+  if (worked) {
+    const int top = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0) atomicMax(iterations, top);
+  }
 }
 
 // Step 1.  Lanes of a warp hold consecutive points, so equal segment starts
@@ -216,7 +572,8 @@ __global__ void __launch_bounds__(256)
                 int32_t* __restrict__ e, uint8_t* __restrict__ flag, double* __restrict__ num,
                 double* __restrict__ seglen, unsigned long long* __restrict__ segmax,
                 uint32_t* __restrict__ segarg, unsigned long long* __restrict__ counter,
-                int* __restrict__ iterations) {
+                const DpCtl* __restrict__ ctl, int* __restrict__ iterations) {
+  if (ctl->n_long == 0u && ctl->irregular == 0u) return;  // the same in every CTA
   cg::grid_group grid = cg::this_grid();
   __shared__ unsigned long long kept;
   int64_t it = 0;
@@ -239,31 +596,78 @@ __global__ void __launch_bounds__(256)
       break;
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *iterations = (int)it;
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicMax(iterations, (int)it);
 }
 
-__global__ void k_dp_flags(const uint8_t* __restrict__ flag, int64_t n,
-                           uint32_t* __restrict__ kept32, uint8_t* __restrict__ keep) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p <= n; p += stride) {
-    const uint32_t k = p < n ? (flag[p] & kKept) : 0u;
-    kept32[p] = k;
+// Compaction, kCompact points per CTA.  First the mask and each CTA's count...
+constexpr int kCompactThreads = 256, kCompact = 2048;
+__global__ void __launch_bounds__(kCompactThreads)
+    k_dp_flags(const uint8_t* __restrict__ flag, int64_t n, uint8_t* __restrict__ keep,
+               uint32_t* __restrict__ counts) {
+  const int64_t base = (int64_t)blockIdx.x * kCompact;
+  int mine = 0;
+#pragma unroll
+  for (int r = 0; r < kCompact / kCompactThreads; ++r) {
+    const int64_t p = base + r * kCompactThreads + threadIdx.x;
+    const int k = p < n ? (flag[p] & kKept) : 0;
     if (p < n) keep[p] = (uint8_t)k;
+    mine += k;
+  }
+  __shared__ int total;
+  if (threadIdx.x == 0) total = 0;
+  __syncthreads();
+  mine = __reduce_add_sync(0xffffffffu, mine);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&total, mine);
+  __syncthreads();
+  // one more entry than CTAs, zero, so that the scan ends with the total
+  if (threadIdx.x == 0) {
+    counts[blockIdx.x] = (uint32_t)total;
+    if (blockIdx.x == gridDim.x - 1) counts[gridDim.x] = 0u;
   }
 }
 
-__global__ void k_dp_compact(const double2* __restrict__ xy, int64_t n,
-                             const uint32_t* __restrict__ kept32, const uint32_t* __restrict__ pos,
-                             double2* __restrict__ out, const int64_t* __restrict__ off,
-                             int64_t ntraj, int64_t* __restrict__ out_off) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += stride)
-    if (out && kept32[p]) out[pos[p]] = xy[p];
-  if (out_off)
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k <= ntraj; k += stride) {
-      const int64_t o = off ? min(max(off[k], (int64_t)0), n) : (k == 0 ? 0 : n);
-      out_off[k] = pos[o];
+// ... then, with the scan of the counts, each kept point to its place, and the
+// number of kept points before each point (pos, when the offsets are wanted).
+__global__ void __launch_bounds__(kCompactThreads)
+    k_dp_compact(const double2* __restrict__ xy, int64_t n, const uint8_t* __restrict__ keep,
+                 const uint32_t* __restrict__ first, double2* __restrict__ out,
+                 uint32_t* __restrict__ pos, int* __restrict__ total) {
+  __shared__ uint32_t warps[kCompactThreads / 32];
+  const int64_t base = (int64_t)blockIdx.x * kCompact;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *total = (int)first[gridDim.x];
+  if (!out && !pos) return;
+  uint32_t before = first[blockIdx.x];
+#pragma unroll
+  for (int r = 0; r < kCompact / kCompactThreads; ++r) {
+    const int64_t p = base + r * kCompactThreads + threadIdx.x;
+    const bool k = p < n && keep[p];
+    const unsigned m = __ballot_sync(0xffffffffu, k);
+    if (lane == 0) warps[warp] = __popc(m);
+    __syncthreads();
+    uint32_t mine = before, all = 0;
+    for (int w = 0; w < kCompactThreads / 32; ++w) {
+      if (w < warp) mine += warps[w];
+      all += warps[w];
     }
+    mine += __popc(m & ((1u << lane) - 1u));
+    if (p < n) {
+      if (pos) pos[p] = mine;
+      if (k && out) out[mine] = xy[p];
+    }
+    before += all;
+    __syncthreads();
+  }
+  if (pos && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) pos[n] = before;
+}
+
+__global__ void k_dp_offsets(const uint32_t* __restrict__ pos, const int64_t* __restrict__ off,
+                             int64_t ntraj, int64_t n, int64_t* __restrict__ out_off) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k <= ntraj; k += stride) {
+    const int64_t o = off ? min(max(off[k], (int64_t)0), n) : (k == 0 ? 0 : n);
+    out_off[k] = pos[o];
+  }
 }
 
 int grid_for(int64_t n) {
@@ -273,15 +677,23 @@ int grid_for(int64_t n) {
 
 }  // namespace
 
+namespace {
+
+// Blocks of the compaction and the words it needs.
+int64_t dp_blocks(int64_t n) { return std::max<int64_t>(1, (n + kCompact - 1) / kCompact); }
+
+}  // namespace
+
 size_t dp_workspace_bytes(int64_t n) {
-  const size_t m = (size_t)n + 1;
-  return 256 * 14 + m * (4 + 4 + 1 + 16 + 8 + 8 + 8 + 4 + 4) +
-         4 * (scan_temp_words((int64_t)m, 2048) + 64);
+  const size_t m = (size_t)n + 1, nb = (size_t)dp_blocks(n) + 1;
+  return 256 * 16 + m * (4 + 4 + 1 + 16 + 8 + 8 + 8 + 4) + sizeof(uint32_t) * (m / 3 + 1) +
+         sizeof(uint32_t) * 2 * nb + 4 * (scan_temp_words((int64_t)nb, 2048) + 64);
 }
 
 cudaError_t launch_dp(const double* xy, int64_t n, const int64_t* off, int64_t ntraj, double eps,
                       uint8_t* keep, double* out_xy, int64_t* out_off, void* ws,
-                      CallScalars* scal, int64_t* n_kept, int* iterations, cudaStream_t st) {
+                      CallScalars* scal, int64_t* n_kept, int* iterations, int* err_word,
+                      cudaStream_t st) {
   const size_t m = (size_t)n + 1;
   char* w = static_cast<char*>(ws);
   size_t o = 0;
@@ -293,25 +705,65 @@ cudaError_t launch_dp(const double* xy, int64_t n, const int64_t* off, int64_t n
   double* num = reinterpret_cast<double*>(take(8 * m));
   double* seglen = reinterpret_cast<double*>(take(8 * m));
   uint32_t* segarg = reinterpret_cast<uint32_t*>(take(8 * m));
-  uint32_t* kept32 = reinterpret_cast<uint32_t*>(take(4 * m));
   uint32_t* pos = reinterpret_cast<uint32_t*>(take(4 * m));
-  unsigned long long* counter = reinterpret_cast<unsigned long long*>(take(16));
-  int* iters_dev = reinterpret_cast<int*>(take(sizeof(int)));
-  uint32_t* scan_temp = reinterpret_cast<uint32_t*>(take(4 * (scan_temp_words((int64_t)m, 2048) + 64)));
+  const uint32_t list_cap = (uint32_t)(m / 3 + 1);
+  uint32_t* list = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * list_cap));
+  // counters, cleared together: points kept per iteration, the plan
+  unsigned long long* counter = reinterpret_cast<unsigned long long*>(take(16 + sizeof(DpCtl)));
+  DpCtl* ctl = reinterpret_cast<DpCtl*>(counter + 2);
+  const int64_t nb = dp_blocks(n);
+  uint32_t* counts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (nb + 1)));
+  uint32_t* first = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (nb + 1)));
+  uint32_t* scan_temp =
+      reinterpret_cast<uint32_t*>(take(4 * (scan_temp_words(nb + 1, 2048) + 64)));
   const double2* P = reinterpret_cast<const double2*>(xy);
-  const int g = grid_for(n);
+  int* iters_dev = &scal->pad[0];  // read back with the error word
   cudaError_t err = cudaSuccess;
-  int it = 0;
   if (n > 0) {
-    k_dp_init<<<g, 256, 0, st>>>(P, n, off, ntraj, s, e, flag, segmax, segarg, seglen, scal);
-    note_launches(1);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    if ((err = cudaMemsetAsync(counter, 0, 16, st)) != cudaSuccess) return err;
-    // all CTAs of the cooperative launch must be resident at once
+    if ((err = cudaMemsetAsync(counter, 0, 16 + sizeof(DpCtl), st)) != cudaSuccess) return err;
     int dev = 0, per_sm = 0, sms = 0;
     if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
     if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
       return err;
+    // Trajectories of up to a quarter above the mean, the bulk of a call's, run
+    // with the shared memory they need, so that many CTAs
+    // share an SM; longer ones get the most a CTA can have, and those beyond
+    // that go to the level kernel.
+    const int64_t mean = n / std::max<int64_t>(ntraj, 1);
+    int local_max = kLocalMax;
+    int short_max = (int)std::min<int64_t>(kLocalMax,
+                                           std::max<int64_t>(256, (5 * mean / 4 + 127) / 128 * 128));
+    if (ntraj > 0xffffffffll) local_max = short_max = 2;  // 32-bit list: none is local
+    k_dp_plan<<<(unsigned)((ntraj + 255) / 256), 256, 0, st>>>(
+        P, off, ntraj, n, flag, scal, short_max, local_max, ctl, list, list_cap, iters_dev);
+    k_dp_init<<<grid_for(n), 256, 0, st>>>(P, n, off, ntraj, s, e, flag, segmax, segarg, seglen,
+                                           local_max, ctl, scal);
+    note_launches(2);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    for (int cls = 0; cls < 2; ++cls) {
+      const int m = cls ? local_max : short_max;
+      // trajectories that can be on the list
+      const int64_t most = std::min<int64_t>(ntraj, n / (cls ? short_max + 1 : 3));
+      if (most < 1 || (cls && local_max <= short_max)) continue;
+      // two warps for the usual track of 500 points (0.34 ms per call on 4000 of
+      // them; 0.40 with one warp, 0.36 with four)
+      const int threads = 32 * std::min(16, std::max(1, m / 320));
+      const size_t smem = dp_local_smem(m);
+      if ((err = cudaFuncSetAttribute(k_dp_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)dp_local_smem(kLocalMax))) !=
+          cudaSuccess)
+        return err;
+      if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dp_local, threads,
+                                                               smem)) != cudaSuccess)
+        return err;
+      if (per_sm < 1) return cudaErrorLaunchOutOfResources;
+      const int gl = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * sms, most));
+      k_dp_local<<<gl, threads, smem, st>>>(P, off, n, eps, m, cls, ctl, list, list_cap, flag,
+                                            scal, iters_dev);
+      note_launches(1);
+      if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    }
+    // all CTAs of the cooperative launch must be resident at once
     if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dp_levels, 256, 0)) !=
         cudaSuccess)
       return err;
@@ -321,34 +773,33 @@ cudaError_t launch_dp(const double* xy, int64_t n, const int64_t* off, int64_t n
     const int gl = (int)std::min<int64_t>((int64_t)std::min(per_sm, 4) * sms, (n + 255) / 256);
     void* args[] = {(void*)&P, (void*)&n, (void*)&eps, (void*)&s, (void*)&e, (void*)&flag,
                     (void*)&num, (void*)&seglen, (void*)&segmax, (void*)&segarg,
-                    (void*)&counter, (void*)&iters_dev};
+                    (void*)&counter, (void*)&ctl, (void*)&iters_dev};
     err = cudaLaunchCooperativeKernel((const void*)k_dp_levels, dim3(gl), dim3(256), args, 0, st);
     note_launches(1);
     if (err != cudaSuccess) return err;
-    if ((err = cudaMemcpyAsync(&it, iters_dev, sizeof(int), cudaMemcpyDeviceToHost, st)) !=
-        cudaSuccess)
-      return err;
-    if ((err = cudaStreamSynchronize(st)) != cudaSuccess) return err;
   }
-  if (iterations) *iterations = it;
-  k_dp_flags<<<grid_for(n + 1), 256, 0, st>>>(flag, n, kept32, keep);
+  k_dp_flags<<<(unsigned)nb, kCompactThreads, 0, st>>>(flag, n, keep, counts);
   note_launches(1);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  if ((err = launch_exclusive_scan(kept32, pos, (int64_t)m, 2048, scan_temp, st)) != cudaSuccess)
+  if ((err = launch_exclusive_scan(counts, first, nb + 1, 2048, scan_temp, st)) != cudaSuccess)
     return err;
-  if (out_xy || out_off) {
-    k_dp_compact<<<grid_for(std::max<int64_t>(n, ntraj + 1)), 256, 0, st>>>(
-        P, n, kept32, pos, reinterpret_cast<double2*>(out_xy), off, ntraj, out_off);
+  k_dp_compact<<<(unsigned)nb, kCompactThreads, 0, st>>>(
+      P, n, keep, first, reinterpret_cast<double2*>(out_xy), out_off ? pos : nullptr,
+      &scal->pad[1]);
+  note_launches(1);
+  if (out_off) {
+    k_dp_offsets<<<grid_for(ntraj + 1), 256, 0, st>>>(pos, off, ntraj, n, out_off);
     note_launches(1);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
-  if (n_kept) {
-    uint32_t total = 0;
-    if ((err = cudaMemcpyAsync(&total, pos + n, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
-      return err;
-    if ((err = cudaStreamSynchronize(st)) != cudaSuccess) return err;
-    *n_kept = total;
-  }
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  // everything the host wants, in one copy and one wait
+  CallScalars hs;
+  if ((err = cudaMemcpyAsync(&hs, scal, sizeof(hs), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+    return err;
+  if ((err = cudaStreamSynchronize(st)) != cudaSuccess) return err;
+  if (n_kept) *n_kept = (uint32_t)hs.pad[1];
+  if (iterations) *iterations = hs.pad[0];
+  *err_word = hs.err;
   return cudaSuccess;
 }
 

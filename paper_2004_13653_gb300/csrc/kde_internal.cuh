@@ -34,8 +34,30 @@ struct CallScalars {
   unsigned wmax_bits; // bit pattern of max |w| (non-negative floats order as ints)
   int timeout_where;  // role id of the first wait that gave up
   int negw;           // nonzero when some weight is negative
-  int pad[60];        // keep the struct 256 bytes
+  int pad[60];        // keep the struct 256 bytes (pad[0], pad[1]: Douglas-Peucker's
+                      // iterations and kept points)
 };
+
+#ifdef __CUDACC__
+// v as hi + lo in FP32, within 2^-47 |v|: hi is v with its mantissa cut to 24
+// bits, lo the other 29, taken from the bits of v.  Rounding v to FP32,
+// widening and subtracting costs four FP64-rate conversions and adds, and
+// this GPU does 2 of those per SM and clock (0.016 of the FP32 rate); this is
+// integer and FP32 work but for numbers below 2^-74 or above 2^126.
+__device__ __forceinline__ float2 split_bits(double v) {
+  const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+  const unsigned e = (h >> 20) & 0x7ffu, sign = h & 0x80000000u;
+  if (e - 949u < 201u) {
+    // exponent 8 bits of the 11 and the top 23 mantissa bits; 896 = the
+    // difference of the biases flips the exponent's top bit
+    const unsigned hi = ((__funnelshift_l(l, h, 3) & 0x7fffffffu) ^ 0x40000000u) | sign;
+    const float scale = __uint_as_float(((e - 948u) << 23) | sign);  // 2^(e - 1075)
+    return make_float2(__uint_as_float(hi), (float)(l & 0x1fffffffu) * scale);
+  }
+  const float hi = __double2float_rn(v);
+  return make_float2(hi, __double2float_rn(v - (double)hi));
+}
+#endif
 
 // One factor k(s) of each Table 1 kernel without its constant; the constant
 // squared and 1/(N h^2) are applied once to the sum.
@@ -401,11 +423,13 @@ cudaError_t launch_binned(const double* xy, int64_t n, const int64_t* off, int64
                           unsigned long long* added, float* out, cudaStream_t s);
 
 // Douglas-Peucker compression of every trajectory (level-synchronous;
-// synchronous on `s`).  ws: dp_workspace_bytes(n) bytes.
+// synchronous on `s`; err_word: the error bits of scal).  ws:
+// dp_workspace_bytes(n) bytes; scal: zeroed.
 size_t dp_workspace_bytes(int64_t n);
 cudaError_t launch_dp(const double* xy, int64_t n, const int64_t* off, int64_t ntraj, double eps,
                       uint8_t* keep, double* out_xy, int64_t* out_off, void* ws,
-                      CallScalars* scal, int64_t* n_kept, int* iterations, cudaStream_t s);
+                      CallScalars* scal, int64_t* n_kept, int* iterations, int* err_word,
+                      cudaStream_t s);
 
 // Path (b): Gaussian as a tcgen05 contraction.
 struct TcPlan {
