@@ -1491,13 +1491,23 @@ int kde_grid_binned(const double* points, const int64_t* traj_offsets, int64_t n
     return fail(KDE_EINVAL, "misaligned offsets or counts");
   cudaStream_t s = stream_of(opts);
   const int64_t cells = (int64_t)nx * ny;
+  // the trajectories' end bits share the row buffer; where they would need more
+  // than that and the workspace does not have it, the call does without them
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t r = off; off = align256(off + bytes); return r; };
-  const size_t o_added = take(sizeof(unsigned long long));
+  const size_t o_added = take(2 * sizeof(unsigned long long));
   const size_t o_counts = take(counts_out ? 0 : sizeof(int) * (size_t)cells);
-  const size_t o_rows = take(sizeof(float) * (size_t)cells);
+  const size_t row_bytes = sizeof(float) * (size_t)cells;
+  const bool want_ends = traj_offsets && interpolate && n > 0;
+  const size_t end_bytes = want_ends ? binned_ends_bytes(n) : 0;
+  bool ends = want_ends;
+  const size_t o_rows = take(std::max(row_bytes, end_bytes));
   void* wsv = nullptr;
   rc = acquire_workspace(opts, off, s, &wsv);
+  if (rc == KDE_ENOMEM && end_bytes > row_bytes) {
+    ends = false;
+    rc = acquire_workspace(opts, align256(o_rows + row_bytes), s, &wsv);
+  }
   if (rc) return rc;
   char* base = static_cast<char*>(wsv);
   int* counts = counts_out ? reinterpret_cast<int*>(counts_out) : reinterpret_cast<int*>(base + o_counts);
@@ -1505,7 +1515,8 @@ int kde_grid_binned(const double* points, const int64_t* traj_offsets, int64_t n
   const int win = binned_window(kernel_id, h, cell, window);
   KDE_CUDA(launch_binned(points, n, traj_offsets, ntraj, grid_origin[0], grid_origin[1], cell, nx,
                          ny, h, kernel_id, win, interpolate, counts,
-                         reinterpret_cast<float*>(base + o_rows), added, out, s),
+                         reinterpret_cast<float*>(base + o_rows),
+                         ends ? reinterpret_cast<uint32_t*>(base + o_rows) : nullptr, added, out, s),
            "binned estimator");
   if (interpolated || (opts && (opts->flags & KDE_FLAG_SYNC))) {
     unsigned long long hv = 0;

@@ -4,19 +4,22 @@
 // interpolation (Eq. InterX / InterY), and M_D is convolved with a
 // window x window stencil of a Table 1 kernel (Eq. 7).
 //
-// Counting: one thread per fix; the cell index is floor((x - o) / cell) with
-// the FP64 division correctly rounded (a multiply by 1/cell decides it except
-// within rounding distance of a cell edge), and the interpolated cells are
-// floor(i + (c/c_max) di + 1/2) with c = 1..c_max-1, evaluated with
-// explicitly rounded FP64 operations (no fused multiply-add), so the counts
-// are bit-identical to a CPU evaluation.
+// Counting: the cell index is floor((x - o) / cell) with the FP64 division
+// correctly rounded, and the interpolated cells are
+// floor(i + (c/c_max) di + 1/2) with c = 1..c_max-1, evaluated with explicitly
+// rounded FP64 operations (no fused multiply-add), so the counts are
+// bit-identical to a CPU evaluation.  GB300 does 2 FP64 operations per SM and
+// clock, so both are decided in FP32 and integers wherever those cannot
+// differ from the FP64 evaluation, and in FP64 in the rest (one fix in a
+// million; interpolated cells that fall half way between two).
 // Integer atomics make the counts independent of scheduling.
 //
 // Convolution: the Table 1 kernels are products, so the 2-D stencil
 // f(s,t) = k(s cell/h) k(t cell/h) / (N h^2) is applied as a row pass and a
-// column pass; each pass stages a tile plus its halo in shared memory and
-// keeps the 1-D stencil in registers.
+// column pass, each thread computing several outputs per value it reads.
 #include <math.h>
+
+#include <algorithm>
 
 #include "kde_internal.cuh"
 
@@ -42,97 +45,274 @@ __device__ __forceinline__ int64_t cell_index(double v, double o, double d, doub
   return (int64_t)f;
 }
 
-__global__ void k_count(const double* __restrict__ xy, int64_t n,
-                        const int64_t* __restrict__ off, int64_t ntraj, double ox, double oy,
-                        double cell, double inv_cell, int nx, int ny, int interpolate,
-                        int* __restrict__ counts, unsigned long long* __restrict__ added) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  unsigned long long my_added = 0;
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += stride) {
-    const int64_t i = cell_index(xy[2 * p], ox, cell, inv_cell, nx);
-    const int64_t j = cell_index(xy[2 * p + 1], oy, cell, inv_cell, ny);
-    if (i < 0 || j < 0) continue;
-    atomicAdd(&counts[j * nx + i], 1);
-    if (!interpolate || p + 1 >= n) continue;
-    // the fix's trajectory: the last k with off[k] <= p
-    int64_t next_start = n;
-    if (off) {
-      int64_t lo = 0, hi = ntraj - 1;
-      while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (off[mid] <= p) lo = mid; else hi = mid - 1;
-      }
-      next_start = off[lo + 1];
+// The same index from FP32: t = v - o as hi + lo, an estimate of the quotient,
+// and the remainder r = t - i d, which one FMA gives to 2^-24 d (i d_hi is
+// exact in it and nearly cancels hi).  Where r is inside (0, d) by more than
+// the rounding of all of it, i is the floor of the exact quotient, which lies
+// far from an integer, so the correctly rounded one has the same floor.  Near a
+// cell edge (about 1e-6 of the fixes) and for quotients beyond 2^21 cell_index
+// decides.
+struct CellMap {
+  double o, d, inv_d;
+  float dh, dl, inv, margin;  // d = dh + dl, 1 / d, 2^-21 d
+  int n;
+};
+__device__ __forceinline__ int cell_of(double v, const CellMap& m) {
+  const double t = __dsub_rn(v, m.o);
+  const float2 s = split_bits(t);
+  const float est = floorf(s.x * m.inv);
+  const float r = fmaf(-est, m.dh, s.x) + fmaf(-est, m.dl, s.y);
+  if (fabsf(est) < 2097152.f) {
+    // the estimate is off by at most one
+    float i = est, q = r;
+    if (r < 0.f) {
+      i -= 1.f;
+      q += m.dh;
+    } else if (r >= m.dh) {
+      i += 1.f;
+      q -= m.dh;
     }
-    if (p + 1 >= next_start) continue;
-    const int64_t i1 = cell_index(xy[2 * p + 2], ox, cell, inv_cell, nx);
-    const int64_t j1 = cell_index(xy[2 * p + 3], oy, cell, inv_cell, ny);
-    if (i1 < 0 || j1 < 0) continue;
-    const int64_t di = i1 - i, dj = j1 - j;
-    const int64_t adi = di < 0 ? -di : di, adj = dj < 0 ? -dj : dj;
-    const int64_t cmax = adi > adj ? adi : adj;
-    for (int64_t c = 1; c < cmax; ++c) {
-      const double t = __ddiv_rn((double)c, (double)cmax);
-      const int64_t ic = (int64_t)floor(__dadd_rn(__dadd_rn((double)i, __dmul_rn(t, (double)di)), 0.5));
-      const int64_t jc = (int64_t)floor(__dadd_rn(__dadd_rn((double)j, __dmul_rn(t, (double)dj)), 0.5));
-      atomicAdd(&counts[jc * nx + ic], 1);
-      ++my_added;
-    }
+    if (q > m.margin && m.dh - q > m.margin) return i >= 0.f && i < (float)m.n ? (int)i : -1;
   }
-  if (my_added) atomicAdd(added, my_added);
+  return (int)cell_index(v, m.o, m.d, m.inv_d, m.n);
 }
 
+// Bits of the fixes that end a trajectory (their successor belongs to another
+// one), from the offsets; *irregular is set when the offsets do not rise, and
+// the counting then searches them per fix.
+__global__ void k_traj_ends(const int64_t* __restrict__ off, int64_t ntraj, int64_t n,
+                            uint32_t* __restrict__ ends, unsigned* __restrict__ irregular) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int64_t e = -1;
+  if (k < ntraj) {
+    e = off[k + 1];
+    if (e < off[k]) atomicOr(irregular, 1u);
+    --e;
+  }
+  const bool in = e >= 0 && e < n;
+  const uint32_t word = in ? (uint32_t)(e >> 5) : 0xffffffffu;
+  const uint32_t bit = in ? 1u << (e & 31) : 0u;
+  // neighbouring trajectories of a few fixes share words: one atomic per word
+  const unsigned peers = __match_any_sync(0xffffffffu, word);
+  const uint32_t bits = __reduce_or_sync(peers, bit);
+  if (in && (threadIdx.x & 31) == __ffs(peers) - 1) atomicOr(ends + word, bits);
+}
+
+// The cells skipped between the cells (i, j) and (i1, j1), added to the
+// counts; returns how many.  The coordinate that moves by c_max steps by one;
+// the other one is floor(j + c dj / c_max + 1/2), a remainder in integers
+// (Bresenham's).  The FP64 evaluation can differ only where that is an exact
+// integer (a tie) and c / c_max is not exact, or for moves so long or cells so
+// far that its rounding reaches 1 / (2 c_max); those are evaluated in FP64.
+__device__ __forceinline__ int fill_gap(int i, int j, int i1, int j1, int nx,
+                                        int* __restrict__ counts) {
+  const int64_t di = (int64_t)i1 - i, dj = (int64_t)j1 - j;
+  const int64_t adi = di < 0 ? -di : di, adj = dj < 0 ? -dj : dj;
+  const int64_t cmax = adi > adj ? adi : adj;
+  if (cmax < 2) return 0;
+  auto exact = [&](int64_t c, int from, int64_t d) {
+    const double t = __ddiv_rn((double)c, (double)cmax);
+    return (int64_t)floor(__dadd_rn(__dadd_rn((double)from, __dmul_rn(t, (double)d)), 0.5));
+  };
+  if (cmax >= 1 << 18) {
+    for (int64_t c = 1; c < cmax; ++c)
+      atomicAdd(&counts[exact(c, j, dj) * nx + exact(c, i, di)], 1);
+    return (int)(cmax - 1);
+  }
+  const int m = (int)cmax;
+  const bool pow2 = (m & (m - 1)) == 0;
+  const bool along_x = adi >= adj;  // equal: both step by one, whichever is taken
+  const int step = along_x ? (di < 0 ? -1 : 1) : (dj < 0 ? -1 : 1);
+  const int slope = 2 * (int)(along_x ? dj : di);
+  int major = along_x ? i : j, minor = along_x ? j : i, rem = m;
+  const int minor0 = minor;
+  for (int c = 1; c < m; ++c) {
+    major += step;
+    rem += slope;
+    if (rem >= 2 * m) {
+      ++minor;
+      rem -= 2 * m;
+    } else if (rem < 0) {
+      --minor;
+      rem += 2 * m;
+    }
+    const int at = rem == 0 && !pow2 ? (int)exact(c, minor0, slope / 2) : minor;
+    const int64_t cell = along_x ? (int64_t)at * nx + major : (int64_t)major * nx + at;
+    atomicAdd(&counts[cell], 1);
+  }
+  return m - 1;
+}
+
+// A warp takes kCountRounds x 32 consecutive fixes; each fix's cell is found
+// once, the cell before it comes from the neighbouring lane (lane 0: from the
+// last round).  ends: bits of the fixes that end a trajectory; null (no
+// scratch for them) or *irregular set: the offsets are searched per fix.
+// Bound by the L2 atomics (one per fix and interpolated cell).  20M fixes x
+// 4096^2, interpolated: 4.21 ms with every index and cell in FP64, the
+// successor's cell found again and a search of the offsets per fix; 0.33 now.
+constexpr int kCountRounds = 16;
+__global__ void __launch_bounds__(256)
+    k_count(const double2* __restrict__ xy, int64_t n, const int64_t* __restrict__ off,
+            int64_t ntraj, const uint32_t* __restrict__ ends,
+            const unsigned* __restrict__ irregular, const __grid_constant__ CellMap mx,
+            const __grid_constant__ CellMap my, int interpolate, int* __restrict__ counts,
+            unsigned long long* __restrict__ added) {
+  const int lane = threadIdx.x & 31, nx = mx.n;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const bool search = off && (!ends || *irregular);
+  const int64_t last_end = off ? off[ntraj] : n;  // no fix from here on has a successor
+  int my_added = 0;
+  unsigned long long total = 0;
+  for (int64_t b = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32 * kCountRounds;
+       b < n; b += warps * 32 * kCountRounds) {
+    double2 v = b + lane < n ? xy[b + lane] : make_double2(0.0, 0.0);
+    int last_i = -1, last_j = -1;  // cell of the fix before this round's first
+    if (interpolate && b > 0 && lane == 31) {
+      const double2 w = xy[b - 1];
+      last_i = cell_of(w.x, mx);
+      last_j = cell_of(w.y, my);
+    }
+    uint32_t last_ends = ends && interpolate && b > 0 ? ends[(b >> 5) - 1] : 0u;
+    for (int r = 0; r < kCountRounds; ++r) {
+      const int64_t p = b + r * 32 + lane;
+      if (b + r * 32 >= n) break;
+      const double2 now = v;
+      if (r + 1 < kCountRounds && p + 32 < n) v = xy[p + 32];
+      int i = -1, j = -1;
+      if (p < n) {
+        i = cell_of(now.x, mx);
+        j = cell_of(now.y, my);
+        if (i >= 0 && j >= 0) atomicAdd(&counts[(int64_t)j * nx + i], 1);
+      }
+      if (!interpolate) continue;
+      int pi = __shfl_up_sync(0xffffffffu, i, 1), pj = __shfl_up_sync(0xffffffffu, j, 1);
+      const int ci = __shfl_sync(0xffffffffu, last_i, 31), cj = __shfl_sync(0xffffffffu, last_j, 31);
+      if (lane == 0) {
+        pi = ci;
+        pj = cj;
+      }
+      last_i = i;
+      last_j = j;
+      // does the fix before p end its trajectory?
+      bool next = p > 0 && p < n && pi >= 0 && pj >= 0 && i >= 0 && j >= 0;
+      if (off && !search) {
+        const uint32_t word = ends[(b >> 5) + r];
+        const uint32_t e = lane ? word >> (lane - 1) : last_ends >> 31;
+        last_ends = word;
+        next = next && !(e & 1u) && p < last_end;
+      } else if (search && next) {
+        int64_t lo = 0, hi = ntraj - 1;  // the last k with off[k] <= p - 1
+        while (lo < hi) {
+          const int64_t mid = (lo + hi + 1) >> 1;
+          if (off[mid] <= p - 1) lo = mid; else hi = mid - 1;
+        }
+        next = p < off[lo + 1];
+      }
+      if (next) my_added += fill_gap(pi, pj, i, j, nx, counts);
+    }
+    total += (unsigned)my_added;
+    my_added = 0;
+  }
+  for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+  if (lane == 0 && total) atomicAdd(added, total);
+}
+
+// The stencil by distance back from an output's last cell: k[u] multiplies the
+// value u cells after the first of its window; zeros up to a multiple of four.
 struct Stencil {
-  float k[2 * kMaxHalf + 1];
+  float k[2 * kMaxHalf + 2];
 };
 
-constexpr int kTile = 128;     // outputs per block of the row pass
-constexpr int kColTile = 64;   // rows per block of the column pass (static smem < 48 KB)
-
-// Row pass: R(i, j) = sum_s k_s M(i - s, j) (cells outside the grid are zero).
-// Rows are strided over gridDim.y (which is capped at 65535).
-__global__ void k_conv_rows(const int* __restrict__ counts, int nx, int ny, int a,
-                            const __grid_constant__ Stencil st, float* __restrict__ R) {
-  __shared__ float line[kTile + 2 * kMaxHalf];
-  const int i0 = blockIdx.x * kTile;
+// Row pass: R(i, j) = sum_u k_u M(i - a + u, j) (cells outside the grid are
+// zero), u falling.  A block takes kRowTile columns of one row; a thread four
+// neighbouring ones, so each 16-byte read of the staged line feeds 16 FMAs (one
+// output per thread read 4 bytes per FMA: 107 us on 4096^2 with 35 taps, 58
+// now).  Rows are strided over gridDim.y (which is capped at 65535).
+constexpr int kRowThreads = 128, kRowTile = 4 * kRowThreads;
+__global__ void __launch_bounds__(kRowThreads)
+    k_conv_rows(const int* __restrict__ counts, int nx, int ny, int a,
+                const __grid_constant__ Stencil st, float* __restrict__ R) {
+  __shared__ __align__(16) float line[kRowTile + 2 * kMaxHalf + 6];
+  const int i0 = blockIdx.x * kRowTile, t = threadIdx.x;
+  const int taps4 = (2 * a + 4) / 4;  // groups of four taps
+  const int width = min(kRowTile, nx - i0);
   for (int j = blockIdx.y; j < ny; j += gridDim.y) {
-    for (int t = threadIdx.x; t < kTile + 2 * a; t += blockDim.x) {
-      const int i = i0 - a + t;
-      line[t] = (i >= 0 && i < nx) ? (float)counts[(int64_t)j * nx + i] : 0.f;
+    const int* row = counts + (int64_t)j * nx;
+    for (int x = t; x < kRowTile + 4 * taps4 + 4; x += kRowThreads) {
+      const int i = i0 - a + x;
+      if (x < kRowTile + 2 * kMaxHalf + 6)
+        line[x] = (i >= 0 && i < nx && x < width + 2 * a) ? (float)row[i] : 0.f;
     }
     __syncthreads();
-    const int i = i0 + threadIdx.x;
-    if (threadIdx.x < kTile && i < nx) {
-      float acc = 0.f;
-      for (int s = -a; s <= a; ++s) acc = fmaf(st.k[s + a], line[threadIdx.x + a - s], acc);
-      R[(int64_t)j * nx + i] = acc;
+    if (4 * t < width) {
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      const float4* v4 = reinterpret_cast<const float4*>(line) + t;
+      float4 hi = v4[taps4];
+      for (int g = taps4 - 1; g >= 0; --g) {
+        const float4 lo = v4[g];
+        const float w[7] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z};
+#pragma unroll
+        for (int u = 3; u >= 0; --u) {
+          const float k = st.k[4 * g + u];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[c] = fmaf(k, w[c + u], acc[c]);
+        }
+        hi = lo;
+      }
+      float* out = R + (int64_t)j * nx + i0 + 4 * t;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (4 * t + c < width) out[c] = acc[c];
     }
     __syncthreads();
   }
 }
 
-// Column pass: out(i, j) = norm sum_t k_t R(i, j - t); block = 32 columns x
-// kColTile rows, each thread walks its column.
-__global__ void k_conv_cols(const float* __restrict__ R, int nx, int ny, int a,
-                            const __grid_constant__ Stencil st, float norm,
-                            float* __restrict__ out) {
-  __shared__ float col[kColTile + 2 * kMaxHalf][33];
-  const int i0 = blockIdx.x * 32, j0 = blockIdx.y * kColTile;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8 threads
-  for (int r = ty; r < kColTile + 2 * a; r += 8) {
-    const int j = j0 - a + r, i = i0 + tx;
-    col[r][tx] = (j >= 0 && j < ny && i < nx) ? R[(int64_t)j * nx + i] : 0.f;
-  }
+// Column pass: out(i, j) = norm sum_u k_u R(i, j - a + u), u falling.  A block
+// takes kColTile columns x kColRows rows; a thread four columns 32 apart and
+// eight consecutive rows, and walks the rows of their common window once from
+// its end: each value feeds eight FMAs, with coefficients that are zero outside
+// an output's window (added zeros change nothing).  The block's rows stay in
+// L1.  Staging 64 rows x 32 columns with one output per thread and step: 90 us
+// on 4096^2 with 35 taps, 65 now.
+constexpr int kColTile = 128, kColRows = 64;
+__global__ void __launch_bounds__(256)
+    k_conv_cols(const float* __restrict__ R, int nx, int ny, int a,
+                const __grid_constant__ Stencil st, float norm, float* __restrict__ out) {
+  // k with eight zeros on either side
+  __shared__ __align__(16) float kz[2 * kMaxHalf + 2 + 24];
+  for (int x = threadIdx.x; x < 2 * kMaxHalf + 26; x += 256)
+    kz[x] = x >= 8 && x - 8 <= 2 * a ? st.k[x - 8] : 0.f;
   __syncthreads();
-  const int i = i0 + tx;
-  if (i >= nx) return;
-  for (int r = ty; r < kColTile; r += 8) {
-    const int j = j0 + r;
-    if (j >= ny) break;
-    float acc = 0.f;
-    for (int t = -a; t <= a; ++t) acc = fmaf(st.k[t + a], col[r + a - t][tx], acc);
-    out[(int64_t)j * nx + i] = acc * norm;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int i0 = blockIdx.x * kColTile + tx, j0 = blockIdx.y * kColRows + 8 * ty;
+  if (i0 >= nx || j0 >= ny) return;
+  float acc[8][4];
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+  const int last = min(j0 + 7 + a, ny - 1), first = max(j0 - a, 0);
+#pragma unroll 2
+  for (int j = last; j >= first; --j) {
+    const float* row = R + (int64_t)j * nx + i0;
+    float v[4], k[8];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = i0 + 32 * c < nx ? __ldg(row + 32 * c) : 0.f;
+    // output row j0 + r takes tap u = j - (j0 + r) + a
+#pragma unroll
+    for (int r = 0; r < 8; ++r) k[r] = kz[8 + j - j0 - r + a];
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(k[r], v[c], acc[r][c]);
   }
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (j0 + r < ny && i0 + 32 * c < nx)
+        out[(int64_t)(j0 + r) * nx + i0 + 32 * c] = acc[r][c] * norm;
 }
 
 // One factor k(s) of a Table 1 kernel with its constant, in double (host side).
@@ -159,6 +339,8 @@ double table1_factor(int kid, double s) {
 
 }  // namespace
 
+size_t binned_ends_bytes(int64_t n) { return sizeof(uint32_t) * (size_t)((n + 31) / 32); }
+
 int binned_window(int kid, double h, double cell, int window) {
   if (window > 0) return window;
   const double r = h / cell;
@@ -169,28 +351,51 @@ int binned_window(int kid, double h, double cell, int window) {
 cudaError_t launch_binned(const double* xy, int64_t n, const int64_t* off, int64_t ntraj,
                           double ox, double oy, double cell, int nx, int ny, double h, int kid,
                           int window, int interpolate, int* counts, float* rowbuf,
-                          unsigned long long* added, float* out, cudaStream_t s) {
+                          uint32_t* ends, unsigned long long* added, float* out, cudaStream_t s) {
   const int a = (window - 1) / 2;
   if (window < 1 || (window & 1) == 0 || a > kMaxHalf) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(int) * (size_t)nx * ny, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(added, 0, sizeof(unsigned long long), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(added, 0, 2 * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
+  // added: the count, then the irregular flag
+  unsigned* irregular = reinterpret_cast<unsigned*>(added + 1);
   if (n > 0) {
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    k_count<<<(int)blocks, 256, 0, s>>>(xy, n, off, ntraj, ox, oy, cell, 1.0 / cell, nx, ny,
-                                        interpolate, counts, added);
+    if (interpolate && off && ends) {
+      if ((e = cudaMemsetAsync(ends, 0, binned_ends_bytes(n), s)) != cudaSuccess) return e;
+      k_traj_ends<<<(unsigned)((ntraj + 255) / 256), 256, 0, s>>>(off, ntraj, n, ends, irregular);
+      note_launches(1);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    auto map = [&](double o, int cells) {
+      CellMap m;
+      m.o = o;
+      m.d = cell;
+      m.inv_d = 1.0 / cell;
+      m.dh = (float)cell;
+      m.dl = (float)(cell - (double)m.dh);
+      m.inv = (float)m.inv_d;
+      m.margin = m.dh * 0x1p-21f;
+      // cells too small or too large for FP32 go to the FP64 index
+      if (!(cell > 1e-30 && cell < 1e30)) m.inv = INFINITY;
+      m.n = cells;
+      return m;
+    };
+    const int64_t per_block = 8 * 32 * kCountRounds;
+    const int64_t blocks = std::min<int64_t>((n + per_block - 1) / per_block, 152 * 8);
+    k_count<<<(int)blocks, 256, 0, s>>>(reinterpret_cast<const double2*>(xy), n, off, ntraj, ends,
+                                        irregular, map(ox, nx), map(oy, ny), interpolate, counts,
+                                        added);
     note_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  Stencil st;
-  for (int t = -a; t <= a; ++t) st.k[t + a] = (float)table1_factor(kid, t * cell / h);
+  Stencil st = {};
+  for (int u = 0; u <= 2 * a; ++u) st.k[u] = (float)table1_factor(kid, (a - u) * cell / h);
   const float norm = n > 0 ? (float)(1.0 / ((double)n * h * h)) : 0.0f;
-  k_conv_rows<<<dim3((nx + kTile - 1) / kTile, ny < 65535 ? ny : 65535), kTile, 0, s>>>(
+  k_conv_rows<<<dim3((nx + kRowTile - 1) / kRowTile, ny < 65535 ? ny : 65535), kRowThreads, 0, s>>>(
       counts, nx, ny, a, st, rowbuf);
   note_launches(1);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_conv_cols<<<dim3((nx + 31) / 32, (ny + kColTile - 1) / kColTile), 256, 0, s>>>(
+  k_conv_cols<<<dim3((nx + kColTile - 1) / kColTile, (ny + kColRows - 1) / kColRows), 256, 0, s>>>(
       rowbuf, nx, ny, a, st, norm, out);
   note_launches(1);
   return cudaGetLastError();

@@ -417,10 +417,14 @@ cudaError_t launch_sum(const double* v, int64_t n, double* partial, double* resu
 // The paper's binned estimator: count matrix with interpolation (Algorithm 3)
 // and the separable window x window convolution of Eq. 7.
 int binned_window(int kid, double h, double cell, int window);
+// added: two 64-bit words; ends: binned_ends_bytes(n) bytes of scratch for the
+// trajectories' ends, free again when the row pass writes rowbuf (so the two
+// may share memory), or null (the offsets are then searched per fix).
+size_t binned_ends_bytes(int64_t n);
 cudaError_t launch_binned(const double* xy, int64_t n, const int64_t* off, int64_t ntraj,
                           double ox, double oy, double cell, int nx, int ny, double h, int kid,
                           int window, int interpolate, int* counts, float* rowbuf,
-                          unsigned long long* added, float* out, cudaStream_t s);
+                          uint32_t* ends, unsigned long long* added, float* out, cudaStream_t s);
 
 // Douglas-Peucker compression of every trajectory (level-synchronous;
 // synchronous on `s`; err_word: the error bits of scal).  ws:
