@@ -347,6 +347,7 @@ struct BatchPlan {
          off_sp_tail = 0, off_sp_temp = 0, off_sp_part = 0;
   CutoffSizes cz;
   bool host_pts = false, host_w = false, host_out = false;
+  size_t upload_end;  // the uploaded region is [off_scal, upload_end)
   size_t off_scal, off_pts, off_wts, off_tab_prep, off_tab_tc, off_tab_cut, off_tab_red;
   size_t off_co_keys[2], off_co_vals[2], off_co_hist, off_co_start,
       off_co_spts, off_co_sw, off_co_order, off_co_totals, off_co_ranges, off_co_ocount, off_hxy,
@@ -680,15 +681,17 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
 
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t r = off; off = align256(off + bytes); return r; };
-  P->off_scal = take(sizeof(CallScalars) * (size_t)(count + 1));
   P->off_pts = take(sizeof(float4) * (size_t)P->total_pad);
   P->off_wts = take(sizeof(float) * (size_t)P->total_pad);
+  // the scalars (zeros) and the tables lie together and are uploaded together
+  P->off_scal = take(sizeof(CallScalars) * (size_t)(count + 1));
   P->off_tab_prep = take(sizeof(PrepInst) * (size_t)count);
   P->off_tab_tc = take(sizeof(TcInst) * (size_t)std::max(P->n_tc, 1));
   P->off_tab_cut = take(sizeof(CutInst) * (size_t)std::max(P->n_cut + P->n_sparse, 1));
   P->off_tab_red = take(sizeof(ReduceInst) * (size_t)std::max(P->n_reduce, 1));
   for (TcFamily& f : P->fam)
     if (!f.sched.empty()) f.off_sched = take(sizeof(uint32_t) * f.sched.size());
+  P->upload_end = off;
   for (int k = 0; k < count; ++k) {
     InstPlan& I = P->in[k];
     I.off_gxt = take(sizeof(float2) * (size_t)A[k].nx);
@@ -756,6 +759,19 @@ int acquire_workspace(const kde_opts* o, size_t need, cudaStream_t s, void** ws)
   return library_workspace(need, ws);
 }
 
+// The scalars (zeros) and the one table entry of a single-instance call, which
+// lie next to each other: CallScalars, then PrepInst.
+struct SingleTables {
+  CallScalars scal;
+  PrepInst prep;
+};
+static_assert(sizeof(CallScalars) == 256 && sizeof(PrepInst) % 16 == 0, "one upload for both");
+cudaError_t upload_single(const PrepInst& q, cudaStream_t s) {
+  SingleTables t = {};
+  t.prep = q;
+  return launch_upload(&t, sizeof(t), q.scal, s);
+}
+
 // The bin-key kernel's FP32 constants of a sort instance (set after its
 // geometry and reach).
 void set_key_constants(CutInst& q) {
@@ -801,7 +817,6 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   float4* pts = reinterpret_cast<float4*>(base + P.off_pts);
   float* wts = reinterpret_cast<float*>(base + P.off_wts);
 
-  KDE_CUDA(cudaMemsetAsync(scal, 0, sizeof(CallScalars) * (size_t)(count + 1), s), "clear scalars");
   const double* xy0 = A[0].points;
   const float* w0 = A[0].weights;
   if (P.host_pts) {
@@ -842,12 +857,9 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     q.begin = I.prep_begin;
     q.ox = a->origin_x;
     q.oy = a->origin_y;
-    q.sigma = kernel_sigma(kid_of(a), a->h);
-    q.cell_sigma = a->cell * q.sigma;
+    set_scale(q, kernel_sigma(kid_of(a), a->h), a->cell, lonlat ? &merc : nullptr);
     q.nx = a->nx;
     q.ny = a->ny;
-    q.lonlat = lonlat ? 1 : 0;
-    q.merc = merc;
   }
   auto part_of = [&](int k) {
     return P.in[k].splits > 1 ? reinterpret_cast<float*>(base + P.in[k].off_part) : out_dev[k];
@@ -980,18 +992,16 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   TcInst* d_tc = reinterpret_cast<TcInst*>(base + P.off_tab_tc);
   CutInst* d_cut = reinterpret_cast<CutInst*>(base + P.off_tab_cut);
   ReduceInst* d_red = reinterpret_cast<ReduceInst*>(base + P.off_tab_red);
-  KDE_CUDA(launch_upload(prep.data(), sizeof(PrepInst) * prep.size(), d_prep, s), "upload tables");
-  if (!tct.empty())
-    KDE_CUDA(launch_upload(tct.data(), sizeof(TcInst) * tct.size(), d_tc, s), "upload tables");
-  if (!cut.empty())
-    KDE_CUDA(launch_upload(cut.data(), sizeof(CutInst) * cut.size(), d_cut, s), "upload tables");
-  if (!red.empty())
-    KDE_CUDA(launch_upload(red.data(), sizeof(ReduceInst) * red.size(), d_red, s), "upload tables");
-  for (const TcFamily& f : P.fam)
-    if (!f.sched.empty())
-      KDE_CUDA(launch_upload(f.sched.data(), sizeof(uint32_t) * f.sched.size(), base + f.off_sched,
-                             s),
-               "upload schedule");
+  std::vector<unsigned char> up(P.upload_end - P.off_scal, 0);
+  auto stage = [&](size_t off, const void* src, size_t bytes) {
+    if (bytes) memcpy(up.data() + (off - P.off_scal), src, bytes);
+  };
+  stage(P.off_tab_prep, prep.data(), sizeof(PrepInst) * prep.size());
+  stage(P.off_tab_tc, tct.data(), sizeof(TcInst) * tct.size());
+  stage(P.off_tab_cut, cut.data(), sizeof(CutInst) * cut.size());
+  stage(P.off_tab_red, red.data(), sizeof(ReduceInst) * red.size());
+  for (const TcFamily& f : P.fam) stage(f.off_sched, f.sched.data(), sizeof(uint32_t) * f.sched.size());
+  KDE_CUDA(launch_upload(up.data(), up.size(), scal, s), "upload tables");
 
   // ---- launches
   KDE_CUDA(launch_prepare(d_prep, count, P.total_pad, P.max_side, s), "prepare points");
@@ -1283,16 +1293,14 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
   q.ox = a->origin_x;
   q.oy = a->origin_y;
   // offsets in bandwidths (window kernel) or in h sqrt(2 ln 2) (contractions)
-  q.sigma = use_tc ? kernel_sigma(KDE_GAUSSIAN, a->h) : 1.0 / a->h;
-  q.cell_sigma = a->cell * q.sigma;
+  set_scale(q, use_tc ? kernel_sigma(KDE_GAUSSIAN, a->h) : 1.0 / a->h, a->cell, nullptr);
   q.nx = a->nx;
   q.ny = a->ny;
   double* ht = reinterpret_cast<double*>(base + o_ht);
   double* lt = reinterpret_cast<double*>(base + o_lt);
   double* part = reinterpret_cast<double*>(base + o_part);
   double* res = reinterpret_cast<double*>(base + o_res);
-  KDE_CUDA(cudaMemsetAsync(q.scal, 0, sizeof(CallScalars), s), "clear scalars");
-  KDE_CUDA(launch_upload(&q, sizeof(q), base + o_tab, s), "upload tables");
+  KDE_CUDA(upload_single(q, s), "upload tables");
   KDE_CUDA(launch_prepare(reinterpret_cast<PrepInst*>(base + o_tab), 1, n_pad,
                           std::max(a->nx, a->ny), s),
            "prepare points");
@@ -1391,8 +1399,7 @@ int kde_lscv_grid(const kde_args* a, const float* F, double* loss, float* grad_F
   q.begin = 0;
   q.ox = a->origin_x;
   q.oy = a->origin_y;
-  q.sigma = 1.0 / a->h;
-  q.cell_sigma = a->cell / a->h;
+  set_scale(q, 1.0 / a->h, a->cell, nullptr);
   q.nx = a->nx;
   q.ny = a->ny;
   double* loo = reinterpret_cast<double*>(base + o_loo);
@@ -1401,9 +1408,8 @@ int kde_lscv_grid(const kde_args* a, const float* F, double* loss, float* grad_F
   double* part = reinterpret_cast<double*>(base + o_part);
   double* res = reinterpret_cast<double*>(base + o_res);
   const size_t np = sum_partials(std::max<int64_t>(n, sq_blocks)) + 1;
-  KDE_CUDA(cudaMemsetAsync(q.scal, 0, sizeof(CallScalars), s), "clear scalars");
+  KDE_CUDA(upload_single(q, s), "upload tables");
   KDE_CUDA(cudaMemsetAsync(res, 0, sizeof(double) * 4, s), "clear results");
-  KDE_CUDA(launch_upload(&q, sizeof(q), base + o_tab, s), "upload tables");
   KDE_CUDA(launch_prepare(reinterpret_cast<PrepInst*>(base + o_tab), 1, n_pad,
                           std::max(a->nx, a->ny), s),
            "prepare points");

@@ -34,7 +34,7 @@ constexpr int kMaxHalf = 127;  // window half-width limit (window <= 255)
 // 3 ulp of the exact quotient, the rounded division within half an ulp, so
 // unless the product lies within 4e-15 relative of an integer both have the
 // same floor; only those rare cases divide.
-__device__ __forceinline__ int64_t cell_index(double v, double o, double d, double inv_d, int n) {
+__device__ __noinline__ int64_t cell_index(double v, double o, double d, double inv_d, int n) {
   const double t = __dsub_rn(v, o);
   const double q = __dmul_rn(t, inv_d);
   double f = floor(q);
@@ -59,7 +59,7 @@ struct CellMap {
 };
 __device__ __forceinline__ int cell_of(double v, const CellMap& m) {
   const double t = __dsub_rn(v, m.o);
-  const float2 s = split_bits(t);
+  const float2 s = split_double(t);
   const float est = floorf(s.x * m.inv);
   const float r = fmaf(-est, m.dh, s.x) + fmaf(-est, m.dl, s.y);
   if (fabsf(est) < 2097152.f) {

@@ -865,9 +865,7 @@ cudaError_t launch_lookback_timeout_probe(uint32_t* buf, CallScalars* err, uint6
   uint32_t* chunk_ctr = ghist + kDigits;
   cudaError_t e = cudaMemsetAsync(buf, 0, sizeof(uint32_t) * lookback_probe_words(), s);
   if (e != cudaSuccess) return e;
-  const uint32_t one = 1;
-  // a kernel-parameter write keeps the probe free of host-to-device copies
-  e = launch_upload(&one, sizeof(one), chunk_ctr, s);
+  e = cudaMemsetAsync(chunk_ctr, 1, 1, s);  // the counter's lowest byte: 1
   if (e != cudaSuccess) return e;
   k_radix_pass<<<1, kSortThreads, 0, s>>>(keys, vals, m, 0, 8, ghist, chunk_ctr, status, keys_out,
                                           vals_out, nullptr, nullptr, nullptr, nullptr, 0, err,

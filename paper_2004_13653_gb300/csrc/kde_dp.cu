@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(512)
     bool bad = false;
     for (int i = tid; i < len; i += nt) {
       const double2 p = P[i];
-      const float2 x = split_bits(p.x - o.x), y = split_bits(p.y - o.y);
+      const float2 x = split_double(p.x - o.x), y = split_double(p.y - o.y);
       // an infinite or undefined coordinate: the high word's exponent is full
       bad |= ((unsigned)__double2hiint(p.x) & 0x7ff00000u) == 0x7ff00000u ||
              ((unsigned)__double2hiint(p.y) & 0x7ff00000u) == 0x7ff00000u;

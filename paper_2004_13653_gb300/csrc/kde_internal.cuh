@@ -39,23 +39,34 @@ struct CallScalars {
 };
 
 #ifdef __CUDACC__
-// v as hi + lo in FP32, within 2^-47 |v|: hi is v with its mantissa cut to 24
-// bits, lo the other 29, taken from the bits of v.  Rounding v to FP32,
-// widening and subtracting costs four FP64-rate conversions and adds, and
-// this GPU does 2 of those per SM and clock (0.016 of the FP32 rate); this is
-// integer and FP32 work but for numbers below 2^-74 or above 2^126.
+// v is zero or between 2^-74 and 2^126 in magnitude.
+__device__ __forceinline__ bool bits_in_range(double v) {
+  const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  return (h >> 20) - 949u < 201u || (h | (unsigned)__double2loint(v)) == 0u;
+}
+// v (in that range) as hi + lo in FP32, within 2^-47 |v|: hi is v with its
+// mantissa cut to 24 bits, lo the other 29, taken from the bits of v.  Rounding
+// v to FP32, widening and subtracting costs four operations on the FP64 pipe,
+// which takes 16 cycles of an SM for each warp instruction; this is integer
+// and FP32 work.
 __device__ __forceinline__ float2 split_bits(double v) {
   const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
   const unsigned e = (h >> 20) & 0x7ffu, sign = h & 0x80000000u;
-  if (e - 949u < 201u) {
-    // exponent 8 bits of the 11 and the top 23 mantissa bits; 896 = the
-    // difference of the biases flips the exponent's top bit
-    const unsigned hi = ((__funnelshift_l(l, h, 3) & 0x7fffffffu) ^ 0x40000000u) | sign;
-    const float scale = __uint_as_float(((e - 948u) << 23) | sign);  // 2^(e - 1075)
-    return make_float2(__uint_as_float(hi), (float)(l & 0x1fffffffu) * scale);
-  }
+  // exponent 8 bits of the 11 and the top 23 mantissa bits; 896 = the
+  // difference of the biases flips the exponent's top bit
+  const unsigned hi = ((__funnelshift_l(l, h, 3) & 0x7fffffffu) ^ 0x40000000u) | sign;
+  const unsigned scale = ((e - 948u) << 23) | sign;  // 2^(e - 1075)
+  return make_float2(__uint_as_float(e ? hi : 0u),
+                     (float)(l & 0x1fffffffu) * __uint_as_float(e ? scale : 0u));
+}
+// Any v.  The FP64 form is a call, so that the usual case does not execute it
+// under a false predicate (which would still take its cycles).
+static __device__ __noinline__ float2 split_any(double v) {
   const float hi = __double2float_rn(v);
   return make_float2(hi, __double2float_rn(v - (double)hi));
+}
+__device__ __forceinline__ float2 split_double(double v) {
+  return bits_in_range(v) ? split_bits(v) : split_any(v);
 }
 #endif
 
@@ -118,7 +129,7 @@ struct MercParams {
 // Parameters of the projection at standard latitude lat0_deg (|lat0| < 90).
 MercParams mercator_params(double lat0_deg);
 
-struct PrepInst {
+struct alignas(16) PrepInst {
   const double* xy;  // caller's points (device): metres, or (lon, lat) degrees when lonlat
   const float* w;    // caller's weights (device) or null
   float4* pts;       // prepared points, n_pad entries
@@ -131,7 +142,17 @@ struct PrepInst {
   int nx, ny;
   int lonlat;       // 1: xy holds (lon, lat) degrees, projected here with merc
   MercParams merc;
+  int usual;        // sigma allows the FP32-pair form of the scaling
+  // merc's x, and y's first terms, with the centring and scaling in them:
+  // X = lon lon_scale + lon_off; Y = lat_off + lat_scale d + lat_q d^2 +
+  // sigma (c3 d^3 + ...) for |d| <= range_f
+  double lon_scale, lon_off, lat_scale, lat_off;
+  float2 sigma2, lat_q;  // pairs of FP32 numbers
+  float range_f;
 };
+// Sets q's scale (offsets in units of 1 / sigma) and, with m, the projection of
+// its (lon, lat) points; q's origin is set before.
+void set_scale(PrepInst& q, double sigma, double cell, const MercParams* m);
 
 struct TcInst {
   const float4* pts;
@@ -277,7 +298,8 @@ struct ReduceInst {
 };
 
 // Write `bytes` host bytes to device memory `dst` in stream order (kernel
-// launches carrying the bytes as parameters; capturable).
+// launches carrying the bytes as parameters; capturable).  nbytes is a multiple
+// of 16, dst 16-byte aligned.
 cudaError_t launch_upload(const void* bytes, size_t nbytes, void* dst, cudaStream_t s);
 
 // -------------------------------------------------------------- launches

@@ -166,8 +166,7 @@ extern "C" int kde_grid_noalloc(const double* points, const float* weights, int6
   q.begin = 0;
   q.ox = grid_origin[0];
   q.oy = grid_origin[1];
-  q.sigma = kernel_sigma(kernel_id, h);
-  q.cell_sigma = cell * q.sigma;
+  set_scale(q, kernel_sigma(kernel_id, h), cell, nullptr);
   q.nx = nx;
   q.ny = ny;
   const double c1 = kernel_const_1d(kernel_id);

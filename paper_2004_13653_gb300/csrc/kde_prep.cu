@@ -123,6 +123,80 @@ __device__ __forceinline__ float2 split_hi_lo(double v) {
   return make_float2(hi, lo);
 }
 
+__device__ __forceinline__ bool finite_bits(double v) {
+  return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
+}
+// v is zero or between 2^-60 and 2^100: split_bits and products with a scale
+// of 2^-60 .. 2^60 then neither overflow nor lose bits to underflow
+__device__ __forceinline__ bool plain_range(double v) {
+  const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  return (h >> 20) - 963u < 160u || (h | (unsigned)__double2loint(v)) == 0u;
+}
+
+// (x, y) + (z, w), both sums of two FP32 numbers, within a few 2^-47 of the
+// larger
+__device__ __forceinline__ float2 add_pairs(float2 a, float2 b) {
+  const float s = a.x + b.x, bb = s - a.x;
+  const float e = ((a.x - (s - bb)) + (b.x - bb)) + (a.y + b.y);
+  const float hi = s + e;
+  return make_float2(hi, e - (hi - s));
+}
+// the product, within 2^-46 of it
+__device__ __forceinline__ float2 mul_pairs(float2 a, float2 b) {
+  const float p = a.x * b.x;
+  const float e = fmaf(a.x, b.x, -p) + fmaf(a.x, b.y, a.y * b.x);
+  const float hi = p + e;
+  return make_float2(hi, e - (hi - p));
+}
+
+// Any point, in FP64 but for the split; a NaN in x: not finite.
+__device__ __noinline__ float4 prepare_any(double2 v, const PrepInst& I) {
+  const double2 m = I.lonlat ? mercator_xy(v, I.merc) : v;
+  const double x = (m.x - I.ox) * I.sigma, y = (m.y - I.oy) * I.sigma;
+  const float2 X = split_hi_lo(x), Y = split_hi_lo(y);
+  return make_float4(finite_bits(x) && finite_bits(y) ? X.x : __uint_as_float(0x7fffffffu), X.y,
+                     Y.x, Y.y);
+}
+
+// The usual points: metres, and (lon, lat) near the standard latitude.  The
+// FP64 pipe takes 16 cycles of an SM per warp instruction, so what needs
+// FP64's 53 bits (the differences of projected coordinates, and the constant
+// and linear terms of the projection with the centring and scaling in them)
+// stays there, two or three operations a point, and the rest runs on pairs of
+// FP32 numbers, whose 2^-46 is far below the 2^-24 of every use of the result.
+// False: prepare_any decides.
+__device__ __forceinline__ bool prepare_usual(double2 v, const PrepInst& I, float4& r) {
+  float2 X, Y;
+  if (!I.lonlat) {
+    const double x = v.x - I.ox, y = v.y - I.oy;
+    if (!(plain_range(x) && plain_range(y))) return false;
+    X = mul_pairs(split_bits(x), I.sigma2);
+    Y = mul_pairs(split_bits(y), I.sigma2);
+  } else {
+    // Eq. 1-4 as in mercator_xy: the quadratic term is a few hundred metres,
+    // the terms beyond it a few
+    const MercParams& m = I.merc;
+    const double dd = fma(v.y, kPi / 180.0, -m.phi0);
+    const double x = fma(v.x, I.lon_scale, I.lon_off), y = fma(dd, I.lat_scale, I.lat_off);
+    if (!(plain_range(dd) && plain_range(x) && plain_range(y))) return false;
+    const float2 d = split_bits(dd);
+    if (!(fabsf(d.x) <= I.range_f)) return false;
+    X = split_bits(x);
+    float t = m.c[4];
+    t = fmaf(t, d.x, m.c[3]);
+    t = fmaf(t, d.x, m.c[2]);
+    t = fmaf(t, d.x, m.c[1]);
+    t = fmaf(t, d.x, m.c[0]);
+    const float sq = d.x * d.x;
+    const float sq_lo = fmaf(d.x, d.x, -sq) + 2.f * d.x * d.y;
+    float2 q = mul_pairs(make_float2(sq, sq_lo), I.lat_q);
+    q.y = fmaf(t * I.sigma2.x, d.x * sq, q.y);
+    Y = add_pairs(split_bits(y), q);
+  }
+  r = make_float4(X.x, X.y, Y.x, Y.y);
+  return true;
+}
+
 // Instance of flattened index p: the last entry whose begin <= p.
 template <class T>
 __device__ __forceinline__ int find_instance(const T* tab, int ninst, int64_t p) {
@@ -134,64 +208,110 @@ __device__ __forceinline__ int find_instance(const T* tab, int ninst, int64_t p)
   return lo;
 }
 
+constexpr int kPerWarp = 64;  // divides every instance's n_pad
+
 // Centre, scale, split; weights copied (unit when w == NULL); padding zeroed;
 // max |w| reduced per instance for the tensor path's operand scaling.  Every
-// instance's n_pad is a multiple of 512, so a warp never straddles two.
-__global__ void k_prepare(const PrepInst* __restrict__ tab, int ninst, int64_t total) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += stride) {
-    const PrepInst& I = tab[find_instance(tab, ninst, g)];
-    const int64_t p = g - I.begin;
-    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-    float wv = 0.f;
-    bool bad = false;
-    unsigned wbits = 0;
-    if (p < I.n) {
-      double2 v = reinterpret_cast<const double2*>(I.xy)[p];
-      if (I.lonlat) v = mercator_xy(v, I.merc);  // Eq. 1-4 fused into the centring
-      const double X = (v.x - I.ox) * I.sigma;
-      const double Y = (v.y - I.oy) * I.sigma;
-      wv = I.w ? I.w[p] : 1.0f;
-      if (isfinite(X) && isfinite(Y) && isfinite(wv)) {
-        const float2 sx = split_hi_lo(X), sy = split_hi_lo(Y);
-        r = make_float4(sx.x, sx.y, sy.x, sy.y);
-        wbits = __float_as_uint(fabsf(wv));
-      } else {
-        bad = true;
-        wv = 0.f;
+// instance's n_pad is a multiple of 512, so a warp's points never straddle two.  The
+// blocks from table_block on fill the cell-centre tables (one launch for
+// both).  1M points: 29.6 us with every step in FP64, 13 now (HBM: 6 us);
+// 20M (lon, lat) points: 0.897 -> 0.160 ms (HBM: 0.12 ms).  A warp keeps its
+// maximum over all its points and skips the atomic when it would not change
+// anything.
+__global__ void __launch_bounds__(256)
+    k_prepare(const PrepInst* __restrict__ tab, int ninst, int64_t total, int table_block,
+              int blocks_per_side) {
+  if ((int)blockIdx.x >= table_block) {
+    const int b = (int)blockIdx.x - table_block;
+    const PrepInst& I = tab[b / blocks_per_side];
+    const int t = (b % blocks_per_side) * blockDim.x + threadIdx.x;
+    if (t >= max(I.nx, I.ny)) return;
+    const float2 c = split_hi_lo(((double)t + 0.5) * I.cell_sigma);
+    if (t < I.nx) I.gxt[t] = c;
+    if (t < I.ny) I.gyt[t] = c;
+    return;
+  }
+  // A warp takes kPerWarp consecutive points at a time, all of one instance,
+  // and has their loads in flight together.
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)table_block * (blockDim.x >> 5);
+  unsigned wmax = 0;
+  bool bad = false, neg = false;
+  const PrepInst* cur = nullptr;
+  auto flush = [&]() {
+    const unsigned top = __reduce_max_sync(0xffffffffu, wmax);
+    const unsigned anybad = __any_sync(0xffffffffu, bad), anyneg = __any_sync(0xffffffffu, neg);
+    if (lane == 0) {
+      if (top > *(volatile unsigned*)&cur->scal->wmax_bits) atomicMax(&cur->scal->wmax_bits, top);
+      if (anybad) atomicOr(&cur->scal->err, kErrNonFinite);
+      if (anyneg) atomicOr(&cur->scal->negw, 1);
+    }
+    wmax = 0;
+    bad = neg = false;
+  };
+  for (int64_t g0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kPerWarp;
+       g0 < total; g0 += warps * kPerWarp) {
+    const PrepInst* ip = tab + (ninst > 1 ? find_instance(tab, ninst, g0) : 0);
+    if (ip != cur) {
+      if (cur) flush();
+      cur = ip;
+    }
+    const PrepInst& I = *ip;
+    const int64_t p0 = g0 - I.begin + lane;
+    double2 v[kPerWarp / 32];
+    float w[kPerWarp / 32];
+#pragma unroll
+    for (int u = 0; u < kPerWarp / 32; ++u) {
+      const int64_t p = p0 + 32 * u;
+      v[u] = p < I.n ? reinterpret_cast<const double2*>(I.xy)[p] : make_double2(0.0, 0.0);
+      w[u] = p < I.n ? (I.w ? I.w[p] : 1.0f) : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < kPerWarp / 32; ++u) {
+      const int64_t p = p0 + 32 * u;
+      float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (p < I.n) {
+        if (!(I.usual && prepare_usual(v[u], I, r))) r = prepare_any(v[u], I);
+        if (!(r.x != r.x) && isfinite(w[u])) {
+          wmax = max(wmax, __float_as_uint(fabsf(w[u])));
+        } else {
+          bad = true;
+          r = make_float4(0.f, 0.f, 0.f, 0.f);
+          w[u] = 0.f;
+        }
       }
-    }
-    I.pts[p] = r;
-    I.wts[p] = wv;
-    // warp-level max, one atomic per warp (all lanes share the instance)
-    for (int o = 16; o > 0; o >>= 1) wbits = max(wbits, __shfl_xor_sync(0xffffffffu, wbits, o));
-    const unsigned anybad = __any_sync(0xffffffffu, bad);
-    const unsigned anyneg = __any_sync(0xffffffffu, wv < 0.f);
-    if ((threadIdx.x & 31) == 0) {
-      if (wbits) atomicMax(&I.scal->wmax_bits, wbits);
-      if (anybad) atomicOr(&I.scal->err, kErrNonFinite);
-      if (anyneg) atomicOr(&I.scal->negw, 1);
+      I.pts[p] = r;
+      I.wts[p] = w[u];
+      neg |= w[u] < 0.f;
     }
   }
+  if (cur) flush();
 }
 
-// Cell-centre tables: blockIdx.y = instance.
-__global__ void k_grid_tables(const PrepInst* __restrict__ tab) {
-  const PrepInst& I = tab[blockIdx.y];
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < max(I.nx, I.ny);
-       t += gridDim.x * blockDim.x) {
-    if (t < I.nx) I.gxt[t] = split_hi_lo(((double)t + 0.5) * I.cell_sigma);
-    if (t < I.ny) I.gyt[t] = split_hi_lo(((double)t + 0.5) * I.cell_sigma);
-  }
-}
-
-constexpr int kBlobBytes = 31 * 1024;
-struct Blob {
-  unsigned char bytes[kBlobBytes];
+// Table bytes carried by a launch's parameters; the small form keeps the
+// parameters of the usual call (one instance) short.
+constexpr int kBlobBytes = 31 * 1024, kSmallBlobBytes = 2 * 1024;
+template <int BYTES>
+struct __align__(16) Blob {
+  unsigned char bytes[BYTES];
 };
 
-__global__ void k_upload(const __grid_constant__ Blob blob, int nbytes, unsigned char* dst) {
-  for (int i = threadIdx.x; i < nbytes; i += blockDim.x) dst[i] = blob.bytes[i];
+template <int BYTES>
+__global__ void k_upload(const __grid_constant__ Blob<BYTES> blob, int nwords, uint4* dst) {
+  for (int i = threadIdx.x; i < nwords; i += blockDim.x)
+    dst[i] = reinterpret_cast<const uint4*>(blob.bytes)[i];
+}
+
+template <int BYTES>
+cudaError_t upload_chunk(const unsigned char* src, size_t len, unsigned char* dst,
+                         cudaStream_t s) {
+  static Blob<BYTES> blob;  // staging for the launch parameters (copied at launch)
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
+  memcpy(blob.bytes, src, len);
+  k_upload<BYTES><<<1, 256, 0, s>>>(blob, (int)(len / 16), reinterpret_cast<uint4*>(dst));
+  note_launches(1);
+  return cudaGetLastError();
 }
 
 int blocks_for(int64_t n, int threads) {
@@ -218,32 +338,50 @@ cudaError_t launch_mercator(const double* lonlat, int64_t n, double lat0_deg, do
   return cudaGetLastError();
 }
 
+namespace {
+float2 pair_of(double v) {
+  const float hi = (float)v;
+  return make_float2(hi, (float)(v - (double)hi));
+}
+}  // namespace
+
+void set_scale(PrepInst& q, double sigma, double cell, const MercParams* m) {
+  q.sigma = sigma;
+  q.cell_sigma = cell * sigma;
+  // a scale outside the plain range sends every point to prepare_any
+  const bool plain = sigma >= 0x1p-60 && sigma <= 0x1p60;
+  q.usual = plain ? 1 : 0;
+  q.sigma2 = plain ? pair_of(sigma) : make_float2(0.f, 0.f);
+  q.lonlat = m ? 1 : 0;
+  if (!m) return;
+  q.merc = *m;
+  q.lon_scale = m->kx * sigma;
+  q.lon_off = -q.ox * sigma;
+  q.lat_scale = m->c1 * sigma;
+  q.lat_off = (m->y0 - q.oy) * sigma;
+  q.lat_q = pair_of(m->c2 * sigma);
+  q.range_f = (float)m->range;
+}
+
 cudaError_t launch_prepare(const PrepInst* tab, int ninst, int64_t total_pad, int max_side,
                            cudaStream_t s) {
   if (ninst <= 0) return cudaSuccess;
-  if (total_pad > 0) {
-    k_prepare<<<blocks_for(total_pad, 256), 256, 0, s>>>(tab, ninst, total_pad);
-    note_launches(1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  dim3 grid((max_side + 255) / 256, ninst);
-  k_grid_tables<<<grid, 256, 0, s>>>(tab);
+  const int per_side = (max_side + 255) / 256;
+  const int points = total_pad > 0 ? blocks_for(total_pad, 8 * kPerWarp) : 0;
+  k_prepare<<<points + ninst * per_side, 256, 0, s>>>(tab, ninst, total_pad, points, per_side);
   note_launches(1);
   return cudaGetLastError();
 }
 
 cudaError_t launch_upload(const void* bytes, size_t nbytes, void* dst, cudaStream_t s) {
-  static Blob blob;  // staging for the launch parameters (copied at launch)
-  static std::mutex mu;
-  std::lock_guard<std::mutex> lock(mu);
   const unsigned char* src = static_cast<const unsigned char*>(bytes);
+  unsigned char* to = static_cast<unsigned char*>(dst);
+  if (nbytes % 16) return cudaErrorInvalidValue;
   for (size_t off = 0; off < nbytes; off += kBlobBytes) {
-    const int len = (int)std::min<size_t>(kBlobBytes, nbytes - off);
-    memcpy(blob.bytes, src + off, len);
-    k_upload<<<1, 256, 0, s>>>(blob, len, static_cast<unsigned char*>(dst) + off);
-    note_launches(1);
-    cudaError_t e = cudaGetLastError();
+    const size_t len = std::min<size_t>(kBlobBytes, nbytes - off);
+    const cudaError_t e = len <= kSmallBlobBytes
+                              ? upload_chunk<kSmallBlobBytes>(src + off, len, to + off, s)
+                              : upload_chunk<kBlobBytes>(src + off, len, to + off, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -128,26 +128,31 @@ __global__ void __launch_bounds__(kTailThreads) k_sparse_tails(SparseCtl sp) {
   list_tails(sp, cnt, warp_sum);
 }
 
-// The whole work list of at most kTailThreads tiles in one CTA: totals (a warp
-// per tile), both exclusive scans (a tile per thread) and the tails.  Five
-// launches of a few microseconds each become one (1024^2: 35 us -> 7 us with
-// the totals' rows over the lanes).
+// The work list of at most kTailThreads tiles in one CTA: totals (a warp per
+// tile; with have_totals k_sparse_totals has done them), both exclusive scans
+// (a tile per thread) and the tails.  Five launches of a few microseconds each
+// become one (1024^2, 16 tiles: 35 us -> 12 us), or two beyond 32 tiles, whose
+// bin ranges, FP64, would queue on the one SM's FP64 pipe (256 tiles: 84 us).
 __global__ void __launch_bounds__(kTailThreads)
     k_sparse_plan(const TcInst* __restrict__ tab, int ninst, SparseCtl sp,
-                  uint32_t* __restrict__ tile_total, uint32_t* __restrict__ piece_begin,
-                  uint32_t* __restrict__ full_begin) {
+                  bool have_totals, uint32_t* __restrict__ tile_total,
+                  uint32_t* __restrict__ piece_begin, uint32_t* __restrict__ full_begin) {
   __shared__ uint32_t cnt[kTailKeys];
   __shared__ uint32_t warp_sum[kTailThreads / 32];
   __shared__ uint32_t totals[kTailThreads];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int t = warp; t < sp.tiles_total; t += kTailThreads / 32) {
-    const uint32_t total = tile_points(tab, ninst, t);
-    if (lane == 0) totals[t] = total;
+  if (have_totals) {
+    if (tid < sp.tiles_total) totals[tid] = tile_total[tid];
+  } else {
+    for (int t = warp; t < sp.tiles_total; t += kTailThreads / 32) {
+      const uint32_t total = tile_points(tab, ninst, t);
+      if (lane == 0) totals[t] = total;
+    }
   }
   __syncthreads();
   const uint32_t L = (uint32_t)sp.piece_len;
   const uint32_t total = tid < sp.tiles_total ? totals[tid] : 0u;
-  if (tid < sp.tiles_total) tile_total[tid] = total;
+  if (tid < sp.tiles_total && !have_totals) tile_total[tid] = total;
   const uint32_t full = total / L, pieces = full + (total % L ? 1u : 0u);
 #pragma unroll
   for (int which = 0; which < 2; ++which) {
@@ -227,19 +232,23 @@ cudaError_t launch_sparse_plan(const TcInst* tab, int ninst, const SparseCtl& sp
                                CallScalars* err, cudaStream_t s) {
   (void)err;
   if (sp.piece_len <= 0) return cudaErrorInvalidValue;
-  if (sp.tiles_total <= kTailThreads) {
-    k_sparse_plan<<<1, kTailThreads, 0, s>>>(tab, ninst, sp, const_cast<uint32_t*>(sp.tile_total),
+  const int m = sp.tiles_total + 1;
+  const bool one_cta = sp.tiles_total <= kTailThreads, split = sp.tiles_total > 32;
+  cudaError_t e = cudaSuccess;
+  if (split) {
+    k_sparse_totals<<<(m + 7) / 8, 256, 0, s>>>(
+        tab, ninst, sp, const_cast<uint32_t*>(sp.tile_total), npieces, nfull);
+    note_launches(1);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  if (one_cta) {
+    k_sparse_plan<<<1, kTailThreads, 0, s>>>(tab, ninst, sp, split,
+                                             const_cast<uint32_t*>(sp.tile_total),
                                              const_cast<uint32_t*>(sp.piece_begin),
                                              const_cast<uint32_t*>(sp.full_begin));
     note_launches(1);
     return cudaGetLastError();
   }
-  const int m = sp.tiles_total + 1;
-  k_sparse_totals<<<(m + 7) / 8, 256, 0, s>>>(
-      tab, ninst, sp, const_cast<uint32_t*>(sp.tile_total), npieces, nfull);
-  note_launches(1);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   e = launch_exclusive_scan(npieces, const_cast<uint32_t*>(sp.piece_begin), m, 2048, scan_temp, s);
   if (e != cudaSuccess) return e;
   e = launch_exclusive_scan(nfull, const_cast<uint32_t*>(sp.full_begin), m, 2048, scan_temp, s);
