@@ -137,21 +137,46 @@ __global__ void __launch_bounds__(256, COLS == 1 ? 5 : (COLS == 2 ? 4 : (COLS ==
   }
 }
 
-// Fixed-order block sums of a double array: partial[b] = sum of block b's slice.
-__global__ void k_sum_blocks(const double* __restrict__ v, int64_t n, int64_t per_block,
-                             double* __restrict__ partial) {
-  __shared__ double sh[256];
-  const int64_t b0 = (int64_t)blockIdx.x * per_block;
-  const int64_t b1 = min(b0 + per_block, n);
+// Fixed-order sums of up to kMaxSums double arrays in two launches: the first
+// sums slices of kSumSlice numbers (block x: slice, y: array), the second the
+// slices' sums.
+constexpr int kMaxSums = 3, kSumThreads = 1024;
+constexpr int64_t kSumSlice = 8192;  // one round of kSumThreads x 8 numbers
+struct SumSet {
+  SumJob job[kMaxSums];
+};
+template <int THREADS>
+__device__ __forceinline__ double block_sum(const double* __restrict__ v, int64_t b0, int64_t b1) {
+  __shared__ double sh[THREADS / 32];
   double acc = 0.0;
-  for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) acc += v[i];
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
+  constexpr int kAhead = 8;
+  for (int64_t i = b0 + threadIdx.x; i < b1; i += (int64_t)kAhead * THREADS) {
+    double x[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) x[u] = i + u * THREADS < b1 ? v[i + u * THREADS] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) acc += x[u];
   }
-  if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  double r = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < THREADS / 32; ++w) r += sh[w];
+  return r;
+}
+__global__ void __launch_bounds__(kSumThreads) k_sum_slices(const __grid_constant__ SumSet s) {
+  const SumJob& j = s.job[blockIdx.y];
+  const int64_t b0 = (int64_t)blockIdx.x * kSumSlice;
+  if (b0 >= j.n && blockIdx.x > 0) return;
+  const double r = block_sum<kSumThreads>(j.v, b0, min(b0 + kSumSlice, j.n));
+  if (threadIdx.x == 0) j.partial[blockIdx.x] = r;
+}
+__global__ void __launch_bounds__(256) k_sum_totals(const __grid_constant__ SumSet s) {
+  const SumJob& j = s.job[blockIdx.x];
+  const int64_t slices = j.n > 0 ? (j.n + kSumSlice - 1) / kSumSlice : 1;
+  const double r = block_sum<256>(j.partial, 0, slices);
+  if (threadIdx.x == 0) *j.result = r;
 }
 
 // ----------------------------------------------------------------- LSCV
@@ -176,58 +201,102 @@ __global__ void k_lscv_grid(const float* __restrict__ F, int64_t cells, double t
   if (threadIdx.x == 0) sq_part[blockIdx.x] = sh[0];
 }
 
+// exp(-c^2 t^2 / 2) for 0 <= t <= 1, c the cell in bandwidths: a polynomial in
+// t^2 (the series of exp, cut where its terms fall below 2^-56), with the
+// coefficients set on the host; for narrow bandwidths (many terms) the exp()
+// of the library.
+constexpr int kMaxTerms = 14;
+struct CellGauss {
+  double c[kMaxTerms];  // (-c^2/2)^k / k!
+  double a;             // -c^2/2
+  int terms;            // 0: use exp()
+};
+__device__ __forceinline__ double cell_gauss(double t, const CellGauss& g) {
+  const double z = t * t;
+  if (g.terms == 0) return exp(g.a * z);
+  double r = g.c[g.terms - 1];
+  for (int k = g.terms - 2; k >= 0; --k) r = fma(r, z, g.c[k]);
+  return r;
+}
+
+// One axis of a point's own term at its two neighbouring cell centres (offsets
+// -t and 1 - t cells; k0, k1: 1 where that cell is in the grid): with weights
+// 1 - t and t, factors e and offsets d in bandwidths,
+//   p = sum w e,  q = sum w e d^2,  dp = d p / d x (in bandwidths: weights' and
+//   factors' slopes, sum (+-e / c + w e d)).
+struct AxisTerm {
+  double p, q, dp;
+};
+__device__ __forceinline__ AxisTerm axis_term(double t, double k0, double k1, double c, double inv_c,
+                                              const CellGauss& g) {
+  const double u = 1.0 - t;
+  const double e0 = k0 * cell_gauss(t, g), e1 = k1 * cell_gauss(u, g);
+  const double d0 = -c * t, d1 = c * u;
+  const double a0 = u * e0, a1 = t * e1;
+  const double b0 = a0 * d0, b1 = a1 * d1;
+  AxisTerm r;
+  r.p = a0 + a1;
+  r.q = fma(b0, d0, b1 * d1);
+  r.dp = fma(e1 - e0, inv_c, b0 + b1);
+  return r;
+}
+
 // Per point: the leave-one-out term w_p bilerp(F - F_p, x_p) (the bilinear
 // sample of F between cell centres, zero outside, minus the same sample of
 // the point's own term F_p = w_p S, S = exp(-r^2/2h^2)/(2 pi N h^2)), the
 // loss's direct partials (through the bilinear weights, w_p and F_p), and the
 // scatter of -(2/N) w_p beta into the FP64 cotangent (atomic adds; in FP64
-// their order does not show in the FP32 result).  FP64 throughout.
-__global__ void k_lscv_points(const float4* __restrict__ pts, const float* __restrict__ wts,
-                              int64_t n, const float* __restrict__ F, int nx, int ny,
-                              double cells_per_h, double cell_h, double inv_cell, double inv_h,
-                              double inv_N, double self_term, double* __restrict__ G,
-                              float* __restrict__ gw_direct, float* __restrict__ gxy_direct,
-                              double* __restrict__ loo, double* __restrict__ hdir) {
+// their order does not show in the FP32 result).  FP64 throughout, which
+// bounds it (16 SM cycles per warp instruction): S and the bilinear weights
+// are products over the axes, so the sums over the four cells are products of
+// two-cell sums, and the four exponentials are values of one polynomial.
+// 1.47M points: 655 us with the four cells one by one, 368 now.
+__global__ void __launch_bounds__(256)
+    k_lscv_points(const float4* __restrict__ pts, const float* __restrict__ wts, int64_t n,
+                  const float* __restrict__ F, int nx, int ny, double cells_per_h, double cell_h,
+                  double inv_cell, double inv_h, double inv_N, double self_term,
+                  const __grid_constant__ CellGauss cg, double* __restrict__ G,
+                  float* __restrict__ gw_direct, float* __restrict__ gxy_direct,
+                  double* __restrict__ loo, double* __restrict__ hdir) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += stride) {
     const float4 P = pts[p];
     const double w = wts[p];
-    const double X = (double)P.x + (double)P.y, Y = (double)P.z + (double)P.w;  // in h
-    const double fx = X * cells_per_h - 0.5;
-    const double fy = Y * cells_per_h - 0.5;
+    const double fx = fma((double)P.x + (double)P.y, cells_per_h, -0.5);  // in cells
+    const double fy = fma((double)P.z + (double)P.w, cells_per_h, -0.5);
     const double fi = floor(fx), fj = floor(fy);
     const double ax = fx - fi, ay = fy - fj;
-    double v = 0.0, sv = 0.0, dvx = 0.0, dvy = 0.0, dsx = 0.0, dsy = 0.0, sh = 0.0;
-#pragma unroll
-    for (int b = 0; b < 2; ++b)
-#pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const double ii = fi + a, jj = fj + b;
-        if (ii < 0 || jj < 0 || ii >= nx || jj >= ny) continue;
-        const int64_t q = (int64_t)jj * nx + (int64_t)ii;
-        const double wx = a ? ax : 1.0 - ax, wy = b ? ay : 1.0 - ay, ww = wx * wy;
-        const double ex = (a ? 1.0 : -1.0) * wy * inv_cell;  // d(wx wy)/dx_p
-        const double ey = (b ? 1.0 : -1.0) * wx * inv_cell;
-        const double dx = (ii + 0.5) * cell_h - X, dy = (jj + 0.5) * cell_h - Y;  // in h
-        const double r2 = dx * dx + dy * dy;
-        const double S = self_term * exp(-0.5 * r2);
-        const double f = F[q];
-        v += ww * f;
-        sv += ww * S;
-        dvx += ex * f;
-        dvy += ey * f;
-        dsx += ex * S + ww * S * dx * inv_h;
-        dsy += ey * S + ww * S * dy * inv_h;
-        sh += ww * S * (r2 - 2.0) * inv_h;
-        if (G) atomicAdd(&G[q], -2.0 * inv_N * w * ww);
-      }
+    // the cell in 32 bits: far outside either way gives cells outside the grid
+    const int i = (int)fmin(fmax(fi, -2.0), 2147483000.0);
+    const int j = (int)fmin(fmax(fj, -2.0), 2147483000.0);
+    const bool x0 = i >= 0 && i < nx, x1 = i >= -1 && i + 1 < nx;
+    const bool y0 = j >= 0 && j < ny, y1 = j >= -1 && j + 1 < ny;
+    const int64_t q = (int64_t)j * nx + i;
+    const double f00 = x0 && y0 ? F[q] : 0.f, f10 = x1 && y0 ? F[q + 1] : 0.f;
+    const double f01 = x0 && y1 ? F[q + nx] : 0.f, f11 = x1 && y1 ? F[q + nx + 1] : 0.f;
+    const double g0 = f10 - f00, g1 = f11 - f01;
+    const double r0 = fma(ax, g0, f00), r1 = fma(ax, g1, f01);
+    const double v = fma(ay, r1 - r0, r0);
+    const double dvx = fma(ay, g1 - g0, g0), dvy = r1 - r0;  // times 1 / cell
+    const AxisTerm X = axis_term(ax, x0 ? 1.0 : 0.0, x1 ? 1.0 : 0.0, cell_h, cells_per_h, cg);
+    const AxisTerm Y = axis_term(ay, y0 ? 1.0 : 0.0, y1 ? 1.0 : 0.0, cell_h, cells_per_h, cg);
+    const double sv = self_term * X.p * Y.p;
+    if (G) {
+      const double k = -2.0 * inv_N * w;
+      const double k0 = k * (1.0 - ay), k1 = k * ay;
+      if (x0 && y0) atomicAdd(&G[q], k0 * (1.0 - ax));
+      if (x1 && y0) atomicAdd(&G[q + 1], k0 * ax);
+      if (x0 && y1) atomicAdd(&G[q + nx], k1 * (1.0 - ax));
+      if (x1 && y1) atomicAdd(&G[q + nx + 1], k1 * ax);
+    }
     if (gw_direct) gw_direct[p] = (float)(-2.0 * inv_N * (v - 2.0 * w * sv));
     if (gxy_direct) {
-      gxy_direct[2 * p] = (float)(-2.0 * inv_N * w * (dvx - w * dsx));
-      gxy_direct[2 * p + 1] = (float)(-2.0 * inv_N * w * (dvy - w * dsy));
+      const double ws = w * self_term * inv_h;
+      gxy_direct[2 * p] = (float)(-2.0 * inv_N * w * fma(-ws * X.dp, Y.p, dvx * inv_cell));
+      gxy_direct[2 * p + 1] = (float)(-2.0 * inv_N * w * fma(-ws * Y.dp, X.p, dvy * inv_cell));
     }
     loo[p] = w * (v - w * sv);
-    hdir[p] = w * w * sh;
+    hdir[p] = w * w * inv_h * self_term * (fma(X.q, Y.p, X.p * Y.q) - 2.0 * X.p * Y.p);
   }
 }
 
@@ -244,18 +313,19 @@ int grid_blocks(int64_t n, int threads, int cap) {
 
 }  // namespace
 
-size_t sum_partials(int64_t n) { return (size_t)((n + 65535) / 65536) + 1; }
+size_t sum_partials(int64_t n) { return (size_t)((n + kSumSlice - 1) / kSumSlice) + 1; }
 
-cudaError_t launch_sum(const double* v, int64_t n, double* partial, double* result,
-                       cudaStream_t s) {
-  const int64_t per = 65536;
-  const int nb = (int)std::max<int64_t>(1, (n + per - 1) / per);
-  k_sum_blocks<<<nb, 256, 0, s>>>(v, n, per, partial);
-  note_launches(1);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_sum_blocks<<<1, 256, 0, s>>>(partial, nb, nb, result);
-  note_launches(1);
+cudaError_t launch_sums(const SumJob* jobs, int count, cudaStream_t s) {
+  if (count < 1 || count > kMaxSums) return cudaErrorInvalidValue;
+  SumSet set = {};
+  int64_t most = 1;
+  for (int k = 0; k < count; ++k) {
+    set.job[k] = jobs[k];
+    most = std::max<int64_t>(most, (jobs[k].n + kSumSlice - 1) / kSumSlice);
+  }
+  k_sum_slices<<<dim3((unsigned)most, count), kSumThreads, 0, s>>>(set);
+  k_sum_totals<<<count, 256, 0, s>>>(set);
+  note_launches(2);
   return cudaGetLastError();
 }
 
@@ -294,9 +364,18 @@ cudaError_t launch_lscv(const float4* pts, const float* wts, int64_t n, const fl
   if (e != cudaSuccess) return e;
   if (n > 0) {
     const double self = 1.0 / (2.0 * 3.14159265358979323846) / ((double)n * h * h);
+    CellGauss cg = {};
+    cg.a = -0.5 * (cell / h) * (cell / h);
+    double term = 1.0;
+    int k = 0;
+    for (; k < kMaxTerms && fabs(term) >= 0x1p-56; ++k) {
+      cg.c[k] = term;
+      term *= cg.a / (k + 1);
+    }
+    cg.terms = fabs(term) < 0x1p-56 ? k : 0;
     k_lscv_points<<<grid_blocks(n, 256, 152 * 16), 256, 0, s>>>(
         pts, wts, n, F, nx, ny, h / cell, cell / h, 1.0 / cell, 1.0 / h, 1.0 / (double)n, self,
-        Gd, gw_direct, gxy_direct, loo, hdir);
+        cg, Gd, gw_direct, gxy_direct, loo, hdir);
     note_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

@@ -211,12 +211,18 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint64_t ehi = desc_swz(st, 2u, 1024u), elo = desc_swz(st + kEBytes, 2u, 1024u);
             const uint64_t thi = desc_swz(st + 2 * kEBytes, 2u, 1024u);
             const uint64_t tlo = desc_swz(st + 2 * kEBytes + kTBytes, 2u, 1024u);
+            // the small products first: a step's truncation is relative to the
+            // accumulator, which they leave nearly empty in the first stage
 #pragma unroll
             for (int k = 0; k < kK / 16; ++k) {
               const uint64_t dk = (uint64_t)(2 * k);
-              mma_f16(acc, ehi + dk, thi + dk, kIdesc, (ks == 0 && k == 0) ? 0u : 1u);
-              mma_f16(acc, ehi + dk, tlo + dk, kIdesc, 1u);
+              mma_f16(acc, ehi + dk, tlo + dk, kIdesc, (ks == 0 && k == 0) ? 0u : 1u);
               mma_f16(acc, elo + dk, thi + dk, kIdesc, 1u);
+            }
+#pragma unroll
+            for (int k = 0; k < kK / 16; ++k) {
+              const uint64_t dk = (uint64_t)(2 * k);
+              mma_f16(acc, ehi + dk, thi + dk, kIdesc, 1u);
             }
             mma_commit(&empty[s]);
           }

@@ -287,6 +287,10 @@ int sparse_sort_bin(int nx, int ny, int instances) {
 // per window cell and point).
 constexpr double kAdjointTcRatio = 0.006;
 
+// Points from which the adjoint's window form sorts them and works in groups:
+// below, the sort's launches cost more than the groups save.
+constexpr int64_t kAdjGroupPoints = 16384;
+
 // Tensor-core instances that share a tile shape and pipeline stage: one
 // persistent launch over their work items.
 struct TcFamily {
@@ -1262,31 +1266,61 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
     const double nxp = std::ceil(a->nx / 256.0) * 256.0, nyp = std::ceil(a->ny / 256.0) * 256.0;
     use_tc = win > kAdjointTcRatio * nxp * nyp;
   }
-  size_t off = 0;
-  auto take = [&](size_t bytes) { size_t r = off; off = align256(off + bytes); return r; };
-  const size_t o_scal = take(sizeof(CallScalars));
-  const size_t o_tab = take(sizeof(PrepInst));
-  const size_t o_pts = take(sizeof(float4) * n_pad);
-  const size_t o_wts = take(sizeof(float) * n_pad);
-  const size_t o_gxt = take(sizeof(float2) * a->nx);
-  const size_t o_gyt = take(sizeof(float2) * a->ny);
-  const size_t o_ht = take(sizeof(double) * a->n);
-  const size_t o_lt = take(sizeof(double) * a->n);
-  const size_t o_part = take(sizeof(double) * 2 * sum_partials(a->n));
-  const size_t o_res = take(sizeof(double) * 2);
-  const size_t o_tc = take(use_tc ? adjoint_tc_workspace(a->nx, a->ny) : 0);
+  // The window form in groups needs the points in bin order and the room for
+  // it; without that room the window kernel takes one point at a time.
+  const int R = adj_group_radius(a->cell, a->h);
+  const CutoffGeom geo = cutoff_geometry(a->nx, a->ny, a->cell / a->h, 8.0, kAdjBin);
+  bool group = !use_tc && adj_group_fits(R) && a->n >= kAdjGroupPoints;
+  const CutoffSizes cz = group ? cutoff_sizes(n_pad, geo.nbins) : CutoffSizes{};
+  struct {
+    size_t scal, tab, cut, pts, wts, gxt, gyt, ht, lt, res, tc;
+    size_t keys[2], vals[2], hist, start, spts, sw, list, ctr;
+  } o = {};
+  auto layout = [&]() {
+    size_t off = 0;
+    auto take = [&](size_t bytes) { size_t r = off; off = align256(off + bytes); return r; };
+    o.scal = take(sizeof(CallScalars));
+    o.tab = take(sizeof(PrepInst));
+    if (group) o.cut = take(sizeof(CutInst));
+    o.pts = take(sizeof(float4) * n_pad);
+    o.wts = take(sizeof(float) * n_pad);
+    o.gxt = take(sizeof(float2) * a->nx);
+    o.gyt = take(sizeof(float2) * a->ny);
+    o.ht = take(sizeof(double) * a->n);
+    o.lt = take(sizeof(double) * a->n);
+    o.res = take(sizeof(double) * 2);
+    o.tc = take(use_tc ? adjoint_tc_workspace(a->nx, a->ny) : 0);
+    if (group) {
+      const size_t u = sizeof(uint32_t);
+      for (int k = 0; k < 2; ++k) {
+        o.keys[k] = take(u * n_pad);
+        o.vals[k] = take(u * n_pad);
+      }
+      o.hist = take(u * cz.hist_words);
+      o.start = take(u * ((size_t)geo.nbins + 1));
+      o.spts = take(sizeof(float4) * n_pad);
+      o.sw = take(sizeof(float) * n_pad);
+      o.list = take(sizeof(int4) * ((size_t)n_pad / kAdjGroup + geo.nbins + 2));
+      o.ctr = take(u * 2);
+    }
+    return off;
+  };
   void* wsv = nullptr;
-  rc = acquire_workspace(opts, off, s, &wsv);
+  rc = acquire_workspace(opts, layout(), s, &wsv);
+  if (rc == KDE_ENOMEM && group) {
+    group = false;
+    rc = acquire_workspace(opts, layout(), s, &wsv);
+  }
   if (rc) return rc;
   char* base = static_cast<char*>(wsv);
   PrepInst q = {};
   q.xy = a->points;
   q.w = a->weights;
-  q.pts = reinterpret_cast<float4*>(base + o_pts);
-  q.wts = reinterpret_cast<float*>(base + o_wts);
-  q.gxt = reinterpret_cast<float2*>(base + o_gxt);
-  q.gyt = reinterpret_cast<float2*>(base + o_gyt);
-  q.scal = reinterpret_cast<CallScalars*>(base + o_scal);
+  q.pts = reinterpret_cast<float4*>(base + o.pts);
+  q.wts = reinterpret_cast<float*>(base + o.wts);
+  q.gxt = reinterpret_cast<float2*>(base + o.gxt);
+  q.gyt = reinterpret_cast<float2*>(base + o.gyt);
+  q.scal = reinterpret_cast<CallScalars*>(base + o.scal);
   q.n = a->n;
   q.n_pad = n_pad;
   q.begin = 0;
@@ -1296,21 +1330,83 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
   set_scale(q, use_tc ? kernel_sigma(KDE_GAUSSIAN, a->h) : 1.0 / a->h, a->cell, nullptr);
   q.nx = a->nx;
   q.ny = a->ny;
-  double* ht = reinterpret_cast<double*>(base + o_ht);
-  double* lt = reinterpret_cast<double*>(base + o_lt);
-  double* part = reinterpret_cast<double*>(base + o_part);
-  double* res = reinterpret_cast<double*>(base + o_res);
-  KDE_CUDA(upload_single(q, s), "upload tables");
-  KDE_CUDA(launch_prepare(reinterpret_cast<PrepInst*>(base + o_tab), 1, n_pad,
+  double* ht = reinterpret_cast<double*>(base + o.ht);
+  double* lt = reinterpret_cast<double*>(base + o.lt);
+  double* part = reinterpret_cast<double*>(q.pts);  // done with when the sums run
+  double* res = reinterpret_cast<double*>(base + o.res);
+  if (group) {
+    CutInst ci = {};
+    ci.n = a->n;
+    ci.n_pad = n_pad;
+    ci.inv_binw = geo.inv_binw;
+    ci.ext_x = geo.ext_x;
+    ci.ext_y = geo.ext_y;
+    ci.reach = 8.0;
+    ci.range_reach = range_reach(8.0, geo);
+    ci.cs = a->cell / a->h;
+    set_key_constants(ci);
+    ci.nbx = geo.nbx;
+    ci.nby = geo.nby;
+    ci.nx = a->nx;
+    ci.ny = a->ny;
+    ci.kid = KDE_GAUSSIAN;
+    std::vector<unsigned char> up(o.pts - o.scal, 0);
+    memcpy(up.data() + (o.tab - o.scal), &q, sizeof(q));
+    memcpy(up.data() + (o.cut - o.scal), &ci, sizeof(ci));
+    KDE_CUDA(launch_upload(up.data(), up.size(), q.scal, s), "upload tables");
+  } else {
+    KDE_CUDA(upload_single(q, s), "upload tables");
+  }
+  KDE_CUDA(launch_prepare(reinterpret_cast<PrepInst*>(base + o.tab), 1, n_pad,
                           std::max(a->nx, a->ny), s),
            "prepare points");
+  const int sms = sm_count();
   if (use_tc) {
-    const int sms = sm_count();
     const int ctas = (opts && opts->max_ctas > 0) ? std::min(opts->max_ctas, sms) : sms;
     KDE_CUDA(launch_adjoint_gauss_tc(q.pts, q.wts, a->n, grad_out, q.gxt, q.gyt, a->nx, a->ny,
                                      a->cell, a->h, grad_points, grad_weights, ht, lt,
-                                     base + o_tc, ctas, s),
+                                     base + o.tc, ctas, s),
              "adjoint contractions");
+  } else if (group) {
+    CutoffScratch cs = {};
+    for (int k = 0; k < 2; ++k) {
+      cs.keys[k] = reinterpret_cast<uint32_t*>(base + o.keys[k]);
+      cs.vals[k] = reinterpret_cast<uint32_t*>(base + o.vals[k]);
+    }
+    cs.hist = reinterpret_cast<uint32_t*>(base + o.hist);
+    cs.start = reinterpret_cast<uint32_t*>(base + o.start);
+    cs.spts = reinterpret_cast<float4*>(base + o.spts);
+    cs.sw = reinterpret_cast<float*>(base + o.sw);
+    cs.err = q.scal;
+    KDE_CUDA(launch_bin_sort(reinterpret_cast<CutInst*>(base + o.cut), 1, n_pad, geo.nbins, q.pts,
+                             q.wts, cz, cs, s, true),
+             "bin sort");
+    AdjGroupArgs g = {};
+    g.pts = cs.spts;
+    g.wts = cs.sw;
+    g.vals = cs.vals[cz.passes & 1];
+    g.start = cs.start;
+    g.n = a->n;
+    g.m = n_pad;
+    g.nbx = geo.nbx;
+    g.nbins = geo.nbins;
+    g.nx = a->nx;
+    g.ny = a->ny;
+    g.R = R;
+    g.sms = sms;
+    g.list = reinterpret_cast<int4*>(base + o.list);
+    g.counters = reinterpret_cast<uint32_t*>(base + o.ctr);
+    g.G = grad_out;
+    g.gxt = q.gxt;
+    g.gyt = q.gyt;
+    g.c = (float)(1.0 / (2.0 * 3.14159265358979323846 * (double)a->n * a->h * a->h));
+    g.inv_h = (float)(1.0 / a->h);
+    g.grad_xy = grad_points;
+    g.grad_w = grad_weights;
+    g.hterm = ht;
+    g.lterm = lt;
+    g.err = q.scal;
+    KDE_CUDA(launch_adjoint_group(g, s), "adjoint");
   } else {
     KDE_CUDA(launch_adjoint_gauss(q.pts, q.wts, a->n, grad_out, q.gxt, q.gyt, a->nx, a->ny,
                                   a->cell, a->h, grad_points, grad_weights, ht, lt, s),
@@ -1319,27 +1415,23 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
   const bool sync = grad_h || (opts && (opts->flags & KDE_FLAG_SYNC));
   if (grad_h) {
     const size_t np = sum_partials(a->n);
-    KDE_CUDA(launch_sum(ht, a->n, part, res, s), "sum");
-    KDE_CUDA(launch_sum(lt, a->n, part + np, res + 1, s), "sum");
+    const SumJob jobs[2] = {{ht, a->n, part, res}, {lt, a->n, part + np, res + 1}};
+    KDE_CUDA(launch_sums(jobs, 2, s), "sum");
   }
   if (sync) {
     double hres[2] = {0.0, 0.0};
-    int err = 0, err_tc = 0, where = 0;
+    CallScalars hs = {}, ts = {};
     if (grad_h)
       KDE_CUDA(cudaMemcpyAsync(hres, res, sizeof(hres), cudaMemcpyDeviceToHost, s), "read result");
-    KDE_CUDA(cudaMemcpyAsync(&err, &q.scal->err, sizeof(int), cudaMemcpyDeviceToHost, s),
-             "read status");
-    if (use_tc) {
-      const CallScalars* ts = reinterpret_cast<const CallScalars*>(base + o_tc);
-      KDE_CUDA(cudaMemcpyAsync(&err_tc, &ts->err, sizeof(int), cudaMemcpyDeviceToHost, s),
+    KDE_CUDA(cudaMemcpyAsync(&hs, q.scal, sizeof(hs), cudaMemcpyDeviceToHost, s), "read status");
+    if (use_tc)
+      KDE_CUDA(cudaMemcpyAsync(&ts, base + o.tc, sizeof(ts), cudaMemcpyDeviceToHost, s),
                "read status");
-      KDE_CUDA(cudaMemcpyAsync(&where, &ts->timeout_where, sizeof(int), cudaMemcpyDeviceToHost, s),
-               "read status");
-    }
     KDE_CUDA(cudaStreamSynchronize(s), "synchronize");
-    if (err & kErrNonFinite) return fail(KDE_EDATA, "non-finite coordinate or weight");
-    if (err_tc & kErrTimeout)
-      return fail(KDE_ETIMEOUT, "a device-side wait of the adjoint gave up (role %d)", where);
+    if (hs.err & kErrNonFinite) return fail(KDE_EDATA, "non-finite coordinate or weight");
+    if ((hs.err | ts.err) & kErrTimeout)
+      return fail(KDE_ETIMEOUT, "a device-side wait of the adjoint gave up (role %d)",
+                  hs.err & kErrTimeout ? hs.timeout_where : ts.timeout_where);
     // dL/dh = -(2/h) sum G F + sum_p h-terms, with sum G F = sum_p w_p dL/dw_p
     if (grad_h) *grad_h = -2.0 / a->h * hres[1] + hres[0];
   }
@@ -1380,7 +1472,6 @@ int kde_lscv_grid(const kde_args* a, const float* F, double* loss, float* grad_F
   const size_t o_hd = take(sizeof(double) * std::max<int64_t>(n, 1));
   const size_t o_sq = take(sizeof(double) * sq_blocks);
   const size_t o_gd = take(grad_F ? sizeof(double) * (size_t)a->nx * a->ny : 0);
-  const size_t o_part = take(sizeof(double) * 3 * (sum_partials(std::max<int64_t>(n, sq_blocks)) + 1));
   const size_t o_res = take(sizeof(double) * 4);
   void* wsv = nullptr;
   rc = acquire_workspace(opts, off, s, &wsv);
@@ -1405,7 +1496,7 @@ int kde_lscv_grid(const kde_args* a, const float* F, double* loss, float* grad_F
   double* loo = reinterpret_cast<double*>(base + o_loo);
   double* hd = reinterpret_cast<double*>(base + o_hd);
   double* sq = reinterpret_cast<double*>(base + o_sq);
-  double* part = reinterpret_cast<double*>(base + o_part);
+  double* part = reinterpret_cast<double*>(q.pts);  // done with when the sums run
   double* res = reinterpret_cast<double*>(base + o_res);
   const size_t np = sum_partials(std::max<int64_t>(n, sq_blocks)) + 1;
   KDE_CUDA(upload_single(q, s), "upload tables");
@@ -1417,11 +1508,10 @@ int kde_lscv_grid(const kde_args* a, const float* F, double* loss, float* grad_F
                        grad_F ? reinterpret_cast<double*>(base + o_gd) : nullptr, grad_F,
                        grad_w_direct, grad_points_direct, sq, sq_blocks, loo, hd, s),
            "LSCV");
-  KDE_CUDA(launch_sum(sq, sq_blocks, part, res, s), "sum");
-  if (n > 0) {
-    KDE_CUDA(launch_sum(loo, n, part + np, res + 1, s), "sum");
-    KDE_CUDA(launch_sum(hd, n, part + 2 * np, res + 2, s), "sum");
-  }
+  const SumJob jobs[3] = {{sq, sq_blocks, part, res},
+                          {loo, n, part + np, res + 1},
+                          {hd, n, part + 2 * np, res + 2}};
+  KDE_CUDA(launch_sums(jobs, n > 0 ? 3 : 1, s), "sum");
   double hres[4];
   int err = 0;
   KDE_CUDA(cudaMemcpyAsync(hres, res, sizeof(hres), cudaMemcpyDeviceToHost, s), "read result");

@@ -156,7 +156,8 @@ __device__ __forceinline__ unsigned long long status_word(int pass, bool incl, u
 // per-digit counts, then walks back over earlier chunks until it meets an
 // inclusive prefix, publishes its own inclusive prefix and scatters: position
 // = (keys of smaller digits) + (same digit in earlier chunks) + rank.  The
-// last pass writes the permuted points and weights instead of the indices.
+// last pass writes the permuted points and weights instead of the indices
+// (last = 1), or beside them (2).
 // A wait that does not end within the limit records a timeout in err; the
 // positions are then bounded, not correct.
 __global__ void __launch_bounds__(kSortThreads)
@@ -261,6 +262,7 @@ __global__ void __launch_bounds__(kSortThreads)
     if (last) {
       spts[pos] = prepared[v];
       sw[pos] = wts[v];
+      if (last == 2) vals_out[pos] = v;
     } else {
       vals_out[pos] = v;
     }
@@ -817,7 +819,7 @@ CutoffSizes cutoff_sizes(int64_t m, int64_t total_bins) {
 
 cudaError_t launch_bin_sort(const CutInst* tab, int ninst, int64_t m, int64_t total_bins,
                             const float4* prepared, const float* prepared_w, const CutoffSizes& z,
-                            CutoffScratch ws, cudaStream_t s) {
+                            CutoffScratch ws, cudaStream_t s, bool indices) {
   if (ninst <= 0 || m <= 0) return cudaSuccess;
   if (z.passes < 1 || z.passes > kMaxPasses) return cudaErrorInvalidValue;
   unsigned long long* status = reinterpret_cast<unsigned long long*>(ws.hist);
@@ -831,7 +833,7 @@ cudaError_t launch_bin_sort(const CutInst* tab, int ninst, int64_t m, int64_t to
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   int cur = 0;
   for (int pass = 0; pass < z.passes; ++pass) {
-    const int last = pass == z.passes - 1;
+    const int last = pass == z.passes - 1 ? (indices ? 2 : 1) : 0;
     k_radix_pass<<<z.nchunks, kSortThreads, 0, s>>>(ws.keys[cur], ws.vals[cur], m, pass,
                                                     8 * z.passes, ghist, chunk_ctr, status,
                                                     ws.keys[cur ^ 1],

@@ -391,9 +391,11 @@ CutoffSizes cutoff_sizes(int64_t m, int64_t total_bins);
 // 8-bit pass is then one kernel whose chunk offsets come from a decoupled
 // look-back (bounded waits, recorded in ws.err); the last pass writes the
 // permuted points.  ws.hist holds z.hist_words words of look-back state.
+// With indices, the last pass also leaves the points' indices in the prepared
+// arrays in ws.vals[z.passes & 1].
 cudaError_t launch_bin_sort(const CutInst* tab, int ninst, int64_t m, int64_t total_bins,
                             const float4* prepared, const float* prepared_w, const CutoffSizes& z,
-                            CutoffScratch ws, cudaStream_t s);
+                            CutoffScratch ws, cudaStream_t s, bool indices = false);
 // The bounded wait of the sort's look-back, made to run out: one radix pass
 // over two chunks of zero keys runs as the second chunk while the first never
 // publishes, so it gives up after limit_ns and records a timeout (role 31) in
@@ -413,6 +415,29 @@ cudaError_t launch_adjoint_gauss(const float4* pts, const float* wts, int64_t n,
                                  const float2* gxt, const float2* gyt, int nx, int ny,
                                  double cell, double h, float* grad_xy, float* grad_w,
                                  double* hterm, double* lterm, cudaStream_t s);
+// The same for points sorted into kAdjBin-cell bins (launch_bin_sort with their
+// indices): groups of kAdjGroup points of a bin share their window.
+constexpr int kAdjBin = 8, kAdjGroup = 64;
+struct AdjGroupArgs {
+  const float4* pts;        // in bin order, offsets in bandwidths
+  const float* wts;
+  const uint32_t* vals;     // the caller's index of each
+  const uint32_t* start;    // bin starts; start[nbins]: first point beyond reach
+  int64_t n, m;             // points, and with the padding
+  int nbx, nbins, nx, ny, R, sms;
+  int4* list;               // [m / kAdjGroup + nbins + 2]
+  uint32_t* counters;       // [2]
+  const float* G;
+  const float2 *gxt, *gyt;
+  float c, inv_h;           // 1/(2 pi n h^2), 1/h
+  float* grad_xy;
+  float* grad_w;
+  double *hterm, *lterm;    // [m], in bin order
+  const CallScalars* err;
+};
+int adj_group_radius(double cell, double h);  // window half-width R, cells
+bool adj_group_fits(int R);
+cudaError_t launch_adjoint_group(const AdjGroupArgs& a, cudaStream_t s);
 // The same adjoint as two tcgen05 contractions (points prepared in the
 // Gaussian's units, sigma = 1/(h sqrt(2 ln 2)), and their cell tables):
 // U = G B and V = G^T A with the points' operands generated on chip.  ws:
@@ -430,11 +455,16 @@ cudaError_t launch_lscv(const float4* pts, const float* wts, int64_t n, const fl
                         int ny, double cell, double h, double* Gd, float* G, float* gw_direct,
                         float* gxy_direct, double* sq_part, int sq_blocks, double* loo,
                         double* hdir, cudaStream_t s);
-// Fixed-order sum of n doubles into *result (device); partial needs
-// sum_partials(n) doubles.
+// Fixed-order sums of up to three arrays of doubles into *result (device);
+// partial: sum_partials(n) doubles.
+struct SumJob {
+  const double* v;
+  int64_t n;
+  double* partial;
+  double* result;
+};
 size_t sum_partials(int64_t n);
-cudaError_t launch_sum(const double* v, int64_t n, double* partial, double* result,
-                       cudaStream_t s);
+cudaError_t launch_sums(const SumJob* jobs, int count, cudaStream_t s);
 
 // The paper's binned estimator: count matrix with interpolation (Algorithm 3)
 // and the separable window x window convolution of Eq. 7.

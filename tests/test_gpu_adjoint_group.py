@@ -1,0 +1,106 @@
+"""The adjoint's window form in groups of sorted points: against the FP64 oracle
+and against the one-point form (which a workspace without room for the sort
+still takes), at the edges of the groups, the bins, the thread tiles (window
+half-widths 12, 28 and 44) and the grid."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from kde_testutil import TOL_GRAD, rel_linf
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2004_13653_gb300 as kde  # noqa: E402
+
+# two FP32 evaluations of sums of up to 96 x 96 products each: 2 sqrt(2 x 96)
+# roundings of 2^-24 relative to the largest value, with a margin of six
+SAME = 1e-5
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    kde.load(build_if_stale=True)
+
+
+def dev(a, dt):
+    return torch.as_tensor(np.ascontiguousarray(a), dtype=dt, device="cuda")
+
+
+def backward(wl, w, G, workspace=None, want_w=True):
+    pts, grad = dev(wl.xy, torch.float64), dev(G, torch.float32)
+    wt = None if w is None else dev(w, torch.float32)
+    gxy = torch.full((wl.n, 2), float("nan"), device="cuda")
+    gw = torch.full((wl.n,), float("nan"), device="cuda")
+    gh = ctypes.c_double(0.0)
+    a = kde.make_args(pts, wt, wl.origin, wl.cell, wl.nx, wl.ny, wl.h, "gaussian", grad)
+    o = kde.make_opts("simt", 0, torch.cuda.current_stream(), workspace)
+    kde.check(kde.load().kde_grid_backward(
+        ctypes.byref(a), grad.data_ptr(), gxy.data_ptr(), gw.data_ptr() if want_w else None,
+        ctypes.byref(gh), ctypes.byref(o)))
+    return gxy.cpu().numpy(), gw.cpu().numpy(), gh.value
+
+
+def one_point_workspace(wl):
+    """What the call needs without the sort: 20 bytes per padded point, 16 per
+    point of FP64 terms, the tables."""
+    pad = (wl.n + 511) // 512 * 512
+    size = 1024 + 20 * pad + 16 * wl.n + 8 * (wl.nx + wl.ny) + 10 * 256
+    return torch.empty(size, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("n,nx,ny,h_cells", [
+    (16384, 96, 80, 1.3),     # R = 12: the smallest thread tile
+    (16385, 97, 81, 1.4),     # R = 13: one cell more
+    (20000, 160, 120, 3.3),   # R = 28
+    (20001, 161, 121, 3.4),   # R = 29
+    (17000, 256, 203, 5.3),   # R = 44: the largest window
+    (17000, 256, 203, 5.4),   # R = 45: one point at a time
+    (30000, 40, 9, 2.0),      # windows wider than the grid, hundreds of points per bin
+    (16400, 3, 500, 1.0),
+])
+def test_matches_one_point_form_and_oracle(n, nx, ny, h_cells):
+    wl = workloads.random_points(31, n, 10.0 * max(nx, ny), 10.0, nx, ny, 10.0 * h_cells,
+                                 oracle.GAUSSIAN)
+    wl.w[::5] *= -1.0
+    G = np.random.default_rng(1).normal(0, 1, (ny, nx))
+    gxy, gw, gh = backward(wl, wl.w, G)
+    sxy, sw, sh = backward(wl, wl.w, G, workspace=one_point_workspace(wl))
+    assert rel_linf(gxy, sxy) <= SAME and rel_linf(gw, sw) <= SAME
+    assert gh == pytest.approx(sh, rel=1e-4)
+    sel = np.random.default_rng(2).choice(n, 300, replace=False)
+    sub = wl.xy[sel]
+    rw, rxy, _ = oracle.kde_vjp_gauss(sub, wl.w[sel], wl.origin, wl.cell, nx, ny, wl.h, G)
+    scale = len(sel) / n  # the density's 1/N
+    assert rel_linf(gw[sel], rw * scale) <= TOL_GRAD
+    assert rel_linf(gxy[sel], rxy * scale) <= TOL_GRAD
+
+
+def test_clusters_empty_bins_far_points_and_missing_outputs():
+    """Bins with 1, 64, 65 and thousands of points, points out of every cell's
+    reach (exact zeros), unit weights, no weight gradient."""
+    rng = np.random.default_rng(7)
+    parts = [np.full((64, 2), 405.0) + rng.random((64, 2)), np.full((65, 2), 885.0) + rng.random((65, 2)),
+             np.array([[1200.0, 300.0]]), rng.normal(700.0, 30.0, (16500, 2)),
+             np.array([[-900.0, 100.0], [5000.0, 700.0], [100.0, 9e5]])]
+    local = np.concatenate(parts)
+    n = len(local)
+    wl = workloads.Workload("clusters", local, np.ones(n, np.float32), 1280.0, 10.0, 128, 110, 20.0,
+                            oracle.GAUSSIAN, np.array([0, n]), 0)
+    G = rng.normal(0, 1, (110, 128))
+    gxy, gw, gh = backward(wl, None, G)
+    sxy, sw, sh = backward(wl, None, G, workspace=one_point_workspace(wl))
+    assert not gxy[-3:].any() and not gw[-3:].any()
+    assert rel_linf(gxy, sxy) <= SAME and rel_linf(gw, sw) <= SAME
+    assert gh == pytest.approx(sh, rel=1e-4)
+    again = backward(wl, None, G)
+    np.testing.assert_array_equal(again[0], gxy)
+    assert again[2] == gh
+    nxy, nw, _ = backward(wl, None, G, want_w=False)
+    np.testing.assert_array_equal(nxy, gxy)
+    assert np.isnan(nw).all()
