@@ -287,6 +287,21 @@ int sparse_sort_bin(int nx, int ny, int instances) {
 // per window cell and point).
 constexpr double kAdjointTcRatio = 0.006;
 
+// The contraction form of the adjoint sorts its points into bins of about one
+// tile of points each (8 to 64 cells a side) where that leaves a tile less
+// than two thirds of the grid.
+int adj_tc_bin(const kde_args* a) {
+  const double side = std::sqrt(128.0 * (double)a->nx * a->ny / (double)std::max<int64_t>(a->n, 1));
+  int bin = 8;
+  while (bin < 64 && bin < side) bin *= 2;
+  return bin;
+}
+bool adj_tc_sorts(const kde_args* a) {
+  const double span = 16.0 * a->h / a->cell + adj_tc_bin(a) + 64.0;  // cells, rounded up to steps
+  return a->n >= 4096 && std::min(span, (double)a->nx) * std::min(span, (double)a->ny) <
+                             0.67 * (double)a->nx * (double)a->ny;
+}
+
 // Points from which the adjoint's window form sorts them and works in groups:
 // below, the sort's launches cost more than the groups save.
 constexpr int64_t kAdjGroupPoints = 16384;
@@ -1266,11 +1281,16 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
     const double nxp = std::ceil(a->nx / 256.0) * 256.0, nyp = std::ceil(a->ny / 256.0) * 256.0;
     use_tc = win > kAdjointTcRatio * nxp * nyp;
   }
-  // The window form in groups needs the points in bin order and the room for
-  // it; without that room the window kernel takes one point at a time.
+  // The window form in groups, and the contractions over the cells near each
+  // tile of points, need the points in bin order and the room for it; without
+  // that room the window kernel takes one point at a time, the contractions
+  // the whole grid.
   const int R = adj_group_radius(a->cell, a->h);
-  const CutoffGeom geo = cutoff_geometry(a->nx, a->ny, a->cell / a->h, 8.0, kAdjBin);
-  bool group = !use_tc && adj_group_fits(R) && a->n >= kAdjGroupPoints;
+  const double sigma = use_tc ? kernel_sigma(KDE_GAUSSIAN, a->h) : 1.0 / a->h;
+  const double reach = use_tc ? kAdjTcReach : 8.0;
+  const int bin = use_tc ? adj_tc_bin(a) : kAdjBin;
+  const CutoffGeom geo = cutoff_geometry(a->nx, a->ny, a->cell * sigma, reach, bin);
+  bool group = use_tc ? adj_tc_sorts(a) : adj_group_fits(R) && a->n >= kAdjGroupPoints;
   const CutoffSizes cz = group ? cutoff_sizes(n_pad, geo.nbins) : CutoffSizes{};
   struct {
     size_t scal, tab, cut, pts, wts, gxt, gyt, ht, lt, res, tc;
@@ -1300,7 +1320,8 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
       o.start = take(u * ((size_t)geo.nbins + 1));
       o.spts = take(sizeof(float4) * n_pad);
       o.sw = take(sizeof(float) * n_pad);
-      o.list = take(sizeof(int4) * ((size_t)n_pad / kAdjGroup + geo.nbins + 2));
+      o.list = take(use_tc ? adjoint_tc_ranges_bytes(a->n)
+                           : sizeof(int4) * ((size_t)n_pad / kAdjGroup + geo.nbins + 2));
       o.ctr = take(u * 2);
     }
     return off;
@@ -1327,7 +1348,7 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
   q.ox = a->origin_x;
   q.oy = a->origin_y;
   // offsets in bandwidths (window kernel) or in h sqrt(2 ln 2) (contractions)
-  set_scale(q, use_tc ? kernel_sigma(KDE_GAUSSIAN, a->h) : 1.0 / a->h, a->cell, nullptr);
+  set_scale(q, sigma, a->cell, nullptr);
   q.nx = a->nx;
   q.ny = a->ny;
   double* ht = reinterpret_cast<double*>(base + o.ht);
@@ -1341,9 +1362,9 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
     ci.inv_binw = geo.inv_binw;
     ci.ext_x = geo.ext_x;
     ci.ext_y = geo.ext_y;
-    ci.reach = 8.0;
-    ci.range_reach = range_reach(8.0, geo);
-    ci.cs = a->cell / a->h;
+    ci.reach = reach;
+    ci.range_reach = range_reach(reach, geo);
+    ci.cs = a->cell * sigma;
     set_key_constants(ci);
     ci.nbx = geo.nbx;
     ci.nby = geo.nby;
@@ -1361,14 +1382,8 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
                           std::max(a->nx, a->ny), s),
            "prepare points");
   const int sms = sm_count();
-  if (use_tc) {
-    const int ctas = (opts && opts->max_ctas > 0) ? std::min(opts->max_ctas, sms) : sms;
-    KDE_CUDA(launch_adjoint_gauss_tc(q.pts, q.wts, a->n, grad_out, q.gxt, q.gyt, a->nx, a->ny,
-                                     a->cell, a->h, grad_points, grad_weights, ht, lt,
-                                     base + o.tc, ctas, s),
-             "adjoint contractions");
-  } else if (group) {
-    CutoffScratch cs = {};
+  CutoffScratch cs = {};
+  if (group) {
     for (int k = 0; k < 2; ++k) {
       cs.keys[k] = reinterpret_cast<uint32_t*>(base + o.keys[k]);
       cs.vals[k] = reinterpret_cast<uint32_t*>(base + o.vals[k]);
@@ -1381,6 +1396,16 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
     KDE_CUDA(launch_bin_sort(reinterpret_cast<CutInst*>(base + o.cut), 1, n_pad, geo.nbins, q.pts,
                              q.wts, cz, cs, s, true),
              "bin sort");
+  }
+  if (use_tc) {
+    const int ctas = (opts && opts->max_ctas > 0) ? std::min(opts->max_ctas, sms) : sms;
+    KDE_CUDA(launch_adjoint_gauss_tc(group ? cs.spts : q.pts, group ? cs.sw : q.wts,
+                                     group ? cs.vals[cz.passes & 1] : nullptr,
+                                     group ? reinterpret_cast<int4*>(base + o.list) : nullptr,
+                                     group ? q.scal : nullptr, a->n, grad_out, q.gxt, q.gyt, a->nx, a->ny, a->cell, a->h,
+                                     grad_points, grad_weights, ht, lt, base + o.tc, ctas, s),
+             "adjoint contractions");
+  } else if (group) {
     AdjGroupArgs g = {};
     g.pts = cs.spts;
     g.wts = cs.sw;

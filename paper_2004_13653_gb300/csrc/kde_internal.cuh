@@ -444,9 +444,16 @@ cudaError_t launch_adjoint_group(const AdjGroupArgs& a, cudaStream_t s);
 // adjoint_tc_workspace(nx, ny) bytes (the cotangent's FP16 tiles and a status
 // word); errors of its waits are recorded in ws's CallScalars.
 size_t adjoint_tc_workspace(int nx, int ny);
-cudaError_t launch_adjoint_gauss_tc(const float4* pts, const float* wts, int64_t n, const float* G,
-                                    const float2* gxt, const float2* gyt, int nx, int ny,
-                                    double cell, double h, float* grad_xy, float* grad_w,
+// vals, ranges: the points in bin order with their indices, and
+// adjoint_tc_ranges_bytes(n) of scratch for each tile's cells, and the scalars
+// the sort reports to; or all null: the caller's order, every tile over the
+// whole grid.  hterm and lterm are in the order of pts.
+constexpr double kAdjTcReach = 6.8;  // +-8 bandwidths in units of h sqrt(2 ln 2)
+size_t adjoint_tc_ranges_bytes(int64_t n);
+cudaError_t launch_adjoint_gauss_tc(const float4* pts, const float* wts, const uint32_t* vals,
+                                    int4* ranges, const CallScalars* sort_err, int64_t n,
+                                    const float* G, const float2* gxt, const float2* gyt, int nx,
+                                    int ny, double cell, double h, float* grad_xy, float* grad_w,
                                     double* hterm, double* lterm, void* ws, int max_ctas,
                                     cudaStream_t s);
 // Gd: FP64 scratch for the cotangent (cells), G: FP32 cotangent out; loo and
