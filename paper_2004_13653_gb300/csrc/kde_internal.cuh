@@ -321,6 +321,7 @@ cudaError_t launch_prepare(const PrepInst* tab, int ninst, int64_t total_pad, in
 // Path (a): FP32 SIMT direct sum into part[S][ny][nx] (scaled).
 // scratch: simt_scratch_bytes(nx, ny, splits) of device memory for the
 // running sums, or nullptr to keep them in shared memory (fewer CTAs per SM).
+constexpr int kSimtCtasPerSm = 4;  // with scratch
 size_t simt_scratch_bytes(int nx, int ny, int splits);
 cudaError_t launch_simt(int kid, const float4* pts, const float* wts, int64_t n_pad,
                         const float2* gxt, const float2* gyt, int nx, int ny, int splits,

@@ -7,8 +7,7 @@
 // 8 x 8 cells (columns 4t..4t+3 and 64+4t..64+4t+3, eight consecutive rows):
 // per point two 16-byte reads of each table and 64 FMAs.  The tables are
 // double-buffered, so one barrier per batch separates a batch's tabulation
-// from its use; each point's table reads are issued while the previous
-// point's FMAs run, and the next batch's points are loaded into registers
+// from its use, and the next batch's points are loaded into registers
 // while the current batch is accumulated.  Points arrive in tiles of 256;
 // each thread sums one tile in registers and adds that partial into a
 // (hi, lo) running sum (in global scratch, or in shared memory for callers
@@ -46,10 +45,14 @@ __device__ __forceinline__ TableRow table_row(const float* KX, const float* KY, 
 
 // GRUN: the (hi, lo) running sums live in global scratch (64 KB per CTA,
 // touched once per 256 points, so they stay in L2), which leaves shared
-// memory to the tables and three CTAs per SM; otherwise in shared memory (two
-// CTAs per SM, for callers that give no scratch).
+// memory to the tables and four CTAs per SM; otherwise in shared memory (two
+// CTAs per SM, for callers that give no scratch).  Bound by instruction issue
+// (1.4 instructions per FMA) with the latencies four warps per scheduler leave
+// open: 1M points x 512^2 in 11.9 ms = 22 Tpair/s of 37; three CTAs per SM with
+// the next point's table row loaded ahead: 12.9 ms, packed two-lane FMAs (which
+// issue half as often, at three CTAs per SM): 14.5 ms.
 template <int KID, bool GRUN>
-__global__ void __launch_bounds__(kThreads, GRUN ? 3 : 2)
+__global__ void __launch_bounds__(kThreads, GRUN ? kSimtCtasPerSm : 2)
     k_simt(const float4* __restrict__ pts, const float* __restrict__ wts, int64_t n_pad,
            int64_t per_split, const float2* __restrict__ gxt, const float2* __restrict__ gyt,
            int nx, int ny, float scale, float2* __restrict__ grun, float* __restrict__ part) {
@@ -136,11 +139,9 @@ __global__ void __launch_bounds__(kThreads, GRUN ? 3 : 2)
       }
       __syncthreads();
       fetch(base + bb + kBatch);
-      TableRow cur = table_row(KX, KY, 0, tx, ty);
 #pragma unroll 4
       for (int q = 0; q < kBatch; ++q) {
-        TableRow nxt = cur;
-        if (q + 1 < kBatch) nxt = table_row(KX, KY, q + 1, tx, ty);
+        const TableRow cur = table_row(KX, KY, q, tx, ty);
         const float kx[8] = {cur.xa.x, cur.xa.y, cur.xa.z, cur.xa.w,
                              cur.xb.x, cur.xb.y, cur.xb.z, cur.xb.w};
         const float ky[8] = {cur.ya.x, cur.ya.y, cur.ya.z, cur.ya.w,
@@ -149,7 +150,6 @@ __global__ void __launch_bounds__(kThreads, GRUN ? 3 : 2)
         for (int b = 0; b < 8; ++b)
 #pragma unroll
           for (int a = 0; a < 8; ++a) acc[b][a] = fmaf(kx[a], ky[b], acc[b][a]);
-        cur = nxt;
       }
     }
     // this tile's partials into the running sums; after the last tile the
