@@ -822,13 +822,69 @@ void set_key_constants(CutInst& q) {
   q.key_inv = (float)q.inv_binw;
 }
 
+// Whether the call names nothing of how its Gaussian density is computed: no
+// path, tiling, cap on the CTAs, or workspace.
+bool plain_gauss(const kde_args* a, const kde_opts* o) {
+  return kid_of(a) == KDE_GAUSSIAN &&
+         (!o || (o->path == KDE_PATH_AUTO && !o->tile_n && !o->k_chunk && !o->split_k &&
+                 !o->stage_points && !o->max_ctas && !o->workspace &&
+                 !(o->flags & (KDE_FLAG_CTA_PAIR | KDE_FLAG_ONE_CTA | KDE_FLAG_SKIP_ZERO))));
+}
+
+// A small Gaussian density on device buffers: one launch, no scratch (but for
+// the status word of a synchronous call).
+int run_small_gauss(const kde_args* a, const kde_opts* o, bool sync) {
+  cudaStream_t s = stream_of(o);
+  PrepInst q = {};
+  q.xy = a->points;
+  q.w = a->weights;
+  q.n = a->n;
+  q.ox = a->origin_x;
+  q.oy = a->origin_y;
+  MercParams merc;
+  const bool lonlat = o && (o->flags & KDE_FLAG_LONLAT);
+  if (lonlat) merc = mercator_params(o->lat0_deg);
+  set_scale(q, kernel_sigma(KDE_GAUSSIAN, a->h), a->cell, lonlat ? &merc : nullptr);
+  q.nx = a->nx;
+  q.ny = a->ny;
+  CallScalars* scal = nullptr;
+  if (sync) {
+    void* wsv = nullptr;
+    int rc = acquire_workspace(o, sizeof(CallScalars), s, &wsv);
+    if (rc) return rc;
+    scal = static_cast<CallScalars*>(wsv);
+    KDE_CUDA(cudaMemsetAsync(scal, 0, sizeof(CallScalars), s), "clear scalars");
+  }
+  const float scale =
+      (float)(1.0 / (2.0 * 3.14159265358979323846 * (double)a->n * a->h * a->h));
+  cudaEvent_t* ev = o ? static_cast<cudaEvent_t*>(o->timing_events) : nullptr;
+  if (ev) KDE_CUDA(cudaEventRecord(ev[0], s), "record start event");
+  KDE_CUDA(launch_small_gauss(q, scale, a->out, scal, sm_count(), s), "small density");
+  if (ev) KDE_CUDA(cudaEventRecord(ev[1], s), "record end event");
+  if (sync) {
+    CallScalars hs;
+    KDE_CUDA(cudaMemcpyAsync(&hs, scal, sizeof(hs), cudaMemcpyDeviceToHost, s), "read status");
+    KDE_CUDA(cudaStreamSynchronize(s), "synchronize");
+    if (hs.err & kErrNonFinite)
+      return fail(KDE_EDATA, "instance 0: non-finite coordinate or weight");
+  }
+  g_err[0] = 0;
+  return KDE_OK;
+}
+
 // Plan, lay out, upload and launch every instance of a batch on one stream.
+// single: the call is one density (not a batch of one, which is computed like
+// an instance of any batch).
 int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling* tiles,
-              bool force_sync) {
+              bool force_sync, bool single = false) {
   for (int k = 0; k < count; ++k) {
     int rc = validate(&A[k], o);
     if (rc) return rc;
   }
+  if (single && plain_gauss(A, o) && small_gauss_fits(A->n, A->nx, A->ny) &&
+      memory_kind(A->points) == 0 && (!A->weights || memory_kind(A->weights) == 0) &&
+      memory_kind(A->out) == 0)
+    return run_small_gauss(A, o, force_sync || (o && (o->flags & KDE_FLAG_SYNC)));
   BatchPlan P;
   int rc = make_plan(A, count, o, tiles, true, true, &P);
   // AUTO's block-sparse plan is a choice: where its work list or workspace is
@@ -1206,14 +1262,14 @@ int kde_grid(const double* points, const float* weights, int64_t n, const double
   kde_opts o;
   kde_default_opts(&o);
   o.stream = g_plain_stream;
-  return run_batch(&a, 1, &o, nullptr, true);
+  return run_batch(&a, 1, &o, nullptr, true, true);
 }
 
 void kde_set_stream(void* stream) { g_plain_stream = stream; }
 
 int kde_grid_ex(const kde_args* a, const kde_opts* opts) {
   if (!a) return fail(KDE_EINVAL, "args is NULL");
-  return run_batch(a, 1, opts, nullptr, false);
+  return run_batch(a, 1, opts, nullptr, false, true);
 }
 
 int kde_workspace_size(const kde_args* a, const kde_opts* opts, size_t* bytes) {

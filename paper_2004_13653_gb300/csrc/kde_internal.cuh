@@ -327,6 +327,12 @@ cudaError_t launch_simt(int kid, const float4* pts, const float* wts, int64_t n_
                         const float2* gxt, const float2* gyt, int nx, int ny, int splits,
                         float scale, float2* scratch, float* part, cudaStream_t s);
 
+// Small Gaussian densities (kde_small.cu): q as for the prepare kernel, without
+// its tables and scalars; scal: where non-finite input is recorded, or null.
+bool small_gauss_fits(int64_t n, int nx, int ny);
+cudaError_t launch_small_gauss(const PrepInst& q, float scale, float* out, CallScalars* scal,
+                               int sms, cudaStream_t s);
+
 // Sum each instance's S partial grids in fixed order (s = 0, 1, ...).
 cudaError_t launch_reduce(const ReduceInst* tab, int ninst, int64_t total_cells, cudaStream_t s);
 

@@ -79,7 +79,8 @@ def test_matches_dense_and_oracle(n, nx, ny, h_cells, weights):
 
 
 def test_wide_bandwidth_and_small_grids_stay_dense():
-    for wl in (case(40_000, 300, 280, 40.0), case(2000, 64, 64, 0.6), case(500, 900, 900, 2.0)):
+    # (at most 6e7 point-cell pairs of at most 16384 points go to neither)
+    for wl in (case(40_000, 300, 280, 40.0), case(20_000, 64, 64, 0.6), case(500, 900, 900, 2.0)):
         pts, w = on_device(wl)
         a = density(wl, pts, w).cpu().numpy()
         d = density(wl, pts, w, path="tc_split16").cpu().numpy()
