@@ -257,40 +257,48 @@ constexpr double kSparseReach = 6.45;
 double sparse_reach_cells(const kde_args* a) {
   return kSparseReach / (a->cell * kernel_sigma(KDE_GAUSSIAN, a->h));
 }
-double sparse_tiles_per_point(double reach_cells, int bin, int tiles) {
-  return std::min((double)tiles, (256.0 + 2.0 * reach_cells + bin) / 256.0);
+double sparse_tiles_per_point(double reach_cells, int bin, int tiles, int side) {
+  return std::min((double)tiles, (side + 2.0 * reach_cells + bin) / side);
 }
-double sparse_tiles_average(double reach_cells, int bin, int n, int tiles) {
+double sparse_tiles_average(double reach_cells, int bin, int n, int tiles, int side) {
   double cells = 0.0;  // of the axis that lie within each tile's reach
   for (int t = 0; t < tiles; ++t) {
-    const double lo = std::max(0.0, 256.0 * t - reach_cells - bin);
-    const double hi = std::min((double)n, 256.0 * (t + 1) + reach_cells);
+    const double lo = std::max(0.0, (double)side * t - reach_cells - bin);
+    const double hi = std::min((double)n, (double)side * (t + 1) + reach_cells);
     cells += std::max(0.0, hi - lo);
   }
   return cells / n;
 }
 
+// Microseconds of a block-sparse split-FP16 contraction on tiles of `side`
+// cells, all SMs on it: per 64 points and tile a CTA of 128 x 128 tiles takes
+// about 1570 SM cycles, a pair of 256 x 256 ones 1950 of two SMs.  The tiles
+// per point are taken halfway between points spread evenly and points all in
+// the middle (tracks lie somewhere between).
+double sparse_contraction_us(const kde_args* a, int bin, int side) {
+  const int tm = (a->nx + side - 1) / side, tn = (a->ny + side - 1) / side;
+  const double rc = sparse_reach_cells(a);
+  const double most = sparse_tiles_per_point(rc, bin, tm, side) *
+                      sparse_tiles_per_point(rc, bin, tn, side);
+  const double even = sparse_tiles_average(rc, bin, a->nx, tm, side) *
+                      sparse_tiles_average(rc, bin, a->ny, tn, side);
+  return (double)a->n * 0.5 * (most + even) * (side == 128 ? 8.25e-5 : 2.06e-4);
+}
+
 // AUTO's choice between the dense and the block-sparse contraction of a
 // Gaussian instance, from the time each takes on this GPU: dense about 1.92e9
-// FLOP per microsecond, block-sparse 1.8e9 on the (tile, point) pairs within
-// reach and about 80 us + 60 us per million points of sort, work list and
-// reduce.  The pairs are taken halfway between points spread evenly and points
-// all in the middle (tracks lie somewhere between).  The block-sparse
-// contraction skips only products that are exactly zero, so the choice never
-// changes what is summed.  It is taken where it should be 10% ahead; near the
-// line either costs about the same (300,007 points x 777 x 1111, reach 421
-// cells: dense 1.27 ms, block-sparse 1.18 ms), far from it the block-sparse
-// one wins by the ratio of the pairs (20M x 4096^2, reach 31 cells: 1030 ms
-// against 8.7 ms).
+// FLOP per microsecond; block-sparse as above and about 80 us + 60 us per
+// million points of sort, work list and reduce.  The block-sparse contraction
+// skips only products that are exactly zero, so the choice never changes what
+// is summed.  It is taken where it should be 10% ahead; near the line either
+// costs about the same, far from it the block-sparse one wins by the ratio of
+// the pairs (20M x 4096^2, reach 31 cells: 1030 ms against 5.3 ms).
 bool auto_sparse(const kde_args* a, int bin) {
   const int tm = (a->nx + 255) / 256, tn = (a->ny + 255) / 256;
-  const double rc = sparse_reach_cells(a);
-  const double per_tile = (double)a->n * 65536.0 * 6.0;
-  const double dense = per_tile * tm * tn / 1.92e9;
-  const double most = sparse_tiles_per_point(rc, bin, tm) * sparse_tiles_per_point(rc, bin, tn);
-  const double even = sparse_tiles_average(rc, bin, a->nx, tm) *
-                      sparse_tiles_average(rc, bin, a->ny, tn);
-  const double sparse = per_tile * 0.5 * (most + even) / 1.8e9 + 80.0 + 60e-6 * (double)a->n;
+  const double dense = (double)a->n * 65536.0 * 6.0 * tm * tn / 1.92e9;
+  const double sparse = std::min(sparse_contraction_us(a, bin, 128),
+                                 sparse_contraction_us(a, bin, 256)) +
+                        80.0 + 60e-6 * (double)a->n;
   return 1.1 * sparse < dense;
 }
 
@@ -341,6 +349,10 @@ struct TcFamily {
   // longest-processing-time-first assignment; empty = round robin
   std::vector<uint32_t> sched;
   size_t off_sched = 0;
+  // block-sparse family (plan.skip_zero = the side of its tiles): its work list
+  int tiles_total = 0, piece_len = 0, max_pieces = 0;
+  size_t off_total = 0, off_np = 0, off_pb = 0, off_nf = 0, off_fb = 0, off_tail = 0,
+         off_temp = 0, off_part = 0;
 };
 
 // Longest processing time first: the items, longest first, each to the CTA
@@ -384,10 +396,7 @@ struct BatchPlan {
   int64_t cut_slice_bins = 0;  // output blocks of cutoff instances that split heavy blocks
   bool sparse = false;  // some tensor-core instances are block-sparse
   bool auto_sparse = false;  // ... by AUTO's choice: the dense plan does as well
-  int n_sparse = 0, sparse_fam = -1;
-  int tiles_total = 0, piece_len = 0, max_pieces = 0;
-  size_t off_sp_total = 0, off_sp_np = 0, off_sp_pb = 0, off_sp_nf = 0, off_sp_fb = 0,
-         off_sp_tail = 0, off_sp_temp = 0, off_sp_part = 0;
+  int n_sparse = 0;
   CutoffSizes cz;
   bool host_pts = false, host_w = false, host_out = false;
   size_t upload_end;  // the uploaded region is [off_scal, upload_end)
@@ -503,11 +512,20 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       f.pair = 1;
       f.tile_n = 256;
       f.stage_points = 64;
-      f.skip_zero = 1;
-      // sorted points put a whole chunk's mass on the same cells, so the
-      // accumulators are drained every 64 points: the tensor core's FP32
-      // accumulation then loses no more than the dense contraction's does
-      if (!(o && o->k_chunk) && f.split16) kc = 64;
+      // 128-cell tiles are split-FP16's; CTA pairs (256 cells) where they are
+      // the faster, or asked for
+      const int bin = sparse_sort_bin(A[k].nx, A[k].ny, n_tc_all);
+      const bool pairs = !f.split16 || (o && ((o->flags & KDE_FLAG_CTA_PAIR) || o->tile_n)) ||
+                         (tiles && ((tiles[k].flags & KDE_FLAG_CTA_PAIR) || tiles[k].tile_n));
+      f.skip_zero = !pairs && sparse_contraction_us(&A[k], bin, 128) <
+                                  sparse_contraction_us(&A[k], bin, 256)
+                        ? 128
+                        : 256;
+      // sorted points put a whole chunk's mass on the same cells, so accumulators
+      // are drained every stage (on 128-cell tiles, where the small products have
+      // their own, every other one): the tensor core's FP32 accumulation then
+      // loses no more than the dense contraction's does
+      if (f.split16 && !(o && o->k_chunk)) kc = f.skip_zero == 128 ? 128 : 64;
       P->auto_sparse = P->auto_sparse || !want_sparse;
     }
     if (tiles) {
@@ -558,7 +576,6 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     }
     if (I.sparse) {
       P->sparse = true;
-      P->sparse_fam = I.fam;
       ++P->n_sparse;
     }
   }
@@ -570,9 +587,10 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     InstPlan& I = P->in[k];
     if (is_tc(I.path)) {
       const TcPlan& f = P->fam[I.fam].plan;
-      const int tile_m = f.pair ? 256 : 128;
+      const int tile_m = I.sparse ? f.skip_zero : f.pair ? 256 : 128;
       I.tiles_m = (a->nx + tile_m - 1) / tile_m;
-      I.tiles_n = (a->ny + f.tile_n - 1) / f.tile_n;
+      const int tile_n = I.sparse ? f.skip_zero : f.tile_n;
+      I.tiles_n = (a->ny + tile_n - 1) / tile_n;
       fam_cost[I.fam] += (double)I.tiles_m * I.tiles_n * (double)I.n_pad;
     }
   }
@@ -645,11 +663,12 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       f.items += P->in[k].items;
     }
   }
-  if (P->sparse) {
+  for (TcFamily& sf : P->fam) {
+    const int side = sf.plan.skip_zero;
+    if (!side) continue;
     // bins of the block-sparse instances follow the cutoff bins in the sort
     double est = 0.0;
     int64_t bound = 0;
-    const TcFamily& sf = P->fam[P->sparse_fam];
     for (int k : sf.order) {
       const kde_args* a = &A[k];
       InstPlan& I = P->in[k];
@@ -660,39 +679,39 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       P->total_bins += I.geo.nbins;
       I.cut_begin = P->cut_m;
       P->cut_m += I.n_pad;
-      I.tile_begin = P->tiles_total;
-      P->tiles_total += I.tiles_m * I.tiles_n;
+      I.tile_begin = sf.tiles_total;
+      sf.tiles_total += I.tiles_m * I.tiles_n;
       const double rc = sparse_reach_cells(a);
-      est += (double)I.n_pad * sparse_tiles_per_point(rc, I.geo.bin, I.tiles_m) *
-             sparse_tiles_per_point(rc, I.geo.bin, I.tiles_n);
+      est += (double)I.n_pad * sparse_tiles_per_point(rc, I.geo.bin, I.tiles_m, side) *
+             sparse_tiles_per_point(rc, I.geo.bin, I.tiles_n, side);
     }
-    // pieces of about an eighth of each CTA pair's share, in whole drain chunks
-    const int clusters = std::max(1, ctas / 2);
+    // pieces of about an eighth of each CTA's (pair's) share, in whole drain chunks
+    const int clusters = std::max(1, side == 128 ? ctas : ctas / 2);
     int64_t L = (int64_t)(est / (8.0 * clusters));
     L = std::max<int64_t>(2048, std::min<int64_t>(kSparseMaxPiece, L));
     for (int k : sf.order) {  // whole accumulator chunks of every instance
       const int64_t kc = std::max(P->in[k].k_chunk, sf.plan.stage_points);
       L = (L + kc - 1) / kc * kc;
     }
-    P->piece_len = (int)L;
+    sf.piece_len = (int)L;
     for (int k : sf.order) {
       const kde_args* a = &A[k];
       const InstPlan& I = P->in[k];
-      // a bin of b cells lies within the reach r of the tiles t with
-      // 256 t in (x - 255.5 - r, x + b - 0.5 + r), x its first cell: at most
-      // floor((b + 255 + 2 r) / 256) + 1 of them along an axis (the hundredth
+      // a bin of b cells lies within the reach r of the tiles t of S cells with
+      // S t in (x - S + 0.5 - r, x + b - 0.5 + r), x its first cell: at most
+      // floor((b + S - 1 + 2 r) / S) + 1 of them along an axis (the hundredth
       // of a cell covers the rounding of the ranges' FP64)
       const double rc = range_reach(kSparseReach, I.geo) /
                         (a->cell * kernel_sigma(KDE_GAUSSIAN, a->h));
       const int64_t per_axis = (int64_t)std::min(
-          1e6, std::floor((I.geo.bin + 255.0 + 2.0 * rc + 0.01) / 256.0) + 1.0);
+          1e6, std::floor((I.geo.bin + side - 1.0 + 2.0 * rc + 0.01) / side) + 1.0);
       const int64_t reach_tiles = std::min<int64_t>(per_axis, I.tiles_m) *
                                   std::min<int64_t>(per_axis, I.tiles_n);
       bound += (I.n_pad * reach_tiles + L - 1) / L + (int64_t)I.tiles_m * I.tiles_n;
     }
-    if (bound > (1 << 24) || P->tiles_total > (1 << 26))
+    if (bound > (1 << 24) || sf.tiles_total > (1 << 26))
       return fail(KDE_EINVAL, "block-sparse work list too large (%lld pieces)", (long long)bound);
-    P->max_pieces = (int)bound;
+    sf.max_pieces = (int)bound;
   }
   if (P->total_bins >= ((int64_t)1 << 31)) return fail(KDE_EINVAL, "too many bins in one batch");
   if (P->cut_m >= ((int64_t)1 << 32)) return fail(KDE_EINVAL, "too many points to sort in one batch");
@@ -756,16 +775,17 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     P->off_co_ranges = take(sizeof(int4) * (size_t)std::max<int64_t>(P->cut_bins, 1));
     P->off_co_ocount = take(u * kCutOcountWords);
   }
-  if (P->sparse) {
-    const size_t u = sizeof(uint32_t);
-    P->off_sp_total = take(u * (size_t)P->tiles_total);
-    P->off_sp_np = take(u * ((size_t)P->tiles_total + 1));
-    P->off_sp_pb = take(u * ((size_t)P->tiles_total + 1));
-    P->off_sp_nf = take(u * ((size_t)P->tiles_total + 1));
-    P->off_sp_fb = take(u * ((size_t)P->tiles_total + 1));
-    P->off_sp_tail = take(u * (size_t)P->tiles_total);
-    P->off_sp_temp = take(u * sparse_scan_words(P->tiles_total));
-    P->off_sp_part = take(sizeof(float) * 65536 * (size_t)P->max_pieces);
+  for (TcFamily& f : P->fam) {
+    if (!f.plan.skip_zero) continue;
+    const size_t u = sizeof(uint32_t), tiles = (size_t)f.tiles_total;
+    f.off_total = take(u * tiles);
+    f.off_np = take(u * (tiles + 1));
+    f.off_pb = take(u * (tiles + 1));
+    f.off_nf = take(u * (tiles + 1));
+    f.off_fb = take(u * (tiles + 1));
+    f.off_tail = take(u * tiles);
+    f.off_temp = take(u * sparse_scan_words(f.tiles_total));
+    f.off_part = take(sizeof(float) * f.plan.skip_zero * f.plan.skip_zero * (size_t)f.max_pieces);
   }
   P->off_hxy = take(P->host_pts ? sizeof(double) * 2 * (size_t)A[0].n : 0);
   P->off_hw = take(P->host_w ? sizeof(float) * (size_t)A[0].n : 0);
@@ -1056,7 +1076,8 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   }
   const int n_cut_only = (int)cut.size();
   if (P.sparse) {  // bin-sort entries of the block-sparse instances, after the cutoff ones
-    for (int k : P.fam[P.sparse_fam].order) {
+    for (int k : P.tc_order) {
+      if (!P.in[k].sparse) continue;
       const InstPlan& I = P.in[k];
       CutInst q = {};
       q.gxt = prep[k].gxt;
@@ -1146,41 +1167,36 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     KDE_CUDA(cudaEventCreateWithFlags(&join, cudaEventDisableTiming), "create event");
     KDE_CUDA(cudaEventRecord(fork, s), "fork to the side stream");
   }
-  SparseCtl sp;
-  const TcInst* d_sp = nullptr;  // the block-sparse family's instances
-  if (P.sparse) {
-    d_sp = d_tc + P.fam[P.sparse_fam].tab_begin;
-    sp.piece_begin = reinterpret_cast<const uint32_t*>(base + P.off_sp_pb);
-    sp.full_begin = reinterpret_cast<const uint32_t*>(base + P.off_sp_fb);
-    sp.tail_tile = reinterpret_cast<const uint32_t*>(base + P.off_sp_tail);
-    sp.tile_total = reinterpret_cast<const uint32_t*>(base + P.off_sp_total);
-    sp.part = reinterpret_cast<float*>(base + P.off_sp_part);
-    sp.tiles_total = P.tiles_total;
-    sp.piece_len = P.piece_len;
-    sp.max_pieces = P.max_pieces;
-    KDE_CUDA(launch_sparse_plan(d_sp, P.n_sparse, sp,
-                                reinterpret_cast<uint32_t*>(base + P.off_sp_np),
-                                reinterpret_cast<uint32_t*>(base + P.off_sp_nf),
-                                reinterpret_cast<uint32_t*>(base + P.off_sp_temp), batch_scal, s),
-             "block-sparse work list");
-  }
+  auto at = [&](size_t off) { return reinterpret_cast<uint32_t*>(base + off); };
   for (const TcFamily& f : P.fam) {  // one persistent launch per tile family
     const int nf = (int)f.order.size();
+    const TcInst* d_fam = d_tc + f.tab_begin;
     if (f.plan.skip_zero) {
-      KDE_CUDA(launch_tc_pair(f.plan, d_sp, nf, 0, &sp, nullptr, batch_scal, s),
+      SparseCtl sp;
+      sp.piece_begin = at(f.off_pb);
+      sp.full_begin = at(f.off_fb);
+      sp.tail_tile = at(f.off_tail);
+      sp.tile_total = at(f.off_total);
+      sp.part = reinterpret_cast<float*>(base + f.off_part);
+      sp.tiles_total = f.tiles_total;
+      sp.piece_len = f.piece_len;
+      sp.max_pieces = f.max_pieces;
+      sp.side = f.plan.skip_zero;
+      KDE_CUDA(launch_sparse_plan(d_fam, nf, sp, at(f.off_np), at(f.off_nf), at(f.off_temp),
+                                  batch_scal, s),
+               "block-sparse work list");
+      KDE_CUDA(sp.side == 128 ? launch_tc_sparse(f.plan, d_fam, nf, sp, batch_scal, s)
+                              : launch_tc_pair(f.plan, d_fam, nf, 0, &sp, nullptr, batch_scal, s),
                "block-sparse tensor-core contraction");
+      KDE_CUDA(launch_sparse_reduce(d_fam, nf, sp, s), "block-sparse reduce");
       continue;
     }
     if (f.items < 1) continue;
-    const uint32_t* sched =
-        f.sched.empty() ? nullptr : reinterpret_cast<const uint32_t*>(base + f.off_sched);
-    KDE_CUDA(f.plan.pair ? launch_tc_pair(f.plan, d_tc + f.tab_begin, nf, f.items, nullptr, sched,
-                                          batch_scal, s)
-                         : launch_tc(f.plan, d_tc + f.tab_begin, nf, f.items, batch_scal, s),
+    const uint32_t* sched = f.sched.empty() ? nullptr : at(f.off_sched);
+    KDE_CUDA(f.plan.pair ? launch_tc_pair(f.plan, d_fam, nf, f.items, nullptr, sched, batch_scal, s)
+                         : launch_tc(f.plan, d_fam, nf, f.items, batch_scal, s),
              "tensor-core contraction");
   }
-  if (P.sparse)
-    KDE_CUDA(launch_sparse_reduce(d_sp, P.n_sparse, sp, s), "block-sparse reduce");
   for (int k = 0; k < count; ++k) {
     const InstPlan& I = P.in[k];
     if (I.path != KDE_PATH_SIMT_FP32) continue;

@@ -196,10 +196,10 @@ __host__ __device__ inline BinRange block_bins(double cs, double reach, double i
                                                int nby, int cx0, int cy0, int side) {
   return block_bins_rect(cs, reach, inv_binw, nbx, nby, cx0, cy0, side, side);
 }
-// the 256 x 256 tile (tm, tn) of the tensor-core paths
+// the tile (tm, tn) of side x side cells of the block-sparse tensor-core path
 __host__ __device__ inline BinRange tile_bins(double cs, double reach, double inv_binw, int nbx,
-                                              int nby, int tm, int tn) {
-  return block_bins(cs, reach, inv_binw, nbx, nby, tm * 256, tn * 256, 256);
+                                              int nby, int tm, int tn, int side) {
+  return block_bins(cs, reach, inv_binw, nbx, nby, tm * side, tn * side, side);
 }
 
 // Walks the bin-row runs of a block's range (the points of bins lo_bx..hi_bx
@@ -247,7 +247,7 @@ __host__ __device__ inline bool range_empty(const BinRange& br) {
 // Work list of the block-sparse contraction: each tile's points (its bin
 // rows' runs, concatenated) cut into pieces of piece_len points; piece p of
 // a tile has id piece_begin[tile] + p and owns partial tile `id` of `part`
-// (256 x 256 floats, [j_local][i_local]).  The contraction takes the pieces
+// (side x side floats, [j_local][i_local]).  The contraction takes the pieces
 // in schedule order: first every full piece (tile by tile), then the
 // shorter last pieces, longest first (tail_tile), dealt to the CTA pairs in
 // snake order so their loads come out even.  The schedule decides only
@@ -257,8 +257,9 @@ struct SparseCtl {
   const uint32_t* full_begin;   // [tiles_total + 1], exclusive scan of full pieces per tile
   const uint32_t* tail_tile;    // [tiles_total] tiles with a short last piece, longest first
   const uint32_t* tile_total;   // [tiles_total] points that can reach each tile
-  float* part;                  // [max_pieces][256][256]
+  float* part;                  // [max_pieces][side][side]
   int tiles_total, piece_len, max_pieces;
+  int side;                     // cells of a tile's side: 128 (one CTA) or 256 (CTA pair)
 };
 // Longest piece the planner makes.
 constexpr int kSparseMaxPiece = 32768;
@@ -508,7 +509,7 @@ struct TcPlan {
   int splits;        // point-range splits S (partials in part[S])
   int k_chunk;       // points per TMEM accumulator drain
   int ctas;          // persistent CTAs
-  int skip_zero;     // skip (tile, stage) pairs whose operands are all zero
+  int skip_zero;     // block-sparse: the side of the tiles, 128 or 256; 0: dense
   int stage_points;  // 32 or 64 points per pipeline stage
   int pair;          // 1: 256 x 256 tiles on CTA pairs (cta_group::2)
 };
@@ -531,6 +532,10 @@ int pair_clusters(const TcPlan& plan, int n_items);
 cudaError_t launch_tc_pair(const TcPlan& plan, const TcInst* tab, int ninst, int n_items,
                            const SparseCtl* sp, const uint32_t* sched, CallScalars* err,
                            cudaStream_t s);
+// The split-FP16 block-sparse contraction on 128 x 128 tiles, one CTA each
+// (tiles_m / tiles_n of the table count 128-cell tiles; sp.side = 128).
+cudaError_t launch_tc_sparse(const TcPlan& plan, const TcInst* tab, int ninst, const SparseCtl& sp,
+                             CallScalars* err, cudaStream_t s);
 // Block-sparse work list: tile totals, pieces and full pieces per tile and
 // their exclusive scans, the tail pieces ordered longest first.  npieces and
 // nfull are [tiles_total + 1] scratch words.

@@ -10,7 +10,8 @@
 // changes no product, only which zeros are added.
 //
 // The points are sorted into bins of 4 to 32 cells a side (the cutoff path's
-// stable radix sort, with that reach); a 256 x 256 tile then needs only the bins
+// stable radix sort, with that reach); a tile (128 x 128 or
+// 256 x 256 cells) then needs only the bins
 // within reach, i.e. one contiguous run of sorted points per bin row.  This
 // file builds the work list (points per tile, cut into pieces of a fixed
 // length, and the exclusive scan of the pieces per tile) and sums each
@@ -35,11 +36,12 @@ __device__ __forceinline__ int inst_of_tile(const TcInst* __restrict__ tab, int 
 // The points of a tile's bin rows, one warp per tile, the rows over its lanes
 // (one thread per tile was a chain of a hundred dependent reads: 27 us for the
 // 16 tiles of 1024^2).
-__device__ __forceinline__ uint32_t tile_points(const TcInst* __restrict__ tab, int ninst, int t) {
+__device__ __forceinline__ uint32_t tile_points(const TcInst* __restrict__ tab, int ninst, int t,
+                                                int side) {
   const TcInst& I = tab[inst_of_tile(tab, ninst, t)];
   const int local = t - I.tile_begin;
   const int tm = local % I.tiles_m, tn = local / I.tiles_m;
-  const BinRange br = tile_bins(I.cs, I.range_reach, I.inv_binw, I.nbx, I.nby, tm, tn);
+  const BinRange br = tile_bins(I.cs, I.range_reach, I.inv_binw, I.nbx, I.nby, tm, tn, side);
   uint32_t total = 0;  // the sort holds fewer than 2^32 points
   if (br.lo_bx <= br.hi_bx)
     for (int by = br.lo_by + (threadIdx.x & 31); by <= br.hi_by; by += 32) {
@@ -58,7 +60,7 @@ __global__ void k_sparse_totals(const TcInst* __restrict__ tab, int ninst, Spars
   const int t = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (t > sp.tiles_total) return;
   uint32_t total = 0;
-  if (t < sp.tiles_total) total = tile_points(tab, ninst, t);
+  if (t < sp.tiles_total) total = tile_points(tab, ninst, t, sp.side);
   if ((threadIdx.x & 31) != 0) return;
   if (t < sp.tiles_total) tile_total[t] = total;
   npieces[t] = (uint32_t)(((uint64_t)total + sp.piece_len - 1) / sp.piece_len);
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(kTailThreads)
     if (tid < sp.tiles_total) totals[tid] = tile_total[tid];
   } else {
     for (int t = warp; t < sp.tiles_total; t += kTailThreads / 32) {
-      const uint32_t total = tile_points(tab, ninst, t);
+      const uint32_t total = tile_points(tab, ninst, t, sp.side);
       if (lane == 0) totals[t] = total;
     }
   }
@@ -179,32 +181,34 @@ __global__ void __launch_bounds__(kTailThreads)
 }
 
 // out cell (i, j) of tile t = sum over the tile's pieces, in order.  Grid:
-// (tiles, 256 / kRedRows); a thread sums four adjacent columns of one row,
+// (tiles, side^2 / kRedCells); a thread sums four adjacent columns of one row,
 // eight pieces' loads in flight at a time (the adds stay in piece order).
 // Bound by HBM (256 KB per piece); a dense cluster's tile holds most of the
 // pieces, so its rows are spread over 128 blocks and each thread keeps enough
 // bytes in flight: 1.47M points x 1024^2, 16 tiles: 323 us with one column per
 // thread, 16 rows per block and one load at a time.
-constexpr int kRedRows = 2;
-__global__ void __launch_bounds__(64 * kRedRows)
+constexpr int kRedThreads = 128, kRedCells = 4 * kRedThreads;
+__global__ void __launch_bounds__(kRedThreads)
     k_sparse_reduce(const TcInst* __restrict__ tab, int ninst, SparseCtl sp) {
   const int t = blockIdx.x;
   const TcInst& I = tab[inst_of_tile(tab, ninst, t)];
   const int local = t - I.tile_begin;
   const int tm = local % I.tiles_m, tn = local / I.tiles_m;
-  const int il = 4 * (threadIdx.x & 63), i = tm * 256 + il;
-  const int jl = blockIdx.y * kRedRows + (threadIdx.x >> 6), j = tn * 256 + jl;
+  const int cell = blockIdx.y * kRedCells + 4 * threadIdx.x;  // of the tile
+  const int il = cell % sp.side, i = tm * sp.side + il;
+  const int jl = cell / sp.side, j = tn * sp.side + jl;
+  const int64_t cells = (int64_t)sp.side * sp.side;
   if (i >= I.nx || j >= I.ny) return;
   const int p0 = min((int)sp.piece_begin[t], sp.max_pieces);
   const int p1 = min((int)sp.piece_begin[t + 1], sp.max_pieces);
-  const float* src = sp.part + jl * 256 + il;
+  const float* src = sp.part + cell;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   constexpr int kAhead = 8;
   for (int p = p0; p < p1; p += kAhead) {
     float4 v[kAhead];
 #pragma unroll
     for (int u = 0; u < kAhead; ++u)
-      if (p + u < p1) v[u] = __ldcs(reinterpret_cast<const float4*>(src + (int64_t)(p + u) * 65536));
+      if (p + u < p1) v[u] = __ldcs(reinterpret_cast<const float4*>(src + (p + u) * cells));
 #pragma unroll
     for (int u = 0; u < kAhead; ++u)
       if (p + u < p1) {
@@ -260,7 +264,8 @@ cudaError_t launch_sparse_plan(const TcInst* tab, int ninst, const SparseCtl& sp
 
 cudaError_t launch_sparse_reduce(const TcInst* tab, int ninst, const SparseCtl& sp,
                                  cudaStream_t s) {
-  k_sparse_reduce<<<dim3(sp.tiles_total, 256 / kRedRows), 64 * kRedRows, 0, s>>>(tab, ninst, sp);
+  k_sparse_reduce<<<dim3(sp.tiles_total, sp.side * sp.side / kRedCells), kRedThreads, 0, s>>>(
+      tab, ninst, sp);
   note_launches(1);
   return cudaGetLastError();
 }

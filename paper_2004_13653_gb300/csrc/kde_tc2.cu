@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         RunCursor cur;
         if (SPARSE)  // items exist only for tiles whose range holds points
           cur.init(I.start, I.bin_begin, I.nbx,
-                   tile_bins(I.cs, I.range_reach, I.inv_binw, I.nbx, I.nby, itm.tm, itm.tn));
+                   tile_bins(I.cs, I.range_reach, I.inv_binw, I.nbx, I.nby, itm.tm, itm.tn, 256));
         for (int st = 0; ok && st < itm.nst; st += kGroup) {
           if (SPARSE && (g & 1u) != mine) {  // the other loader's stage
             ++g;
@@ -668,7 +668,7 @@ cudaError_t launch_tc_pair(const TcPlan& plan, const TcInst* tab, int ninst, int
                            cudaStream_t s) {
   if (ninst < 1 || plan.ctas < 2 || plan.stage_points != kKS) return cudaErrorInvalidValue;
   if (sp) {
-    if (sp->tiles_total < 1 || sp->piece_len < kKS || sp->piece_len % kKS) return cudaErrorInvalidValue;
+    if (sp->side != 256 || sp->tiles_total < 1 || sp->piece_len < kKS || sp->piece_len % kKS) return cudaErrorInvalidValue;
     return plan.split16 ? launch_pair<true, true>(plan, tab, ninst, 0, *sp, nullptr, err, s)
                         : launch_pair<false, true>(plan, tab, ninst, 0, *sp, nullptr, err, s);
   }
