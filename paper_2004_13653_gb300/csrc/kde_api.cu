@@ -305,9 +305,11 @@ bool auto_sparse(const kde_args* a, int bin) {
 // Side of the block-sparse sort bins, in cells: a tile reads every point of
 // the bins within its reach, (256 + 2 reach + bin)^2 cells' worth, so finer
 // bins mean fewer products; the bins of one call stay within the 2^16 that
-// two radix passes sort (kSparseBin = 32 where even those are more).
+// two radix passes sort (kSparseBin = 32 where even those are more).  Below 8
+// the runs of a row get too short for the loaders: 1M points x 1024^2, reach
+// 20 cells, takes 328 us per call with 4-cell bins and 312 with 8.
 int sparse_sort_bin(int nx, int ny, int instances) {
-  for (int bin = 4; bin < kSparseBin; bin *= 2)
+  for (int bin = 8; bin < kSparseBin; bin *= 2)
     if (((int64_t)(nx + bin - 1) / bin) * ((ny + bin - 1) / bin) * instances <= 65536) return bin;
   return kSparseBin;
 }
