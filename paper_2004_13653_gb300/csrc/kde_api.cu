@@ -240,7 +240,8 @@ struct InstPlan {
   int bin_begin;
   int obx, oby, out_begin;  // cutoff: output blocks of kCutoffBin cells, first CTA
   int64_t cut_begin;
-  int tile_begin;  // block-sparse: first tile in the batch's tile numbering
+  int tile_begin;  // block-sparse, wide gather: first tile in its family's numbering
+  bool wide;       // cutoff path: the wide gather on 32 x 32-cell tiles
 };
 
 // Block-sparse skipping: reach of a Gaussian operand in prepared units
@@ -387,6 +388,32 @@ std::vector<uint32_t> lpt_schedule(const std::vector<int64_t>& cost, int cluster
   return t;
 }
 
+// Tiles of `side` cells that a bin's points can be within reach of, at most: a
+// bin of b cells lies within the reach r (cells) of the tiles t with
+// side t in (x - side + 0.5 - r, x + b - 0.5 + r), x its first cell: at most
+// floor((b + side - 1 + 2 r) / side) + 1 of them along an axis (the hundredth
+// of a cell covers the rounding of the ranges' FP64).
+int64_t reach_tiles(double reach_cells, const InstPlan& I, int side) {
+  const int64_t per_axis = (int64_t)std::min(
+      1e6, std::floor((I.geo.bin + side - 1.0 + 2.0 * reach_cells + 0.01) / side) + 1.0);
+  return std::min<int64_t>(per_axis, I.tiles_m) * std::min<int64_t>(per_axis, I.tiles_n);
+}
+
+// Whether a compact kernel's instance takes the wide gather: supports of more
+// than 16 cells a side from the point, and half a million (tile, point) pairs,
+// enough pieces to fill the GPU.  Epanechnikov and radial quartic, us per call,
+// 16 x 16 blocks against 32 x 32 tiles: 1M points x 1024^2 at reach 12 cells
+// 387 / 333 and 600 / 618, at 20 cells 772 / 449 and 1393 / 928; 200,000 points
+// x 512^2 at 20 cells 269 / 164 and 406 / 287; 20,000 points x 256^2 at 20 cells
+// 100 / 111 and 121 / 173, 2,000 points 70 / 74 and 71 / 110.
+constexpr int kWidePiece = 8192;
+bool wide_gather(const kde_args* a) {
+  const double reach = a->h / a->cell;
+  const double tx = std::min(1.0 + 2.0 * reach / kWideSide, (a->nx + kWideSide - 1.0) / kWideSide);
+  const double ty = std::min(1.0 + 2.0 * reach / kWideSide, (a->ny + kWideSide - 1.0) / kWideSide);
+  return reach > 16.0 && (double)a->n * tx * ty >= 5e5;
+}
+
 struct BatchPlan {
   int count;
   std::vector<InstPlan> in;
@@ -396,6 +423,13 @@ struct BatchPlan {
   int n_tc = 0, n_cut = 0, n_simt = 0, n_reduce = 0, tc_items = 0, max_side = 1;
   int64_t total_pad = 0, cut_m = 0, total_bins = 0, reduce_cells = 0, cut_bins = 0;
   int64_t cut_slice_bins = 0;  // output blocks of cutoff instances that split heavy blocks
+  // the cutoff instances of the wide gather, by piece length; their table
+  // entries follow the tensor-core ones
+  std::vector<TcFamily> wide;
+  int n_wide = 0;
+  // whether the plan holds a choice that may be undone for want of workspace
+  bool chosen() const { return auto_sparse || n_wide; }
+  bool sorts() const { return n_cut || n_wide || sparse; }
   bool sparse = false;  // some tensor-core instances are block-sparse
   bool auto_sparse = false;  // ... by AUTO's choice: the dense plan does as well
   int n_sparse = 0;
@@ -499,6 +533,7 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   for (int k = 0; k < count; ++k) {
     InstPlan& I = P->in[k];
     I.fam = -1;
+    I.wide = false;
     I.split_req = o ? o->split_k : 0;
     I.sparse = false;
     if (!is_tc(I.path)) continue;
@@ -632,6 +667,10 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       I.items = (int)(tiles * splits);
       P->fam[I.fam].order.push_back(k);
       ++P->n_tc;
+    } else if (allow_sparse && wide_gather(a)) {  // cutoff, laid out below
+      splits = 1;
+      I.wide = true;
+      ++P->n_wide;
     } else {  // cutoff
       splits = 1;
       I.geo = cutoff_geometry(a->nx, a->ny, a->cell / a->h, 1.0,
@@ -664,6 +703,47 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       P->tc_order.push_back(k);
       f.items += P->in[k].items;
     }
+  }
+  // the wide gather's bins follow the cutoff bins in the sort
+  int n_wide_tab = 0;
+  for (int k = 0; k < count; ++k) {
+    const kde_args* a = &A[k];
+    InstPlan& I = P->in[k];
+    if (!I.wide) continue;
+    I.geo = cutoff_geometry(a->nx, a->ny, a->cell / a->h, 1.0, sparse_sort_bin(a->nx, a->ny, 1));
+    I.bin_begin = (int)P->total_bins;
+    P->total_bins += I.geo.nbins;
+    I.cut_begin = P->cut_m;
+    P->cut_m += I.n_pad;
+    I.tiles_m = (a->nx + kWideSide - 1) / kWideSide;
+    I.tiles_n = (a->ny + kWideSide - 1) / kWideSide;
+    const int64_t tiles = (int64_t)I.tiles_m * I.tiles_n;
+    const int64_t visits =
+        I.n_pad * reach_tiles(range_reach(1.0, I.geo) * a->h / a->cell, I, kWideSide);
+    // pieces of kWidePiece points (1M points x 1000 x 900, reach 40: 885 us per call
+    // with 2048, 832 with 4096, 808 with 8192), longer ones where their partial tiles
+    // would take more than a gigabyte (a function of the instance alone, so
+    // that it is computed the same way in any batch)
+    int L = kWidePiece;
+    while (L < kSparseMaxPiece && visits / L > (1 << 17)) L *= 2;
+    int f = 0;
+    while (f < (int)P->wide.size() && P->wide[f].piece_len != L) ++f;
+    if (f == (int)P->wide.size()) {
+      P->wide.push_back(TcFamily());
+      P->wide[f].piece_len = L;
+    }
+    TcFamily& wf = P->wide[f];
+    const int64_t bound = wf.max_pieces + (visits + L - 1) / L + tiles;
+    if (bound > (1 << 24) || wf.tiles_total + tiles > (1 << 26))
+      return fail(KDE_EINVAL, "compact work list too large (%lld pieces)", (long long)bound);
+    wf.max_pieces = (int)bound;
+    I.tile_begin = wf.tiles_total;
+    wf.tiles_total += (int)tiles;
+    wf.order.push_back(k);
+  }
+  for (TcFamily& f : P->wide) {
+    f.tab_begin = P->n_tc + n_wide_tab;
+    n_wide_tab += (int)f.order.size();
   }
   for (TcFamily& sf : P->fam) {
     const int side = sf.plan.skip_zero;
@@ -699,17 +779,9 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     for (int k : sf.order) {
       const kde_args* a = &A[k];
       const InstPlan& I = P->in[k];
-      // a bin of b cells lies within the reach r of the tiles t of S cells with
-      // S t in (x - S + 0.5 - r, x + b - 0.5 + r), x its first cell: at most
-      // floor((b + S - 1 + 2 r) / S) + 1 of them along an axis (the hundredth
-      // of a cell covers the rounding of the ranges' FP64)
       const double rc = range_reach(kSparseReach, I.geo) /
                         (a->cell * kernel_sigma(KDE_GAUSSIAN, a->h));
-      const int64_t per_axis = (int64_t)std::min(
-          1e6, std::floor((I.geo.bin + side - 1.0 + 2.0 * rc + 0.01) / side) + 1.0);
-      const int64_t reach_tiles = std::min<int64_t>(per_axis, I.tiles_m) *
-                                  std::min<int64_t>(per_axis, I.tiles_n);
-      bound += (I.n_pad * reach_tiles + L - 1) / L + (int64_t)I.tiles_m * I.tiles_n;
+      bound += (I.n_pad * reach_tiles(rc, I, side) + L - 1) / L + (int64_t)I.tiles_m * I.tiles_n;
     }
     if (bound > (1 << 24) || sf.tiles_total > (1 << 26))
       return fail(KDE_EINVAL, "block-sparse work list too large (%lld pieces)", (long long)bound);
@@ -748,8 +820,9 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   // the scalars (zeros) and the tables lie together and are uploaded together
   P->off_scal = take(sizeof(CallScalars) * (size_t)(count + 1));
   P->off_tab_prep = take(sizeof(PrepInst) * (size_t)count);
-  P->off_tab_tc = take(sizeof(TcInst) * (size_t)std::max(P->n_tc, 1));
-  P->off_tab_cut = take(sizeof(CutInst) * (size_t)std::max(P->n_cut + P->n_sparse, 1));
+  P->off_tab_tc = take(sizeof(TcInst) * (size_t)std::max(P->n_tc + P->n_wide, 1));
+  P->off_tab_cut = take(sizeof(CutInst) *
+                         (size_t)std::max(P->n_cut + P->n_wide + P->n_sparse, 1));
   P->off_tab_red = take(sizeof(ReduceInst) * (size_t)std::max(P->n_reduce, 1));
   for (TcFamily& f : P->fam)
     if (!f.sched.empty()) f.off_sched = take(sizeof(uint32_t) * f.sched.size());
@@ -762,7 +835,7 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     I.off_run = I.path == KDE_PATH_SIMT_FP32 ? take(simt_scratch_bytes(A[k].nx, A[k].ny, I.splits))
                                              : 0;
   }
-  if (P->n_cut || P->sparse) {
+  if (P->sorts()) {
     const size_t u = sizeof(uint32_t);
     for (int k = 0; k < 2; ++k) {
       P->off_co_keys[k] = take(u * (size_t)P->cut_m);
@@ -777,8 +850,7 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     P->off_co_ranges = take(sizeof(int4) * (size_t)std::max<int64_t>(P->cut_bins, 1));
     P->off_co_ocount = take(u * kCutOcountWords);
   }
-  for (TcFamily& f : P->fam) {
-    if (!f.plan.skip_zero) continue;
+  auto take_list = [&](TcFamily& f, size_t tile_bytes) {
     const size_t u = sizeof(uint32_t), tiles = (size_t)f.tiles_total;
     f.off_total = take(u * tiles);
     f.off_np = take(u * (tiles + 1));
@@ -787,8 +859,11 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     f.off_fb = take(u * (tiles + 1));
     f.off_tail = take(u * tiles);
     f.off_temp = take(u * sparse_scan_words(f.tiles_total));
-    f.off_part = take(sizeof(float) * f.plan.skip_zero * f.plan.skip_zero * (size_t)f.max_pieces);
-  }
+    f.off_part = take(tile_bytes * (size_t)f.max_pieces);
+  };
+  for (TcFamily& f : P->fam)
+    if (f.plan.skip_zero) take_list(f, sizeof(float) * f.plan.skip_zero * f.plan.skip_zero);
+  for (TcFamily& f : P->wide) take_list(f, sizeof(float2) * kWideSide * kWideSide);
   P->off_hxy = take(P->host_pts ? sizeof(double) * 2 * (size_t)A[0].n : 0);
   P->off_hw = take(P->host_w ? sizeof(float) * (size_t)A[0].n : 0);
   P->off_hout = take(P->host_out ? sizeof(float) * (size_t)A[0].nx * A[0].ny : 0);
@@ -911,7 +986,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   int rc = make_plan(A, count, o, tiles, true, true, &P);
   // AUTO's block-sparse plan is a choice: where its work list or workspace is
   // out of reach, the call runs dense as an explicit TC_SPLIT16 call does
-  if (rc && P.auto_sparse) {
+  if (rc && P.chosen()) {
     P = BatchPlan();
     rc = make_plan(A, count, o, tiles, true, false, &P);
   }
@@ -923,7 +998,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   const bool sync = force_sync || (o && (o->flags & KDE_FLAG_SYNC)) || (P.host_out && !host_async);
   void* wsv = nullptr;
   rc = acquire_workspace(o, P.total, s, &wsv);
-  if (rc == KDE_ENOMEM && P.auto_sparse) {
+  if (rc == KDE_ENOMEM && P.chosen()) {
     P = BatchPlan();
     rc = make_plan(A, count, o, tiles, true, false, &P);
     if (rc) return rc;
@@ -989,13 +1064,28 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     const double c = kid >= kRadial ? kernel_const_radial(kid - kRadial) : c1 * c1;
     return A[k].n > 0 ? (float)(c / ((double)A[k].n * A[k].h * A[k].h)) : 0.0f;
   };
+  auto sorted_inst = [&](TcInst& q, int k, double reach) {  // points in bin order
+    const InstPlan& I = P.in[k];
+    q.pts = reinterpret_cast<const float4*>(base + P.off_co_spts);
+    q.wts = reinterpret_cast<const float*>(base + P.off_co_sw);
+    q.part = out_dev[k];  // the reduce writes the output
+    q.start = reinterpret_cast<const uint32_t*>(base + P.off_co_start);
+    q.cs = prep[k].cell_sigma;
+    q.reach = reach;
+    q.range_reach = range_reach(reach, I.geo);
+    q.inv_binw = I.geo.inv_binw;
+    q.nbx = I.geo.nbx;
+    q.nby = I.geo.nby;
+    q.bin_begin = I.bin_begin;
+    q.tile_begin = I.tile_begin;
+  };
   int item_begin = 0;
   for (int k : P.tc_order) {
     const kde_args* a = &A[k];
     const InstPlan& I = P.in[k];
     const TcFamily& fam = P.fam[I.fam];
     if (k == fam.order.front()) item_begin = 0;  // each family numbers its own items
-    TcInst q;
+    TcInst q = {};
     q.pts = prep[k].pts;
     q.wts = prep[k].wts;
     q.gxt = prep[k].gxt;
@@ -1015,29 +1105,30 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     q.base_scale = a->n > 0 ? (float)(0x1p-30 / (2.0 * 3.14159265358979323846 * (double)a->n *
                                                  a->h * a->h))
                             : 0.0f;
-    q.start = nullptr;
-    q.cs = q.reach = q.inv_binw = q.range_reach = 0.0;
-    q.nbx = q.nby = q.bin_begin = q.tile_begin = 0;
-    if (I.sparse) {  // points in bin order; the sparse reduce writes the output
-      q.pts = reinterpret_cast<const float4*>(base + P.off_co_spts);
-      q.wts = reinterpret_cast<const float*>(base + P.off_co_sw);
-      q.part = out_dev[k];
-      q.start = reinterpret_cast<const uint32_t*>(base + P.off_co_start);
-      q.cs = prep[k].cell_sigma;
-      q.reach = kSparseReach;
-      q.range_reach = range_reach(kSparseReach, I.geo);
-      q.inv_binw = I.geo.inv_binw;
-      q.nbx = I.geo.nbx;
-      q.nby = I.geo.nby;
-      q.bin_begin = I.bin_begin;
-      q.tile_begin = I.tile_begin;
-    }
+    if (I.sparse) sorted_inst(q, k, kSparseReach);
     item_begin += I.items;
     tct.push_back(q);
   }
+  for (const TcFamily& f : P.wide)
+    for (int k : f.order) {
+      TcInst q = {};
+      q.gxt = prep[k].gxt;
+      q.gyt = prep[k].gyt;
+      q.scal = scal + k;
+      q.n_pad = P.in[k].n_pad;
+      q.nx = A[k].nx;
+      q.ny = A[k].ny;
+      q.tiles_m = P.in[k].tiles_m;
+      q.tiles_n = P.in[k].tiles_n;
+      q.splits = 1;
+      q.base_scale = compact_scale(k);
+      q.kid = kid_of(&A[k]);
+      sorted_inst(q, k, 1.0);
+      tct.push_back(q);
+    }
   for (int k = 0; k < count; ++k) {
     const InstPlan& I = P.in[k];
-    if (I.path == KDE_PATH_CUTOFF) {
+    if (I.path == KDE_PATH_CUTOFF && !I.wide) {
       CutInst q = {};
       q.gxt = prep[k].gxt;
       q.gyt = prep[k].gyt;
@@ -1077,10 +1168,12 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     }
   }
   const int n_cut_only = (int)cut.size();
-  if (P.sparse) {  // bin-sort entries of the block-sparse instances, after the cutoff ones
-    for (int k : P.tc_order) {
-      if (!P.in[k].sparse) continue;
+  if (P.sparse || P.n_wide) {
+    // bin-sort entries of the instances that only need the sort, after the
+    // gather's
+    for (int k = 0; k < count; ++k) {
       const InstPlan& I = P.in[k];
+      if (!I.sparse && !I.wide) continue;
       CutInst q = {};
       q.gxt = prep[k].gxt;
       q.gyt = prep[k].gyt;
@@ -1092,16 +1185,16 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       q.inv_binw = I.geo.inv_binw;
       q.ext_x = I.geo.ext_x;
       q.ext_y = I.geo.ext_y;
-      q.reach = kSparseReach;
-      q.range_reach = range_reach(kSparseReach, I.geo);
-      q.cs = A[k].cell * kernel_sigma(KDE_GAUSSIAN, A[k].h);
+      q.reach = I.sparse ? kSparseReach : 1.0;
+      q.range_reach = range_reach(q.reach, I.geo);
+      q.cs = prep[k].cell_sigma;
       set_key_constants(q);
       q.nbx = I.geo.nbx;
       q.nby = I.geo.nby;
       q.bin_begin = I.bin_begin;
       q.nx = A[k].nx;
       q.ny = A[k].ny;
-      q.kid = KDE_GAUSSIAN;
+      q.kid = kid_of(&A[k]);
       cut.push_back(q);
     }
     // cut_begin must increase along the table for the key kernel's search
@@ -1128,7 +1221,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   cudaEvent_t* ev = o ? static_cast<cudaEvent_t*>(o->timing_events) : nullptr;
   if (ev) KDE_CUDA(cudaEventRecord(ev[0], s), "record start event");
   CutoffScratch cs;
-  if (P.n_cut || P.sparse) {
+  if (P.sorts()) {
     for (int k = 0; k < 2; ++k) {
       cs.keys[k] = reinterpret_cast<uint32_t*>(base + P.off_co_keys[k]);
       cs.vals[k] = reinterpret_cast<uint32_t*>(base + P.off_co_vals[k]);
@@ -1149,7 +1242,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
   // instances, whose contraction needs the sort first, the small sort kernels
   // move there as well (they fit beside the contraction's CTAs).  The two
   // sides write disjoint buffers, so results do not change.
-  const bool overlap = P.n_cut && P.n_tc;
+  const bool overlap = (P.n_cut || P.n_wide) && P.n_tc;
   const bool sort_aside = overlap && !P.sparse;
   cudaStream_t s2 = s;
   cudaEvent_t fork = nullptr, join = nullptr;
@@ -1160,7 +1253,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
         if (*x) cudaEventDestroy(*x);
     }
   } guard{{&fork, &join}};
-  if ((P.n_cut || P.sparse) && !sort_aside)
+  if (P.sorts() && !sort_aside)
     KDE_CUDA(launch_bin_sort(d_cut, (int)cut.size(), P.cut_m, P.total_bins, pts, wts, P.cz, cs, s),
              "bin sort");
   if (overlap) {
@@ -1170,20 +1263,35 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     KDE_CUDA(cudaEventRecord(fork, s), "fork to the side stream");
   }
   auto at = [&](size_t off) { return reinterpret_cast<uint32_t*>(base + off); };
+  auto work_list = [&](const TcFamily& f, int side) {
+    SparseCtl sp;
+    sp.piece_begin = at(f.off_pb);
+    sp.full_begin = at(f.off_fb);
+    sp.tail_tile = at(f.off_tail);
+    sp.tile_total = at(f.off_total);
+    sp.part = reinterpret_cast<float*>(base + f.off_part);
+    sp.tiles_total = f.tiles_total;
+    sp.piece_len = f.piece_len;
+    sp.max_pieces = f.max_pieces;
+    sp.side = side;
+    return sp;
+  };
+  auto compact = [&](cudaStream_t cs_stream) {  // the compact instances' gathers
+    for (const TcFamily& f : P.wide) {
+      const int nf = (int)f.order.size();
+      const SparseCtl sp = work_list(f, kWideSide);
+      cudaError_t e = launch_sparse_plan(d_tc + f.tab_begin, nf, sp, at(f.off_np), at(f.off_nf),
+                                         at(f.off_temp), batch_scal, cs_stream);
+      if (e == cudaSuccess) e = launch_cutoff_wide(d_tc + f.tab_begin, nf, sp, batch_scal, cs_stream);
+      if (e != cudaSuccess) return e;
+    }
+    return launch_cutoff_eval(d_cut, n_cut_only, P.cut_bins, P.cut_slice_bins, cs, cs_stream);
+  };
   for (const TcFamily& f : P.fam) {  // one persistent launch per tile family
     const int nf = (int)f.order.size();
     const TcInst* d_fam = d_tc + f.tab_begin;
     if (f.plan.skip_zero) {
-      SparseCtl sp;
-      sp.piece_begin = at(f.off_pb);
-      sp.full_begin = at(f.off_fb);
-      sp.tail_tile = at(f.off_tail);
-      sp.tile_total = at(f.off_total);
-      sp.part = reinterpret_cast<float*>(base + f.off_part);
-      sp.tiles_total = f.tiles_total;
-      sp.piece_len = f.piece_len;
-      sp.max_pieces = f.max_pieces;
-      sp.side = f.plan.skip_zero;
+      const SparseCtl sp = work_list(f, f.plan.skip_zero);
       KDE_CUDA(launch_sparse_plan(d_fam, nf, sp, at(f.off_np), at(f.off_nf), at(f.off_temp),
                                   batch_scal, s),
                "block-sparse work list");
@@ -1213,13 +1321,11 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       KDE_CUDA(launch_bin_sort(d_cut, (int)cut.size(), P.cut_m, P.total_bins, pts, wts, P.cz, cs,
                                s2),
                "bin sort");
-    KDE_CUDA(launch_cutoff_eval(d_cut, n_cut_only, P.cut_bins, P.cut_slice_bins, cs, s2),
-             "cutoff evaluation");
+    KDE_CUDA(compact(s2), "cutoff evaluation");
     KDE_CUDA(cudaEventRecord(join, s2), "join from the side stream");
     KDE_CUDA(cudaStreamWaitEvent(s, join, 0), "join the side stream");
-  } else if (P.n_cut) {
-    KDE_CUDA(launch_cutoff_eval(d_cut, n_cut_only, P.cut_bins, P.cut_slice_bins, cs, s),
-             "cutoff evaluation");
+  } else if (P.n_cut || P.n_wide) {
+    KDE_CUDA(compact(s), "cutoff evaluation");
   }
   if (ev) KDE_CUDA(cudaEventRecord(ev[1], s), "record end event");
   if (P.n_reduce) KDE_CUDA(launch_reduce(d_red, P.n_reduce, P.reduce_cells, s), "split-K reduce");
@@ -1296,7 +1402,7 @@ int kde_workspace_size(const kde_args* a, const kde_opts* opts, size_t* bytes) {
   if (rc) return rc;
   BatchPlan pl;
   rc = make_plan(a, 1, opts, nullptr, true, true, &pl);
-  if (rc && pl.auto_sparse) {
+  if (rc && pl.chosen()) {
     pl = BatchPlan();
     rc = make_plan(a, 1, opts, nullptr, true, false, &pl);
   }

@@ -169,6 +169,7 @@ struct TcInst {
   double cs, reach, inv_binw;  // cell and reach in prepared units, 1 / bin width
   double range_reach;          // reach plus the bin keys' FP32 rounding margin (ranges use it)
   int nbx, nby, bin_begin, tile_begin;
+  int kid;  // the wide gather's kernel (part: the output; base_scale: its constant)
 };
 
 // Points of bin rows lo_by..hi_by, columns lo_bx..hi_bx can reach the block
@@ -240,6 +241,39 @@ struct RunCursor {
     return (int64_t)ra + (v - vr);
   }
 };
+// The RunCursor walk with 32-bit positions (a block's or slice's reach list
+// and the sorted points number fewer than 2^32): fewer registers in the
+// gather, whose occupancy its register count sets.
+struct RunCursor32 {
+  const uint32_t* row;  // start + row0 + by * nbx
+  int nbx, lo_bx, hi_bx, by, hi_by;
+  uint32_t vr, ra, rb;
+  __device__ __forceinline__ void load_run() {
+    ra = __ldg(row + lo_bx);
+    rb = __ldg(row + hi_bx + 1);
+  }
+  __device__ __forceinline__ void init(const uint32_t* start, int row0, int nbx_,
+                                       const BinRange& br) {
+    nbx = nbx_;
+    lo_bx = br.lo_bx;
+    hi_bx = br.hi_bx;
+    by = br.lo_by;
+    hi_by = br.hi_by;
+    row = start + row0 + by * nbx;
+    vr = 0;
+    load_run();
+  }
+  // index of position v (v below the range's total, not decreasing)
+  __device__ __forceinline__ uint32_t map(uint32_t v) {
+    while (v >= vr + (rb - ra) && by < hi_by) {
+      vr += rb - ra;
+      ++by;
+      row += nbx;
+      load_run();
+    }
+    return ra + (v - vr);
+  }
+};
 __host__ __device__ inline bool range_empty(const BinRange& br) {
   return br.lo_bx > br.hi_bx || br.lo_by > br.hi_by;
 }
@@ -257,9 +291,10 @@ struct SparseCtl {
   const uint32_t* full_begin;   // [tiles_total + 1], exclusive scan of full pieces per tile
   const uint32_t* tail_tile;    // [tiles_total] tiles with a short last piece, longest first
   const uint32_t* tile_total;   // [tiles_total] points that can reach each tile
-  float* part;                  // [max_pieces][side][side]
+  float* part;                  // [max_pieces][side][side] ((hi, lo) pairs for the wide gather)
   int tiles_total, piece_len, max_pieces;
-  int side;                     // cells of a tile's side: 128 (one CTA) or 256 (CTA pair)
+  int side;                     // cells of a tile's side: 128 (one CTA), 256 (CTA pair) or
+                                // kWideSide (the compact kernels' wide gather)
 };
 // Longest piece the planner makes.
 constexpr int kSparseMaxPiece = 32768;
@@ -544,6 +579,11 @@ cudaError_t launch_sparse_plan(const TcInst* tab, int ninst, const SparseCtl& sp
                                uint32_t* npieces, uint32_t* nfull, uint32_t* scan_temp,
                                CallScalars* err, cudaStream_t s);
 // Sum each tile's piece partials in order into the instance outputs.
+// The wide gather of the compact kernels over the work list's pieces, and the
+// sum of the pieces (kde_cutoff_wide.cu).
+constexpr int kWideSide = 32;
+cudaError_t launch_cutoff_wide(const TcInst* tab, int ninst, const SparseCtl& sp, CallScalars* err,
+                               cudaStream_t s);
 cudaError_t launch_sparse_reduce(const TcInst* tab, int ninst, const SparseCtl& sp,
                                  cudaStream_t s);
 
