@@ -674,7 +674,7 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     } else {  // cutoff
       splits = 1;
       I.geo = cutoff_geometry(a->nx, a->ny, a->cell / a->h, 1.0,
-                              cutoff_sort_bin(a->nx, a->ny, a->h / a->cell));
+                              cutoff_sort_bin(a->n, a->nx, a->ny, a->h / a->cell));
       I.bin_begin = (int)P->total_bins;
       P->total_bins += I.geo.nbins;
       I.obx = (a->nx + kCutoffBin - 1) / kCutoffBin;
@@ -1155,6 +1155,13 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       q.kid = kid_of(&A[k]);
       q.scale = compact_scale(k);
       q.slice = I.geo.bin == 4;
+      uint32_t bits;
+      const float side = (float)q.cs;
+      memcpy(&bits, &side, sizeof(bits));
+      bits &= 0xFFFFFFC0u;
+      memcpy(&q.cs_hi, &bits, sizeof(bits));
+      q.cs_lo = (float)(q.cs - (double)q.cs_hi);
+      q.drop_reach = (float)q.range_reach;
       cut.push_back(q);
     }
     if (I.splits > 1) {

@@ -6,9 +6,10 @@
 // outside the grid are dropped), the (key, index) pairs are sorted with a
 // stable LSD radix sort, and each 16x16-cell output block is then computed by
 // one CTA that reads the points of the sort bins within reach of its cells,
-// in sorted order: its eight warps take 32-point batches in turn, tabulate
-// the x and y kernel factors of the block's 16 columns and 16 rows in shared
-// memory, and each thread adds the outer products into its eight cells.  The
+// in sorted order: its eight warps take 32-point batches in turn, keep the
+// points within reach of the block, tabulate the x and y kernel factors of the
+// block's 16 columns and 16 rows for 16 of them at a time in shared memory, and
+// each thread adds the outer products into its eight cells.  The
 // blocks run heaviest first; a block with thousands of points within reach is
 // split into four row slices, one CTA each, and light blocks share a CTA two
 // at a time, four warps each.  Nothing is accumulated with atomics, and the
@@ -29,7 +30,8 @@ constexpr int kSortThreads = 512;   // 16 warps
 constexpr int kSortRounds = 8;      // 32-element rounds per warp
 constexpr int kSortChunk = kSortThreads * kSortRounds;  // 4096 keys per block
 constexpr int kMaxPasses = 4;     // 8-bit digits of 32-bit keys
-constexpr int kBatch = 32;          // points per shared-memory batch (one per lane)
+constexpr int kBatch = 32;          // points read at a time (one per lane)
+constexpr int kStep = 16;           // points whose factors are tabulated at a time
 
 template <class T>
 __device__ __forceinline__ int find_by(const T* tab, int ninst, int64_t v, int64_t T::*field) {
@@ -283,26 +285,36 @@ __global__ void k_bin_bounds(const uint32_t* __restrict__ skeys, int64_t m, int 
 }
 
 
-// Accumulate one batch's outer products into a thread's cells: columns cx,
-// cx+1 of RPL rows from cy0 (acc[2 r + c]); RPL = 4 for a whole 16-row
-// block, 1 for a 4-row slice of a heavy block.  Product kernels from
-// tabulated factors, radial kernels from tabulated squared offsets and the
-// profile per pair.  Per point one 8-byte and one 4*RPL-byte table read feed
-// 2*RPL FMAs.
+// Shared-memory tables of one point group: points within reach that wait for
+// their turn (x and y, hi and lo; weights), and the factors of kStep of them.
+// A row of factors is four floats longer than its 16 so that eight lanes'
+// 16-byte stores, a row each, take all the banks.
+constexpr int kRow = kBin + 4;
+struct GroupTables {
+  float2 P[2][kBatch + kStep];
+  float W[kBatch + kStep];
+  __align__(16) float K[2][kStep][kRow];
+};
+
+// Accumulate the outer products of the first cnt <= kStep waiting points into a
+// thread's cells: columns cx, cx+1 of RPL rows from cy0 (acc[2 r + c]); RPL = 4
+// for a whole 16-row block, 1 for a 4-row slice of a heavy block.  Product
+// kernels from tabulated factors, radial kernels from tabulated squared offsets
+// and the profile per pair.  Per point one 8-byte and one 4*RPL-byte table read
+// feed 2*RPL FMAs.
 template <int KID, bool RADIAL, int RPL>
-__device__ __forceinline__ void accumulate(const float (*KX)[kBin], const float (*KY)[kBin],
-                                           const float* sW, int cnt, int cx, int cy0,
+__device__ __forceinline__ void accumulate(const GroupTables& T, int cnt, int cx, int cy0,
                                            float (&acc)[2 * RPL]) {
   static_assert(RPL == 4 || RPL == 1, "rows per lane");
   auto load_y = [&](int c, float (&y)[RPL]) {
     if constexpr (RPL == 4) {
-      const float4 v = *reinterpret_cast<const float4*>(&KY[c][cy0]);
+      const float4 v = *reinterpret_cast<const float4*>(&T.K[1][c][cy0]);
       y[0] = v.x;
       y[1] = v.y;
       y[2] = v.z;
       y[3] = v.w;
     } else {
-      y[0] = KY[c][cy0];
+      y[0] = T.K[1][c][cy0];
     }
   };
   int c = 0;
@@ -312,7 +324,7 @@ __device__ __forceinline__ void accumulate(const float (*KX)[kBin], const float 
       float y[2][RPL];
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        kx[u] = *reinterpret_cast<const float2*>(&KX[c + u][cx]);
+        kx[u] = *reinterpret_cast<const float2*>(&T.K[0][c + u][cx]);
         load_y(c + u, y[u]);
       }
 #pragma unroll
@@ -326,11 +338,11 @@ __device__ __forceinline__ void accumulate(const float (*KX)[kBin], const float 
     }
   }
   for (; c < cnt; ++c) {
-    const float2 kx = *reinterpret_cast<const float2*>(&KX[c][cx]);
+    const float2 kx = *reinterpret_cast<const float2*>(&T.K[0][c][cx]);
     float y[RPL];
     load_y(c, y);
     if (RADIAL) {
-      const float w = sW[c];
+      const float w = T.W[c];
 #pragma unroll
       for (int r = 0; r < RPL; ++r) {
         acc[2 * r] = fmaf(w, kradial<KID>(kx.x + y[r]), acc[2 * r]);
@@ -342,6 +354,34 @@ __device__ __forceinline__ void accumulate(const float (*KX)[kBin], const float 
         acc[2 * r] = fmaf(kx.x, y[r], acc[2 * r]);
         acc[2 * r + 1] = fmaf(kx.y, y[r], acc[2 * r + 1]);
       }
+    }
+  }
+}
+
+// The factors of the first cnt <= kStep waiting points, lanes l and l + 16 for
+// point l's columns and rows: the offset from cell j is that from the item's
+// first cell, g0, plus j times the cell's side (its upper 18 bits, whose product
+// with j is exact, and the rest).  A slice has 4 rows.
+template <int KID, bool RADIAL, int RPL>
+__device__ __forceinline__ void tabulate(GroupTables& T, int cnt, int lane, float2 g0, float cs_hi,
+                                         float cs_lo) {
+  const int axis = lane >> 4, pt = lane & (kStep - 1);
+  if (pt < cnt) {
+    const float2 p = T.P[axis][pt];
+    const float w = axis && !RADIAL ? T.W[pt] : 1.0f;
+    const float dh = g0.x - p.x, dl = g0.y - p.y;
+    float4* row = reinterpret_cast<float4*>(&T.K[axis][pt][0]);
+#pragma unroll
+    for (int q = 0; q < kBin / 4; ++q) {
+      if (RPL == 1 && q > 0 && axis) break;
+      float v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float j = (float)(4 * q + e);
+        const float u = fmaf(j, cs_hi, dh) + fmaf(j, cs_lo, dl);
+        v[e] = RADIAL ? u * u : w * kfactor<KID>(u);
+      }
+      row[q] = make_float4(v[0], v[1], v[2], v[3]);
     }
   }
 }
@@ -458,14 +498,6 @@ __global__ void k_cut_order_scatter(const CutInst* __restrict__ tab, int ninst,
   order[first[key] + atomicAdd(&ocount[kCutOrderKeys + key], 1u)] = (uint32_t)blk;
 }
 
-// Shared-memory tables of one point group.
-struct GroupTables {
-  float4 P[kBatch];
-  float W[kBatch];
-  __align__(16) float KX[kBatch][kBin];
-  __align__(16) float KY[kBatch][kBin];
-};
-
 constexpr int kSliceRows = 4;
 // dynamic shared memory of the gather: the groups' tables, then their running sums
 constexpr size_t kCutTablesBytes = sizeof(GroupTables) * kGroups;
@@ -477,26 +509,42 @@ constexpr int kSlices = kBin / kSliceRows;  // items per heavy block
 // reach those rows are the runs of the sort bins in range br, one run per bin
 // row; their concatenation is cut into kBatch-point batches, and group g of
 // the block's NG takes batches g, g+NG, g+2NG, ... (fetching the next while computing
-// the current; the warp synchronises only itself) and adds each batch into
-// the (hi, lo) running sums of its cells with a two-sum; the running sums
-// live in shared memory (run[r * 32] for cell r of this lane), which keeps
-// the kernel at 64 registers and four CTAs per SM.
+// the current; the warp synchronises only itself).  The bins hold half as many
+// points again as reach the item at a reach of 3 cells: the others, whose
+// factors are zeros, are dropped, and the rest wait until there are kStep.
+// After 32 points the products go into the (hi, lo) running sums of the cells
+// with a two-sum; the running sums live in shared memory (run[r * 32] for cell r
+// of this lane), which keeps the kernel at 64 registers and four CTAs per SM.
+// Bound by shared memory's 128 bytes per clock to the registers and by the
+// latency of the point reads: with every point of the bins computed, and its
+// factors made a cell per lane from a broadcast of the point, 4M points x 1024^2
+// took 664 us per call at a reach of 3 cells, 1080 at 6 and 1292 at 12; now 543,
+// 781 and 936.
 template <int KID, bool RADIAL, int RPL, int NG>
 __device__ __forceinline__ void cutoff_group(const CutInst& I, const float4* __restrict__ P,
                                              const float* __restrict__ W,
                                              const uint32_t* __restrict__ start, int bx, int by,
                                              int y_off, const BinRange& br, int64_t total, int g,
                                              int lane, GroupTables& T, float2* run) {
+  static_assert(kGroupThreads == 2 * kStep && kBatch == kGroupThreads && kBatch % kStep == 0,
+                "table roles");
   const int nx = I.nx, ny = I.ny;
-  const int x0 = bx * kBin, y0 = by * kBin;
-  const int cx = 2 * (lane & 7), cy0 = y_off + RPL * (lane >> 3);
-  // table role: column (and row) ej for the points of one parity, c = 2k + half
-  constexpr int kEvalPts = kBatch * kBin / kGroupThreads;
-  static_assert(kGroupThreads == 2 * kBin && kBatch == kGroupThreads, "table roles");
-  const int ej = lane & (kBin - 1), half = lane >> 4;
-  const float2 gxe = I.gxt[min(x0 + ej, nx - 1)];
-  const float2 gye = I.gyt[min(y0 + ej, ny - 1)];
-  if (total == 0) return;
+  const int x0 = bx * kBin, y0 = by * kBin + y_off;
+  const int cx = 2 * (lane & 7), cy0 = RPL * (lane >> 3);
+  if (total == 0 || y0 >= ny) return;  // a ragged block's slice may have no row
+  const float2 g0 = lane < kStep ? I.gxt[x0] : I.gyt[y0];
+  // the item's reach, widened as the bin ranges are: points beyond it have a
+  // factor of exactly zero at every cell
+  float x_lo, x_hi, y_lo, y_hi;
+  {
+    const float2 a = I.gxt[x0], b = I.gxt[min(x0 + kBin - 1, nx - 1)];
+    const float2 c = I.gyt[y0], d = I.gyt[min(y0 + 4 * RPL - 1, ny - 1)];
+    x_lo = (a.x + a.y) - I.drop_reach;
+    x_hi = (b.x + b.y) + I.drop_reach;
+    y_lo = (c.x + c.y) - I.drop_reach;
+    y_hi = (d.x + d.y) + I.drop_reach;
+  }
+  const float cs_hi = I.cs_hi, cs_lo = I.cs_lo;
   RunCursor32 cur;
   cur.init(start, I.bin_begin, I.nbx, br);
   constexpr uint32_t kStride = NG * kBatch;
@@ -509,47 +557,69 @@ __device__ __forceinline__ void cutoff_group(const CutInst& I, const float4* __r
     pf = P[p];
     wf = W[p];
   }
-  for (uint32_t b0 = g * kBatch; b0 < total32; b0 += kStride, v += kStride) {
-    const int cnt = (int)min((uint32_t)kBatch, total32 - b0);
-    __syncwarp();  // the warp's previous batch is consumed
-    if (lane < cnt) {
-      T.P[lane] = pf;
-      T.W[lane] = wf;
-    }
-    __syncwarp();
-    if (v + kStride < total32) {  // next batch, in flight
-      const uint32_t p = cur.map(v + kStride);
-      pf = P[p];
-      wf = W[p];
-    }
-    // the two half-warps write rows 2k and 2k+1: conflict-free
-#pragma unroll 4
-    for (int k = 0; k < kEvalPts; ++k) {
-      const int c = 2 * k + half;
-      if (c < cnt) {
-        const float4 p = T.P[c];
-        const float u = (gxe.x - p.x) + (gxe.y - p.y), w = (gye.x - p.z) + (gye.y - p.w);
-        if (RADIAL) {
-          T.KX[c][ej] = u * u;
-          T.KY[c][ej] = w * w;
-        } else {
-          T.KX[c][ej] = kfactor<KID>(u);
-          T.KY[c][ej] = T.W[c] * kfactor<KID>(w);
-        }
-      }
-    }
-    __syncwarp();
-    float acc[2 * RPL];
+  float acc[2 * RPL];
 #pragma unroll
-    for (int r = 0; r < 2 * RPL; ++r) acc[r] = 0.f;
-    accumulate<KID, RADIAL, RPL>(T.KX, T.KY, T.W, cnt, cx, cy0, acc);
+  for (int r = 0; r < 2 * RPL; ++r) acc[r] = 0.f;
+  int held = 0, waiting = 0;  // points in acc, and in the tables
+  auto flush = [&]() {
 #pragma unroll
     for (int r = 0; r < 2 * RPL; ++r) {
       float2 x = run[r * kGroupThreads];
       two_sum_acc(x, acc[r]);
       run[r * kGroupThreads] = x;
+      acc[r] = 0.f;
     }
+  };
+  for (uint32_t b0 = g * kBatch;; b0 += kStride, v += kStride) {
+    const bool more = b0 < total32;
+    if (more) {
+      const float X = pf.x + pf.y, Y = pf.z + pf.w;
+      const bool in = v < total32 && X >= x_lo && X <= x_hi && Y >= y_lo && Y <= y_hi;
+      const uint32_t mask = __ballot_sync(0xffffffffu, in);
+      if (in) {
+        const int e = waiting + __popc(mask & ((1u << lane) - 1u));
+        T.P[0][e] = make_float2(pf.x, pf.y);
+        T.P[1][e] = make_float2(pf.z, pf.w);
+        T.W[e] = wf;
+      }
+      waiting += __popc(mask);
+      __syncwarp();
+      if (v + kStride < total32) {  // next batch, in flight
+        const uint32_t p = cur.map(v + kStride);
+        pf = P[p];
+        wf = W[p];
+      }
+    }
+    while (waiting >= (more ? kStep : 1)) {  // at the end, the points left too
+      const int cnt = min(waiting, kStep);
+      tabulate<KID, RADIAL, RPL>(T, cnt, lane, g0, cs_hi, cs_lo);
+      __syncwarp();
+      accumulate<KID, RADIAL, RPL>(T, cnt, cx, cy0, acc);
+      held += cnt;
+      waiting -= cnt;
+      if (held >= kBatch) {
+        flush();
+        held = 0;
+      }
+      // the points left, at most 31, move to the front
+      float2 px = make_float2(0.f, 0.f), py = px;
+      float w = 0.f;
+      if (lane < waiting) {
+        px = T.P[0][lane + kStep];
+        py = T.P[1][lane + kStep];
+        w = T.W[lane + kStep];
+      }
+      __syncwarp();
+      if (lane < waiting) {
+        T.P[0][lane] = px;
+        T.P[1][lane] = py;
+        T.W[lane] = w;
+      }
+      __syncwarp();
+    }
+    if (!more) break;
   }
+  flush();
 }
 
 // Points of the sort bins in range br (the runs of its bin rows).
@@ -761,7 +831,7 @@ CutoffGeom cutoff_geometry(int nx, int ny, double cs, double reach, int bin) {
   return g;
 }
 
-int cutoff_sort_bin(int nx, int ny, double reach_cells) {
+int cutoff_sort_bin(int64_t n, int nx, int ny, double reach_cells) {
   // an output block reads about (16 + 2 reach + bin)^2 cells' points, of which
   // (16 + 2 reach)^2 can reach it; finer bins mean more bins to sort
   int bin = reach_cells <= 6.0 ? 4 : reach_cells <= 16.0 ? 8 : 16;

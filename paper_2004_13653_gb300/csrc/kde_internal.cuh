@@ -320,6 +320,9 @@ struct CutInst {
   int nbx, nby, bin_begin, nx, ny, kid;
   int obx, oby, out_begin;
   float scale;
+  // the gather's FP32 constants: the cell's side (its upper 18 bits and the
+  // rest), and the reach beyond which points are dropped (range_reach)
+  float cs_hi, cs_lo, drop_reach;
   // heavy output blocks (4096 or more points within reach) are computed as
   // four 4-row slices: set for supports of at most 6 cells (4-cell sort bins),
   // where a slice reads about half of the block's points
@@ -401,7 +404,7 @@ inline double range_reach(double reach, const CutoffGeom& g) {
 // The cutoff path's sort-bin side for a support of reach_cells cells: small
 // enough that an output block reads little beyond its support's reach, large
 // enough that the number of bins stays bounded.
-int cutoff_sort_bin(int nx, int ny, double reach_cells);
+int cutoff_sort_bin(int64_t n, int nx, int ny, double reach_cells);
 struct CutoffScratch {
   uint32_t* keys[2];
   uint32_t* vals[2];
