@@ -681,7 +681,7 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       I.oby = (a->ny + kCutoffBin - 1) / kCutoffBin;
       I.out_begin = (int)P->cut_bins;
       P->cut_bins += (int64_t)I.obx * I.oby;
-      if (I.geo.bin == 4) P->cut_slice_bins += (int64_t)I.obx * I.oby;
+      if (cutoff_slices(a->nx, a->ny, a->h / a->cell)) P->cut_slice_bins += (int64_t)I.obx * I.oby;
       I.cut_begin = P->cut_m;
       P->cut_m += I.n_pad;
       ++P->n_cut;
@@ -1154,7 +1154,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       q.ny = A[k].ny;
       q.kid = kid_of(&A[k]);
       q.scale = compact_scale(k);
-      q.slice = I.geo.bin == 4;
+      q.slice = cutoff_slices(A[k].nx, A[k].ny, A[k].h / A[k].cell);
       uint32_t bits;
       const float side = (float)q.cs;
       memcpy(&bits, &side, sizeof(bits));
@@ -1292,7 +1292,8 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       if (e == cudaSuccess) e = launch_cutoff_wide(d_tc + f.tab_begin, nf, sp, batch_scal, cs_stream);
       if (e != cudaSuccess) return e;
     }
-    return launch_cutoff_eval(d_cut, n_cut_only, P.cut_bins, P.cut_slice_bins, cs, cs_stream);
+    return launch_cutoff_eval(d_cut, n_cut_only, P.cut_bins, P.cut_slice_bins, cs, sm_count(),
+                              cs_stream);
   };
   for (const TcFamily& f : P.fam) {  // one persistent launch per tile family
     const int nf = (int)f.order.size();

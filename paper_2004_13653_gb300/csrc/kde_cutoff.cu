@@ -1,8 +1,8 @@
 // Path (c): the compact kernels of Table 1 evaluated over their support only.
 //
 // With the indicator of Eq. 8 a point contributes to the cells within one
-// bandwidth of it.  Every point gets the key of its sort bin (4, 8 or 16
-// cells a side, chosen from the bandwidth; points farther than a bandwidth
+// bandwidth of it.  Every point gets the key of its sort bin (4, 8 or
+// 16 cells a side, cutoff_sort_bin; points farther than a bandwidth
 // outside the grid are dropped), the (key, index) pairs are sorted with a
 // stable LSD radix sort, and each 16x16-cell output block is then computed by
 // one CTA that reads the points of the sort bins within reach of its cells,
@@ -10,11 +10,11 @@
 // points within reach of the block, tabulate the x and y kernel factors of the
 // block's 16 columns and 16 rows for 16 of them at a time in shared memory, and
 // each thread adds the outer products into its eight cells.  The
-// blocks run heaviest first; a block with thousands of points within reach is
-// split into four row slices, one CTA each, and light blocks share a CTA two
-// at a time, four warps each.  Nothing is accumulated with atomics, and the
+// blocks run heaviest first; a block with thousands of points within reach may be
+// split into four row slices, one CTA each, light blocks share a CTA two at a
+// time, four warps each, and blocks that no point reaches get their zeros.  Nothing is accumulated with atomics, and the
 // order of every sum is fixed, so results are reproducible bit for bit.  The
-// same sort, with 32-cell bins and a wider reach, orders the points of the
+// same sort, with a wider reach, orders the points of the
 // block-sparse tensor-core path.
 #include "kde_internal.cuh"
 #include "kernel_factors.cuh"
@@ -483,11 +483,12 @@ __global__ void k_cut_order_scatter(const CutInst* __restrict__ tab, int ninst,
       first[k] = acc;
       acc += ocount[k];
     }
-    // the blocks to be split into slices come first and the light ones last;
-    // the gather needs the count of the first and the position of the second
+    // the blocks to be split into slices come first, then the others, the light
+    // ones and those without a point: the gather needs where each kind begins
     if (blockIdx.x == 0) {
       ocount[2 * kCutOrderKeys] = first[kCutOrderClasses - 1];
       ocount[2 * kCutOrderKeys + 1] = first[kLightKey];
+      ocount[2 * kCutOrderKeys + 2] = first[0];
     }
   }
   __syncthreads();
@@ -498,6 +499,7 @@ __global__ void k_cut_order_scatter(const CutInst* __restrict__ tab, int ninst,
   order[first[key] + atomicAdd(&ocount[kCutOrderKeys + key], 1u)] = (uint32_t)blk;
 }
 
+constexpr int kCutCtasPerSm = 4;
 constexpr int kSliceRows = 4;
 // dynamic shared memory of the gather: the groups' tables, then their running sums
 constexpr size_t kCutTablesBytes = sizeof(GroupTables) * kGroups;
@@ -660,155 +662,209 @@ __device__ __forceinline__ void group_dispatch(const CutInst& I, const float4* _
   }
 }
 
-// One CTA of kGroups one-warp point groups per item: first the four slices of
-// every heavy block, then the other blocks, each in the order list's
-// heaviest-first order, and last the light blocks two at a time, groups 0-3
-// on the first and 4-7 on the second (CTAs past the last item return at once).  A whole
+// One item by a CTA of kGroups one-warp point groups.  A whole
 // block's eight cells per thread, or a slice's two, are summed over the groups
 // in group order at the end, so every cell is computed by one CTA in a fixed
 // order and results are reproducible bit for bit.  Blocks of 16 cells spread a
 // dense region over many CTAs; the finer sort bins keep the points an item
 // reads close to those its cells' supports actually reach.
-__global__ void __launch_bounds__(kGroups * kGroupThreads)
-    k_cutoff(const CutInst* __restrict__ tab, int ninst, const float4* __restrict__ P,
-             const float* __restrict__ W, const uint32_t* __restrict__ start,
-             const uint32_t* __restrict__ order, const uint32_t* __restrict__ totals,
-             const int4* __restrict__ ranges, const uint32_t* __restrict__ heavy_count,
-             int nblocks, const CallScalars* __restrict__ err) {
-  // the groups' tables, then their running sums (cell r of lane l of group g
-  // at part[g][r][l])
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int4 s_rg[2];
-  __shared__ uint32_t s_total[2];
-  __shared__ int s_blk[2];
-  GroupTables* tables = reinterpret_cast<GroupTables*>(smem);
-  float2 (*part)[8][kGroupThreads] =
-      reinterpret_cast<float2 (*)[8][kGroupThreads]>(smem + kCutTablesBytes);
+struct ItemShared {
+  int4 rg[2];
+  uint32_t total[2];
+  int blk[2];
+  int64_t next;  // the CTA's next item
+};
+// thread 0 takes the CTA's next item
+__device__ __forceinline__ void take_next(uint32_t* ctr, ItemShared& S) {
+  if (threadIdx.x == 0) S.next = (int64_t)gridDim.x + atomicAdd(ctr, 1u);
+}
+
+// two light blocks: half h = g / 4 takes the block at order position
+// pos0 + h with its four groups
+__device__ __forceinline__ void light_item(const CutInst* __restrict__ tab, int ninst,
+                                           const float4* __restrict__ P,
+                                           const float* __restrict__ W,
+                                           const uint32_t* __restrict__ start,
+                                           const uint32_t* __restrict__ order,
+                                           const uint32_t* __restrict__ totals,
+                                           const int4* __restrict__ ranges, int64_t pos0,
+                                           int64_t end, GroupTables& T,
+                                           float2 (*part)[8][kGroupThreads], ItemShared& S) {
   const int g = threadIdx.x / kGroupThreads, lane = threadIdx.x % kGroupThreads;
-  GroupTables& T = tables[g];
-  // after a timed-out sort the bin starts may not rise, and positions taken
-  // from them could leave the sorted points: compute nothing (the call
-  // reports the timeout)
-  if (*reinterpret_cast<const volatile int*>(&err->err) & kErrSortTimeout) return;
-  const int64_t heavy = __ldg(heavy_count);
-  const int64_t light = __ldg(heavy_count + 1);  // order position of the first light block
-  const int64_t singles = kSlices * heavy + (light - heavy);
-  const int64_t item = blockIdx.x;
-  if (item >= singles + ((int64_t)nblocks - light + 1) / 2) return;
-  if (item >= singles) {
-    // two light blocks: half h = g / 4 takes the block at order position
-    // light + 2 (item - singles) + h with its four groups
-    const int half = g >> 2, gh = g & 3;
-    const int64_t pos = light + 2 * (item - singles) + half;
-    const bool has = pos < nblocks;
-    if (has && gh == 0 && lane == 0) {
-      const int blk = (int)__ldg(order + pos);
-      s_blk[half] = blk;
-      s_rg[half] = __ldg(ranges + blk);
-      s_total[half] = __ldg(totals + blk);
-    }
-    __syncthreads();
-    if (has) {
-      int bx, by;
-      const CutInst& I = output_block(tab, ninst, s_blk[half], bx, by);
-      const int4 rg = s_rg[half];
-      const BinRange br = {rg.x, rg.y, rg.z, rg.w};
-#pragma unroll
-      for (int r = 0; r < 8; ++r) part[g][r][lane] = make_float2(0.f, 0.f);
-      group_dispatch<4, 4>(I, P, W, start, bx, by, 0, br, s_total[half], gh, lane, T,
-                           &part[g][0][lane]);
-    }
-    __syncthreads();  // every group's running sums are final
-    if (has) {
-      // group gh of the half combines cells 2 gh and 2 gh + 1 of every
-      // thread's eight over the half's four groups, in order
-      int bx, by;
-      const CutInst& I = output_block(tab, ninst, s_blk[half], bx, by);
-      const int cx = 2 * (lane & 7), cy0 = 4 * (lane >> 3);
-#pragma unroll
-      for (int rr = 0; rr < 2; ++rr) {
-        const int r = 2 * gh + rr;
-        float2 sum = part[4 * half][r][lane];
-#pragma unroll
-        for (int h = 1; h < 4; ++h) {
-          const float2 o = part[4 * half + h][r][lane];
-          two_sum_acc(sum, o.x);
-          sum.y += o.y;
-        }
-        const int x = bx * kBin + cx + (r & 1), y = by * kBin + cy0 + (r >> 1);
-        if (x < I.nx && y < I.ny) I.out[(int64_t)y * I.nx + x] = (sum.x + sum.y) * I.scale;
-      }
-    }
-    return;
-  }
-  {
-    int64_t pos;
-    int slice;
-    if (item < kSlices * heavy) {
-      pos = item / kSlices;
-      slice = (int)(item % kSlices);
-    } else {
-      pos = heavy + (item - kSlices * heavy);
-      slice = -1;
-    }
+  const int half = g >> 2, gh = g & 3;
+  const int64_t pos = pos0 + half;
+  const bool has = pos < end;
+  if (has && gh == 0 && lane == 0) {
     const int blk = (int)__ldg(order + pos);
+    S.blk[half] = blk;
+    S.rg[half] = __ldg(ranges + blk);
+    S.total[half] = __ldg(totals + blk);
+  }
+  __syncthreads();
+  if (has) {
     int bx, by;
-    const CutInst& I = output_block(tab, ninst, blk, bx, by);
-    if (threadIdx.x == 0) {
-      if (slice < 0) {
-        s_rg[0] = __ldg(ranges + blk);
-        s_total[0] = __ldg(totals + blk);
-      } else {  // the slice's own bin range and point count
-        const BinRange b = block_bins_rect(I.cs, I.range_reach, I.inv_binw, I.nbx, I.nby,
-                                           bx * kBin, by * kBin + slice * kSliceRows, kBin,
-                                           kSliceRows);
-        s_rg[0] = make_int4(b.lo_bx, b.hi_bx, b.lo_by, b.hi_by);
-        s_total[0] = range_total(start, I.bin_begin, I.nbx, b);
-      }
-    }
-    __syncthreads();
-    const int4 rg = s_rg[0];
+    const CutInst& I = output_block(tab, ninst, S.blk[half], bx, by);
+    const int4 rg = S.rg[half];
     const BinRange br = {rg.x, rg.y, rg.z, rg.w};
-    const int64_t total = s_total[0];
-    if (slice < 0) {
 #pragma unroll
-      for (int r = 0; r < 8; ++r) part[g][r][lane] = make_float2(0.f, 0.f);
-      group_dispatch<4, kGroups>(I, P, W, start, bx, by, 0, br, total, g, lane, T,
-                                 &part[g][0][lane]);
-      __syncthreads();  // every group's running sums are final
-      // group g combines cell r = g of every thread's eight, over the groups in
-      // order (the same order for every block and run)
-      static_assert(kGroups == 8, "one cell of eight per group");
-      const int r = g;
-      const int cx = 2 * (lane & 7), cy0 = 4 * (lane >> 3);
-      float2 sum = part[0][r][lane];
+    for (int r = 0; r < 8; ++r) part[g][r][lane] = make_float2(0.f, 0.f);
+    group_dispatch<4, 4>(I, P, W, start, bx, by, 0, br, S.total[half], gh, lane, T,
+                         &part[g][0][lane]);
+  }
+  __syncthreads();  // every group's running sums are final
+  if (has) {
+    // group gh of the half combines cells 2 gh and 2 gh + 1 of every
+    // thread's eight over the half's four groups, in order
+    int bx, by;
+    const CutInst& I = output_block(tab, ninst, S.blk[half], bx, by);
+    const int cx = 2 * (lane & 7), cy0 = 4 * (lane >> 3);
 #pragma unroll
-      for (int h = 1; h < kGroups; ++h) {
-        const float2 o = part[h][r][lane];
+    for (int rr = 0; rr < 2; ++rr) {
+      const int r = 2 * gh + rr;
+      float2 sum = part[4 * half][r][lane];
+#pragma unroll
+      for (int h = 1; h < 4; ++h) {
+        const float2 o = part[4 * half + h][r][lane];
         two_sum_acc(sum, o.x);
         sum.y += o.y;
       }
       const int x = bx * kBin + cx + (r & 1), y = by * kBin + cy0 + (r >> 1);
       if (x < I.nx && y < I.ny) I.out[(int64_t)y * I.nx + x] = (sum.x + sum.y) * I.scale;
-    } else {
-      part[g][0][lane] = make_float2(0.f, 0.f);
-      part[g][1][lane] = make_float2(0.f, 0.f);
-      group_dispatch<1, kGroups>(I, P, W, start, bx, by, slice * kSliceRows, br, total, g, lane, T,
-                        &part[g][0][lane]);
-      __syncthreads();
-      if (threadIdx.x < 2 * kGroupThreads) {  // 64 cells, one thread each
-        const int l = threadIdx.x >> 1, r = threadIdx.x & 1;
-        float2 sum = part[0][r][l];
+    }
+  }
+}
+
+// a whole block (slice < 0) or a slice of one
+__device__ __forceinline__ void block_item(const CutInst* __restrict__ tab, int ninst,
+                                           const float4* __restrict__ P,
+                                           const float* __restrict__ W,
+                                           const uint32_t* __restrict__ start, int blk, int slice,
+                                           const uint32_t* __restrict__ totals,
+                                           const int4* __restrict__ ranges, GroupTables& T,
+                                           float2 (*part)[8][kGroupThreads], uint32_t* ctr,
+                                           ItemShared& S) {
+  const int g = threadIdx.x / kGroupThreads, lane = threadIdx.x % kGroupThreads;
+  int bx, by;
+  const CutInst& I = output_block(tab, ninst, blk, bx, by);
+  if (threadIdx.x == 0) {
+    if (slice < 0) {
+      S.rg[0] = __ldg(ranges + blk);
+      S.total[0] = __ldg(totals + blk);
+    } else {  // the slice's own bin range and point count
+      const BinRange b = block_bins_rect(I.cs, I.range_reach, I.inv_binw, I.nbx, I.nby, bx * kBin,
+                                         by * kBin + slice * kSliceRows, kBin, kSliceRows);
+      S.rg[0] = make_int4(b.lo_bx, b.hi_bx, b.lo_by, b.hi_by);
+      S.total[0] = range_total(start, I.bin_begin, I.nbx, b);
+    }
+  }
+  __syncthreads();
+  const int4 rg = S.rg[0];
+  const BinRange br = {rg.x, rg.y, rg.z, rg.w};
+  const int64_t total = S.total[0];
+  if (slice < 0) {
 #pragma unroll
-        for (int h = 1; h < kGroups; ++h) {
-          const float2 o = part[h][r][l];
-          two_sum_acc(sum, o.x);
-          sum.y += o.y;
+    for (int r = 0; r < 8; ++r) part[g][r][lane] = make_float2(0.f, 0.f);
+    group_dispatch<4, kGroups>(I, P, W, start, bx, by, 0, br, total, g, lane, T,
+                               &part[g][0][lane]);
+    __syncthreads();  // every group's running sums are final
+    take_next(ctr, S);
+    // group g combines cell r = g of every thread's eight, over the groups in
+    // order (the same order for every block and run)
+    static_assert(kGroups == 8, "one cell of eight per group");
+    const int r = g;
+    const int cx = 2 * (lane & 7), cy0 = 4 * (lane >> 3);
+    float2 sum = part[0][r][lane];
+#pragma unroll
+    for (int h = 1; h < kGroups; ++h) {
+      const float2 o = part[h][r][lane];
+      two_sum_acc(sum, o.x);
+      sum.y += o.y;
+    }
+    const int x = bx * kBin + cx + (r & 1), y = by * kBin + cy0 + (r >> 1);
+    if (x < I.nx && y < I.ny) I.out[(int64_t)y * I.nx + x] = (sum.x + sum.y) * I.scale;
+  } else {
+    part[g][0][lane] = make_float2(0.f, 0.f);
+    part[g][1][lane] = make_float2(0.f, 0.f);
+    group_dispatch<1, kGroups>(I, P, W, start, bx, by, slice * kSliceRows, br, total, g, lane, T,
+                               &part[g][0][lane]);
+    __syncthreads();
+    take_next(ctr, S);
+    if (threadIdx.x < 2 * kGroupThreads) {  // 64 cells, one thread each
+      const int l = threadIdx.x >> 1, r = threadIdx.x & 1;
+      float2 sum = part[0][r][l];
+#pragma unroll
+      for (int h = 1; h < kGroups; ++h) {
+        const float2 o = part[h][r][l];
+        two_sum_acc(sum, o.x);
+        sum.y += o.y;
+      }
+      const int x = bx * kBin + 2 * (l & 7) + r, y = by * kBin + slice * kSliceRows + (l >> 3);
+      if (x < I.nx && y < I.ny) I.out[(int64_t)y * I.nx + x] = (sum.x + sum.y) * I.scale;
+    }
+  }
+}
+
+// The items, taken from a counter by CTAs that stay: first the four slices of
+// every heavy block, then the other blocks, each in the order list's
+// heaviest-first order, then the light blocks two at a time, groups 0-3 on the
+// first and 4-7 on the second, and last the blocks that no point reaches, whose
+// zeros a warp writes, 32 blocks an item.  The counts are known on the device
+// only; a CTA for every item there could be was 65,536 launches at 4096^2, most
+// of which found nothing to do.
+constexpr int kEmptyPerItem = 32;
+__global__ void __launch_bounds__(kGroups * kGroupThreads, 4)
+    k_cutoff(const CutInst* __restrict__ tab, int ninst, const float4* __restrict__ P,
+             const float* __restrict__ W, const uint32_t* __restrict__ start,
+             const uint32_t* __restrict__ order, const uint32_t* __restrict__ totals,
+             const int4* __restrict__ ranges, uint32_t* __restrict__ counts, int nblocks,
+             const CallScalars* __restrict__ err) {
+  // the groups' tables, then their running sums (cell r of lane l of group g
+  // at part[g][r][l])
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ ItemShared S;
+  GroupTables* tables = reinterpret_cast<GroupTables*>(smem);
+  float2 (*part)[8][kGroupThreads] =
+      reinterpret_cast<float2 (*)[8][kGroupThreads]>(smem + kCutTablesBytes);
+  const int g = threadIdx.x / kGroupThreads, lane = threadIdx.x % kGroupThreads;
+  // after a timed-out sort the bin starts may not rise, and positions taken
+  // from them could leave the sorted points: compute nothing (the call
+  // reports the timeout)
+  if (*reinterpret_cast<const volatile int*>(&err->err) & kErrSortTimeout) return;
+  // blocks to split, and the order positions of the first light and empty ones
+  const int64_t heavy = __ldg(counts), light = __ldg(counts + 1), empty = __ldg(counts + 2);
+  const int64_t slices = kSlices * heavy, singles = slices + (light - heavy);
+  const int64_t pairs = singles + (empty - light + 1) / 2;
+  const int64_t items = pairs + (nblocks - empty + kEmptyPerItem - 1) / kEmptyPerItem;
+  int64_t item = blockIdx.x;
+  while (item < items) {
+    // a CTA takes its next item when its long item ends (one taken before would
+    // wait for it: 4M points x 1024^2 at a reach of 14 cells 1243 us against
+    // 1056), and while it computes a short one
+    if (item >= singles) take_next(counts + 3, S);
+    if (item < singles) {
+      const bool slice = item < slices;
+      const int64_t pos = slice ? item / kSlices : heavy + (item - slices);
+      block_item(tab, ninst, P, W, start, (int)__ldg(order + pos),
+                 slice ? (int)(item % kSlices) : -1, totals, ranges, tables[g], part, counts + 3, S);
+    } else if (item < pairs) {
+      light_item(tab, ninst, P, W, start, order, totals, ranges, light + 2 * (item - singles),
+                 empty, tables[g], part, S);
+    } else {
+      for (int k = g; k < kEmptyPerItem; k += kGroups) {
+        const int64_t pos = empty + kEmptyPerItem * (item - pairs) + k;
+        if (pos >= nblocks) break;
+        int bx, by;
+        const CutInst& I = output_block(tab, ninst, (int)__ldg(order + pos), bx, by);
+        const int x = bx * kBin + (lane & 15);
+        for (int r = lane >> 4; r < kBin; r += 2) {
+          const int y = by * kBin + r;
+          if (x < I.nx && y < I.ny) I.out[(int64_t)y * I.nx + x] = 0.f * I.scale;
         }
-        const int x = bx * kBin + 2 * (l & 7) + r, y = by * kBin + slice * kSliceRows + (l >> 3);
-        if (x < I.nx && y < I.ny) I.out[(int64_t)y * I.nx + x] = (sum.x + sum.y) * I.scale;
       }
     }
+    __syncthreads();  // the item's shared memory is free, and S.next there
+    item = S.next;
+    __syncthreads();
   }
 }
 
@@ -831,12 +887,29 @@ CutoffGeom cutoff_geometry(int nx, int ny, double cs, double reach, int bin) {
   return g;
 }
 
+// Sort bins of 8 cells, 16 beyond a reach of 12.  A block reads the points of
+// about (16 + 2 reach + bin)^2 cells and computes the (16 + 2 reach)^2 cells'
+// that reach it; finer bins mean more bins to sort and to find, and three radix
+// passes sooner.  4-, 8- and 16-cell bins, us per call: 1M points x 1024^2 at a
+// reach of 3 cells 199 / 203 / 223, x 2048^2 275 / 254 / 258, 8M x 4096^2 1385 /
+// 1270 / 1258, 200,000 x 4096^2 at 14 cells 430 / 376 / 342, 8M 2594 / 2434 /
+// 2324.  4-cell bins only where the reach is short (a block then reads fewest
+// points beyond it), the points many and the bins still two passes' worth.
 int cutoff_sort_bin(int64_t n, int nx, int ny, double reach_cells) {
-  // an output block reads about (16 + 2 reach + bin)^2 cells' points, of which
-  // (16 + 2 reach)^2 can reach it; finer bins mean more bins to sort
-  int bin = reach_cells <= 6.0 ? 4 : reach_cells <= 16.0 ? 8 : 16;
+  const int64_t bins4 = (int64_t)((nx + 3) / 4) * ((ny + 3) / 4);
+  const bool fine = reach_cells <= 4.0 && n >= (1 << 18) && n >= 8 * bins4 && bins4 <= 65536;
+  int bin = fine ? 4 : reach_cells <= 12.0 ? 8 : 16;
   while (bin < 64 && ((int64_t)(nx + bin - 1) / bin) * ((ny + bin - 1) / bin) > (1 << 24)) bin *= 2;
   return bin;
+}
+
+// The four slices read (4 + 2 reach + bin) / (16 + 2 reach + bin) of the block's
+// points each: up to 6 cells of reach that costs little; beyond, they pay where
+// the grid has too few blocks to fill the GPU (200,000 points x 256^2 at 8
+// cells: 178 us whole, 139 sliced; 1M x 1024^2 at 14 cells: 352 and 470).
+bool cutoff_slices(int nx, int ny, double reach_cells) {
+  const double blocks = ((nx + kBin - 1) / kBin) * (double)((ny + kBin - 1) / kBin);
+  return reach_cells <= 6.0 || blocks * reach_cells <= 8192.0;
 }
 
 CutoffSizes cutoff_sizes(int64_t m, int64_t total_bins) {
@@ -913,7 +986,7 @@ cudaError_t launch_lookback_timeout_probe(uint32_t* buf, CallScalars* err, uint6
 }
 
 cudaError_t launch_cutoff_eval(const CutInst* tab, int ninst, int64_t cut_bins, int64_t slice_bins,
-                               const CutoffScratch& ws, cudaStream_t s) {
+                               const CutoffScratch& ws, int sms, cudaStream_t s) {
   if (ninst <= 0 || cut_bins <= 0) return cudaSuccess;
   if (cut_bins > 0x7fffffff || !ws.err) return cudaErrorInvalidValue;
   const int nb = (int)cut_bins, grid = (nb + 255) / 256;
@@ -923,10 +996,10 @@ cudaError_t launch_cutoff_eval(const CutInst* tab, int ninst, int64_t cut_bins, 
   k_cut_block_totals<<<grid, 256, 0, s>>>(tab, ninst, ws.start, nb, ws.totals, ws.ranges,
                                           ws.ocount);
   k_cut_order_scatter<<<grid, 256, 0, s>>>(tab, ninst, ws.totals, nb, ws.ocount, ws.order);
-  // one CTA per item: every block, plus three more slices for each block of a
-  // slicing instance that may turn out heavy
-  const int64_t ctas = (int64_t)nb + (int64_t)(kSlices - 1) * slice_bins;
-  if (ctas > 0x7fffffff) return cudaErrorInvalidValue;
+  // as many CTAs as stay on the GPU, or as there can be items: every block, and
+  // three more for each block of a slicing instance that may turn out heavy
+  const int64_t ctas = std::min((int64_t)nb + (int64_t)(kSlices - 1) * slice_bins,
+                                (int64_t)kCutCtasPerSm * sms);
   if ((e = cudaFuncSetAttribute(k_cutoff, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kCutSmemBytes)) != cudaSuccess)
     return e;

@@ -324,8 +324,7 @@ struct CutInst {
   // rest), and the reach beyond which points are dropped (range_reach)
   float cs_hi, cs_lo, drop_reach;
   // heavy output blocks (4096 or more points within reach) are computed as
-  // four 4-row slices: set for supports of at most 6 cells (4-cell sort bins),
-  // where a slice reads about half of the block's points
+  // four 4-row slices (cutoff_slices)
   int slice;
 };
 
@@ -405,6 +404,8 @@ inline double range_reach(double reach, const CutoffGeom& g) {
 // enough that an output block reads little beyond its support's reach, large
 // enough that the number of bins stays bounded.
 int cutoff_sort_bin(int64_t n, int nx, int ny, double reach_cells);
+// Whether its heavy output blocks are computed in slices.
+bool cutoff_slices(int nx, int ny, double reach_cells);
 struct CutoffScratch {
   uint32_t* keys[2];
   uint32_t* vals[2];
@@ -416,16 +417,16 @@ struct CutoffScratch {
   uint32_t* totals; // [cutoff output blocks] points within reach of each block
   int4* ranges;     // [cutoff output blocks] each block's sort-bin range (BinRange)
   uint32_t* ocount; // [kCutOcountWords] per-key block counts and cursors, blocks to split,
-                    // position of the first light block
+                    // positions of the first light and the first empty block, item counter
   CallScalars* err; // where a timed-out wait of the sort's look-back is recorded
 };
 // Weight classes of the cutoff path's output blocks (by points within reach:
 // 66 classes, and the same again above them for the heavy blocks the gather
 // splits into row slices); the ocount scratch holds their counts, their
-// cursors and the number of blocks to be split.
+// cursors, where the kinds of blocks begin and the gather's item counter.
 constexpr int kCutOrderClasses = 66;
 constexpr int kCutOrderKeys = 2 * kCutOrderClasses;
-constexpr int kCutOcountWords = 2 * kCutOrderKeys + 2;
+constexpr int kCutOcountWords = 2 * kCutOrderKeys + 4;
 struct CutoffSizes {
   int nchunks, passes;
   size_t hist_words;
@@ -451,9 +452,9 @@ cudaError_t launch_lookback_timeout_probe(uint32_t* buf, CallScalars* err, uint6
                                           cudaStream_t s);
 // The cutoff evaluation of the first ninst instances (output blocks
 // 0..cut_bins-1, of which slice_bins belong to instances with CutInst::slice
-// set): one CTA per block, or per 4-row slice of a heavy block.
+// set): blocks and 4-row slices of heavy blocks, by CTAs that stay.
 cudaError_t launch_cutoff_eval(const CutInst* tab, int ninst, int64_t cut_bins, int64_t slice_bins,
-                               const CutoffScratch& ws, cudaStream_t s);
+                               const CutoffScratch& ws, int sms, cudaStream_t s);
 
 // Adjoint of the Gaussian density (points prepared with sigma = 1/h) and the
 // grid LSCV loss.  hterm / lterm: per-point FP64 terms of dL/dh.
