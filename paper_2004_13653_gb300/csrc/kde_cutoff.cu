@@ -369,7 +369,8 @@ __device__ __forceinline__ void tabulate(GroupTables& T, int cnt, int lane, floa
   if (pt < cnt) {
     const float2 p = T.P[axis][pt];
     const float w = axis && !RADIAL ? T.W[pt] : 1.0f;
-    const float dh = g0.x - p.x, dl = g0.y - p.y;
+    const float2 d0 = pair_offset(g0, p);
+    const float dh = d0.x, dl = d0.y;
     float4* row = reinterpret_cast<float4*>(&T.K[axis][pt][0]);
 #pragma unroll
     for (int q = 0; q < kBin / 4; ++q) {

@@ -84,6 +84,15 @@ __device__ __forceinline__ float kradial(float q) {
   }
 }
 
+// g - p of two (hi, lo) pairs as a (hi, lo) pair: the hi parts' difference is
+// kept exactly, so that adding multiples of the cell's side to it loses no more
+// than the rounding of the sum.
+__device__ __forceinline__ float2 pair_offset(float2 g, float2 p) {
+  const float d = g.x - p.x, b = d - g.x;
+  const float e = (g.x - (d - b)) - (p.x + b);
+  return make_float2(d, (g.y - p.y) + e);
+}
+
 __device__ __forceinline__ void two_sum_acc(float2& run, float v) {
   const float s = run.x + v;
   const float bb = s - run.x;

@@ -55,3 +55,24 @@ def test_items(n, nx, ny, h_cells, kid):
         np.add.at(count, (a, b), s)
     near = count.cumsum(0).cumsum(1)[:ny, :nx] > 0
     assert (F[~near] == 0.0).all()
+
+
+@pytest.mark.parametrize("h_cells", [0.02, 0.3, 0.75])
+def test_supports_below_a_cell_near_the_origin(h_cells):
+    """Offsets from a block's first cell are up to 16 / h_cells bandwidths, of
+    which a point's own cell leaves less than one: FP32 must not round the
+    former (1e-6 bounds the result, whose slope per bandwidth is up to 1.5)."""
+    rng = np.random.default_rng(943)
+    nx, ny = 40, 37
+    wl = workloads.random_points(944, 4000, 400.0, 10.0, nx, ny, 10.0 * h_cells, oracle.QUARTIC)
+    cell = rng.integers(0, (nx, ny), (4000, 2))
+    wl.local[:] = 10.0 * (cell + 0.5 + rng.uniform(-1.0, 1.0, (4000, 2)) * h_cells)
+    F = kde.grid(torch.as_tensor(np.ascontiguousarray(wl.xy), dtype=torch.float64, device="cuda"),
+                 torch.as_tensor(wl.w, dtype=torch.float32, device="cuda"), wl.origin, wl.cell,
+                 nx, ny, wl.h, oracle.QUARTIC, flags=kde.FLAG_SYNC).cpu().numpy()
+    ref = oracle.kde_grid(wl.xy, wl.w, wl.origin, wl.cell, nx, ny, wl.h, oracle.QUARTIC)
+    cells = np.flatnonzero(ref.reshape(-1) > 0.01 * ref.max())
+    err = np.abs(F.reshape(-1)[cells] - ref.reshape(-1)[cells]) / ref.reshape(-1)[cells]
+    # a factor near the support's edge is steep relative to its value: 1% of the
+    # maximum still leaves u's error amplified by at most 2 * 1.5 / sqrt(0.01)
+    assert err.max() <= 30 * 2.0 ** -22
