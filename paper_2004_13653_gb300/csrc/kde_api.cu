@@ -192,22 +192,24 @@ int choose_tc_splits(int64_t tiles, int ctas, int64_t n_pad) {
   return best;
 }
 
-// Point-range splits of the SIMT path: the CTAs (tiles x splits) run `slots` at
-// a time, so the call takes as many rounds as that fills, each as long as one
-// split's points.  The split count with the fewest point-rounds wins, the
-// smaller one on a near tie; a split has at least 4096 points, which keeps the
-// partial grids' share small.  (Enough splits for six CTAs per SM, without a
-// look at the rounds, gave 928 CTAs for 456 slots on 512^2: two rounds and a
-// third of 16 CTAs, 15.2 ms for 1M points; whole rounds: 12.9 ms, and 11.9 ms
-// with four CTAs per SM.)
-int choose_simt_splits(int64_t tiles, int64_t slots, int64_t n_pad) {
-  const int64_t most = std::max<int64_t>(1, std::min<int64_t>(64, n_pad / 4096));
+// Point-range splits of the SIMT path.  A CTA (a tile's split) computes its
+// points at the same rate whether it shares its SM with three others or follows
+// them, but a quarter slower alone, so a call takes as long as the CTAs of the
+// SM that gets most of them: their points, 128 more for a CTA's start, a third
+// of a split while the last one ends alone, and the partial grids' traffic
+// (in points: 46 ns each).  Splits of 4096 points at least, four CTAs per SM at
+// a time, gave one split of 20,000 points x 128^2 259 us for 2 to 4 CTAs' work;
+// now 58.  The smaller count wins on a near tie.
+int choose_simt_splits(int64_t tiles, int64_t cells, int sms, int64_t n_pad, int most) {
   int best = 1;
   double best_cost = 0.0;
-  for (int64_t s = 1; s <= most; ++s) {
+  for (int64_t s = 1; s <= std::min<int64_t>(most, std::max<int64_t>(1, n_pad / 256)); ++s) {
     const int64_t per = ((n_pad + s - 1) / s + 255) / 256 * 256;  // whole register tiles
     const int64_t used = (n_pad + per - 1) / per;                 // splits with points
-    const double cost = (double)((tiles * used + slots - 1) / slots) * (double)per;
+    if (used < s) continue;                                       // a smaller s is the same
+    const int64_t ctas = tiles * used;
+    const double cost = (double)((ctas + sms - 1) / sms) * (per + 128.0) * (ctas <= sms ? 1.25 : 1.0) +
+                        0.3 * (double)per + (used > 1 ? 4.3e-5 * (double)cells * used : 0.0);
     if (s == 1 || cost < 0.99 * best_cost) {
       best = (int)s;
       best_cost = cost;
@@ -228,7 +230,7 @@ struct InstPlan {
   int path;
   int splits;
   int64_t n_pad, prep_begin;
-  size_t off_gxt, off_gyt, off_part, off_run;  // off_run: SIMT running sums
+  size_t off_gxt, off_gyt, off_part;
   // tensor-core path: the instance's tile family and accumulator chunk;
   // sparse: block-sparse skipping (asked for, or AUTO's choice)
   int fam, k_chunk, split_req;
@@ -427,8 +429,9 @@ struct BatchPlan {
   // entries follow the tensor-core ones
   std::vector<TcFamily> wide;
   int n_wide = 0;
+  bool simt_splits = false;  // some SIMT instance has more than two splits
   // whether the plan holds a choice that may be undone for want of workspace
-  bool chosen() const { return auto_sparse || n_wide; }
+  bool chosen() const { return auto_sparse || n_wide || simt_splits; }
   bool sorts() const { return n_cut || n_wide || sparse; }
   bool sparse = false;  // some tensor-core instances are block-sparse
   bool auto_sparse = false;  // ... by AUTO's choice: the dense plan does as well
@@ -443,8 +446,9 @@ struct BatchPlan {
       off_hout, total;
 };
 
-// allow_sparse: whether AUTO may choose the block-sparse contraction (false
-// when its workspace cannot be had).
+// allow_sparse: whether the plan may choose what needs more workspace, the
+// block-sparse contraction, the wide gather and many SIMT splits (false when
+// that workspace cannot be had).
 int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling* tiles,
               bool probe_memory, bool allow_sparse, BatchPlan* P) {
   P->count = count;
@@ -637,8 +641,11 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     int splits = I.split_req;
     if (I.path == KDE_PATH_SIMT_FP32) {
       if (splits == 0) {
+        // without a choice of the workspace, no more than two: their partial
+        // grids take what the running sums of one would in global memory
         splits = choose_simt_splits((int64_t)((a->nx + 127) / 128) * ((a->ny + 63) / 64),
-                                    (int64_t)kSimtCtasPerSm * sms, I.n_pad);
+                                    (int64_t)a->nx * a->ny, sms, I.n_pad, allow_sparse ? 64 : 2);
+        P->simt_splits = P->simt_splits || splits > 2;
       }
       ++P->n_simt;
     } else if (is_tc(I.path) && I.sparse) {
@@ -832,8 +839,6 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     I.off_gxt = take(sizeof(float2) * (size_t)A[k].nx);
     I.off_gyt = take(sizeof(float2) * (size_t)A[k].ny);
     I.off_part = I.splits > 1 ? take(sizeof(float) * (size_t)A[k].nx * A[k].ny * I.splits) : 0;
-    I.off_run = I.path == KDE_PATH_SIMT_FP32 ? take(simt_scratch_bytes(A[k].nx, A[k].ny, I.splits))
-                                             : 0;
   }
   if (P->sorts()) {
     const size_t u = sizeof(uint32_t);
@@ -1124,6 +1129,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       q.base_scale = compact_scale(k);
       q.kid = kid_of(&A[k]);
       sorted_inst(q, k, 1.0);
+      split_side(q.cs, &q.cs_hi, &q.cs_lo);
       tct.push_back(q);
     }
   for (int k = 0; k < count; ++k) {
@@ -1155,12 +1161,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
       q.kid = kid_of(&A[k]);
       q.scale = compact_scale(k);
       q.slice = cutoff_slices(A[k].nx, A[k].ny, A[k].h / A[k].cell);
-      uint32_t bits;
-      const float side = (float)q.cs;
-      memcpy(&bits, &side, sizeof(bits));
-      bits &= 0xFFFFFFC0u;
-      memcpy(&q.cs_hi, &bits, sizeof(bits));
-      q.cs_lo = (float)(q.cs - (double)q.cs_hi);
+      split_side(q.cs, &q.cs_hi, &q.cs_lo);
       q.drop_reach = (float)q.range_reach;
       cut.push_back(q);
     }
@@ -1319,8 +1320,9 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     const InstPlan& I = P.in[k];
     if (I.path != KDE_PATH_SIMT_FP32) continue;
     KDE_CUDA(launch_simt(kid_of(&A[k]), prep[k].pts, prep[k].wts, I.n_pad, prep[k].gxt,
-                         prep[k].gyt, A[k].nx, A[k].ny, I.splits, compact_scale(k),
-                         reinterpret_cast<float2*>(base + I.off_run), part_of(k), s),
+                         prep[k].gyt, A[k].nx, A[k].ny, prep[k].cell_sigma, I.splits,
+                         compact_scale(k),
+                         part_of(k), s),
              "SIMT direct sum");
   }
   if (overlap) {

@@ -360,8 +360,8 @@ __device__ __forceinline__ void accumulate(const GroupTables& T, int cnt, int cx
 
 // The factors of the first cnt <= kStep waiting points, lanes l and l + 16 for
 // point l's columns and rows: the offset from cell j is that from the item's
-// first cell, g0, plus j times the cell's side (its upper 18 bits, whose product
-// with j is exact, and the rest).  A slice has 4 rows.
+// first cell, g0, plus j times the cell's side (pair_offset).  A slice has 4
+// rows.
 template <int KID, bool RADIAL, int RPL>
 __device__ __forceinline__ void tabulate(GroupTables& T, int cnt, int lane, float2 g0, float cs_hi,
                                          float cs_lo) {

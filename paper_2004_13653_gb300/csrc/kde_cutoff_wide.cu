@@ -141,8 +141,7 @@ __device__ __forceinline__ void point_products(const Factors& f, Cells& acc) {
 
 // The products of the first m <= kStep waiting points.  Lanes l and l + 16 make
 // point l's 32 column and 32 row factors: the offset from cell j is that from
-// the tile's first cell plus j times the cell's side (its upper 18 bits, whose
-// product with j is exact, and the rest).
+// the tile's first cell plus j times the cell's side (pair_offset).
 template <int KID, bool RADIAL>
 __device__ __forceinline__ void step(WarpTables& T, int m, int lane, float2 g0, float cs_hi,
                                      float cs_lo, int cx, int cy, Cells& acc) {
@@ -186,8 +185,7 @@ __device__ __forceinline__ void warp_piece(const TcInst& I, const BinRange& br, 
                                            uint32_t begin, uint32_t end, int warp, int lane,
                                            WarpTables& T) {
   const float2 g0 = lane < 16 ? I.gxt[tm * kSide] : I.gyt[tn * kSide];
-  const float cs_hi = __uint_as_float(__float_as_uint((float)I.cs) & 0xFFFFFFC0u);
-  const float cs_lo = (float)(I.cs - (double)cs_hi);
+  const float cs_hi = I.cs_hi, cs_lo = I.cs_lo;
   // the tile's reach, widened as the bin ranges are: FP32 coordinates beyond it
   // have a factor of exactly zero at every cell
   const float rr = (float)I.range_reach;

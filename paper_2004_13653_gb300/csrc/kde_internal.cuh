@@ -110,6 +110,13 @@ inline double kernel_sigma(int kid, double h) {
   return kid == KDE_GAUSSIAN ? 1.0 / (h * 1.17741002251547469101) : 1.0 / h;
 }
 
+// A cell's side as a multiple of 2^-18 (from 64 on, the nearest FP32 number) and
+// the rest, for offsets of whole cells (pair_offset).
+inline void split_side(double cs, float* hi, float* lo) {
+  *hi = cs < 64.0 ? (float)(nearbyint(cs * 0x1p18) * 0x1p-18) : (float)cs;
+  *lo = (float)(cs - (double)*hi);
+}
+
 // ------------------------------------------------------- instance tables
 // Every launch is driven by a table of per-instance descriptors that lives in
 // the workspace; a single density is a batch of one.  Tables are written by
@@ -169,7 +176,10 @@ struct TcInst {
   double cs, reach, inv_binw;  // cell and reach in prepared units, 1 / bin width
   double range_reach;          // reach plus the bin keys' FP32 rounding margin (ranges use it)
   int nbx, nby, bin_begin, tile_begin;
-  int kid;  // the wide gather's kernel (part: the output; base_scale: its constant)
+  // the wide gather's kernel and cell side (part: the output; base_scale: its
+  // constant)
+  int kid;
+  float cs_hi, cs_lo;
 };
 
 // Points of bin rows lo_by..hi_by, columns lo_bx..hi_bx can reach the block
@@ -320,8 +330,7 @@ struct CutInst {
   int nbx, nby, bin_begin, nx, ny, kid;
   int obx, oby, out_begin;
   float scale;
-  // the gather's FP32 constants: the cell's side (its upper 18 bits and the
-  // rest), and the reach beyond which points are dropped (range_reach)
+  // the gather's FP32 constants: the cell's side (split_side), and the reach beyond which points are dropped (range_reach)
   float cs_hi, cs_lo, drop_reach;
   // heavy output blocks (4096 or more points within reach) are computed as
   // four 4-row slices (cutoff_slices)
@@ -356,14 +365,12 @@ cudaError_t launch_mercator(const double* lonlat, int64_t n, double lat0_deg, do
 cudaError_t launch_prepare(const PrepInst* tab, int ninst, int64_t total_pad, int max_side,
                            cudaStream_t s);
 
-// Path (a): FP32 SIMT direct sum into part[S][ny][nx] (scaled).
-// scratch: simt_scratch_bytes(nx, ny, splits) of device memory for the
-// running sums, or nullptr to keep them in shared memory (fewer CTAs per SM).
-constexpr int kSimtCtasPerSm = 4;  // with scratch
-size_t simt_scratch_bytes(int nx, int ny, int splits);
+// Path (a): FP32 SIMT direct sum into part[S][ny][nx] (scaled).  cs: cell side in
+// prepared units.
+constexpr int kSimtCtasPerSm = 4;
 cudaError_t launch_simt(int kid, const float4* pts, const float* wts, int64_t n_pad,
-                        const float2* gxt, const float2* gyt, int nx, int ny, int splits,
-                        float scale, float2* scratch, float* part, cudaStream_t s);
+                        const float2* gxt, const float2* gyt, int nx, int ny, double cs,
+                        int splits, float scale, float* part, cudaStream_t s);
 
 // Small Gaussian densities (kde_small.cu): q as for the prepare kernel, without
 // its tables and scalars; scal: where non-finite input is recorded, or null.

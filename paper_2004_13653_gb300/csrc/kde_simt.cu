@@ -10,13 +10,13 @@
 // from its use, and the next batch's points are loaded into registers
 // while the current batch is accumulated.  Points arrive in tiles of 256;
 // each thread sums one tile in registers and adds that partial into a
-// (hi, lo) running sum (in global scratch, or in shared memory for callers
-// without scratch) with an error-free two-sum, so the result does not degrade
-// with the number of points a cell sees.  The factors and the order of every sum are
-// those of a thread that evaluates its own factors, so the result does not
-// depend on the tabulation.
+// (hi, lo) running sum with an error-free two-sum, so the result does not
+// degrade with the number of points a cell sees.  The running sums of a CTA's
+// 8192 cells, 64 KB, live in tensor memory, which this path has no other use
+// for: four CTAs take all of an SM's.
 #include "kde_internal.cuh"
 #include "kernel_factors.cuh"
+#include "tc_ptx.cuh"
 
 namespace kde {
 namespace {
@@ -26,7 +26,11 @@ constexpr int kTileX = 128;    // cells along x per CTA
 constexpr int kTileY = 64;     // cells along y per CTA
 constexpr int kPtsTile = 256;  // points per register partial (two-sum cadence)
 constexpr int kBatch = 32;     // points per factor table
-constexpr int kTable = kBatch * (kTileX + kTileY);  // floats per table buffer
+constexpr uint32_t kRunCols = 128;  // tensor memory columns of a CTA's running sums
+// a table row, a point's x and y factors, is four floats longer than these, so
+// that eight lanes' 16-byte stores, a row each, take all the banks
+constexpr int kRow = kTileX + kTileY + 4;
+constexpr int kTable = kBatch * kRow;  // floats per table buffer
 
 struct TableRow {
   float4 xa, xb, ya, yb;
@@ -36,39 +40,51 @@ __device__ __forceinline__ TableRow table_row(const float* KX, const float* KY, 
                                               int ty) {
   // columns 4tx.. and 64+4tx..: a half-warp reads 256 contiguous bytes
   TableRow r;
-  r.xa = *reinterpret_cast<const float4*>(KX + q * kTileX + tx * 4);
-  r.xb = *reinterpret_cast<const float4*>(KX + q * kTileX + 64 + tx * 4);
-  r.ya = *reinterpret_cast<const float4*>(KY + q * kTileY + ty * 8);
-  r.yb = *reinterpret_cast<const float4*>(KY + q * kTileY + ty * 8 + 4);
+  r.xa = *reinterpret_cast<const float4*>(KX + q * kRow + tx * 4);
+  r.xb = *reinterpret_cast<const float4*>(KX + q * kRow + 64 + tx * 4);
+  r.ya = *reinterpret_cast<const float4*>(KY + q * kRow + ty * 8);
+  r.yb = *reinterpret_cast<const float4*>(KY + q * kRow + ty * 8 + 4);
   return r;
 }
 
-// GRUN: the (hi, lo) running sums live in global scratch (64 KB per CTA,
-// touched once per 256 points, so they stay in L2), which leaves shared
-// memory to the tables and four CTAs per SM; otherwise in shared memory (two
-// CTAs per SM, for callers that give no scratch).  Bound by instruction issue
-// (1.4 instructions per FMA) with the latencies four warps per scheduler leave
-// open: 1M points x 512^2 in 11.9 ms = 22 Tpair/s of 37; three CTAs per SM with
-// the next point's table row loaded ahead: 12.9 ms, packed two-lane FMAs (which
-// issue half as often, at three CTAs per SM): 14.5 ms.
-template <int KID, bool GRUN>
-__global__ void __launch_bounds__(kThreads, GRUN ? kSimtCtasPerSm : 2)
+// f32x2 arithmetic as the scalar instructions round it (denormals kept).
+__device__ __forceinline__ float2 p_add(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+      "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 p_sub(float2 a, float2 b) {
+  return p_add(a, make_float2(-b.x, -b.y));
+}
+__device__ __forceinline__ float2 p_fma(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+      "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+
+// Bound by the FMA pipe (a packed FMA is two of its cycles) and shared memory's
+// 128 bytes per clock to the registers.  1M points x 512^2: 11.9 ms with the
+// running sums in global memory, a table stage of a cell per lane and scalar
+// FMAs; 11.5 with points per lane and packed FMAs; 9.6 with the sums in tensor
+// memory; 9.3 = 28 Tpair/s with twice the splits (choose_simt_splits).
+template <int KID>
+__global__ void __launch_bounds__(kThreads, kSimtCtasPerSm)
     k_simt(const float4* __restrict__ pts, const float* __restrict__ wts, int64_t n_pad,
            int64_t per_split, const float2* __restrict__ gxt, const float2* __restrict__ gyt,
-           int nx, int ny, float scale, float2* __restrict__ grun, float* __restrict__ part) {
+           int nx, int ny, float cs_hi, float cs_lo, float scale, float* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char smem[];
   float* tables = reinterpret_cast<float*>(smem);                        // [2][kTable]
   const int tid = threadIdx.x, lane = tid & 31;
   const int tx = tid & 15, ty = tid >> 4;
   const int cx0 = blockIdx.x * kTileX, cy0 = blockIdx.y * kTileY;
-  // running sum of cell c = b * 8 + a of this thread: run[c * kThreads]
-  float2* run;
-  if (GRUN) {
-    const int64_t cta = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    run = grun + cta * 64 * kThreads + tid;
-  } else {
-    run = reinterpret_cast<float2*>(tables + 2 * kTable) + tid;  // [64][kThreads]
-  }
   float* dst = part + (int64_t)blockIdx.z * nx * ny;
   auto cell = [&](int b, int a, int& x, int& y) {
     y = cy0 + ty * 8 + b;
@@ -89,17 +105,31 @@ __global__ void __launch_bounds__(kThreads, GRUN ? kSimtCtasPerSm : 2)
       }
     return;
   }
-  // factor roles: x column tid; y row frow for points fq0 .. fq0 + kBatch/2 - 1
+  __shared__ uint32_t tmem_slot;
+  if (tid < 32) tc::tmem_alloc(&tmem_slot, kRunCols);
+  __syncthreads();
+  // this warp's lanes; row b's eight hi parts at column 16 b, its lo parts after
+  const uint32_t run = tmem_slot + ((uint32_t)(tid >> 5) << 21);
+  {
+    const float zero[16] = {};
+#pragma unroll
+    for (int b = 0; b < 8; ++b) tc::tmem_st16(run + 16 * b, zero);
+    tc::tmem_wait_st();
+  }
+
+  // factor roles: warp w makes columns 32 w.. and rows 16 w.. of every point,
+  // a point per lane
   static_assert(kThreads == kTileX && kThreads == 2 * kTileY, "factor roles");
   static_assert(kPtsTile % kBatch == 0 && kBatch == 32, "one point per lane per batch");
-  const float2 gxr = gxt[min(cx0 + tid, nx - 1)];
-  const int frow = tid & (kTileY - 1), fq0 = (tid / kTileY) * (kBatch / 2);
-  const float2 gyr = gyt[min(cy0 + frow, ny - 1)];
+  const int warp = tid >> 5;
+  const float2 gx0 = gxt[cx0], gy0 = gyt[cy0];
 
   // Every warp holds the points of the next batch in registers, one per
   // lane, loaded while the current batch is accumulated (the global-memory
-  // latency hides behind a whole batch); the tabulation broadcasts them with
-  // shuffles.
+  // latency hides behind a whole batch), and makes their factors lane by lane:
+  // the offset from cell j is that from the tile's first cell plus j times the
+  // cell's side (pair_offset).  A cell per lane, with the points broadcast by shuffles, took three
+  // times as much of shared memory's bandwidth.
   float4 nP;
   float nW;
   auto fetch = [&](int64_t first) {
@@ -112,112 +142,118 @@ __global__ void __launch_bounds__(kThreads, GRUN ? kSimtCtasPerSm : 2)
 
   int buf = 0;
   for (int64_t base = p_begin; base < p_end; base += kPtsTile) {
-    float acc[8][8];
+    float2 acc[8][4];
 #pragma unroll
     for (int b = 0; b < 8; ++b)
 #pragma unroll
-      for (int a = 0; a < 8; ++a) acc[b][a] = 0.f;
+      for (int a = 0; a < 4; ++a) acc[b][a] = make_float2(0.f, 0.f);
 
     for (int bb = 0; bb < kPtsTile; bb += kBatch, buf ^= 1) {
-      float* KX = tables + buf * kTable;  // [kBatch][kTileX]
-      float* KY = KX + kBatch * kTileX;   // [kBatch][kTileY]
+      float* KX = tables + buf * kTable;  // [kBatch][kRow]
+      float* KY = KX + kTileX;            // the same rows' y factors
       const float4 P = nP;
       const float W = nW;
       // This buffer was last read two batches ago, before the barrier of the
       // previous batch, which every thread has passed.
+      auto factors = [&](float2 d0, int j0, int count, float w, float* row) {
 #pragma unroll 8
-      for (int q = 0; q < kBatch; ++q) {
-        const float px = __shfl_sync(0xffffffffu, P.x, q), pxl = __shfl_sync(0xffffffffu, P.y, q);
-        KX[q * kTileX + tid] = kfactor<KID>((gxr.x - px) + (gxr.y - pxl));
-      }
-#pragma unroll 8
-      for (int k = 0; k < kBatch / 2; ++k) {
-        const int q = fq0 + k;
-        const float py = __shfl_sync(0xffffffffu, P.z, q), pyl = __shfl_sync(0xffffffffu, P.w, q);
-        const float w = __shfl_sync(0xffffffffu, W, q);
-        KY[q * kTileY + frow] = w * kfactor<KID>((gyr.x - py) + (gyr.y - pyl));
-      }
+        for (int q = 0; q < count; q += 4) {
+          float v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float j = (float)(j0 + q + e);
+            v[e] = w * kfactor<KID>(fmaf(j, cs_hi, d0.x) + fmaf(j, cs_lo, d0.y));
+          }
+          *reinterpret_cast<float4*>(row + j0 + q) = make_float4(v[0], v[1], v[2], v[3]);
+        }
+      };
+      factors(pair_offset(gx0, make_float2(P.x, P.y)), 32 * warp, 32, 1.0f, KX + lane * kRow);
+      factors(pair_offset(gy0, make_float2(P.z, P.w)), 16 * warp, 16, W, KY + lane * kRow);
       __syncthreads();
       fetch(base + bb + kBatch);
-#pragma unroll 4
+#pragma unroll 2
       for (int q = 0; q < kBatch; ++q) {
         const TableRow cur = table_row(KX, KY, q, tx, ty);
-        const float kx[8] = {cur.xa.x, cur.xa.y, cur.xa.z, cur.xa.w,
-                             cur.xb.x, cur.xb.y, cur.xb.z, cur.xb.w};
+        const float2 kx[4] = {make_float2(cur.xa.x, cur.xa.y), make_float2(cur.xa.z, cur.xa.w),
+                              make_float2(cur.xb.x, cur.xb.y), make_float2(cur.xb.z, cur.xb.w)};
         const float ky[8] = {cur.ya.x, cur.ya.y, cur.ya.z, cur.ya.w,
                              cur.yb.x, cur.yb.y, cur.yb.z, cur.yb.w};
 #pragma unroll
         for (int b = 0; b < 8; ++b)
 #pragma unroll
-          for (int a = 0; a < 8; ++a) acc[b][a] = fmaf(kx[a], ky[b], acc[b][a]);
+          for (int a = 0; a < 4; ++a)
+            acc[b][a] = p_fma(kx[a], make_float2(ky[b], ky[b]), acc[b][a]);
       }
     }
-    // this tile's partials into the running sums; after the last tile the
-    // sums are the cells' results
-    const bool first = base == p_begin, last = base + kPtsTile >= p_end;
+    // this tile's partials into the running sums, a row at a time
 #pragma unroll
-    for (int b = 0; b < 8; ++b)
+    for (int b = 0; b < 8; ++b) {
+      uint32_t in[16];
+      tc::tmem_ld_async(run + 16 * b, in);
+      tc::tmem_wait_ld();
+      float out[16];
 #pragma unroll
-      for (int a = 0; a < 8; ++a) {
-        float2 r = first ? make_float2(0.f, 0.f) : run[(b * 8 + a) * kThreads];
-        two_sum_acc(r, acc[b][a]);
-        if (last) {
-          int x, y;
-          cell(b, a, x, y);
-          if (x < nx && y < ny) dst[(int64_t)y * nx + x] = (r.x + r.y) * scale;
-        } else {
-          run[(b * 8 + a) * kThreads] = r;
-        }
+      for (int a = 0; a < 8; a += 2) {
+        const float2 r = make_float2(__uint_as_float(in[a]), __uint_as_float(in[a + 1]));
+        const float2 v = acc[b][a / 2], hi = p_add(r, v), t = p_sub(hi, r);
+        const float2 lo = p_add(make_float2(__uint_as_float(in[8 + a]), __uint_as_float(in[9 + a])),
+                                p_add(p_sub(r, p_sub(hi, t)), p_sub(v, t)));
+        out[a] = hi.x;
+        out[a + 1] = hi.y;
+        out[8 + a] = lo.x;
+        out[9 + a] = lo.y;
       }
+      tc::tmem_st16(run + 16 * b, out);
+    }
+    tc::tmem_wait_st();
   }
-}
-
-// 48 KB of tables (+ 64 KB of running sums without global scratch)
-constexpr size_t kSmemTables = 2 * kTable * sizeof(float);
-constexpr size_t kSmemRun = 64 * kThreads * sizeof(float2);
-
-template <int KID, bool GRUN>
-cudaError_t launch_kid(const float4* pts, const float* wts, int64_t n_pad, const float2* gxt,
-                       const float2* gyt, int nx, int ny, int splits, float scale, float2* grun,
-                       float* part, cudaStream_t s) {
-  const size_t smem = GRUN ? kSmemTables : kSmemTables + kSmemRun;
-  // per-device attribute; cheap, so set on every launch
-  cudaError_t e = cudaFuncSetAttribute(k_simt<KID, GRUN>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  int64_t per = (n_pad + splits - 1) / splits;
-  per = (per + kPtsTile - 1) / kPtsTile * kPtsTile;
-  if (per < kPtsTile) per = kPtsTile;
-  dim3 grid((nx + kTileX - 1) / kTileX, (ny + kTileY - 1) / kTileY, splits);
-  k_simt<KID, GRUN><<<grid, kThreads, smem, s>>>(pts, wts, n_pad, per, gxt, gyt, nx, ny, scale,
-                                                 grun, part);
-  note_launches(1);
-  return cudaGetLastError();
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    uint32_t in[16];
+    tc::tmem_ld_async(run + 16 * b, in);
+    tc::tmem_wait_ld();
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      int x, y;
+      cell(b, a, x, y);
+      if (x < nx && y < ny)
+        dst[(int64_t)y * nx + x] = (__uint_as_float(in[a]) + __uint_as_float(in[8 + a])) * scale;
+    }
+  }
+  __syncthreads();
+  if (tid < 32) tc::tmem_dealloc(tmem_slot, kRunCols);
 }
 
 template <int KID>
 cudaError_t launch_kid(const float4* pts, const float* wts, int64_t n_pad, const float2* gxt,
-                       const float2* gyt, int nx, int ny, int splits, float scale, float2* grun,
+                       const float2* gyt, int nx, int ny, double cs, int splits, float scale,
                        float* part, cudaStream_t s) {
-  return grun ? launch_kid<KID, true>(pts, wts, n_pad, gxt, gyt, nx, ny, splits, scale, grun,
-                                      part, s)
-              : launch_kid<KID, false>(pts, wts, n_pad, gxt, gyt, nx, ny, splits, scale, grun,
-                                       part, s);
+  constexpr size_t smem = 2 * kTable * sizeof(float);
+  // per-device attribute; cheap, so set on every launch
+  cudaError_t e = cudaFuncSetAttribute(k_simt<KID>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  int64_t per = (n_pad + splits - 1) / splits;
+  per = (per + kPtsTile - 1) / kPtsTile * kPtsTile;
+  if (per < kPtsTile) per = kPtsTile;
+  float cs_hi, cs_lo;
+  split_side(cs, &cs_hi, &cs_lo);
+  dim3 grid((nx + kTileX - 1) / kTileX, (ny + kTileY - 1) / kTileY, splits);
+  k_simt<KID><<<grid, kThreads, smem, s>>>(pts, wts, n_pad, per, gxt, gyt, nx, ny, cs_hi,
+                                           cs_lo, scale, part);
+  note_launches(1);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
-size_t simt_scratch_bytes(int nx, int ny, int splits) {
-  return (size_t)((nx + kTileX - 1) / kTileX) * ((ny + kTileY - 1) / kTileY) * splits * kSmemRun;
-}
-
 cudaError_t launch_simt(int kid, const float4* pts, const float* wts, int64_t n_pad,
-                        const float2* gxt, const float2* gyt, int nx, int ny, int splits,
-                        float scale, float2* scratch, float* part, cudaStream_t s) {
+                        const float2* gxt, const float2* gyt, int nx, int ny, double cs, int splits,
+                        float scale, float* part, cudaStream_t s) {
   switch (kid) {
-#define KDE_CASE(K) \
-  case K:           \
-    return launch_kid<K>(pts, wts, n_pad, gxt, gyt, nx, ny, splits, scale, scratch, part, s);
+#define KDE_CASE(K)                                                                          \
+  case K:                                                                                    \
+    return launch_kid<K>(pts, wts, n_pad, gxt, gyt, nx, ny, cs, splits, scale, part, s);
     KDE_CASE(KDE_UNIFORM)
     KDE_CASE(KDE_TRIANGULAR)
     KDE_CASE(KDE_EPANECHNIKOV)

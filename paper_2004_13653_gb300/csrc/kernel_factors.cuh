@@ -84,13 +84,17 @@ __device__ __forceinline__ float kradial(float q) {
   }
 }
 
-// g - p of two (hi, lo) pairs as a (hi, lo) pair: the hi parts' difference is
-// kept exactly, so that adding multiples of the cell's side to it loses no more
-// than the rounding of the sum.
+// g - p of two (hi, lo) pairs, as a multiple of 2^-18 (or of a larger power of
+// two) and the rest; nothing of it is lost.  split_side's parts of the cell's
+// side are made alike, so that the offset from the j-th cell after g,
+//   fmaf(j, side hi, hi) + fmaf(j, side lo, lo),
+// has an exact first term wherever a kernel is not zero (below 64 in size), and
+// the sum's rounding, as g_j - p from a table of the cells has.
 __device__ __forceinline__ float2 pair_offset(float2 g, float2 p) {
   const float d = g.x - p.x, b = d - g.x;
   const float e = (g.x - (d - b)) - (p.x + b);
-  return make_float2(d, (g.y - p.y) + e);
+  const float hi = (d + 48.0f) - 48.0f;  // 48 = 1.5 * 2^23 * 2^-18
+  return make_float2(hi, (d - hi) + ((g.y - p.y) + e));
 }
 
 __device__ __forceinline__ void two_sum_acc(float2& run, float v) {
