@@ -15,7 +15,8 @@
 // Terms beyond a point's own +-8 bandwidths but inside the shared window are
 // added where the other form leaves them out (they are below e^-32).
 // Bound by FP32 FMA issue.  1.47M points x 1024^2, h = 3.07 cells: 3.33 ms one
-// warp per point, 0.79 ms in groups (0.9 with the sort).
+// warp per point, 0.79 ms in groups (0.9 with the sort), 0.75 with the inner loops
+// ended at the window's 58 cells instead of the 64 of the tables.
 #include <algorithm>
 
 #include "kde_internal.cuh"
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(kThreads)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // after a timed-out sort the bin starts are not trusted: compute nothing
   if (*reinterpret_cast<const volatile int*>(&err->err) & kErrSortTimeout) return;
+  const int wu = kAdjBin + 2 * R;  // the window's cells, of the W (a multiple of 32) computed
   const uint32_t n_items = *count;
   for (;;) {
     __syncthreads();
@@ -180,7 +182,7 @@ __global__ void __launch_bounds__(kThreads)
         const float* a0 = sA + pb * WP;
         const float* g0 = sG + blk * WP;
 #pragma unroll 1
-        for (int i = 0; i < W; i += 4) {
+        for (int i = 0; i < wu; i += 4) {
           float4 a[8];
 #pragma unroll
           for (int s = 0; s < 8; ++s)
@@ -241,7 +243,7 @@ __global__ void __launch_bounds__(kThreads)
         const float* b0 = sB + 8 * pb;
         const float* g0 = sG + 4 * blk;
 #pragma unroll 2
-        for (int j = 0; j < W; ++j) {
+        for (int j = 0; j < wu; ++j) {
           const float4 b1 = *reinterpret_cast<const float4*>(b0 + j * kPP);
           const float4 b2 = *reinterpret_cast<const float4*>(b0 + j * kPP + 4);
           const float b[8] = {b1.x, b1.y, b1.z, b1.w, b2.x, b2.y, b2.z, b2.w};
