@@ -474,11 +474,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             const float2 y = fma2(make_float2(v0, v1), make_float2(v0, v1),
                                   make_float2(-15.f, -15.f));
             const float x0 = ex2_neg(y.x), x1 = ex2_neg(y.y);
-            const float h0 = __uint_as_float(__float_as_uint(x0) & 0xFFFFE000u);
-            const float h1 = __uint_as_float(__float_as_uint(x1) & 0xFFFFE000u);
-            const float2 l = sub2(make_float2(x0, x1), make_float2(h0, h1));
-            const __half2 hh = __floats2half2_rn(h0, h1);
-            const __half2 ll = __floats2half2_rn(l.x, l.y);
+            const __half2 hh = __floats2half2_rn(x0, x1);
+            const __half2 ll = __floats2half2_rn(minus_half(x0, __low2half(hh)),
+                                                 minus_half(x1, __high2half(hh)));
             hw[e2] = *reinterpret_cast<const uint32_t*>(&hh);
             lw[e2] = *reinterpret_cast<const uint32_t*>(&ll);
           }

@@ -393,12 +393,12 @@ __global__ void __launch_bounds__(kThreads, 1)
               const float2 u = add2(P2[e2], ng2);   // point - cell, in units of h sqrt(2 ln 2)
               const float2 y = fma2(u, u, N2[e2]);  // u^2 - exponent offset
               const float v0 = ex2_neg(y.x), v1 = ex2_neg(y.y);
-              // hi = v with 11 significant bits (exact in FP16), lo = v - hi
-              const float h0 = __uint_as_float(__float_as_uint(v0) & 0xFFFFE000u);
-              const float h1 = __uint_as_float(__float_as_uint(v1) & 0xFFFFE000u);
-              const float2 l = sub2(make_float2(v0, v1), make_float2(h0, h1));
-              const __half2 hh = __floats2half2_rn(h0, h1);
-              const __half2 ll = __floats2half2_rn(l.x, l.y);
+              // hi = v rounded to FP16, lo = v - hi (one instruction each; masking hi
+              // out of v and subtracting it took three for two: 5.31 ms, now 5.21 for
+              // 20M points x 4096^2)
+              const __half2 hh = __floats2half2_rn(v0, v1);
+              const __half2 ll = __floats2half2_rn(minus_half(v0, __low2half(hh)),
+                                                   minus_half(v1, __high2half(hh)));
               hw[e2] = *reinterpret_cast<const uint32_t*>(&hh);
               lw[e2] = *reinterpret_cast<const uint32_t*>(&ll);
             }

@@ -2,6 +2,8 @@
 // bounded waits, the tcgen05 MMA / TMEM instructions, and shared-memory
 // matrix descriptors for the 128-byte-swizzled K-major operand layout.
 #pragma once
+#include <cuda_fp16.h>
+
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -298,6 +300,16 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
       "mov.b64 {%0, %1}, rd;\n\t}"
       : "=f"(d.x), "=f"(d.y)
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+
+// v - h, exact for h = v rounded to FP16: the mixed-precision FMA reads the FP16
+// half where it lies.
+__device__ __forceinline__ float minus_half(float v, __half h) {
+  float d;
+  asm("{\n\t.reg .b16 m1;\n\tmov.b16 m1, 0xBC00;\n\tfma.rn.f32.f16 %0, %1, m1, %2;\n\t}"
+      : "=f"(d)
+      : "h"(__half_as_ushort(h)), "f"(v));
   return d;
 }
 // 2^(-y) (MUFU ex2, approximate, subnormals flushed)
