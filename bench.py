@@ -43,18 +43,30 @@ TRAFFIC = {("tc_split16", 4096, 40_000): {
     "bytes": 1255729152 + 527909888}}
 
 
-def sparse_products(xy, origin, cell, nx, ny, h):
+def sparse_geometry(path, cell, nx, ny, h):
+    """Tile side and sort-bin side, in cells, of the block-sparse contraction of
+    one instance: split-FP16 runs on 128 x 128 tiles up to a reach of about 170
+    cells, CTA pairs on 256 x 256; bins of 8 cells, doubled while the grid has
+    more than 2^16 of them (32 at most)."""
+    side = 128 if path == "tc_split16" and 6.45 * h * 1.17741 / cell <= 170 else 256
+    b = 8
+    while b < 32 and ((nx + b - 1) // b) * ((ny + b - 1) // b) > 65536:
+        b *= 2
+    return side, b
+
+
+def sparse_products(xy, origin, cell, nx, ny, h, side=256, bin=32):
     """Point-tile pairs the block-sparse contraction multiplies out: for each
-    256 x 256 tile, the points of the 32 x 32-cell bins within 6.45 h sqrt(2 ln 2)
-    of it (the library's binning, in FP64 here).  Times 65536 cells and 2 FLOP
-    per product this is the contraction's algorithmic work."""
+    tile of side x side cells, the points of the bin x bin-cell sort bins within
+    6.45 h sqrt(2 ln 2) of it (the library's binning, in FP64 here).  Times side^2
+    cells and 2 FLOP per product this is the contraction's algorithmic work."""
     import numpy as np
     sigma = 1.0 / (h * 1.17741002251547469101)
     cs = cell * sigma
     # the library's ranges widen the reach by the FP32 rounding margin of its bin keys
     reach = 6.45 + 1e-6 + 8.0 * 2.0 ** -24 * (max(nx, ny) * cs + 6.45)
-    inv_binw = 1.0 / (32 * cs)
-    nbx, nby = (nx + 31) // 32, (ny + 31) // 32
+    inv_binw = 1.0 / (bin * cs)
+    nbx, nby = (nx + bin - 1) // bin, (ny + bin - 1) // bin
     X = (xy[:, 0] - origin[0]) * sigma
     Y = (xy[:, 1] - origin[1]) * sigma
     keep = (X >= -reach) & (Y >= -reach) & (X <= nx * cs + reach) & (Y <= ny * cs + reach)
@@ -64,11 +76,11 @@ def sparse_products(xy, origin, cell, nx, ny, h):
     S = np.zeros((nby + 1, nbx + 1), np.int64)
     S[1:, 1:] = H.cumsum(0).cumsum(1)
     total = 0
-    for tn in range((ny + 255) // 256):
-        y0, y1 = (tn * 256 + 0.5) * cs - reach, (tn * 256 + 255.5) * cs + reach
+    for tn in range((ny + side - 1) // side):
+        y0, y1 = (tn * side + 0.5) * cs - reach, (tn * side + side - 0.5) * cs + reach
         ly, hy = max(0, int(np.floor(y0 * inv_binw))), min(nby - 1, int(np.floor(y1 * inv_binw)))
-        for tm in range((nx + 255) // 256):
-            x0, x1 = (tm * 256 + 0.5) * cs - reach, (tm * 256 + 255.5) * cs + reach
+        for tm in range((nx + side - 1) // side):
+            x0, x1 = (tm * side + 0.5) * cs - reach, (tm * side + side - 0.5) * cs + reach
             lx = max(0, int(np.floor(x0 * inv_binw)))
             hx = min(nbx - 1, int(np.floor(x1 * inv_binw)))
             total += S[hy + 1, hx + 1] - S[ly, hx + 1] - S[hy + 1, lx] + S[ly, lx]
@@ -76,10 +88,9 @@ def sparse_products(xy, origin, cell, nx, ny, h):
 
 
 def cutoff_pairs(xy, origin, cell, nx, ny, h):
-    """Point-cell pairs the cutoff path evaluates: every 16 x 16-cell output
-    block reads the points of the sort bins (4, 8 or 16 cells, chosen from
-    h/cell) whose points can lie within a bandwidth of its cell centres (the
-    library's binning, in FP64 here)."""
+    """Point-cell pairs of 16 x 16-cell blocks and the points of the sort bins
+    (4, 8 or 16 cells, chosen from h/cell) within a bandwidth of their cell
+    centres: what a gather evaluates that computes every point it reads."""
     import numpy as np
     rc = h / cell
     S = 4 if rc <= 6.0 else 8 if rc <= 16.0 else 16
@@ -111,6 +122,29 @@ def cutoff_pairs(xy, origin, cell, nx, ny, h):
     LX, LY = np.where(ok, LX, 0), np.where(ok, LY, 0)
     reach_pts = C[HY1, HX1] - C[LY, HX1] - C[HY1, LX] + C[LY, LX]
     return int(B * B * reach_pts.sum())
+
+
+def evaluated_pairs(xy, origin, cell, nx, ny, h):
+    """Point-cell pairs the cutoff path evaluates: the points within a bandwidth
+    of a block's cell centres along both axes, times its cells; blocks are 16 x 16
+    cells, and 32 x 32 where the support is more than 16 cells and the (tile,
+    point) pairs number half a million (the library's rule)."""
+    import numpy as np
+    r = h / cell
+
+    def expected(n):  # the rule's tiles per point along one axis
+        return min(1.0 + 2.0 * r / 32, (n + 31.0) / 32)
+    B = 32 if r > 16.0 and len(xy) * expected(nx) * expected(ny) >= 5e5 else 16
+    X = (np.asarray(xy[:, 0], np.float64) - origin[0]) / cell
+    Y = (np.asarray(xy[:, 1], np.float64) - origin[1]) / cell
+
+    def span(c, n):
+        # blocks [B t + 1/2, min(B t + B, n) - 1/2] within r of c
+        last = (n + B - 1) // B - 1
+        lo = np.maximum(np.ceil((c - r - B + 0.5) / B), 0.0)
+        hi = np.minimum(np.floor((c + r - 0.5) / B), last)
+        return np.where(c - r > n - 0.5, 0.0, np.maximum(hi - lo + 1.0, 0.0))
+    return int(B * B * (span(X, nx) * span(Y, ny)).sum())
 
 
 def support_pairs(xy, origin, cell, nx, ny, h):
@@ -381,8 +415,8 @@ def run_ours(args):
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         peak_pairs = alu_peak_pairs(peaks, sms)
         pairs = evals
-        if args.path == "cutoff":  # only the pairs of the bins within reach are evaluated
-            pairs = cutoff_pairs(xy_dev.cpu().numpy().reshape(-1, 2), origin, wl.cell, nx, ny,
+        if args.path == "cutoff":  # only the pairs of blocks and points within reach
+            pairs = evaluated_pairs(xy_dev.cpu().numpy().reshape(-1, 2), origin, wl.cell, nx, ny,
                                  wl.h)
         achieved = pairs / (kernel_ms * 1e-3)
         roof = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_pairs / 1e12,
@@ -398,8 +432,9 @@ def run_ours(args):
         flops = 2.0 * products * evals
         if args.flags & kde.FLAG_SKIP_ZERO:  # only the pairs within reach are multiplied
             xy_proj = xy_dev.cpu().numpy().reshape(-1, 2)  # the projected fixes
-            flops = 2.0 * products * 65536.0 * sparse_products(xy_proj, origin, wl.cell, nx, ny,
-                                                                wl.h)
+            side, sbin = sparse_geometry(args.path, wl.cell, nx, ny, wl.h)
+            flops = 2.0 * products * side * side * sparse_products(
+                xy_proj, origin, wl.cell, nx, ny, wl.h, side, sbin)
         peak = peaks["bf16_tflops_sustained"]
         achieved = flops / (kernel_ms * 1e-3) / 1e12
         roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
@@ -582,11 +617,14 @@ def run_ours(args):
         if sparse_e2e is not None:
             result["block_sparse"]["e2e"] = sparse_e2e
         products = 3 if args.path == "tc_split16" else 1
-        pt = sparse_products(xy_dev.cpu().numpy().reshape(-1, 2), origin, wl.cell, nx, ny, wl.h)
-        flops = 2.0 * products * 65536.0 * pt
+        side, sbin = sparse_geometry(args.path, wl.cell, nx, ny, wl.h)
+        pt = sparse_products(xy_dev.cpu().numpy().reshape(-1, 2), origin, wl.cell, nx, ny, wl.h,
+                             side, sbin)
+        flops = 2.0 * products * side * side * pt
         ach = flops / (result["block_sparse"]["kernel_ms"] * 1e-3) / 1e12
         peak = peaks["bf16_tflops_sustained"]
         result["block_sparse"]["point_tile_pairs"] = pt
+        result["block_sparse"]["tile_side"] = side
         result["block_sparse"]["roofline"] = {
             "bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
             "frac": ach / peak, "traffic": None,
@@ -750,12 +788,12 @@ def configs12_leg(dev, peaks, sms, local):
                       "note": "whole call: centring, contraction and split-K reduce"}
     tc["vs_simt"] = out["config2_gaussian_simt_fp32"]["ms_per_call"] / tc["ms_per_call"]
     cut = out["config2_epanechnikov_cutoff"]
-    pairs = cutoff_pairs(c2.xy, c2.origin, c2.cell, c2.nx, c2.ny, c2.h)
+    pairs = evaluated_pairs(c2.xy, c2.origin, c2.cell, c2.nx, c2.ny, c2.h)
     peak_a = alu_peak_pairs(peaks, sms)
     cut["roofline"] = dict(cutoff_roofline(pairs, support_pairs(c2.xy, c2.origin, c2.cell, c2.nx,
                                                                 c2.ny, c2.h),
                                            cut["ms_per_call"], c2.n, c2.nx, c2.ny, peaks, peak_a),
-                           note="evaluated pairs (16x16-cell blocks x points of the sort bins "
+                           note="evaluated pairs (16x16-cell blocks x points "
                                 "within reach) over the whole call")
     out["config2_points"] = c2.n
     out["clocks"] = clk
@@ -836,7 +874,7 @@ def batched_leg(dev, peaks, sms, local):
         if x.kernel == 6:
             t_roof += 6.0 * x.n * x.nx * x.ny / peak_t
         else:
-            t_roof += cutoff_pairs(x.xy, x.origin, x.cell, x.nx, x.ny, x.h) / peak_a
+            t_roof += evaluated_pairs(x.xy, x.origin, x.cell, x.nx, x.ny, x.h) / peak_a
     pairs = float(sum(x.n * x.nx * x.ny for x in inst))
     del insts, outs, g
     torch.cuda.empty_cache()
@@ -946,14 +984,15 @@ def adjoint_leg(dev, args, local):
         e_xy = float(np.max(np.abs(gxy.cpu().numpy()[sel] - rxy)) / np.max(np.abs(rxy)))
         res[{"simt": "window", "tc_split16": "contractions"}[path] + "_rel_linf_vs_oracle"] = \
             max(e_w, e_xy)
-    n_pad = (wl.n + 511) // 512 * 512
-    pad = lambda v: (v + 255) // 256 * 256
-    flops = 2 * 3 * 2.0 * n_pad * pad(wl.nx) * pad(wl.ny)
+    # the contractions take the cells within 8 h of each tile of sorted points;
+    # counted here are those within 8 h of each point
+    flops = 2 * 3 * 2.0 * support_pairs(wl.xy, wl.origin, wl.cell, wl.nx, wl.ny, 8.0 * h)
     peaks, _ = load_peaks()
     ach = flops / (res["contractions_ms"] * 1e-3) / 1e12
     res["roofline"] = {"bound": "tensor", "achieved": ach, "peak": peaks["bf16_tflops_sustained"],
                        "unit": "TFLOP/s", "frac": ach / peaks["bf16_tflops_sustained"],
-                       "note": "both contractions and the cotangent tiling, whole call"}
+                       "note": "products within +-8 h of the points; whole call: sort, both "
+                               "contractions and the cotangent tiling"}
     res["speedup"] = res["window_ms"] / res["contractions_ms"]
     return res
 

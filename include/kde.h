@@ -87,12 +87,15 @@ typedef enum {
 
 #define KDE_FLAG_SYNC 1u         /* wait for completion and check device flags */
 #define KDE_FLAG_SKIP_ZERO 2u    /* TC paths: block-sparse skipping. Points are */
-                                 /* sorted into small bins and each 256x256    */
-                                 /* tile reads only the bins within 6.45        */
-                                 /* h sqrt(2 ln 2) (~7.6 h) of it; beyond that  */
-                                 /* every FP16 operand is exactly zero, so no   */
-                                 /* product changes (Table 1 Gaussian).  Runs   */
-                                 /* on CTA pairs (KDE_ENOTSUP with ONE_CTA).    */
+                                 /* sorted into small bins and each tile reads  */
+                                 /* only the bins within 6.45 h sqrt(2 ln 2)    */
+                                 /* (~7.6 h) of it; beyond that every FP16      */
+                                 /* operand is exactly zero, so no product      */
+                                 /* changes (Table 1 Gaussian).  Split-FP16     */
+                                 /* runs on 128x128 tiles, one CTA each, or,    */
+                                 /* where that is the faster or CTA_PAIR is     */
+                                 /* named, on 256x256 CTA-pair tiles, FP16 on   */
+                                 /* the latter (KDE_ENOTSUP with ONE_CTA).      */
                                  /* Workspace grows by the piece partials.      */
 #define KDE_FLAG_CTA_PAIR 4u     /* TC paths: 256x256 tiles on pairs of CTAs    */
                                  /* (tcgen05 cta_group::2); the default with    */
@@ -247,10 +250,12 @@ int kde_grid_batched_tiled(const kde_args* inst, const kde_tiling* tiles, int co
  *   dL/dh   = -(2/h) sum_ij G_ij F_ij + c sum_p w_p sum_ij G_ij r^2/h^3 A B,
  * c = 1/(2 pi N h^2), A, B the 1-D Gaussian factors, recomputed on the fly.
  * Two forms: a window kernel that sums each point's +-8h window on the FP32
- * pipes (opts->path KDE_PATH_SIMT_FP32), and, for wide bandwidths, two
+ * pipes (opts->path KDE_PATH_SIMT_FP32; many points are sorted and share
+ * windows in groups), and, for wide bandwidths, two
  * tcgen05 contractions U = G B and V = G^T A (split-FP16, three products;
  * KDE_PATH_TC_SPLIT16 or KDE_PATH_TC_FP16) whose epilogues fold U and V
- * into the per-point sums.  KDE_PATH_AUTO takes the contractions when the
+ * into the per-point sums, over the cells within 8h of each tile of sorted
+ * points.  KDE_PATH_AUTO takes the contractions when the
  * window covers more than 0.6% of the grid padded to 256-cell tiles.
  * Requires a->points on the device and kernel_id == KDE_GAUSSIAN.  dL/dh
  * makes the call synchronous (and reports KDE_ETIMEOUT from the
@@ -317,9 +322,10 @@ int kde_grid_binned(const double* points, const int64_t* traj_offsets, int64_t n
  * metres; keep: device [n] (1 = kept); out_points: device [2n] or NULL,
  * receives the kept points in order; out_offsets: device [ntraj+1] or NULL,
  * the trajectories' bounds in out_points; n_kept, iterations: host, optional.
- * Synchronous: every iteration runs inside one cooperative launch (the loop
- * ends on the device when an iteration keeps no point), and the call reads
- * the iteration count and the kept count back once.  Errors: KDE_EINVAL (n,
+ * Synchronous: trajectories of up to a few thousand points run their iterations
+ * in one launch, a CTA each, and the others all of theirs in one cooperative
+ * launch (the loop ends on the device); the call reads the iteration count and
+ * the kept count back once.  Errors: KDE_EINVAL (n,
  * eps, pointers, alignment, offsets that do not rise from 0 to n), KDE_EDATA
  * (non-finite coordinate), KDE_ECUDA (the device cannot hold the cooperative
  * launch's CTAs at once).

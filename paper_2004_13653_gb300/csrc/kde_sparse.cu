@@ -9,7 +9,7 @@
 // from it along x or along y.  Skipping those (tile, point) pairs therefore
 // changes no product, only which zeros are added.
 //
-// The points are sorted into bins of 4 to 32 cells a side (the cutoff path's
+// The points are sorted into bins of 8 to 32 cells a side (the cutoff path's
 // stable radix sort, with that reach); a tile (128 x 128 or
 // 256 x 256 cells) then needs only the bins
 // within reach, i.e. one contiguous run of sorted points per bin row.  This
