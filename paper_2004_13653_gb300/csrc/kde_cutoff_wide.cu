@@ -23,9 +23,8 @@
 //
 // 1M points x 1000 x 900, reach 40 cells, quartic: 1150 us in 16 x 16 blocks,
 // 838 with the factors tabulated a cell per lane (each point read as a
-// broadcast), 680 now: the FMA pipe takes about two thirds of it (a packed FMA
-// is two cycles), the three float4 reads a point about as much of shared
-// memory's bandwidth.
+// broadcast), 670 now: the three float4 reads a point keep shared memory's data
+// pipe 94% busy, the FMA pipe (a packed FMA is two cycles) 70%.
 #include "kde_internal.cuh"
 #include "kernel_factors.cuh"
 

@@ -113,3 +113,32 @@ def test_smaller_workspace_takes_the_blocks():
         ref = oracle.kde_cells(wl.xy, wl.w, wl.origin, wl.cell, wl.nx, wl.ny, wl.h,
                                oracle.EPANECHNIKOV, np.unique(cells))
         assert rel_linf(F.reshape(-1)[np.unique(cells)], ref) <= TOL_FP32
+
+
+def test_more_than_1024_tiles():
+    """35 x 34 tiles: the work list of several launches."""
+    wl = case(150_000, 1100, 1060, 17.0, oracle.QUARTIC, seed=936)
+    F = kde.grid(*args(wl), oracle.QUARTIC, flags=kde.FLAG_SYNC).cpu().numpy()
+    cells = np.random.default_rng(8).integers(0, wl.nx * wl.ny, 400)
+    cells = np.unique(np.append(cells, int(np.argmax(F))))
+    ref = oracle.kde_cells(wl.xy, wl.w, wl.origin, wl.cell, wl.nx, wl.ny, wl.h, oracle.QUARTIC,
+                           cells)
+    assert rel_linf(F.reshape(-1)[cells], ref) <= TOL_FP32
+
+
+@pytest.mark.parametrize("gauss", [(60_000, 1500, 1300, 1.0), (20_000, 256, 256, 40.0)],
+                         ids=["block_sparse", "dense"])
+def test_beside_a_contraction(gauss):
+    """On the side stream of a batch with a Gaussian: the bits of a call alone."""
+    n, nx, ny, h_cells = gauss
+    wls = [case(150_000, 96, 70, 20.0, oracle.TRIWEIGHT, seed=937),
+           workloads.random_points(938, n, 20.0 * max(nx, ny), 20.0, nx, ny, 20.0 * h_cells,
+                                   oracle.GAUSSIAN),
+           case(90_000, 300, 280, 18.0, oracle.EPANECHNIKOV, seed=939)]
+    kids = ["triweight", "gaussian", "epanechnikov"]
+    names = ("points", "weights", "origin", "cell", "nx", "ny", "h", "kernel")
+    insts = [dict(zip(names, args(w) + (k,))) for w, k in zip(wls, kids)]
+    for _ in range(2):
+        out = kde.grid_batched(insts)
+        for k in (0, 2):
+            assert torch.equal(out[k], kde.grid(*args(wls[k]), kids[k]))
