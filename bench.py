@@ -127,14 +127,15 @@ def cutoff_pairs(xy, origin, cell, nx, ny, h):
 def evaluated_pairs(xy, origin, cell, nx, ny, h):
     """Point-cell pairs the cutoff path evaluates: the points within a bandwidth
     of a block's cell centres along both axes, times its cells; blocks are 16 x 16
-    cells, and 32 x 32 where the support is more than 16 cells and the (tile,
-    point) pairs number half a million (the library's rule)."""
+    cells, and 32 x 32 where the support is more than 16 cells and a tile has
+    2500 points within reach (the library's rule for product kernels)."""
     import numpy as np
     r = h / cell
 
     def expected(n):  # the rule's tiles per point along one axis
         return min(1.0 + 2.0 * r / 32, (n + 31.0) / 32)
-    B = 32 if r > 16.0 and len(xy) * expected(nx) * expected(ny) >= 5e5 else 16
+    visits = len(xy) * expected(nx) * expected(ny)
+    B = 32 if r > 16.0 and visits >= max(2.5e5, 2500.0 * -(-nx // 32) * -(-ny // 32)) else 16
     X = (np.asarray(xy[:, 0], np.float64) - origin[0]) / cell
     Y = (np.asarray(xy[:, 1], np.float64) - origin[1]) / cell
 

@@ -401,19 +401,35 @@ int64_t reach_tiles(double reach_cells, const InstPlan& I, int side) {
   return std::min<int64_t>(per_axis, I.tiles_m) * std::min<int64_t>(per_axis, I.tiles_n);
 }
 
-// Whether a compact kernel's instance takes the wide gather: supports of more
-// than 16 cells a side from the point, and half a million (tile, point) pairs,
-// enough pieces to fill the GPU.  Epanechnikov and radial quartic, us per call,
-// 16 x 16 blocks against 32 x 32 tiles: 1M points x 1024^2 at reach 12 cells
-// 387 / 333 and 600 / 618, at 20 cells 772 / 449 and 1393 / 928; 200,000 points
-// x 512^2 at 20 cells 269 / 164 and 406 / 287; 20,000 points x 256^2 at 20 cells
-// 100 / 111 and 121 / 173, 2,000 points 70 / 74 and 71 / 110.
-constexpr int kWidePiece = 8192;
-bool wide_gather(const kde_args* a) {
+// Whether a compact kernel's instance takes the wide gather: a product kernel
+// (a radial one costs a profile per pair, and the larger tiles hold more pairs
+// beyond the disk), a support of more than 16 cells, and 2500 points within reach
+// of a tile on average, a quarter of a million in all.  Epanechnikov, lane
+// traffic, us per call in 16 x 16 blocks against 32 x 32 tiles: 1M points x 1024^2
+// at reach 17 cells (4150 a tile) 426 / 424, at 28 cells 701 / 572, at 57 cells
+// 1993 / 1303; 200,000 x 512^2 at 28 cells 262 / 199, x 2048^2 (370 a tile) 238 /
+// 275; 50,000 x 1500^2 at 40 cells 150 / 193; radial tricube 1M x 1024^2 at 28
+// cells 2989 / 4444.
+double wide_visits(const kde_args* a) {  // (tile, point) pairs, about
   const double reach = a->h / a->cell;
   const double tx = std::min(1.0 + 2.0 * reach / kWideSide, (a->nx + kWideSide - 1.0) / kWideSide);
   const double ty = std::min(1.0 + 2.0 * reach / kWideSide, (a->ny + kWideSide - 1.0) / kWideSide);
-  return reach > 16.0 && (double)a->n * tx * ty >= 5e5;
+  return (double)a->n * tx * ty;
+}
+bool wide_gather(const kde_args* a) {
+  const double tiles = (double)((a->nx + kWideSide - 1) / kWideSide) *
+                       (double)((a->ny + kWideSide - 1) / kWideSide);
+  return kid_of(a) < kRadial && a->h / a->cell > 16.0 &&
+         wide_visits(a) >= std::max(2.5e5, 2500.0 * tiles);
+}
+// Points of a piece: 8192 (1M points x 1000 x 900, reach 40: 885 us per call with
+// 2048, 832 with 4096, 808 with 8192), fewer while the pieces would not be four
+// for each of the CTAs that run at a time.
+int wide_piece(const kde_args* a) {
+  const double visits = wide_visits(a);
+  int L = 8192;
+  while (L > 512 && visits < 1216.0 * L) L /= 2;
+  return L;
 }
 
 struct BatchPlan {
@@ -727,11 +743,10 @@ int make_plan(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     const int64_t tiles = (int64_t)I.tiles_m * I.tiles_n;
     const int64_t visits =
         I.n_pad * reach_tiles(range_reach(1.0, I.geo) * a->h / a->cell, I, kWideSide);
-    // pieces of kWidePiece points (1M points x 1000 x 900, reach 40: 885 us per call
-    // with 2048, 832 with 4096, 808 with 8192), longer ones where their partial tiles
-    // would take more than a gigabyte (a function of the instance alone, so
-    // that it is computed the same way in any batch)
-    int L = kWidePiece;
+    // longer pieces where their partial tiles would take more than a gigabyte
+    // (a function of the instance alone, so that it is computed the same way in
+    // any batch)
+    int L = wide_piece(a);
     while (L < kSparseMaxPiece && visits / L > (1 << 17)) L *= 2;
     int f = 0;
     while (f < (int)P->wide.size() && P->wide[f].piece_len != L) ++f;

@@ -1,4 +1,4 @@
-// Path (c) for supports of many cells: 32 x 32-cell tiles, one warp each.
+// Path (c), product kernels over supports of many cells: 32 x 32-cell tiles.
 //
 // The gather of kde_cutoff.cu computes 16 x 16-cell blocks: per 32 points a
 // warp tabulates 32 factors a point and then adds 256 products a point, eight
@@ -105,19 +105,15 @@ __device__ __forceinline__ void flush(WarpTables& T, int lane, Cells& acc) {
 // A point's factors at a lane's columns and rows.
 struct Factors {
   float4 x0, x1, y;
-  float w;
 };
-template <bool RADIAL>
 __device__ __forceinline__ Factors load_factors(const WarpTables& T, int c, int cx, int cy) {
   Factors f;
   f.x0 = *reinterpret_cast<const float4*>(&T.K[0][c][cx]);
   f.x1 = *reinterpret_cast<const float4*>(&T.K[0][c][cx + 4]);
   f.y = *reinterpret_cast<const float4*>(&T.K[1][c][cy]);
-  f.w = RADIAL ? T.W[c] : 0.f;
   return f;
 }
 
-template <int KID, bool RADIAL>
 __device__ __forceinline__ void point_products(const Factors& f, Cells& acc) {
   const float2 x[4] = {make_float2(f.x0.x, f.x0.y), make_float2(f.x0.z, f.x0.w),
                        make_float2(f.x1.x, f.x1.y), make_float2(f.x1.z, f.x1.w)};
@@ -126,28 +122,20 @@ __device__ __forceinline__ void point_products(const Factors& f, Cells& acc) {
   for (int r = 0; r < 4; ++r) {
     const float2 yy = make_float2(y[r], y[r]);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (RADIAL) {
-        const float2 q = p_add(x[j], yy);
-        acc.v[r][j] = p_fma(make_float2(f.w, f.w),
-                            make_float2(kradial<KID>(q.x), kradial<KID>(q.y)), acc.v[r][j]);
-      } else {
-        acc.v[r][j] = p_fma(x[j], yy, acc.v[r][j]);
-      }
-    }
+    for (int j = 0; j < 4; ++j) acc.v[r][j] = p_fma(x[j], yy, acc.v[r][j]);
   }
 }
 
 // The products of the first m <= kStep waiting points.  Lanes l and l + 16 make
 // point l's 32 column and 32 row factors: the offset from cell j is that from
 // the tile's first cell plus j times the cell's side (pair_offset).
-template <int KID, bool RADIAL>
+template <int KID>
 __device__ __forceinline__ void step(WarpTables& T, int m, int lane, float2 g0, float cs_hi,
                                      float cs_lo, int cx, int cy, Cells& acc) {
   const int axis = lane >> 4, pt = lane & (kStep - 1);
   if (pt < m) {
     const float2 p = T.P[axis][pt];
-    const float w = axis && !RADIAL ? T.W[pt] : 1.0f;
+    const float w = axis ? T.W[pt] : 1.0f;
     const float2 d0 = pair_offset(g0, p);
     const float dh = d0.x, dl = d0.y;
     float4* row = reinterpret_cast<float4*>(&T.K[axis][pt][0]);
@@ -159,8 +147,8 @@ __device__ __forceinline__ void step(WarpTables& T, int m, int lane, float2 g0, 
         const float2 j = make_float2((float)(4 * q + e), (float)(4 * q + e + 1));
         const float2 u = p_add(p_fma(j, make_float2(cs_hi, cs_hi), make_float2(dh, dh)),
                                p_fma(j, make_float2(cs_lo, cs_lo), make_float2(dl, dl)));
-        v[e] = RADIAL ? u.x * u.x : w * kfactor<KID>(u.x);
-        v[e + 1] = RADIAL ? u.y * u.y : w * kfactor<KID>(u.y);
+        v[e] = w * kfactor<KID>(u.x);
+        v[e + 1] = w * kfactor<KID>(u.y);
       }
       row[q] = make_float4(v[0], v[1], v[2], v[3]);
     }
@@ -168,18 +156,18 @@ __device__ __forceinline__ void step(WarpTables& T, int m, int lane, float2 g0, 
   __syncwarp();
   int c = 0;
   for (; c + 2 <= m; c += 2) {
-    const Factors a = load_factors<RADIAL>(T, c, cx, cy);
-    const Factors b = load_factors<RADIAL>(T, c + 1, cx, cy);
-    point_products<KID, RADIAL>(a, acc);
-    point_products<KID, RADIAL>(b, acc);
+    const Factors a = load_factors(T, c, cx, cy);
+    const Factors b = load_factors(T, c + 1, cx, cy);
+    point_products(a, acc);
+    point_products(b, acc);
   }
-  if (c < m) point_products<KID, RADIAL>(load_factors<RADIAL>(T, c, cx, cy), acc);
+  if (c < m) point_products(load_factors(T, c, cx, cy), acc);
   __syncwarp();  // the tables are consumed
 }
 
 // The batches of one warp: points begin + 32 (warp + 8 k) of the tile's runs,
 // up to end.
-template <int KID, bool RADIAL>
+template <int KID>
 __device__ __forceinline__ void warp_piece(const TcInst& I, const BinRange& br, int tm, int tn,
                                            uint32_t begin, uint32_t end, int warp, int lane,
                                            WarpTables& T) {
@@ -234,7 +222,7 @@ __device__ __forceinline__ void warp_piece(const TcInst& I, const BinRange& br, 
         flush(T, lane, acc);
         held = 0;
       }
-      step<KID, RADIAL>(T, kStep, lane, g0, cs_hi, cs_lo, cx, cy, acc);
+      step<KID>(T, kStep, lane, g0, cs_hi, cs_lo, cx, cy, acc);
       held += kStep;
       waiting -= kStep;
       // the points left, at most 31, move to the front
@@ -257,7 +245,7 @@ __device__ __forceinline__ void warp_piece(const TcInst& I, const BinRange& br, 
   }
   if (waiting) {
     if (held == kBatch) flush(T, lane, acc);
-    step<KID, RADIAL>(T, waiting, lane, g0, cs_hi, cs_lo, cx, cy, acc);
+    step<KID>(T, waiting, lane, g0, cs_hi, cs_lo, cx, cy, acc);
   }
   flush(T, lane, acc);
 }
@@ -331,11 +319,8 @@ __global__ void __launch_bounds__(kThreads, 2)
   const BinRange br = s_br;
   const uint32_t begin = (uint32_t)pc.k_begin, end = (uint32_t)pc.vend;
   switch (I.kid) {
-#define KDE_WIDE(K)                                                                            \
-  case K: warp_piece<K, false>(I, br, pc.tm, pc.tn, begin, end, warp, lane, tables[warp]); break; \
-  case kRadial + K:                                                                            \
-    warp_piece<K, true>(I, br, pc.tm, pc.tn, begin, end, warp, lane, tables[warp]);            \
-    break;
+#define KDE_WIDE(K) \
+  case K: warp_piece<K>(I, br, pc.tm, pc.tn, begin, end, warp, lane, tables[warp]); break;
     KDE_WIDE(KDE_UNIFORM)
     KDE_WIDE(KDE_TRIANGULAR)
     KDE_WIDE(KDE_EPANECHNIKOV)

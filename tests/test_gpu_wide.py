@@ -1,6 +1,6 @@
-"""The compact kernels' gather on 32 x 32-cell tiles (supports of more than 16
-cells, half a million (tile, point) pairs): every kernel and its radial variant
-against the FP64 oracle at the cutoff path's 1e-6, on ragged grids around the
+"""The compact kernels' gather on 32 x 32-cell tiles (product kernels, supports
+of more than 16 cells, dense points; their radial variants stay in 16 x 16
+blocks at the same sizes): every kernel and its radial variant against the FP64 oracle at the cutoff path's 1e-6, on ragged grids around the
 tile's side, tiles of one piece and of many, points outside the grid, signed
 weights; the same results in a batch, under graph capture and again; and the
 16 x 16-cell blocks where the workspace holds no more."""
@@ -105,7 +105,7 @@ def test_smaller_workspace_takes_the_blocks():
     a = args(wl)
     out = torch.empty(wl.ny, wl.nx, device="cuda")
     full = kde.workspace_size(*a, "epanechnikov", out)
-    # the pieces' partial tiles alone take 200,000 x 16 / 8192 x 8 KB = 3 MB
+    # the pieces' partial tiles alone take 200,000 x 16 / 512 x 8 KB = 51 MB
     for size in (full, full - (2 << 20)):
         ws = torch.empty(size, dtype=torch.uint8, device="cuda")
         F = kde.grid(*a, "epanechnikov", workspace=ws, flags=kde.FLAG_SYNC).cpu().numpy()
@@ -117,7 +117,7 @@ def test_smaller_workspace_takes_the_blocks():
 
 def test_more_than_1024_tiles():
     """35 x 34 tiles: the work list of several launches."""
-    wl = case(150_000, 1100, 1060, 17.0, oracle.QUARTIC, seed=936)
+    wl = case(800_000, 1100, 1060, 17.0, oracle.QUARTIC, seed=936)
     F = kde.grid(*args(wl), oracle.QUARTIC, flags=kde.FLAG_SYNC).cpu().numpy()
     cells = np.random.default_rng(8).integers(0, wl.nx * wl.ny, 400)
     cells = np.unique(np.append(cells, int(np.argmax(F))))
