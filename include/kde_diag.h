@@ -50,6 +50,23 @@ int kde_diag_wait_timeout(int64_t limit_ns, void* stream);
 int kde_diag_sort_wait_timeout(int64_t limit_ns, void* stream);
 
 /*
+ * kde_diag_adjoint_list — the work list of the adjoint's window form alone (no
+ * counterpart in the paper): the groups of at most 64 points of every sort bin,
+ * from the bin starts, as kde_grid_backward makes it after its sort.  start:
+ * device, [nbins + 1], the sorted position of each bin's first point and, last,
+ * of the first point beyond every cell's reach; m: the sorted points; list:
+ * device, [m / 64 + nbins + 2][4], 16-byte aligned, receives (bin, first point,
+ * points, 0) in no particular order, bin nbins for the points beyond reach;
+ * counters: device, [2], receives the number of groups and a zero.  With
+ * sort_failed the sort counts as timed out: its bin starts may then be anything,
+ * and nothing is listed.  Without it they have to rise from 0 to at most m.
+ * Synchronous; uses the library workspace.  Errors: KDE_EINVAL (nbins, m,
+ * pointers, alignment), KDE_ENOMEM, KDE_ECUDA.
+ */
+int kde_diag_adjoint_list(const uint32_t* start, int nbins, int64_t m, int sort_failed,
+                          int32_t* list, uint32_t* counters, void* stream);
+
+/*
  * kde_diag_peak_rates — measures, at the clock the GPU runs at, the rates the
  * rooflines of the tensor-core and exp-bound kernels are set against (no
  * counterpart in the paper): rates[0] = tcgen05 kind::f16 MMAs on CTA pairs

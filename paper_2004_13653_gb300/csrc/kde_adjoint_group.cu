@@ -34,10 +34,14 @@ constexpr int kPP = kP + 4;    // row of the y-factor table: 16-byte aligned, sp
 
 // Lists the groups of every bin (first point and count; the order is whatever
 // the atomics give and decides only which CTA takes a group), and those of the
-// points beyond every cell's reach, which only get zeros.
+// points beyond every cell's reach, which only get zeros.  After a timed-out sort
+// the bin starts need not rise, and the differences of two that fall would list
+// groups past the end of the list: nothing is listed then.
 __global__ void __launch_bounds__(256)
     k_adj_groups(const uint32_t* __restrict__ start, int nbins, int64_t m,
-                 int4* __restrict__ list, uint32_t* __restrict__ count) {
+                 int4* __restrict__ list, uint32_t* __restrict__ count,
+                 const CallScalars* __restrict__ err) {
+  if (*reinterpret_cast<const volatile int*>(&err->err) & kErrSortTimeout) return;
   const int b = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
   uint32_t a = 0, n = 0;
   if (b <= nbins) {
@@ -331,12 +335,18 @@ int adj_group_radius(double cell, double h) { return (int)ceil(8.0 * h / cell) +
 // 12 cells per thread at most: 96 x 96 cells and the tables of 64 points take 88 KB
 bool adj_group_fits(int R) { return kAdjBin + 2 * R <= 96; }
 
-cudaError_t launch_adjoint_group(const AdjGroupArgs& a, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(a.counters, 0, 2 * sizeof(uint32_t), s);
+cudaError_t launch_adjoint_list(const AdjGroupArgs& a, cudaStream_t s) {
+  const cudaError_t e = cudaMemsetAsync(a.counters, 0, 2 * sizeof(uint32_t), s);
   if (e != cudaSuccess) return e;
-  k_adj_groups<<<(a.nbins + 1 + 255) / 256, 256, 0, s>>>(a.start, a.nbins, a.m, a.list, a.counters);
+  k_adj_groups<<<(a.nbins + 1 + 255) / 256, 256, 0, s>>>(a.start, a.nbins, a.m, a.list, a.counters,
+                                                         a.err);
   note_launches(1);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_adjoint_group(const AdjGroupArgs& a, cudaStream_t s) {
+  const cudaError_t e = launch_adjoint_list(a, s);
+  if (e != cudaSuccess) return e;
   const int W = kAdjBin + 2 * a.R;
   if (W <= 32) return launch_rt<4>(a, s);
   if (W <= 64) return launch_rt<8>(a, s);

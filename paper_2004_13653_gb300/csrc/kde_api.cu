@@ -1997,6 +1997,34 @@ int kde_diag_exclusive_scan(const uint32_t* in, uint32_t* out, int64_t n, int pe
   return KDE_OK;
 }
 
+int kde_diag_adjoint_list(const uint32_t* start, int nbins, int64_t m, int sort_failed,
+                          int32_t* list, uint32_t* counters, void* stream) {
+  if (nbins < 1 || m < 0 || m >= ((int64_t)1 << 32))
+    return fail(KDE_EINVAL, "nbins must be positive and m in [0, 2^32)");
+  if (!start || !list || !counters) return fail(KDE_EINVAL, "null pointer");
+  if (memory_kind(start) != 0 || memory_kind(list) != 0 || memory_kind(counters) != 0)
+    return fail(KDE_EINVAL, "kde_diag_adjoint_list needs device pointers");
+  if (reinterpret_cast<uintptr_t>(list) & 15) return fail(KDE_EINVAL, "list must be 16-byte aligned");
+  void* ws = nullptr;
+  int rc = library_workspace(sizeof(CallScalars), &ws);
+  if (rc) return rc;
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  CallScalars hs = {};
+  if (sort_failed) hs.err = kErrTimeout | kErrSortTimeout;
+  KDE_CUDA(launch_upload(&hs, sizeof(hs), ws, s), "write status");
+  AdjGroupArgs a = {};
+  a.start = start;
+  a.nbins = nbins;
+  a.m = m;
+  a.list = reinterpret_cast<int4*>(list);
+  a.counters = counters;
+  a.err = static_cast<const CallScalars*>(ws);
+  KDE_CUDA(launch_adjoint_list(a, s), "list of the adjoint's groups");
+  KDE_CUDA(cudaStreamSynchronize(s), "synchronize");
+  g_err[0] = 0;
+  return KDE_OK;
+}
+
 const char* kde_version(void) { return "kde-gb300 0.1 (sm_103a)"; }
 
 }  // extern "C"

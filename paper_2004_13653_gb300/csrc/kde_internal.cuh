@@ -491,6 +491,8 @@ struct AdjGroupArgs {
 };
 int adj_group_radius(double cell, double h);  // window half-width R, cells
 bool adj_group_fits(int R);
+// The list of the groups alone (start, nbins, m, list, counters and err of a).
+cudaError_t launch_adjoint_list(const AdjGroupArgs& a, cudaStream_t s);
 cudaError_t launch_adjoint_group(const AdjGroupArgs& a, cudaStream_t s);
 // The same adjoint as two tcgen05 contractions (points prepared in the
 // Gaussian's units, sigma = 1/(h sqrt(2 ln 2)), and their cell tables):
