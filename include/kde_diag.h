@@ -67,6 +67,21 @@ int kde_diag_adjoint_list(const uint32_t* start, int nbins, int64_t m, int sort_
                           int32_t* list, uint32_t* counters, void* stream);
 
 /*
+ * kde_diag_piece_reduce — the sum of a tiled grid's piece partials alone (no
+ * counterpart in the paper), as the block-sparse contraction (side 128 or 256)
+ * and the wide gather of the compact kernels (side 32) end with it: out(i, j) =
+ * the sum over the pieces piece_begin[t] .. piece_begin[t + 1] - 1 of cell (i, j)'s
+ * tile t, in order; tiles of side x side cells, row by row.  piece_begin: device,
+ * [tiles + 1], any values: those above max_pieces count as max_pieces.  part:
+ * device, 16-byte aligned, [max_pieces][side][side] floats, for side 32 pairs of
+ * floats (a sum's high and low part).  For side 32 a tile of exactly one piece is
+ * left as it is (the gather writes it).  out: device, [ny * nx].  Synchronous;
+ * uses the library workspace.  Errors: KDE_EINVAL, KDE_ENOMEM, KDE_ECUDA.
+ */
+int kde_diag_piece_reduce(const uint32_t* piece_begin, const float* part, int max_pieces, int side,
+                          int nx, int ny, float* out, void* stream);
+
+/*
  * kde_diag_peak_rates — measures, at the clock the GPU runs at, the rates the
  * rooflines of the tensor-core and exp-bound kernels are set against (no
  * counterpart in the paper): rates[0] = tcgen05 kind::f16 MMAs on CTA pairs

@@ -64,7 +64,8 @@ EXPORTS = ("kde_default_opts", "kde_grid", "kde_grid_ex", "kde_workspace_size",
            "kde_last_error", "kde_release", "kde_version", "kde_launch_count",
            "kde_diag_exclusive_scan", "kde_grid_noalloc", "kde_diag_wait_timeout",
            "kde_grid_binned", "kde_dp_simplify", "kde_diag_peak_rates",
-           "kde_diag_sort_wait_timeout", "kde_set_stream", "kde_diag_adjoint_list")
+           "kde_diag_sort_wait_timeout", "kde_set_stream", "kde_diag_adjoint_list",
+           "kde_diag_piece_reduce")
 
 _lib = None
 
@@ -126,6 +127,8 @@ def load(build_if_stale: bool = False) -> ctypes.CDLL:
     lib.kde_diag_sort_wait_timeout.restype = i32
     lib.kde_diag_adjoint_list.argtypes = [vp, i32, i64, i32, vp, vp, vp]
     lib.kde_diag_adjoint_list.restype = i32
+    lib.kde_diag_piece_reduce.argtypes = [vp, vp, i32, i32, i32, i32, vp, vp]
+    lib.kde_diag_piece_reduce.restype = i32
     lib.kde_set_stream.argtypes = [vp]
     lib.kde_set_stream.restype = None
     lib.kde_diag_peak_rates.argtypes = [P(ctypes.c_double * 3), vp]

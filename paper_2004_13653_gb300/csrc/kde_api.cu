@@ -2025,6 +2025,45 @@ int kde_diag_adjoint_list(const uint32_t* start, int nbins, int64_t m, int sort_
   return KDE_OK;
 }
 
+int kde_diag_piece_reduce(const uint32_t* piece_begin, const float* part, int max_pieces, int side,
+                          int nx, int ny, float* out, void* stream) {
+  if (side != 128 && side != 256 && side != kWideSide)
+    return fail(KDE_EINVAL, "side must be 32, 128 or 256");
+  if (nx < 1 || ny < 1 || (int64_t)nx * ny >= (int64_t)1 << 31 || max_pieces < 1 ||
+      max_pieces > (1 << 24))
+    return fail(KDE_EINVAL, "grid or max_pieces out of range");
+  if (!piece_begin || !part || !out) return fail(KDE_EINVAL, "null pointer");
+  if (memory_kind(piece_begin) != 0 || memory_kind(part) != 0 || memory_kind(out) != 0)
+    return fail(KDE_EINVAL, "kde_diag_piece_reduce needs device pointers");
+  if (reinterpret_cast<uintptr_t>(part) & 15) return fail(KDE_EINVAL, "part must be 16-byte aligned");
+  struct alignas(16) Entry {
+    TcInst inst;
+  } t = {};
+  t.inst.part = out;
+  t.inst.nx = nx;
+  t.inst.ny = ny;
+  t.inst.tiles_m = (nx + side - 1) / side;
+  t.inst.tiles_n = (ny + side - 1) / side;
+  t.inst.base_scale = 1.0f;
+  void* ws = nullptr;
+  int rc = library_workspace(sizeof(t), &ws);
+  if (rc) return rc;
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  KDE_CUDA(launch_upload(&t, sizeof(t), ws, s), "upload table");
+  SparseCtl sp = {};
+  sp.piece_begin = piece_begin;
+  sp.part = const_cast<float*>(part);
+  sp.tiles_total = t.inst.tiles_m * t.inst.tiles_n;
+  sp.max_pieces = max_pieces;
+  sp.side = side;
+  const TcInst* tab = static_cast<const TcInst*>(ws);
+  KDE_CUDA(side == kWideSide ? launch_wide_reduce(tab, 1, sp, s) : launch_sparse_reduce(tab, 1, sp, s),
+           "piece reduce");
+  KDE_CUDA(cudaStreamSynchronize(s), "synchronize");
+  g_err[0] = 0;
+  return KDE_OK;
+}
+
 const char* kde_version(void) { return "kde-gb300 0.1 (sm_103a)"; }
 
 }  // extern "C"

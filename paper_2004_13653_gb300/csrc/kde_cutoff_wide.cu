@@ -358,8 +358,8 @@ __global__ void __launch_bounds__(kRedThreads)
     k_wide_reduce(const TcInst* __restrict__ tab, int ninst, SparseCtl sp,
                   const float2* __restrict__ part) {
   const int t = blockIdx.x;
-  const int p0 = min((int)sp.piece_begin[t], sp.max_pieces);
-  const int p1 = min((int)sp.piece_begin[t + 1], sp.max_pieces);
+  const int p0 = bounded_piece(sp.piece_begin[t], sp.max_pieces);
+  const int p1 = bounded_piece(sp.piece_begin[t + 1], sp.max_pieces);
   if (p1 - p0 == 1) return;
   int a = 0, b = ninst - 1;
   while (a < b) {
@@ -391,6 +391,13 @@ __global__ void __launch_bounds__(kRedThreads)
 
 }  // namespace
 
+cudaError_t launch_wide_reduce(const TcInst* tab, int ninst, const SparseCtl& sp, cudaStream_t s) {
+  k_wide_reduce<<<dim3(sp.tiles_total, kCellsPerTile / kRedThreads), kRedThreads, 0, s>>>(
+      tab, ninst, sp, reinterpret_cast<const float2*>(sp.part));
+  note_launches(1);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_cutoff_wide(const TcInst* tab, int ninst, const SparseCtl& sp, CallScalars* err,
                                cudaStream_t s) {
   if (ninst < 1 || sp.side != kSide || sp.tiles_total < 1 || sp.piece_len < 1 || sp.max_pieces < 1)
@@ -400,11 +407,9 @@ cudaError_t launch_cutoff_wide(const TcInst* tab, int ninst, const SparseCtl& sp
   if (e != cudaSuccess) return e;
   float2* part = reinterpret_cast<float2*>(sp.part);
   k_cutoff_wide<<<sp.max_pieces, kThreads, kSmemBytes, s>>>(tab, ninst, sp, part, err);
+  note_launches(1);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_wide_reduce<<<dim3(sp.tiles_total, kCellsPerTile / kRedThreads), kRedThreads, 0, s>>>(
-      tab, ninst, sp, part);
-  note_launches(2);
-  return cudaGetLastError();
+  return launch_wide_reduce(tab, ninst, sp, s);
 }
 
 }  // namespace kde

@@ -306,6 +306,12 @@ struct SparseCtl {
   int side;                     // cells of a tile's side: 128 (one CTA), 256 (CTA pair) or
                                 // kWideSide (the compact kernels' wide gather)
 };
+// A piece index of the work list as the reduces read it: after a timed-out sort
+// the list may hold any 32-bit number, and whatever it holds, no piece outside
+// the partial buffer is read.
+__host__ __device__ inline int bounded_piece(uint32_t piece, int max_pieces) {
+  return piece < (uint32_t)max_pieces ? (int)piece : max_pieces;
+}
 // Longest piece the planner makes.
 constexpr int kSparseMaxPiece = 32768;
 
@@ -597,6 +603,7 @@ cudaError_t launch_sparse_plan(const TcInst* tab, int ninst, const SparseCtl& sp
 constexpr int kWideSide = 32;
 cudaError_t launch_cutoff_wide(const TcInst* tab, int ninst, const SparseCtl& sp, CallScalars* err,
                                cudaStream_t s);
+cudaError_t launch_wide_reduce(const TcInst* tab, int ninst, const SparseCtl& sp, cudaStream_t s);
 cudaError_t launch_sparse_reduce(const TcInst* tab, int ninst, const SparseCtl& sp,
                                  cudaStream_t s);
 

@@ -199,8 +199,8 @@ __global__ void __launch_bounds__(kRedThreads)
   const int jl = cell / sp.side, j = tn * sp.side + jl;
   const int64_t cells = (int64_t)sp.side * sp.side;
   if (i >= I.nx || j >= I.ny) return;
-  const int p0 = min((int)sp.piece_begin[t], sp.max_pieces);
-  const int p1 = min((int)sp.piece_begin[t + 1], sp.max_pieces);
+  const int p0 = bounded_piece(sp.piece_begin[t], sp.max_pieces);
+  const int p1 = bounded_piece(sp.piece_begin[t + 1], sp.max_pieces);
   const float* src = sp.part + cell;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   constexpr int kAhead = 8;

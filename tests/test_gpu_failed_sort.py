@@ -46,3 +46,27 @@ def test_adjoint_lists_nothing_after_a_timed_out_sort(lib, starts):
     groups, counters = listed(lib, starts, 1)
     assert counters.tolist() == [0, 0]
     assert (groups == -7).all()
+
+
+@pytest.mark.parametrize("side", [32, 128, 256])
+@pytest.mark.parametrize("starts", [[0, 2, 2, 5, 6], [2 ** 31, 3, 2 ** 32 - 1, 2 ** 31 + 2, 1],
+                                    [6, 2 ** 31, 0, 2 ** 32 - 6, 5], [0, 7, 2 ** 30, 2, 2 ** 31 - 1]])
+def test_reduces_read_no_piece_outside_their_buffer(lib, side, starts):
+    pieces, nx, ny = 6, 2 * side - 3, 2 * side - 5  # 2 x 2 tiles
+    rng = np.random.default_rng(side)
+    part = rng.integers(-50, 50, (pieces, side, side)).astype(np.float32)  # sums are exact
+    buf = np.stack([part, np.zeros_like(part)], -1) if side == 32 else part
+    buf = torch.as_tensor(buf, device="cuda")
+    begin = torch.as_tensor(np.asarray(starts, dtype=np.uint32).view(np.int32), device="cuda")
+    out = torch.full((ny, nx), 1000.0, device="cuda")
+    kde.check(lib.kde_diag_piece_reduce(begin.data_ptr(), buf.data_ptr(), pieces, side, nx, ny,
+                                        out.data_ptr(), None))
+    got = out.cpu().numpy()
+    for t in range(4):
+        a, b = min(starts[t], pieces), min(starts[t + 1], pieces)
+        y, x = side * (t // 2), side * (t % 2)
+        h, w = min(side, ny - y), min(side, nx - x)
+        want = part[a:max(a, b)].sum(0)[:h, :w]
+        if side == 32 and b - a == 1:
+            want = np.full((h, w), 1000.0)
+        np.testing.assert_array_equal(got[y:y + h, x:x + w], want)
