@@ -331,7 +331,12 @@ cudaError_t launch_rt(const AdjGroupArgs& a, cudaStream_t s) {
 
 }  // namespace
 
-int adj_group_radius(double cell, double h) { return (int)ceil(8.0 * h / cell) + 1; }
+// The points' bins come from FP32 keys, off by up to 3 units of 2^-24 of the
+// coordinate, and the window hangs on the bin: one cell to spare for keys of up to
+// 2^21 cells, one more for every further 2^21 along the longer axis.
+int adj_group_radius(double cell, double h, int nx, int ny) {
+  return (int)ceil(std::min(8.0 * h / cell, 1e6)) + 1 + (std::max(nx, ny) >> 21);
+}
 // 12 cells per thread at most: 96 x 96 cells and the tables of 64 points take 88 KB
 bool adj_group_fits(int R) { return kAdjBin + 2 * R <= 96; }
 

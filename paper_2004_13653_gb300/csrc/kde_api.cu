@@ -1512,7 +1512,7 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
   // tile of points, need the points in bin order and the room for it; without
   // that room the window kernel takes one point at a time, the contractions
   // the whole grid.
-  const int R = adj_group_radius(a->cell, a->h);
+  const int R = adj_group_radius(a->cell, a->h, a->nx, a->ny);
   const double sigma = use_tc ? kernel_sigma(KDE_GAUSSIAN, a->h) : 1.0 / a->h;
   const double reach = use_tc ? kAdjTcReach : 8.0;
   const int bin = use_tc ? adj_tc_bin(a) : kAdjBin;

@@ -495,7 +495,7 @@ struct AdjGroupArgs {
   double *hterm, *lterm;    // [m], in bin order
   const CallScalars* err;
 };
-int adj_group_radius(double cell, double h);  // window half-width R, cells
+int adj_group_radius(double cell, double h, int nx, int ny);  // window half-width R, cells
 bool adj_group_fits(int R);
 // The list of the groups alone (start, nbins, m, list, counters and err of a).
 cudaError_t launch_adjoint_list(const AdjGroupArgs& a, cudaStream_t s);

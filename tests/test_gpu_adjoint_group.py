@@ -104,3 +104,32 @@ def test_clusters_empty_bins_far_points_and_missing_outputs():
     nxy, nw, _ = backward(wl, None, G, want_w=False)
     np.testing.assert_array_equal(nxy, gxy)
     assert np.isnan(nw).all()
+
+
+def own_window(local, w, cell, h, G, n):
+    """FP64 gradients of the points, each over the cells within 10 bandwidths; G: one row."""
+    span = int(np.ceil(10 * h / cell))
+    i = np.floor(local[:, 0] / cell).astype(np.int64)[:, None] + np.arange(-span, span + 1)
+    g = np.where((i >= 0) & (i < len(G)), G[np.clip(i, 0, len(G) - 1)], 0.0)
+    s = ((i + 0.5) * cell - local[:, :1]) / h
+    t = (0.5 * cell - local[:, 1:]) / h
+    f = np.exp(-0.5 * (s * s + t * t)) * g / (2 * np.pi * n * h * h)
+    return (np.stack([(s * f).sum(1), (t * f).sum(1)], 1) * w[:, None] / h, f.sum(1))
+
+
+@pytest.mark.parametrize("nx,cell,h", [(3_000_000, 7.3, 0.9), (34_000_000, 7.3, 0.9),
+                                       (34_000_000, 10.0, 20.0), (100_000_000, 10.0, 3.0)])
+def test_long_axes(nx, cell, h):
+    """The sort's FP32 bin keys are several cells off at the far end of a long axis."""
+    n = 16384
+    rng = np.random.default_rng(nx)
+    local = np.stack([(nx - rng.random(n) * 0.02 * nx) * cell, rng.random(n) * cell], 1)
+    w = (rng.random(n) + 0.5).astype(np.float32)
+    wl = workloads.Workload("long", local, w, nx * cell, cell, nx, 1, h, oracle.GAUSSIAN,
+                            np.array([0, n]), 0)
+    G = rng.standard_normal(nx, dtype=np.float32)
+    gxy, gw, _ = backward(wl, w, G[None])
+    at = wl.xy - np.asarray(wl.origin)
+    rxy, rw = own_window(at, w.astype(np.float64), cell, h, G.astype(np.float64), n)
+    assert rel_linf(gw, rw) <= TOL_GRAD
+    assert rel_linf(gxy, rxy) <= TOL_GRAD
