@@ -13,7 +13,10 @@
 //   dL/dw ~ sum_j B U,  dL/dy ~ sum_j t B U,  dL/dx ~ sum_i s A V,
 //   h-term ~ sum_j t^2 B U + sum_i s^2 A V.
 // Terms beyond a point's own +-8 bandwidths but inside the shared window are
-// added where the other form leaves them out (they are below e^-32).
+// added where the other form leaves them out (they are below e^-32, for a finite
+// cotangent: a group whose window holds an infinity or a NaN, which makes all its
+// sums infinities or NaN, sums each point over its own window instead, so that only
+// the points that reach that cell see it).
 // Bound by FP32 FMA issue.  1.47M points x 1024^2, h = 3.07 cells: 3.33 ms one
 // warp per point, 0.79 ms in groups (0.9 with the sort), 0.75 with the inner loops
 // ended at the window's 58 cells instead of the 64 of the tables.
@@ -71,16 +74,66 @@ struct GroupCfg {
   static constexpr size_t kSmem = sizeof(float) * kFloats;
 };
 
+// The sums of a group's points over their own windows, +-reach cells from the
+// point's cell as in the one-point form, one warp per point, lanes over the columns.
+template <int RT>
+__device__ __noinline__ void own_windows(const float* sm, int np, int ib, int jb, int nx, int ny,
+                                         int reach, double cell_s, float* sum) {
+  using C = GroupCfg<RT>;
+  const float2* sgx = reinterpret_cast<const float2*>(sm + C::kGx);
+  const float2* sgy = reinterpret_cast<const float2*>(sm + C::kGy);
+  const int lane = threadIdx.x & 31;
+  for (int p = threadIdx.x >> 5; p < np; p += kThreads / 32) {
+    const float4 P = reinterpret_cast<const float4*>(sm + C::kPt)[p];
+    const int ic = (int)floor(((double)P.x + (double)P.y) / cell_s);
+    const int jc = (int)floor(((double)P.z + (double)P.w) / cell_s);
+    const int i0 = max(max(ic - reach, 0), ib), i1 = min(min(ic + reach, nx - 1), ib + C::W - 1);
+    const int j0 = max(max(jc - reach, 0), jb), j1 = min(min(jc + reach, ny - 1), jb + C::W - 1);
+    float aw = 0.f, ax = 0.f, ay = 0.f, ah = 0.f;
+    for (int j = j0; j <= j1; ++j) {
+      const float2 gy = sgy[j - jb];
+      const float t = (gy.x - P.z) + (gy.y - P.w), B = gauss(t);
+      float u = 0.f, v = 0.f, x = 0.f;
+      for (int i = i0 + lane; i <= i1; i += 32) {
+        const float2 gx = sgx[i - ib];
+        const float S = (gx.x - P.x) + (gx.y - P.y), A = gauss(S);
+        const float g = sm[C::kG + (j - jb) * C::WP + (i - ib)];
+        u = fmaf(g, A, u);
+        v = fmaf(g, S * A, v);
+        x = fmaf(g, S * (S * A), x);
+      }
+      const float Bu = B * u;
+      aw += Bu;
+      ax = fmaf(B, v, ax);
+      ay = fmaf(t, Bu, ay);
+      ah = fmaf(B, x, fmaf(t * t, Bu, ah));
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      aw += __shfl_xor_sync(0xffffffffu, aw, o);
+      ax += __shfl_xor_sync(0xffffffffu, ax, o);
+      ay += __shfl_xor_sync(0xffffffffu, ay, o);
+      ah += __shfl_xor_sync(0xffffffffu, ah, o);
+    }
+    if (lane == 0) {
+      sum[5 * p] = aw;
+      sum[5 * p + 1] = ay;
+      sum[5 * p + 2] = ah;
+      sum[5 * p + 3] = ax;
+      sum[5 * p + 4] = 0.f;
+    }
+  }
+}
+
 template <int RT>
 __global__ void __launch_bounds__(kThreads)
     k_adj_group(const float4* __restrict__ pts, const float* __restrict__ wts,
                 const uint32_t* __restrict__ vals, int64_t n, const int4* __restrict__ list,
                 const uint32_t* __restrict__ count, uint32_t* __restrict__ next,
                 const float* __restrict__ G, const float2* __restrict__ gxt,
-                const float2* __restrict__ gyt, int nx, int ny, int nbx, int nbins, int R, float c,
-                float inv_h, float* __restrict__ grad_xy, float* __restrict__ grad_w,
-                double* __restrict__ hterm, double* __restrict__ lterm,
-                const CallScalars* __restrict__ err) {
+                const float2* __restrict__ gyt, int nx, int ny, int nbx, int nbins, int R, int reach,
+                double cell_s, float c, float inv_h, float* __restrict__ grad_xy,
+                float* __restrict__ grad_w, double* __restrict__ hterm,
+                double* __restrict__ lterm, const CallScalars* __restrict__ err) {
   using C = GroupCfg<RT>;
   constexpr int W = C::W, WP = C::WP;
   extern __shared__ __align__(16) float sm[];
@@ -174,6 +227,7 @@ __global__ void __launch_bounds__(kThreads)
     }
     __syncthreads();
     const int blk = lane & 7;  // block of cells
+    bool odd = false;  // a sum that is not finite: every point's is when a cell is not
     if (warp < 2) {
       // U: points p = 8 s + pb, rows j = 8 r + blk; four columns per step
       const int pb = (warp << 2) | (lane >> 3);
@@ -232,6 +286,7 @@ __global__ void __launch_bounds__(kThreads)
             sum[5 * p] = aw;
             sum[5 * p + 1] = ay;
             sum[5 * p + 2] = ah;
+            odd |= !(fabsf(aw) + fabsf(ay) + fabsf(ah) < INFINITY);
           }
         }
       }
@@ -288,11 +343,15 @@ __global__ void __launch_bounds__(kThreads)
           if (blk == 0 && p < np) {
             sum[5 * p + 3] = ax;
             sum[5 * p + 4] = ah;
+            odd |= !(fabsf(ax) + fabsf(ah) < INFINITY);
           }
         }
       }
     }
-    __syncthreads();
+    if (__syncthreads_or(odd)) {
+      own_windows<RT>(sm, np, ib, jb, nx, ny, reach, cell_s, sum);
+      __syncthreads();
+    }
     if (tid < np) {
       const uint32_t o = sIdx[tid];
       if (o < n) {  // the caller's order
@@ -324,7 +383,8 @@ cudaError_t launch_rt(const AdjGroupArgs& a, cudaStream_t s) {
   const int grid = (int)std::min<int64_t>((int64_t)per_sm * a.sms, most);
   k_adj_group<RT><<<grid, kThreads, C::kSmem, s>>>(
       a.pts, a.wts, a.vals, a.n, a.list, a.counters, a.counters + 1, a.G, a.gxt, a.gyt, a.nx, a.ny,
-      a.nbx, a.nbins, a.R, a.c, a.inv_h, a.grad_xy, a.grad_w, a.hterm, a.lterm, a.err);
+      a.nbx, a.nbins, a.R, a.reach, a.cell_s, a.c, a.inv_h, a.grad_xy, a.grad_w, a.hterm, a.lterm,
+      a.err);
   note_launches(1);
   return cudaGetLastError();
 }

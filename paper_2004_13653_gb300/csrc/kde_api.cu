@@ -1645,6 +1645,8 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
     g.nx = a->nx;
     g.ny = a->ny;
     g.R = R;
+    g.reach = adj_group_radius(a->cell, a->h, 1, 1);
+    g.cell_s = a->cell / a->h;
     g.sms = sms;
     g.list = reinterpret_cast<int4*>(base + o.list);
     g.counters = reinterpret_cast<uint32_t*>(base + o.ctr);

@@ -485,6 +485,8 @@ struct AdjGroupArgs {
   const uint32_t* start;    // bin starts; start[nbins]: first point beyond reach
   int64_t n, m;             // points, and with the padding
   int nbx, nbins, nx, ny, R, sms;
+  int reach;                // cells to either side of a point's own window
+  double cell_s;            // cell side in bandwidths
   int4* list;               // [m / kAdjGroup + nbins + 2]
   uint32_t* counters;       // [2]
   const float* G;

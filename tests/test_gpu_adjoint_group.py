@@ -133,3 +133,22 @@ def test_long_axes(nx, cell, h):
     rxy, rw = own_window(at, w.astype(np.float64), cell, h, G.astype(np.float64), n)
     assert rel_linf(gw, rw) <= TOL_GRAD
     assert rel_linf(gxy, rxy) <= TOL_GRAD
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
+@pytest.mark.parametrize("h_cells", [0.6, 1.4, 3.3, 5.3])
+def test_non_finite_cotangent_cells(value, h_cells):
+    """Such a cell reaches the points whose own window holds it, no others."""
+    n, nx, ny = 20000, 130, 117
+    wl = workloads.random_points(33, n, 10.0 * nx, 10.0, nx, ny, 10.0 * h_cells, oracle.GAUSSIAN)
+    G = np.random.default_rng(3).normal(0, 1, (ny, nx))
+    clean = backward(wl, wl.w, G)
+    G[40, 51] = value
+    gxy, gw, _ = backward(wl, wl.w, G)
+    sxy, sw, _ = backward(wl, wl.w, G, workspace=one_point_workspace(wl))
+    hit = ~np.isfinite(sw)
+    assert 0 < hit.sum() < n
+    np.testing.assert_array_equal(~np.isfinite(gw), hit)
+    np.testing.assert_array_equal(np.isfinite(gxy), np.isfinite(sxy))
+    assert rel_linf(gw[~hit], clean[1][~hit]) <= SAME
+    assert rel_linf(gxy[~hit], clean[0][~hit]) <= SAME
