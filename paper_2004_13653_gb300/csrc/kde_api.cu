@@ -972,8 +972,7 @@ int run_small_gauss(const kde_args* a, const kde_opts* o, bool sync) {
     scal = static_cast<CallScalars*>(wsv);
     KDE_CUDA(cudaMemsetAsync(scal, 0, sizeof(CallScalars), s), "clear scalars");
   }
-  const float scale =
-      (float)(1.0 / (2.0 * 3.14159265358979323846 * (double)a->n * a->h * a->h));
+  const double scale = 1.0 / (2.0 * 3.14159265358979323846 * (double)a->n * a->h * a->h);
   cudaEvent_t* ev = o ? static_cast<cudaEvent_t*>(o->timing_events) : nullptr;
   if (ev) KDE_CUDA(cudaEventRecord(ev[0], s), "record start event");
   KDE_CUDA(launch_small_gauss(q, scale, a->out, scal, sm_count(), s), "small density");

@@ -381,7 +381,7 @@ cudaError_t launch_simt(int kid, const float4* pts, const float* wts, int64_t n_
 // Small Gaussian densities (kde_small.cu): q as for the prepare kernel, without
 // its tables and scalars; scal: where non-finite input is recorded, or null.
 bool small_gauss_fits(int64_t n, int nx, int ny);
-cudaError_t launch_small_gauss(const PrepInst& q, float scale, float* out, CallScalars* scal,
+cudaError_t launch_small_gauss(const PrepInst& q, double scale, float* out, CallScalars* scal,
                                int sms, cudaStream_t s);
 
 // Sum each instance's S partial grids in fixed order (s = 0, 1, ...).

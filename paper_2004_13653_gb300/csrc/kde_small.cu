@@ -13,6 +13,7 @@
 // path.  2000 points x 64^2: four launches, 18 us of GPU time and 30 us per
 // call on the general path, 6 and 20 us (the host's part) in this form.
 #include <cooperative_groups.h>
+#include <math.h>
 
 #include <algorithm>
 
@@ -35,7 +36,7 @@ struct WarpTables {
 };
 
 __global__ void __launch_bounds__(kThreads)
-    k_small_gauss(const __grid_constant__ PrepInst I, float scale, int tiles_x,
+    k_small_gauss(const __grid_constant__ PrepInst I, float scale, float post, int tiles_x,
                   float* __restrict__ out, CallScalars* __restrict__ scal) {
   __shared__ __align__(16) WarpTables tables[kWarps];
   __shared__ float2 part[kWarps][8][32];
@@ -67,8 +68,9 @@ __global__ void __launch_bounds__(kThreads)
     float w = 0.f;
     if (p < I.n) {
       const double2 v = reinterpret_cast<const double2*>(I.xy)[p];
-      // the density's scale goes into the weights, so that sums overflow only
-      // where the result does
+      // the density's scale goes into the weights, but for a power of two that
+      // leaves what goes in below 2^-14: no weight and no sum overflows then
+      // (n <= 2^14), only a result that does
       const float wv = I.w ? I.w[p] : 1.0f;
       w = wv * scale;
       if (!(I.usual && prepare_usual(v, I, P))) P = prepare_any(v, I);
@@ -131,7 +133,7 @@ __global__ void __launch_bounds__(kThreads)
   }
   if (rank == 0) {
     const int x = x0 + cx + (warp & 1), y = y0 + cy + (warp >> 1);
-    if (x < I.nx && y < I.ny) out[(int64_t)y * I.nx + x] = sum.x + sum.y;
+    if (x < I.nx && y < I.ny) out[(int64_t)y * I.nx + x] = (sum.x + sum.y) * post;
   }
 }
 
@@ -145,8 +147,11 @@ bool small_gauss_fits(int64_t n, int nx, int ny) {
   return n >= 1 && n <= 16384 && (double)n * nx * ny <= 6e7;
 }
 
-cudaError_t launch_small_gauss(const PrepInst& q, float scale, float* out, CallScalars* scal,
+cudaError_t launch_small_gauss(const PrepInst& q, double scale, float* out, CallScalars* scal,
                                int sms, cudaStream_t s) {
+  int e2 = 0;
+  frexp(scale, &e2);  // scale < 2^e2
+  const int post2 = std::max(0, std::min(e2 + 14, 127));
   const int tx = (q.nx + kTile - 1) / kTile, ty = (q.ny + kTile - 1) / kTile;
   const int64_t tiles = (int64_t)tx * ty;
   // clusters as large as leave every warp a batch, up to eight CTAs
@@ -164,7 +169,8 @@ cudaError_t launch_small_gauss(const PrepInst& q, float scale, float* out, CallS
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_small_gauss, q, scale, tx, out, scal);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_small_gauss, q, (float)ldexp(scale, -post2),
+                                           ldexpf(1.0f, post2), tx, out, scal);
   note_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -96,3 +96,34 @@ def test_status_lonlat_plain_call_and_capture():
     with pytest.raises(kde.KDEError) as e:
         kde.grid(pts, w, wl.origin, wl.cell, 64, 64, wl.h, "gaussian", flags=kde.FLAG_SYNC)
     assert e.value.code == kde.KDE_EDATA
+
+
+@pytest.mark.parametrize("n,h,scale,signs", [
+    (2000, 0.02, 3e38, 1),    # overflows near the points: infinities there, numbers elsewhere
+    (2000, 0.02, 3e38, 2),    # the same with weights of both signs: sums that cancel
+    (50, 0.01, 1e38, 1),      # 1 / (2 pi n h^2) times the weight overflows by itself
+    (16384, 1e-3, 1e37, 1),
+])
+def test_only_results_that_overflow_are_infinite(n, h, scale, signs):
+    """Weights near the largest FP32 number and small bandwidths, as the general path
+    has them: an infinity where the density overflows, its value (or zero) elsewhere."""
+    wl = workloads.random_points(73, n, 40.0 * h, h, 40, 40, 1.3 * h, oracle.GAUSSIAN)
+    wl.local[:, 0] *= 0.4  # the far columns are out of every point's reach
+    wl.w = (wl.w * np.float32(scale / np.abs(wl.w).max())).astype(np.float32)
+    if signs == 2:
+        wl.w[::2] *= -1.0
+    assert one_launch(wl)
+    F = density(wl).cpu().numpy()
+    ref = oracle.kde_grid(wl.xy, wl.w, wl.origin, wl.cell, 40, 40, wl.h, oracle.GAUSSIAN)
+    top = float(np.finfo(np.float32).max)
+    sure = np.abs(np.abs(ref) / top - 1.0) > 1e-5  # FP32 decides at the edge
+    assert (np.abs(ref) > top).any() == (signs == 1) and (np.abs(ref) < top).any()
+    assert not np.isnan(F).any()
+    big = (np.abs(ref) > top) & sure
+    np.testing.assert_array_equal(F[big], np.sign(ref[big]) * np.inf)
+    rest = (np.abs(ref) < top) & sure
+    assert np.isfinite(F[rest]).all()
+    # as the FP32 path, relative to the largest value there is (signs: to that of |w|)
+    peak = np.abs(ref).max() if signs == 1 else oracle.kde_grid(
+        wl.xy, np.abs(wl.w), wl.origin, wl.cell, 40, 40, wl.h, oracle.GAUSSIAN).max()
+    assert np.abs(F[rest] - ref[rest]).max() <= TOL_FP32 * peak
