@@ -142,9 +142,15 @@ __global__ void __launch_bounds__(kThreads)
 // GPU time, small against general form: 500 points x 128^2 4.8 / 17.8 us,
 // 2000 x 200^2 (8e7 pairs) 17.7 / 19.5, 8000 x 128^2 (1.3e8) 22.7 / 21.6, 16000 x
 // 64^2 (6.6e7) 22.1 / 24.7, 32000 x 64^2 40 / 31: the line lies where the two
-// meet.
+// meet.  What the kernel computes are whole 16 x 16 tiles, so thin grids have a
+// line of their own, by the tiles' pairs (1 x 3600: 1.2e8 of them 17.5 / 22.4, 2.3e8
+// 31.5 / 28.2, 9.4e8 113 / 67), and so have grids of few points, by the tiles, each
+// of which costs a CTA's start (1 point x 1024^2, 4096 tiles 17.7 / 20.9, x 1500^2
+// 36 / 25, x 2048^2 64 / 21).
 bool small_gauss_fits(int64_t n, int nx, int ny) {
-  return n >= 1 && n <= 16384 && (double)n * nx * ny <= 6e7;
+  const double tiles = (double)((nx + kTile - 1) / kTile) * ((ny + kTile - 1) / kTile);
+  return n >= 1 && n <= 16384 && (double)n * nx * ny <= 6e7 && tiles <= 4096.0 &&
+         (double)n * tiles * (kTile * kTile) <= 1.5e8;
 }
 
 cudaError_t launch_small_gauss(const PrepInst& q, double scale, float* out, CallScalars* scal,

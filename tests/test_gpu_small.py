@@ -127,3 +127,25 @@ def test_only_results_that_overflow_are_infinite(n, h, scale, signs):
     peak = np.abs(ref).max() if signs == 1 else oracle.kde_grid(
         wl.xy, np.abs(wl.w), wl.origin, wl.cell, 40, 40, wl.h, oracle.GAUSSIAN).max()
     assert np.abs(F[rest] - ref[rest]).max() <= TOL_FP32 * peak
+
+
+@pytest.mark.parametrize("n,nx,ny,small", [
+    (2600, 1, 3600, True),        # 1.5e8 pairs of the 225 tiles' cells
+    (2605, 1, 3600, False),
+    (2605, 3600, 1, False),
+    (16384, 1, 3600, False),
+    (3, 1024, 1024, True),        # 4096 tiles
+    (3, 1024, 1025, False),
+    (1, 2048, 2048, False),
+])
+def test_rule_counts_whole_tiles(n, nx, ny, small):
+    wl = workloads.random_points(80 + n, n, 12.0 * max(nx, ny), 12.0, nx, ny, 30.0,
+                                 oracle.GAUSSIAN)
+    if min(nx, ny) == 1:  # onto the grid's one row or column
+        wl.local[:, 1 if ny == 1 else 0] *= 1.0 / 3600
+    assert one_launch(wl) == small
+    F = density(wl).cpu().numpy()
+    cells = np.random.default_rng(n).integers(0, nx * ny, 2000)
+    cells[0] = int(F.argmax())
+    ref = oracle.kde_cells(wl.xy, wl.w, wl.origin, wl.cell, nx, ny, wl.h, oracle.GAUSSIAN, cells)
+    assert rel_linf(F.reshape(-1)[cells], ref) <= (TOL_FP32 if small else 1e-5)
