@@ -56,15 +56,17 @@ int kde_diag_sort_wait_timeout(int64_t limit_ns, void* stream);
  * device, [nbins + 1], the sorted position of each bin's first point and, last,
  * of the first point beyond every cell's reach; m: the sorted points; list:
  * device, [m / 64 + nbins + 2][4], 16-byte aligned, receives (bin, first point,
- * points, 0) in no particular order, bin nbins for the points beyond reach;
- * counters: device, [2], receives the number of groups and a zero.  With
+ * points, 0) in no particular order, bin nbins for up to 1024 points beyond reach;
+ * singles: device, [m], receives the sorted positions of the points that are taken
+ * one by one, the last of a bin where they are fewer than 12; counters: device,
+ * [3], receives the number of groups, a zero and the number of singles.  With
  * sort_failed the sort counts as timed out: its bin starts may then be anything,
  * and nothing is listed.  Without it they have to rise from 0 to at most m.
  * Synchronous; uses the library workspace.  Errors: KDE_EINVAL (nbins, m,
  * pointers, alignment), KDE_ENOMEM, KDE_ECUDA.
  */
 int kde_diag_adjoint_list(const uint32_t* start, int nbins, int64_t m, int sort_failed,
-                          int32_t* list, uint32_t* counters, void* stream);
+                          int32_t* list, uint32_t* singles, uint32_t* counters, void* stream);
 
 /*
  * kde_diag_piece_reduce — the sum of a tiled grid's piece partials alone (no

@@ -125,7 +125,7 @@ def load(build_if_stale: bool = False) -> ctypes.CDLL:
     lib.kde_diag_wait_timeout.restype = i32
     lib.kde_diag_sort_wait_timeout.argtypes = [i64, vp]
     lib.kde_diag_sort_wait_timeout.restype = i32
-    lib.kde_diag_adjoint_list.argtypes = [vp, i32, i64, i32, vp, vp, vp]
+    lib.kde_diag_adjoint_list.argtypes = [vp, i32, i64, i32, vp, vp, vp, vp]
     lib.kde_diag_adjoint_list.restype = i32
     lib.kde_diag_piece_reduce.argtypes = [vp, vp, i32, i32, i32, i32, vp, vp]
     lib.kde_diag_piece_reduce.restype = i32

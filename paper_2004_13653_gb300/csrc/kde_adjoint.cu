@@ -36,10 +36,15 @@ __device__ __forceinline__ float gauss(float s) { return ex2_approx(-0.5f * kLog
 // A window of at most 16 columns takes 2^sub_log2 >= its width lanes per row
 // and 32 / 2^sub_log2 rows at a time (sub_log2 = 5 otherwise).  The launch
 // bounds are the blocks per SM each COLS fits without spilling registers.
-template <int COLS>
+// LIST: the points are those at the sorted positions list[0 .. *list_count), what
+// the groups of kde_adjoint_group.cu leave over.  Their count is known here only:
+// where they are few, a warp takes as few at a time as keep `busy` warps, those
+// that fit the GPU, at work.
+template <int COLS, bool LIST>
 __global__ void __launch_bounds__(256, COLS == 1 ? 5 : (COLS == 2 ? 4 : (COLS == 4 ? 3 : 1)))
     k_adjoint_gauss(const float4* __restrict__ pts, const float* __restrict__ wts, int64_t n,
-                    const float* __restrict__ G, const float2* __restrict__ gxt,
+                    const uint32_t* __restrict__ list, const uint32_t* __restrict__ list_count,
+                    int busy, const uint32_t* __restrict__ vals, const float* __restrict__ G, const float2* __restrict__ gxt,
                     const float2* __restrict__ gyt, int nx, int ny, double cell_s, int R,
                     int sub_log2, float c, float inv_h, float* __restrict__ grad_xy,
                     float* __restrict__ grad_w, double* __restrict__ hterm,
@@ -52,13 +57,24 @@ __global__ void __launch_bounds__(256, COLS == 1 ? 5 : (COLS == 2 ? 4 : (COLS ==
   // lanes in groups of 2^sub_log2 over the columns; group g takes rows g, g + ng, ...
   const int ci = lane & ((1 << sub_log2) - 1), rg = lane >> sub_log2, ng = 32 >> sub_log2;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t pb = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; pb < n;
-       pb += warps * 32) {
+  // batches, and points of a batch: the list's are taken `batches` apart, so that the
+  // warps that run at a time, not the points of one, are neighbours
+  const int64_t count = LIST ? (int64_t)*list_count : n;
+  const int per = LIST ? (int)min((int64_t)32, (count + busy - 1) / busy) : 32;
+  const int64_t batches = count ? (count + per - 1) / per : 0;
+  for (int64_t batch = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; batch < batches;
+       batch += warps) {
     // Lane l prepares point pb + l: its window of cells within R of its cell
     // (X, Y in bandwidths).  This is the FP64 part, so it runs once per point
     // instead of once per lane of the warp.
-    const int64_t pl = pb + lane;
-    if (pl < n) {
+    auto point = [&](int64_t& pl) {  // the lane's point, if it has one
+      const int64_t at = LIST ? batch + lane * batches : batch * 32 + lane;
+      if (lane >= per || at >= count) return false;
+      pl = LIST ? (int64_t)list[at] : at;
+      return true;
+    };
+    int64_t pl;
+    if (point(pl)) {
       const float4 P = pts[pl];
       const double X = (double)P.x + (double)P.y, Y = (double)P.z + (double)P.w;
       const int ic = (int)floor(X / cell_s), jc = (int)floor(Y / cell_s);
@@ -67,7 +83,8 @@ __global__ void __launch_bounds__(256, COLS == 1 ? 5 : (COLS == 2 ? 4 : (COLS ==
                                   min(jc + R, ny - 1));
     }
     __syncwarp();
-    const int cnt = n - pb < 32 ? (int)(n - pb) : 32;
+    const int cnt = (int)min((int64_t)per, LIST ? (count - batch + batches - 1) / batches
+                                                : count - batch * 32);
     for (int q = 0; q < cnt; ++q) {
       const float4 P = sP[wib][q];
       const int4 win = sWin[wib][q];
@@ -123,13 +140,14 @@ __global__ void __launch_bounds__(256, COLS == 1 ? 5 : (COLS == 2 ? 4 : (COLS ==
       if (lane == 0) sSum[wib][q] = make_float4(aw, ax, ay, ah);
     }
     __syncwarp();
-    if (pl < n) {
+    if (point(pl)) {
       const float w = wts[pl];
       const float4 r = sSum[wib][lane];
       const float gw = c * r.x;
-      if (grad_w) grad_w[pl] = gw;
-      grad_xy[2 * pl] = c * w * inv_h * r.y;
-      grad_xy[2 * pl + 1] = c * w * inv_h * r.z;
+      const int64_t to = LIST ? (int64_t)vals[pl] : pl;  // the caller's order
+      if (grad_w) grad_w[to] = gw;
+      grad_xy[2 * to] = c * w * inv_h * r.y;
+      grad_xy[2 * to + 1] = c * w * inv_h * r.z;
       hterm[pl] = (double)c * w * inv_h * r.w;
       lterm[pl] = (double)w * gw;
     }
@@ -329,25 +347,61 @@ cudaError_t launch_sums(const SumJob* jobs, int count, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+namespace {
+
+struct AdjWindow {  // what the one-point kernel's launches share
+  int R, cols, sub_log2;
+  float c, inv_h;
+};
+AdjWindow adj_window(int64_t n, double cell, double h) {
+  AdjWindow w = {};
+  w.R = (int)ceil(8.0 * h / cell) + 1;
+  const int width = 2 * w.R + 1;
+  w.cols = width <= 32 ? 1 : width <= 64 ? 2 : width <= 128 ? 4 : 8;
+  while ((1 << w.sub_log2) < width && w.sub_log2 < 5) ++w.sub_log2;
+  if (w.cols > 1) w.sub_log2 = 5;
+  w.c = (float)(1.0 / (2.0 * 3.14159265358979323846 * (double)n * h * h));
+  w.inv_h = (float)(1.0 / h);
+  return w;
+}
+
+}  // namespace
+
 cudaError_t launch_adjoint_gauss(const float4* pts, const float* wts, int64_t n, const float* G,
                                  const float2* gxt, const float2* gyt, int nx, int ny,
                                  double cell, double h, float* grad_xy, float* grad_w,
                                  double* hterm, double* lterm, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int R = (int)ceil(8.0 * h / cell) + 1;
-  const float c = (float)(1.0 / (2.0 * 3.14159265358979323846 * (double)n * h * h));
-  const int width = 2 * R + 1;
+  const AdjWindow w = adj_window(n, cell, h);
   const int blocks = grid_blocks((n + 31) / 32 * 32, 256, 152 * 64);  // a warp per 32 points
-  int sub_log2 = 0;
-  while ((1 << sub_log2) < width && sub_log2 < 5) ++sub_log2;
-#define KDE_ADJ(C)                                                                          \
-  k_adjoint_gauss<C><<<blocks, 256, 0, s>>>(pts, wts, n, G, gxt, gyt, nx, ny, cell / h, R,    \
-                                            C == 1 ? sub_log2 : 5, c, (float)(1.0 / h),     \
-                                            grad_xy, grad_w, hterm, lterm)
-  if (width <= 32) KDE_ADJ(1);
-  else if (width <= 64) KDE_ADJ(2);
-  else if (width <= 128) KDE_ADJ(4);
+#define KDE_ADJ(C)                                                                             \
+  k_adjoint_gauss<C, false><<<blocks, 256, 0, s>>>(pts, wts, n, nullptr, nullptr, 1, nullptr,   \
+                                                   G, gxt, gyt, nx, ny, cell / h, w.R,          \
+                                                   w.sub_log2, w.c, w.inv_h, grad_xy, grad_w,  \
+                                                   hterm, lterm)
+  if (w.cols == 1) KDE_ADJ(1);
+  else if (w.cols == 2) KDE_ADJ(2);
+  else if (w.cols == 4) KDE_ADJ(4);
   else KDE_ADJ(8);
+#undef KDE_ADJ
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_adjoint_listed(const AdjGroupArgs& a, double cell, double h, cudaStream_t s) {
+  const AdjWindow w = adj_window(a.n, cell, h);
+  // the groups' windows end at 44 cells to either side, so no 8 columns per lane
+  if (w.cols > 4) return cudaErrorInvalidValue;
+  const int resident = (w.cols == 1 ? 5 : w.cols == 2 ? 4 : 3) * a.sms;  // launch bounds
+  const int blocks = std::max(resident, grid_blocks((a.n + 31) / 32 * 32, 256, 152 * 64));
+#define KDE_ADJ(C)                                                                             \
+  k_adjoint_gauss<C, true><<<blocks, 256, 0, s>>>(a.pts, a.wts, a.n, a.singles, a.counters + 2, \
+                                                  8 * resident, a.vals, a.G, a.gxt, a.gyt, a.nx, a.ny,       \
+                                                  cell / h, w.R, w.sub_log2, w.c, w.inv_h,     \
+                                                  a.grad_xy, a.grad_w, a.hterm, a.lterm)
+  if (w.cols == 1) KDE_ADJ(1);
+  else if (w.cols == 2) KDE_ADJ(2);
+  else KDE_ADJ(4);
 #undef KDE_ADJ
   note_launches(1);
   return cudaGetLastError();

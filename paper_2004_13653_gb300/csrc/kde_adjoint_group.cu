@@ -32,36 +32,50 @@ constexpr float kLog2e = 1.44269504088896340736f;
 __device__ __forceinline__ float gauss(float s) { return ex2_approx(-0.5f * kLog2e * s * s); }
 
 constexpr int kP = kAdjGroup;  // points per group
+constexpr uint32_t kFar = 1024;  // points per item beyond every cell's reach
 constexpr int kThreads = 128;  // two warps form U, two form V
 constexpr int kPP = kP + 4;    // row of the y-factor table: 16-byte aligned, spread over the banks
 
 // Lists the groups of every bin (first point and count; the order is whatever
 // the atomics give and decides only which CTA takes a group), and those of the
-// points beyond every cell's reach, which only get zeros.  After a timed-out sort
-// the bin starts need not rise, and the differences of two that fall would list
-// groups past the end of the list: nothing is listed then.
-__global__ void __launch_bounds__(256)
-    k_adj_groups(const uint32_t* __restrict__ start, int nbins, int64_t m,
-                 int4* __restrict__ list, uint32_t* __restrict__ count,
-                 const CallScalars* __restrict__ err) {
-  if (*reinterpret_cast<const volatile int*>(&err->err) & kErrSortTimeout) return;
-  const int b = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
-  uint32_t a = 0, n = 0;
-  if (b <= nbins) {
-    a = start[b];
-    n = (b < nbins ? start[b + 1] : (uint32_t)m) - a;
-  }
-  const uint32_t g = (n + kP - 1) / kP;
-  uint32_t incl = g;
+// points beyond every cell's reach, which only get zeros.  Fewer than kAdjFew points
+// left over in a bin are listed one by one instead, for the one-point form: a
+// group costs its tile however few its points are, as much as about 9 to 17 of them
+// one at a time (points spread evenly, 1M x 4096^2, 4 a bin, h = 3 cells: 6.0 ms
+// in groups, 2.3 one by one; a mixture of lanes, ports and even ones 2.7 and 1.2).  After a timed-out sort the bin starts need not rise,
+// and the differences of two that fall would list groups past the end of the list:
+// nothing is listed then.
+__device__ __forceinline__ uint32_t take_slots(uint32_t mine, uint32_t* count) {
+  const int lane = threadIdx.x & 31;
+  uint32_t incl = mine;
   for (int o = 1; o < 32; o <<= 1) {
     const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += y;
   }
   uint32_t base = 0;
   if (lane == 31 && incl) base = atomicAdd(count, incl);
-  base = __shfl_sync(0xffffffffu, base, 31) + incl - g;
+  return __shfl_sync(0xffffffffu, base, 31) + incl - mine;
+}
+__global__ void __launch_bounds__(256)
+    k_adj_groups(const uint32_t* __restrict__ start, int nbins, int64_t m,
+                 int4* __restrict__ list, uint32_t* __restrict__ singles,
+                 uint32_t* __restrict__ count, const CallScalars* __restrict__ err) {
+  if (*reinterpret_cast<const volatile int*>(&err->err) & kErrSortTimeout) return;
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  uint32_t a = 0, n = 0;
+  if (b <= nbins) {
+    a = start[b];
+    n = (b < nbins ? start[b + 1] : (uint32_t)m) - a;
+  }
+  uint32_t rest = n % kP;
+  if (b == nbins || rest >= (uint32_t)kAdjFew) rest = 0;
+  n -= rest;
+  const uint32_t most = b < nbins ? kP : kFar, g = (n + most - 1) / most;
+  const uint32_t base = take_slots(g, count);
   for (uint32_t k = 0; k < g; ++k)
-    list[base + k] = make_int4(b, (int)(a + k * kP), (int)min((uint32_t)kP, n - k * kP), 0);
+    list[base + k] = make_int4(b, (int)(a + k * most), (int)min(most, n - k * most), 0);
+  const uint32_t first = take_slots(rest, count + 2);
+  for (uint32_t k = 0; k < rest; ++k) singles[first + k] = a + n + k;
 }
 
 template <int RT>
@@ -161,8 +175,8 @@ __global__ void __launch_bounds__(kThreads)
     const int4 it = list[item];
     const int np = it.z;
     if (it.x >= nbins) {  // out of every cell's reach
-      if (tid < np) {
-        const uint32_t p = (uint32_t)it.y + tid;
+      for (int t = tid; t < np; t += kThreads) {
+        const uint32_t p = (uint32_t)it.y + t;
         const uint32_t o = vals[p];
         if (o < n) {
           if (grad_w) grad_w[o] = 0.f;
@@ -401,21 +415,20 @@ int adj_group_radius(double cell, double h, int nx, int ny) {
 bool adj_group_fits(int R) { return kAdjBin + 2 * R <= 96; }
 
 cudaError_t launch_adjoint_list(const AdjGroupArgs& a, cudaStream_t s) {
-  const cudaError_t e = cudaMemsetAsync(a.counters, 0, 2 * sizeof(uint32_t), s);
+  const cudaError_t e = cudaMemsetAsync(a.counters, 0, 3 * sizeof(uint32_t), s);
   if (e != cudaSuccess) return e;
-  k_adj_groups<<<(a.nbins + 1 + 255) / 256, 256, 0, s>>>(a.start, a.nbins, a.m, a.list, a.counters,
-                                                         a.err);
+  k_adj_groups<<<(a.nbins + 1 + 255) / 256, 256, 0, s>>>(a.start, a.nbins, a.m, a.list, a.singles,
+                                                         a.counters, a.err);
   note_launches(1);
   return cudaGetLastError();
 }
 
-cudaError_t launch_adjoint_group(const AdjGroupArgs& a, cudaStream_t s) {
-  const cudaError_t e = launch_adjoint_list(a, s);
+cudaError_t launch_adjoint_group(const AdjGroupArgs& a, double cell, double h, cudaStream_t s) {
+  cudaError_t e = launch_adjoint_list(a, s);
   if (e != cudaSuccess) return e;
   const int W = kAdjBin + 2 * a.R;
-  if (W <= 32) return launch_rt<4>(a, s);
-  if (W <= 64) return launch_rt<8>(a, s);
-  return launch_rt<12>(a, s);
+  e = W <= 32 ? launch_rt<4>(a, s) : W <= 64 ? launch_rt<8>(a, s) : launch_rt<12>(a, s);
+  return e == cudaSuccess ? launch_adjoint_listed(a, cell, h, s) : e;
 }
 
 }  // namespace kde

@@ -339,9 +339,23 @@ bool adj_tc_sorts(const kde_args* a) {
                              0.67 * (double)a->nx * (double)a->ny;
 }
 
-// Points from which the adjoint's window form sorts them and works in groups:
-// below, the sort's launches cost more than the groups save.
-constexpr int64_t kAdjGroupPoints = 16384;
+// Whether the adjoint's window form sorts the points and works in groups.  Below
+// 16384 points the sort's launches cost more than the groups save, and a window of
+// up to 16 cells (h up to 0.75 cells) is too little work per point for it (h = 0.4
+// cells, one by one / groups: 300k x 256^2 137 / 144 us, 1M x 1024^2 381 / 326, but
+// 302 / 383 for 1M of which 95% lie outside a 4096 x 200 grid).  Where the
+// points are many and thin over the grid, their own form may get nearly all of them
+// after a sort for nothing: with fewer than 10 a bin the sort has to be small beside
+// that form, as it is for wide windows (evenly spread points, 300k x 2048^2, 4.6 a
+// bin: h = 1 cell 306 / 379, 2 cells 546 / 628, 4 cells 1442 / 1544; on lanes 288 /
+// 164, 534 / 264, 1397 / 588), and up to 2^16 points the listed ones are spread over
+// more warps than they are alone, which pays for it (50k x 2048^2, evenly spread:
+// 146 / 140, 183 / 185, 387 / 337).
+bool adj_groups_pay(const kde_args* a, int nbins) {
+  const int reach = adj_group_radius(a->cell, a->h, 1, 1);
+  return adj_group_fits(adj_group_radius(a->cell, a->h, a->nx, a->ny)) && reach > 7 &&
+         a->n >= 16384 && (a->n < 1 << 16 || a->n >= 10 * (int64_t)nbins || reach >= 28);
+}
 
 // Tensor-core instances that share a tile shape and pipeline stage: one
 // persistent launch over their work items.
@@ -1516,11 +1530,11 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
   const double reach = use_tc ? kAdjTcReach : 8.0;
   const int bin = use_tc ? adj_tc_bin(a) : kAdjBin;
   const CutoffGeom geo = cutoff_geometry(a->nx, a->ny, a->cell * sigma, reach, bin);
-  bool group = use_tc ? adj_tc_sorts(a) : adj_group_fits(R) && a->n >= kAdjGroupPoints;
+  bool group = use_tc ? adj_tc_sorts(a) : adj_groups_pay(a, geo.nbins);
   const CutoffSizes cz = group ? cutoff_sizes(n_pad, geo.nbins) : CutoffSizes{};
   struct {
     size_t scal, tab, cut, pts, wts, gxt, gyt, ht, lt, res, tc;
-    size_t keys[2], vals[2], hist, start, spts, sw, list, ctr;
+    size_t keys[2], vals[2], hist, start, spts, sw, list, singles, ctr;
   } o = {};
   auto layout = [&]() {
     size_t off = 0;
@@ -1548,7 +1562,8 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
       o.sw = take(sizeof(float) * n_pad);
       o.list = take(use_tc ? adjoint_tc_ranges_bytes(a->n)
                            : sizeof(int4) * ((size_t)n_pad / kAdjGroup + geo.nbins + 2));
-      o.ctr = take(u * 2);
+      o.singles = take(use_tc ? 0 : u * n_pad);
+      o.ctr = take(u * 3);
     }
     return off;
   };
@@ -1648,6 +1663,7 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
     g.cell_s = a->cell / a->h;
     g.sms = sms;
     g.list = reinterpret_cast<int4*>(base + o.list);
+    g.singles = reinterpret_cast<uint32_t*>(base + o.singles);
     g.counters = reinterpret_cast<uint32_t*>(base + o.ctr);
     g.G = grad_out;
     g.gxt = q.gxt;
@@ -1659,7 +1675,7 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
     g.hterm = ht;
     g.lterm = lt;
     g.err = q.scal;
-    KDE_CUDA(launch_adjoint_group(g, s), "adjoint");
+    KDE_CUDA(launch_adjoint_group(g, a->cell, a->h, s), "adjoint");
   } else {
     KDE_CUDA(launch_adjoint_gauss(q.pts, q.wts, a->n, grad_out, q.gxt, q.gyt, a->nx, a->ny,
                                   a->cell, a->h, grad_points, grad_weights, ht, lt, s),
@@ -1999,11 +2015,12 @@ int kde_diag_exclusive_scan(const uint32_t* in, uint32_t* out, int64_t n, int pe
 }
 
 int kde_diag_adjoint_list(const uint32_t* start, int nbins, int64_t m, int sort_failed,
-                          int32_t* list, uint32_t* counters, void* stream) {
+                          int32_t* list, uint32_t* singles, uint32_t* counters, void* stream) {
   if (nbins < 1 || m < 0 || m >= ((int64_t)1 << 32))
     return fail(KDE_EINVAL, "nbins must be positive and m in [0, 2^32)");
-  if (!start || !list || !counters) return fail(KDE_EINVAL, "null pointer");
-  if (memory_kind(start) != 0 || memory_kind(list) != 0 || memory_kind(counters) != 0)
+  if (!start || !list || !singles || !counters) return fail(KDE_EINVAL, "null pointer");
+  if (memory_kind(start) != 0 || memory_kind(list) != 0 || memory_kind(singles) != 0 ||
+      memory_kind(counters) != 0)
     return fail(KDE_EINVAL, "kde_diag_adjoint_list needs device pointers");
   if (reinterpret_cast<uintptr_t>(list) & 15) return fail(KDE_EINVAL, "list must be 16-byte aligned");
   void* ws = nullptr;
@@ -2018,6 +2035,7 @@ int kde_diag_adjoint_list(const uint32_t* start, int nbins, int64_t m, int sort_
   a.nbins = nbins;
   a.m = m;
   a.list = reinterpret_cast<int4*>(list);
+  a.singles = singles;
   a.counters = counters;
   a.err = static_cast<const CallScalars*>(ws);
   KDE_CUDA(launch_adjoint_list(a, s), "list of the adjoint's groups");

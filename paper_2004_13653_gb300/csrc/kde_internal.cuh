@@ -477,7 +477,8 @@ cudaError_t launch_adjoint_gauss(const float4* pts, const float* wts, int64_t n,
                                  double* hterm, double* lterm, cudaStream_t s);
 // The same for points sorted into kAdjBin-cell bins (launch_bin_sort with their
 // indices): groups of kAdjGroup points of a bin share their window.
-constexpr int kAdjBin = 8, kAdjGroup = 64;
+// A bin's last points, where they are fewer than kAdjFew, are taken one by one.
+constexpr int kAdjBin = 8, kAdjGroup = 64, kAdjFew = 12;
 struct AdjGroupArgs {
   const float4* pts;        // in bin order, offsets in bandwidths
   const float* wts;
@@ -488,7 +489,8 @@ struct AdjGroupArgs {
   int reach;                // cells to either side of a point's own window
   double cell_s;            // cell side in bandwidths
   int4* list;               // [m / kAdjGroup + nbins + 2]
-  uint32_t* counters;       // [2]
+  uint32_t* singles;        // [m] sorted positions of the points taken one by one
+  uint32_t* counters;       // [3] groups, groups taken, singles
   const float* G;
   const float2 *gxt, *gyt;
   float c, inv_h;           // 1/(2 pi n h^2), 1/h
@@ -499,9 +501,12 @@ struct AdjGroupArgs {
 };
 int adj_group_radius(double cell, double h, int nx, int ny);  // window half-width R, cells
 bool adj_group_fits(int R);
-// The list of the groups alone (start, nbins, m, list, counters and err of a).
+// The list of the groups alone (start, nbins, m, list, singles, counters and err
+// of a).
 cudaError_t launch_adjoint_list(const AdjGroupArgs& a, cudaStream_t s);
-cudaError_t launch_adjoint_group(const AdjGroupArgs& a, cudaStream_t s);
+// The points of a.singles by the one-point form (kde_adjoint.cu).
+cudaError_t launch_adjoint_listed(const AdjGroupArgs& a, double cell, double h, cudaStream_t s);
+cudaError_t launch_adjoint_group(const AdjGroupArgs& a, double cell, double h, cudaStream_t s);
 // The same adjoint as two tcgen05 contractions (points prepared in the
 // Gaussian's units, sigma = 1/(h sqrt(2 ln 2)), and their cell tables):
 // U = G B and V = G^T A with the points' operands generated on chip.  ws:

@@ -152,3 +152,43 @@ def test_non_finite_cotangent_cells(value, h_cells):
     np.testing.assert_array_equal(np.isfinite(gxy), np.isfinite(sxy))
     assert rel_linf(gw[~hit], clean[1][~hit]) <= SAME
     assert rel_linf(gxy[~hit], clean[0][~hit]) <= SAME
+
+
+@pytest.mark.parametrize("nx,h_cells", [(3_000_000, 1.0), (34_000_000, 1.5), (34_000_000, 3.0)])
+def test_long_axes_with_points_in_clusters(nx, h_cells):
+    """As above, with enough points in a bin for groups of them."""
+    n, cell, per = 16384, 7.3, 64
+    rng = np.random.default_rng(nx)
+    at = np.repeat(nx - rng.integers(0, nx // 50, n // per), per)
+    local = np.stack([(at + rng.random(n) * 4.0) * cell, rng.random(n) * cell], 1)
+    w = (rng.random(n) + 0.5).astype(np.float32)
+    wl = workloads.Workload("long", local, w, nx * cell, cell, nx, 1, h_cells * cell,
+                            oracle.GAUSSIAN, np.array([0, n]), 0)
+    G = rng.standard_normal(nx, dtype=np.float32)
+    gxy, gw, _ = backward(wl, w, G[None])
+    rxy, rw = own_window(wl.xy - np.asarray(wl.origin), w.astype(np.float64), cell, wl.h,
+                         G.astype(np.float64), n)
+    assert rel_linf(gw, rw) <= TOL_GRAD
+    assert rel_linf(gxy, rxy) <= TOL_GRAD
+
+
+@pytest.mark.parametrize("n,side,h_cells,sorts", [
+    (16383, 300, 2.0, False), (16384, 1024, 1.0, True), (16384, 300, 2.0, True),
+    (20011, 128, 3.0, True), (16400, 2048, 5.3, True),
+    (20000, 100, 0.75, False), (20000, 100, 0.76, True),  # windows of 16 and of 18 cells
+    (65535, 900, 2.0, True), (65536, 900, 2.0, False),    # 5.1 points a bin
+    (65536, 640, 2.0, True), (70000, 900, 3.25, False), (70000, 900, 3.3, True),
+])
+def test_bins_with_few_points(n, side, h_cells, sorts):
+    """Points spread evenly, 0.25 to 78 a bin: bins without a group, points left over
+    beside groups, and the lines of the rule that sorts the points at all."""
+    wl = workloads.random_points(34, n, 10.0 * side, 10.0, side, side, 10.0 * h_cells,
+                                 oracle.GAUSSIAN)
+    G = np.random.default_rng(4).normal(0, 1, (side, side))
+    before = kde.launch_count()
+    gxy, gw, gh = backward(wl, wl.w, G)
+    launches = kde.launch_count() - before
+    sxy, sw, sh = backward(wl, wl.w, G, workspace=one_point_workspace(wl))
+    assert (launches > kde.launch_count() - before - launches) == sorts
+    assert rel_linf(gxy, sxy) <= SAME and rel_linf(gw, sw) <= SAME
+    assert gh == pytest.approx(sh, rel=1e-4)

@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 import paper_2004_13653_gb300 as kde  # noqa: E402
 
-M, NBINS, GROUP = 512, 7, 64
+M, NBINS, GROUP, FEW, FAR = 2048, 7, 64, 12, 1024
 ENTRIES = M // GROUP + NBINS + 2
 
 
@@ -23,29 +23,40 @@ def lib():
 def listed(lib, starts, failed):
     start = torch.as_tensor(np.asarray(starts, dtype=np.uint32).view(np.int32), device="cuda")
     groups = torch.full((ENTRIES, 4), -7, dtype=torch.int32, device="cuda")
-    counters = torch.full((2,), -7, dtype=torch.int32, device="cuda")
+    singles = torch.full((M,), -7, dtype=torch.int32, device="cuda")
+    counters = torch.full((3,), -7, dtype=torch.int32, device="cuda")
     kde.check(lib.kde_diag_adjoint_list(start.data_ptr(), NBINS, M, failed, groups.data_ptr(),
-                                        counters.data_ptr(), None))
-    return groups.cpu().numpy(), counters.cpu().numpy()
+                                        singles.data_ptr(), counters.data_ptr(), None))
+    return groups.cpu().numpy(), singles.cpu().numpy(), counters.cpu().numpy()
 
 
-def test_adjoint_groups_of_rising_starts(lib):
-    starts = [0, 0, 1, 65, 129, 194, 194, 500]  # 0, 1, 64, 64, 65, 0, 306 points, 12 beyond reach
-    groups, counters = listed(lib, starts, 0)
-    ends = starts[1:] + [M]
-    want = [(b, a + k, min(GROUP, e - a - k), 0) for b, (a, e) in enumerate(zip(starts, ends))
-            for k in range(0, e - a, GROUP)]
-    assert counters.tolist() == [len(want), 0]
+@pytest.mark.parametrize("starts", [
+    [0, 0, 1, 65, 129, 194, 194, 500],    # 0, 1, 64, 64, 65, 0, 306 points, 1548 beyond reach
+    [3, 14, 26, 101, 177, 177, 188, 2047],  # 11, 12, 64 + 11, 64 + 12, 0, 11, 1859, 1 beyond
+    [0, 0, 0, 0, 0, 0, 0, 0],              # 2048 beyond
+])
+def test_adjoint_groups_of_rising_starts(lib, starts):
+    groups, singles, counters = listed(lib, starts, 0)
+    want, alone = [], []
+    for b, (a, e) in enumerate(zip(starts, starts[1:] + [M])):
+        most = GROUP if b < NBINS else FAR
+        for k in range(a, e, most):
+            if b < NBINS and e - k < FEW:
+                alone += range(k, e)
+            else:
+                want.append((b, k, min(most, e - k), 0))
+    assert counters.tolist() == [len(want), 0, len(alone)]
     assert sorted(map(tuple, groups[:len(want)].tolist())) == want
-    assert (groups[len(want):] == -7).all()
+    assert sorted(singles[:len(alone)].tolist()) == alone
+    assert (groups[len(want):] == -7).all() and (singles[len(alone):] == -7).all()
 
 
-@pytest.mark.parametrize("starts", [[512, 0, 512, 0, 512, 0, 512, 0], [5, 4, 3, 2, 1, 0, 0, 512],
+@pytest.mark.parametrize("starts", [[2048, 0, 2048, 0, 2048, 0, 2048, 0], [5, 4, 3, 2, 1, 0, 0, 2048],
                                     [0, 2 ** 32 - 1, 0, 2 ** 31, 7, 600, 1, 2 ** 31 + 5]])
 def test_adjoint_lists_nothing_after_a_timed_out_sort(lib, starts):
-    groups, counters = listed(lib, starts, 1)
-    assert counters.tolist() == [0, 0]
-    assert (groups == -7).all()
+    groups, singles, counters = listed(lib, starts, 1)
+    assert counters.tolist() == [0, 0, 0]
+    assert (groups == -7).all() and (singles == -7).all()
 
 
 @pytest.mark.parametrize("side", [32, 128, 256])
