@@ -192,3 +192,25 @@ def test_bins_with_few_points(n, side, h_cells, sorts):
     assert (launches > kde.launch_count() - before - launches) == sorts
     assert rel_linf(gxy, sxy) <= SAME and rel_linf(gw, sw) <= SAME
     assert gh == pytest.approx(sh, rel=1e-4)
+
+
+@pytest.mark.parametrize("h_cells", [3.3, 5.3])
+def test_error_no_larger_than_one_point_form(h_cells):
+    """Rms over 20,000 points, a statistic that repeats to a few percent: sums of W
+    terms added from the small ones to the large ones round less than in order."""
+    n, nx, ny = 20000, 190, 170
+    wl = workloads.random_points(35, n, 10.0 * ny, 10.0, nx, ny, 10.0 * h_cells, oracle.GAUSSIAN)
+    G = np.random.default_rng(5).normal(0, 1, (ny, nx)).astype(np.float32)
+    at = wl.xy - np.asarray(wl.origin)
+    s = ((np.arange(nx) + 0.5) * wl.cell - at[:, :1]) / wl.h
+    t = ((np.arange(ny) + 0.5) * wl.cell - at[:, 1:]) / wl.h
+    A, B = np.exp(-0.5 * s * s), np.exp(-0.5 * t * t)
+    U = A @ G.T.astype(np.float64)  # over the columns
+    V = B @ G.astype(np.float64)
+    c = 1.0 / (2 * np.pi * n * wl.h ** 2)
+    rw = c * (B * U).sum(1)
+    rxy = c * wl.w[:, None].astype(np.float64) / wl.h * np.stack([(s * A * V).sum(1), (t * B * U).sum(1)], 1)
+    gxy, gw, _ = backward(wl, wl.w, G)
+    sxy, sw, _ = backward(wl, wl.w, G, workspace=one_point_workspace(wl))
+    for got, one, ref in ((gxy, sxy, rxy), (gw, sw, rw)):
+        assert np.sqrt(((got - ref) ** 2).mean()) <= 0.95 * np.sqrt(((one - ref) ** 2).mean())
