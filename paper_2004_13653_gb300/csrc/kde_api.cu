@@ -1863,7 +1863,8 @@ int kde_grid_binned(const double* points, const int64_t* traj_offsets, int64_t n
   const size_t o_added = take(2 * sizeof(unsigned long long));
   const size_t o_counts = take(counts_out ? 0 : sizeof(int) * (size_t)cells);
   const size_t row_bytes = sizeof(float) * (size_t)cells;
-  const bool want_ends = traj_offsets && interpolate && n > 0;
+  // (few fixes search the offsets: the bits cost two launches, 5 us)
+  const bool want_ends = traj_offsets && interpolate && n >= 1 << 17;
   const size_t end_bytes = want_ends ? binned_ends_bytes(n) : 0;
   bool ends = want_ends;
   const size_t o_rows = take(std::max(row_bytes, end_bytes));

@@ -143,19 +143,19 @@ __device__ __forceinline__ int fill_gap(int i, int j, int i1, int j1, int nx,
   return m - 1;
 }
 
-// A warp takes kCountRounds x 32 consecutive fixes; each fix's cell is found
+// A warp takes `rounds` x 32 consecutive fixes at a time, as many rounds as leave
+// work for every warp (count_rounds); each fix's cell is found
 // once, the cell before it comes from the neighbouring lane (lane 0: from the
 // last round).  ends: bits of the fixes that end a trajectory; null (no
 // scratch for them) or *irregular set: the offsets are searched per fix.
 // Bound by the L2 atomics (one per fix and interpolated cell).  20M fixes x
 // 4096^2, interpolated: 4.21 ms with every index and cell in FP64, the
 // successor's cell found again and a search of the offsets per fix; 0.33 now.
-constexpr int kCountRounds = 16;
 __global__ void __launch_bounds__(256)
     k_count(const double2* __restrict__ xy, int64_t n, const int64_t* __restrict__ off,
             int64_t ntraj, const uint32_t* __restrict__ ends,
             const unsigned* __restrict__ irregular, const __grid_constant__ CellMap mx,
-            const __grid_constant__ CellMap my, int interpolate, int* __restrict__ counts,
+            const __grid_constant__ CellMap my, int interpolate, int rounds, int* __restrict__ counts,
             unsigned long long* __restrict__ added) {
   const int lane = threadIdx.x & 31, nx = mx.n;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -163,8 +163,8 @@ __global__ void __launch_bounds__(256)
   const int64_t last_end = off ? off[ntraj] : n;  // no fix from here on has a successor
   int my_added = 0;
   unsigned long long total = 0;
-  for (int64_t b = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32 * kCountRounds;
-       b < n; b += warps * 32 * kCountRounds) {
+  for (int64_t b = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32 * rounds;
+       b < n; b += warps * 32 * rounds) {
     double2 v = b + lane < n ? xy[b + lane] : make_double2(0.0, 0.0);
     int last_i = -1, last_j = -1;  // cell of the fix before this round's first
     if (interpolate && b > 0 && lane == 31) {
@@ -173,11 +173,11 @@ __global__ void __launch_bounds__(256)
       last_j = cell_of(w.y, my);
     }
     uint32_t last_ends = ends && interpolate && b > 0 ? ends[(b >> 5) - 1] : 0u;
-    for (int r = 0; r < kCountRounds; ++r) {
+    for (int r = 0; r < rounds; ++r) {
       const int64_t p = b + r * 32 + lane;
       if (b + r * 32 >= n) break;
       const double2 now = v;
-      if (r + 1 < kCountRounds && p + 32 < n) v = xy[p + 32];
+      if (r + 1 < rounds && p + 32 < n) v = xy[p + 32];
       int i = -1, j = -1;
       if (p < n) {
         i = cell_of(now.x, mx);
@@ -224,26 +224,35 @@ struct Stencil {
 };
 
 // Row pass: R(i, j) = sum_u k_u M(i - a + u, j) (cells outside the grid are
-// zero), u falling.  A block takes kRowTile columns of one row; a thread four
+// zero), u falling.  LANES threads take 4 LANES columns of one row: a block's 128,
+// or a warp's 32 where a row has no more than that many (four rows a block then).
+// A thread computes four
 // neighbouring ones, so each 16-byte read of the staged line feeds 16 FMAs (one
 // output per thread read 4 bytes per FMA: 107 us on 4096^2 with 35 taps, 58
-// now).  Rows are strided over gridDim.y (which is capped at 65535).
-constexpr int kRowThreads = 128, kRowTile = 4 * kRowThreads;
+// now; 20 x 20000 with 97 taps: 16 so, 20 with a block per row, 17 now).  Rows
+// are strided over gridDim.y (which is capped at 65535).
+constexpr int kRowThreads = 128;
+template <int LANES>
 __global__ void __launch_bounds__(kRowThreads)
     k_conv_rows(const int* __restrict__ counts, int nx, int ny, int a,
                 const __grid_constant__ Stencil st, float* __restrict__ R) {
-  __shared__ __align__(16) float line[kRowTile + 2 * kMaxHalf + 6];
-  const int i0 = blockIdx.x * kRowTile, t = threadIdx.x;
+  constexpr int kRows = kRowThreads / LANES, kTile = 4 * LANES, kLine = kTile + 2 * kMaxHalf + 6;
+  __shared__ __align__(16) float lines[kRows][kLine];
+  const int i0 = blockIdx.x * kTile, t = threadIdx.x % LANES, sub = threadIdx.x / LANES;
+  float* line = lines[sub];
   const int taps4 = (2 * a + 4) / 4;  // groups of four taps
-  const int width = min(kRowTile, nx - i0);
-  for (int j = blockIdx.y; j < ny; j += gridDim.y) {
-    const int* row = counts + (int64_t)j * nx;
-    for (int x = t; x < kRowTile + 4 * taps4 + 4; x += kRowThreads) {
+  const int width = min(kTile, nx - i0);
+  auto sync = []() {
+    if (LANES == 32) __syncwarp();
+    else __syncthreads();
+  };
+  for (int64_t j = (int64_t)blockIdx.y * kRows + sub; j < ny; j += (int64_t)gridDim.y * kRows) {
+    const int* row = counts + j * nx;
+    for (int x = t; x < ((width + 3) & ~3) + 4 * taps4 + 4; x += LANES) {
       const int i = i0 - a + x;
-      if (x < kRowTile + 2 * kMaxHalf + 6)
-        line[x] = (i >= 0 && i < nx && x < width + 2 * a) ? (float)row[i] : 0.f;
+      if (x < kLine) line[x] = (i >= 0 && i < nx && x < width + 2 * a) ? (float)row[i] : 0.f;
     }
-    __syncthreads();
+    sync();
     if (4 * t < width) {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
       const float4* v4 = reinterpret_cast<const float4*>(line) + t;
@@ -259,60 +268,85 @@ __global__ void __launch_bounds__(kRowThreads)
         }
         hi = lo;
       }
-      float* out = R + (int64_t)j * nx + i0 + 4 * t;
+      float* out = R + j * nx + i0 + 4 * t;
 #pragma unroll
       for (int c = 0; c < 4; ++c)
         if (4 * t + c < width) out[c] = acc[c];
     }
-    __syncthreads();
+    sync();
   }
 }
 
 // Column pass: out(i, j) = norm sum_u k_u R(i, j - a + u), u falling.  A block
-// takes kColTile columns x kColRows rows; a thread four columns 32 apart and
+// takes 32 C columns x kColRows rows; a thread C columns 32 apart and
 // eight consecutive rows, and walks the rows of their common window once from
 // its end: each value feeds eight FMAs, with coefficients that are zero outside
-// an output's window (added zeros change nothing).  The block's rows stay in
-// L1.  Staging 64 rows x 32 columns with one output per thread and step: 90 us
-// on 4096^2 with 35 taps, 65 now.
-constexpr int kColTile = 128, kColRows = 64;
+// an output's window (added zeros change nothing).  Step s of the walk needs the
+// coefficients of distances s .. s + 7, which stay in registers, one new one a step.
+// The block's rows stay in L1.  Staging 64 rows x 32 columns with one output per
+// thread and step: 90 us on 4096^2 with 35 taps, 65 with C = 4 and eight coefficients
+// read a step.  C = 1 where the grid has too few blocks of four columns a thread, or
+// fewer than 33 columns (conv_columns).
+constexpr int kColRows = 64;
+template <int C>
 __global__ void __launch_bounds__(256)
     k_conv_cols(const float* __restrict__ R, int nx, int ny, int a,
                 const __grid_constant__ Stencil st, float norm, float* __restrict__ out) {
-  // k with eight zeros on either side
-  __shared__ __align__(16) float kz[2 * kMaxHalf + 2 + 24];
-  for (int x = threadIdx.x; x < 2 * kMaxHalf + 26; x += 256)
-    kz[x] = x >= 8 && x - 8 <= 2 * a ? st.k[x - 8] : 0.f;
+  // kz[8 + m] = k by distance m from the walk's first row; zeros around it
+  __shared__ float kz[2 * kMaxHalf + 1 + 24];
+  for (int x = threadIdx.x; x < 2 * kMaxHalf + 25; x += 256)
+    kz[x] = x >= 8 && x - 8 <= 2 * a ? st.k[2 * a - (x - 8)] : 0.f;
   __syncthreads();
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int i0 = blockIdx.x * kColTile + tx, j0 = blockIdx.y * kColRows + 8 * ty;
+  const int i0 = blockIdx.x * (32 * C) + tx, j0 = blockIdx.y * kColRows + 8 * ty;
   if (i0 >= nx || j0 >= ny) return;
-  float acc[8][4];
+  float acc[8][C];
 #pragma unroll
   for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-  const int last = min(j0 + 7 + a, ny - 1), first = max(j0 - a, 0);
-#pragma unroll 2
-  for (int j = last; j >= first; --j) {
-    const float* row = R + (int64_t)j * nx + i0;
-    float v[4], k[8];
+    for (int c = 0; c < C; ++c) acc[r][c] = 0.f;
+  // output row j0 + r takes the tap at distance s + r - 7 in step s, row top - s; the
+  // coefficient of step s + r is in k[(s + r) % 8]
+  const int top = j0 + 7 + a;
+  const int begin = max(top - (ny - 1), 0) & ~7, end = min(8 + 2 * a, top + 1);  // the grid's rows
+  float k[8];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) v[c] = i0 + 32 * c < nx ? __ldg(row + 32 * c) : 0.f;
-    // output row j0 + r takes tap u = j - (j0 + r) + a
+  for (int r = 0; r < 7; ++r) k[r] = kz[1 + begin + r];
+  for (int s0 = begin; s0 < end; s0 += 8) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r) k[r] = kz[8 + j - j0 - r + a];
+    for (int q = 0; q < 8; ++q) {
+      const int s = s0 + q, j = top - s;
+      k[(q + 7) & 7] = kz[8 + s];
+      float v[C];
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+      for (int c = 0; c < C; ++c)
+        v[c] = j >= 0 && j < ny && i0 + 32 * c < nx ? __ldg(R + (int64_t)j * nx + i0 + 32 * c) : 0.f;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(k[r], v[c], acc[r][c]);
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[r][c] = fmaf(k[(q + r) & 7], v[c], acc[r][c]);
+    }
   }
 #pragma unroll
   for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
+    for (int c = 0; c < C; ++c)
       if (j0 + r < ny && i0 + 32 * c < nx)
         out[(int64_t)(j0 + r) * nx + i0 + 32 * c] = acc[r][c] * norm;
+}
+
+// Rounds of k_count: 16 where every warp of the GPU gets that many (fewer fixes'
+// cells are then found twice), fewer below, one under 311,000 fixes, whose gaps would
+// otherwise be walked one after the other by a few warps (5000 fixes far apart on
+// 512^2: 659 us with a thread per fix, 1170 with 16 rounds).
+int count_rounds(int64_t n) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(16, n / (152 * 8 * 8 * 32)));
+}
+
+// Columns per thread of the column pass.
+int conv_columns(int nx, int ny) {
+  const int64_t blocks = (int64_t)((nx + 127) / 128) * ((ny + kColRows - 1) / kColRows);
+  return nx > 32 && blocks >= 2 * 152 ? 4 : 1;
 }
 
 // One factor k(s) of a Table 1 kernel with its constant, in double (host side).
@@ -380,23 +414,30 @@ cudaError_t launch_binned(const double* xy, int64_t n, const int64_t* off, int64
       m.n = cells;
       return m;
     };
-    const int64_t per_block = 8 * 32 * kCountRounds;
+    const int rounds = count_rounds(n);
+    const int64_t per_block = 8 * 32 * rounds;
     const int64_t blocks = std::min<int64_t>((n + per_block - 1) / per_block, 152 * 8);
     k_count<<<(int)blocks, 256, 0, s>>>(reinterpret_cast<const double2*>(xy), n, off, ntraj, ends,
-                                        irregular, map(ox, nx), map(oy, ny), interpolate, counts,
-                                        added);
+                                        irregular, map(ox, nx), map(oy, ny), interpolate, rounds,
+                                        counts, added);
     note_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   Stencil st = {};
   for (int u = 0; u <= 2 * a; ++u) st.k[u] = (float)table1_factor(kid, (a - u) * cell / h);
   const float norm = n > 0 ? (float)(1.0 / ((double)n * h * h)) : 0.0f;
-  k_conv_rows<<<dim3((nx + kRowTile - 1) / kRowTile, ny < 65535 ? ny : 65535), kRowThreads, 0, s>>>(
-      counts, nx, ny, a, st, rowbuf);
+  if (nx <= 128)
+    k_conv_rows<32><<<dim3(1, std::min((ny + 3) / 4, 65535)), kRowThreads, 0, s>>>(counts, nx, ny, a,
+                                                                                 st, rowbuf);
+  else
+    k_conv_rows<128><<<dim3((nx + 511) / 512, std::min(ny, 65535)), kRowThreads, 0, s>>>(
+        counts, nx, ny, a, st, rowbuf);
   note_launches(1);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_conv_cols<<<dim3((nx + kColTile - 1) / kColTile, (ny + kColRows - 1) / kColRows), 256, 0, s>>>(
-      rowbuf, nx, ny, a, st, norm, out);
+  const int cols = conv_columns(nx, ny);
+  const dim3 tiles((nx + 32 * cols - 1) / (32 * cols), (ny + kColRows - 1) / kColRows);
+  if (cols == 4) k_conv_cols<4><<<tiles, 256, 0, s>>>(rowbuf, nx, ny, a, st, norm, out);
+  else k_conv_cols<1><<<tiles, 256, 0, s>>>(rowbuf, nx, ny, a, st, norm, out);
   note_launches(1);
   return cudaGetLastError();
 }
