@@ -309,6 +309,50 @@ __device__ __forceinline__ int dp_finish(const double2* __restrict__ P,
   return most;
 }
 
+// A lane's points begin, begin + step, ... of segment (s, e) whose upper bound
+// reaches `low`, in FP64: the largest numerator and the first point that has it.
+// tie: another one comes so close below it that the quotients may be equal.
+struct DpBest {
+  double c;
+  int at;
+  bool tie;
+};
+__device__ __forceinline__ DpBest dp_best(const double2* __restrict__ P,
+                                          const float4* __restrict__ q, int begin, int step, int e,
+                                          float4 A, float4 B, double2 Ad, double2 Bd, double len,
+                                          float low, float uR, float tiny) {
+  constexpr double near = 1.0 - 2e-15;
+  DpBest r = {0.0, -1, false};
+  for (int i = begin; i < e; i += step)
+    if (dp_bracket(q[i], A, B, uR, tiny).hi >= low) {
+      const double c = ved_num(P[i], Ad, Bd, len);
+      if (c > r.c) {
+        r.tie = r.tie || (r.at >= 0 && r.c >= __dmul_rn(c, near));
+        r.c = c;
+        r.at = i;
+      } else if (c != r.c && c >= __dmul_rn(r.c, near)) {
+        r.tie = true;
+      }
+    }
+  return r;
+}
+// The first of the lane's points whose VED is the segment's largest: its best one,
+// or, with ties about, by another look at all of them.
+__device__ __forceinline__ uint32_t dp_first(const double2* __restrict__ P,
+                                             const float4* __restrict__ q, int begin, int step,
+                                             int e, float4 A, float4 B, double2 Ad, double2 Bd,
+                                             double len, float low, float uR, float tiny,
+                                             const DpBest& mine, bool ties, double cmax,
+                                             double dmax) {
+  const double from = __dmul_rn(cmax, 1.0 - 1e-15);
+  auto is_it = [&](double c) { return c >= from && (c == cmax || ved_of(c, len) == dmax); };
+  if (!ties) return mine.at >= 0 && is_it(mine.c) ? (uint32_t)mine.at : kNoArg;
+  for (int i = begin; i < e; i += step)
+    if (dp_bracket(q[i], A, B, uR, tiny).hi >= low && is_it(ved_num(P[i], Ad, Bd, len)))
+      return (uint32_t)i;
+  return kNoArg;
+}
+
 // The split of segment (s, e) by one warp, every lane alike; -1: nothing in it
 // is above eps.
 __device__ __forceinline__ int dp_split_warp(const double2* __restrict__ P,
@@ -342,30 +386,125 @@ __device__ __forceinline__ int dp_split_warp(const double2* __restrict__ P,
   // nothing: low is 0 there)
   const double2 Ad = P[s], Bd = P[e];
   const double len = seg_len(Ad, Bd);
-  double cmax = 0.0;
-  for (int i = s + 1 + lane; i < e; i += 32)
-    if (dp_bracket(q[i], A, B, uR, tiny).hi >= low) {
-      const double c = ved_num(P[i], Ad, Bd, len);
-      if (c > cmax) cmax = c;
-    }
+  const DpBest mine = dp_best(P, q, s + 1 + lane, 32, e, A, B, Ad, Bd, len, low, uR, tiny);
+  double cmax = mine.c;
   for (int o = 16; o > 0; o >>= 1) {
     const double c = __shfl_xor_sync(0xffffffffu, cmax, o);
     if (c > cmax) cmax = c;
   }
   const double dmax = cmax == 0.0 ? 0.0 : ved_of(cmax, len);
   if (!(dmax > eps)) return -1;
-  uint32_t first = kNoArg;
-  for (int i = s + 1 + lane; i < e; i += 32)
-    if (first == kNoArg && dp_bracket(q[i], A, B, uR, tiny).hi >= low) {
-      const double c = ved_num(P[i], Ad, Bd, len);
-      if (c >= __dmul_rn(cmax, 1.0 - 1e-15) && (c == cmax || ved_of(c, len) == dmax))
-        first = (uint32_t)i;
-    }
+  const bool ties = __any_sync(0xffffffffu, mine.tie);
+  const uint32_t first = dp_first(P, q, s + 1 + lane, 32, e, A, B, Ad, Bd, len, low, uR, tiny, mine,
+                                  ties, cmax, dmax);
   return (int)__reduce_min_sync(0xffffffffu, first);  // kNoArg = -1
 }
 
+// The split of segment (s, e) by a team of `size` warps, this one its `rank`-th (the
+// same warps of the CTA for all of a team, first its first warp); -1: nothing in it
+// is above eps.  The same decisions as dp_split_warp's, the maxima and the points
+// left taken over the team through shared memory.  Every warp of the CTA calls it
+// alike (warps without a segment: none), for its barriers.
+struct TeamShared {
+  double c[16];
+  float low[16], high[16];
+  int at[16], left[16];
+  uint32_t first[16];
+};
+__device__ __forceinline__ int dp_split_team(const double2* __restrict__ P,
+                                             const float4* __restrict__ q, int s, int e, bool none,
+                                             int first_warp, int rank, int size, float uR,
+                                             float tiny, float eps_lo, float eps_hi, double eps,
+                                             TeamShared& S) {
+  const int lane = threadIdx.x & 31, warp = first_warp + rank;
+  const float4 A = q[s], B = q[e];
+  const int begin = s + 1 + 32 * rank + lane, step = 32 * size;
+  const DpBracket b = dp_bracket(A, A, B, uR, tiny);  // the length's bounds
+  float best_lo = 0.f, top = 0.f, second = 0.f;
+  int at = -1;
+  if (!none)
+    for (int i = begin; i < e; i += step) {
+      const DpBracket c = dp_bracket(q[i], A, B, uR, tiny);
+      best_lo = fmaxf(best_lo, c.lo);
+      if (c.hi > top) {
+        second = top;
+        top = c.hi;
+        at = i;
+      } else {
+        second = fmaxf(second, c.hi);
+      }
+    }
+  float low = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(best_lo)));
+  float high = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(top)));
+  if (lane == 0) {
+    S.low[warp] = low;
+    S.high[warp] = high;
+  }
+  __syncthreads();
+  if (!none)
+    for (int w = first_warp; w < first_warp + size; ++w) {
+      low = fmaxf(low, S.low[w]);
+      high = fmaxf(high, S.high[w]);
+    }
+  const bool closed = none || high < eps_lo * b.len_lo;
+  // the points whose upper bound reaches the largest lower bound
+  const unsigned one = __ballot_sync(0xffffffffu, at >= 0 && top >= low);
+  const unsigned more = __ballot_sync(0xffffffffu, at >= 0 && second >= low && second > 0.f);
+  const int mine = one ? __shfl_sync(0xffffffffu, at, __ffs(one) - 1) : -1;
+  if (lane == 0) {
+    S.left[warp] = more ? 2 : __popc(one);
+    S.at[warp] = mine;
+  }
+  __syncthreads();
+  int left = 0, split = -1;
+  if (!closed)
+    for (int w = first_warp; w < first_warp + size; ++w) {
+      left += S.left[w];
+      if (S.left[w]) split = S.at[w];
+    }
+  const bool exact = !closed && !(left == 1 && low > eps_hi * b.len_hi);
+  if (closed) split = -1;
+  if (!__syncthreads_or(exact)) return split;
+  // undecided somewhere: the points left in FP64
+  const double2 Ad = P[s], Bd = P[e];
+  const double len = seg_len(Ad, Bd);
+  DpBest mine_d = {0.0, -1, false};
+  if (exact) mine_d = dp_best(P, q, begin, step, e, A, B, Ad, Bd, len, low, uR, tiny);
+  double cmax = mine_d.c;
+  for (int o = 16; o > 0; o >>= 1) {
+    const double c = __shfl_xor_sync(0xffffffffu, cmax, o);
+    if (c > cmax) cmax = c;
+  }
+  bool ties = __any_sync(0xffffffffu, mine_d.tie);
+  if (lane == 0) {
+    S.c[warp] = cmax;
+    S.left[warp] = ties;
+  }
+  __syncthreads();
+  if (exact)
+    for (int w = first_warp; w < first_warp + size; ++w) {
+      if (S.c[w] > cmax) cmax = S.c[w];
+      ties |= S.left[w] != 0;
+    }
+  const double dmax = cmax == 0.0 ? 0.0 : ved_of(cmax, len);
+  uint32_t first = kNoArg;
+  if (exact && dmax > eps)
+    first = dp_first(P, q, begin, step, e, A, B, Ad, Bd, len, low, uR, tiny, mine_d, ties, cmax,
+                     dmax);
+  first = __reduce_min_sync(0xffffffffu, first);
+  if (lane == 0) S.first[warp] = first;
+  __syncthreads();
+  if (!exact) return split;
+  for (int w = first_warp; w < first_warp + size; ++w) first = min(first, S.first[w]);
+  return (int)first;  // kNoArg = -1
+}
+
 // list: the trajectories of class cls (0: from the list's start, 1: from its
-// end), each of at most m points.
+// end), each of at most m points.  While a level has fewer segments than half the
+// CTA's warps and one of them is long, the warps share them in teams (one
+// warp a segment left fifteen of sixteen idle at the top of a long track: one of
+// 9000 points on a parabola 264 us per call, 172 so, 181 in the level kernel).
+constexpr int kTeamPoints = 512;
 __global__ void __launch_bounds__(512)
     k_dp_local(const double2* __restrict__ xy, const int64_t* __restrict__ off, int64_t n,
                double eps, int m, int cls, DpCtl* __restrict__ ctl,
@@ -377,7 +516,8 @@ __global__ void __launch_bounds__(512)
   uint32_t* small = longs + 2 * (m / 16);                // [m / 2]
   uint16_t* lvl = reinterpret_cast<uint16_t*>(small + m / 2);  // kept points: level + 1
   uint8_t* st = reinterpret_cast<uint8_t*>(lvl + m);
-  __shared__ uint32_t s_item, s_r, s_small, s_count[2];
+  __shared__ uint32_t s_item, s_r, s_small, s_count[2], s_team[2];
+  __shared__ TeamShared team;
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   const int warp = tid >> 5, warps = nt >> 5;
   if (__ldg(&ctl->irregular)) return;
@@ -386,17 +526,21 @@ __global__ void __launch_bounds__(512)
   const float eps_lo = (float)(eps * (1.0 - 1e-6)), eps_hi = (float)(eps * (1.0 + 1e-6));
   int most = 1;
   bool worked = false;
-  auto list_segment = [&](int s, int e, uint32_t* next, uint32_t* n_next) {
+  auto list_segment = [&](int s, int e, int which) {
     const uint32_t w = (uint32_t)s | ((uint32_t)e << 16);
     if (e - s < 2) return;
-    if (e - s - 1 <= kSmall) small[atomicAdd(&s_small, 1u)] = w;
-    else next[atomicAdd(n_next, 1u)] = w;
+    if (e - s - 1 <= kSmall) {
+      small[atomicAdd(&s_small, 1u)] = w;
+    } else {
+      longs[which * (m / 16) + atomicAdd(&s_count[which], 1u)] = w;
+      if (e - s >= kTeamPoints) s_team[which] = 1u;  // any thread, the same value
+    }
   };
   for (;;) {
     __syncthreads();  // the previous trajectory's state is no longer read
     if (tid == 0) {
       s_item = atomicAdd(&ctl->next[cls], 1u);
-      s_r = s_small = s_count[0] = s_count[1] = 0u;
+      s_r = s_small = s_count[0] = s_count[1] = s_team[0] = s_team[1] = 0u;
     }
     __syncthreads();
     const uint32_t item = s_item;
@@ -420,7 +564,7 @@ __global__ void __launch_bounds__(512)
       st[i] = i == 0 || i == len - 1 ? kKept : 0;
       lvl[i] = 0;
     }
-    if (tid == 0) list_segment(0, len - 1, longs, &s_count[0]);
+    if (tid == 0) list_segment(0, len - 1, 0);
     if (bad) atomicOr(&scal->err, kErrNonFinite);
     const uint32_t rb = __reduce_max_sync(0xffffffffu, __float_as_uint(r));
     if (lane == 0) atomicMax(&s_r, rb);
@@ -432,24 +576,36 @@ __global__ void __launch_bounds__(512)
       const uint32_t count = s_count[it & 1];
       if (!count) break;
       const uint32_t* cur = longs + (it & 1) * (m / 16);
-      uint32_t* next = longs + ((it & 1) ^ 1) * (m / 16);
-      for (uint32_t j = warp; j < count; j += warps) {
-        const int s = (int)(cur[j] & 0xffffu), e = (int)(cur[j] >> 16);
-        const int at = dp_split_warp(P, q, s, e, uR, tiny, eps_lo, eps_hi, eps);
+      // the split of (s, e), by `size` warps of which this is the rank-th
+      auto settle = [&](int s, int e, int at, int rank, int size) {
         if (at < 0) {
-          for (int i = s + 1 + lane; i < e; i += 32) st[i] = kDone;
+          for (int i = s + 1 + 32 * rank + lane; i < e; i += 32 * size) st[i] = kDone;
         } else {
           most = max(most, it + 2);
-          if (lane == 0) {
+          if (rank == 0 && lane == 0) {
             st[at] = kKept;
             lvl[at] = (uint16_t)(it + 1);
-            list_segment(s, at, next, &s_count[(it & 1) ^ 1]);
-            list_segment(at, e, next, &s_count[(it & 1) ^ 1]);
+            list_segment(s, at, (it & 1) ^ 1);
+            list_segment(at, e, (it & 1) ^ 1);
           }
+        }
+      };
+      if (s_team[it & 1] && 2 * (int)count <= warps) {
+        const int size = warps / (int)count, j = warp / size;
+        const bool none = j >= (int)count;
+        const uint32_t w = cur[none ? 0 : j];
+        const int s = (int)(w & 0xffffu), e = (int)(w >> 16), rank = warp - j * size;
+        const int at = dp_split_team(P, q, s, e, none, none ? warp : j * size, none ? 0 : rank,
+                                     none ? 1 : size, uR, tiny, eps_lo, eps_hi, eps, team);
+        if (!none) settle(s, e, at, rank, size);
+      } else {
+        for (uint32_t j = warp; j < count; j += warps) {
+          const int s = (int)(cur[j] & 0xffffu), e = (int)(cur[j] >> 16);
+          settle(s, e, dp_split_warp(P, q, s, e, uR, tiny, eps_lo, eps_hi, eps), 0, 1);
         }
       }
       __syncthreads();
-      if (tid == 0) s_count[it & 1] = 0u;  // the list after next
+      if (tid == 0) s_count[it & 1] = s_team[it & 1] = 0u;  // the list after next
       __syncthreads();
     }
     const uint32_t ns = s_small;
@@ -733,7 +889,11 @@ cudaError_t launch_dp(const double* xy, int64_t n, const int64_t* off, int64_t n
     int local_max = kLocalMax;
     int short_max = (int)std::min<int64_t>(kLocalMax,
                                            std::max<int64_t>(256, (5 * mean / 4 + 127) / 128 * 128));
-    if (ntraj > 0xffffffffll) local_max = short_max = 2;  // 32-bit list: none is local
+    // Brackets cannot tell a straight track's roundings from a VED above an eps this
+    // small (metres), and one SM's FP64 pipe is slower than the GPU's (straight tracks
+    // at eps = 0, level kernel / local: one of 9000 points 0.88 / 4.5 ms, 20,000 of 40
+    // 1.29 / 1.80); and the list holds 32-bit indices.
+    if (eps < 1e-8 || ntraj > 0xffffffffll) local_max = short_max = 2;  // none is local
     k_dp_plan<<<(unsigned)((ntraj + 255) / 256), 256, 0, st>>>(
         P, off, ntraj, n, flag, scal, short_max, local_max, ctl, list, list_cap, iters_dev);
     k_dp_init<<<grid_for(n), 256, 0, st>>>(P, n, off, ntraj, s, e, flag, segmax, segarg, seglen,

@@ -74,3 +74,28 @@ def test_ties_and_flat_tracks():
     xy = np.vstack(parts) + np.array([4096.0, 8192.0])
     for eps in (0.0, 4.0, 7.999, 8.0):
         check(xy, [len(p) for p in parts], eps)
+
+
+@pytest.mark.parametrize("eps", [1e-7, 4.0, 7.999, 8.0])
+def test_long_segments_shared_by_warps(eps):
+    """Tracks whose top levels have fewer segments than the CTA has warps: ties over
+    the whole track, ends of the track as the split, flat and closed tracks."""
+    i = np.arange(9000, dtype=np.float64)
+    zig = np.stack([i, (i % 2) * 8.0], 1)
+    line = np.stack([i, 2.0 * i], 1)
+    plateau = np.stack([i[:3000], np.where((i[:3000] > 100) & (i[:3000] < 2900), 50.0, 0.0)], 1)
+    late = np.stack([i[:5000], np.exp((i[:5000] - 4999.0) / 40.0) * 3000.0], 1)
+    t = np.arange(4000) * (2 * np.pi / 4000)
+    loop = np.stack([1000 * np.cos(t), 1000 * np.sin(t)], 1)
+    loop = np.vstack([loop, loop[:1]])
+    same = np.repeat(np.array([[5.0, 7.0]]), 2000, axis=0)
+    for parts in ([zig], [line], [plateau, late], [loop, same], [zig[:700], late, plateau, line[:1500]]):
+        check(np.vstack(parts) + np.array([4096.0, 8192.0]), [len(q) for q in parts], eps)
+
+
+@pytest.mark.parametrize("lens", [[640], [641], [960, 961], [3000], [9728], [9728] * 3 + [40] * 50])
+@pytest.mark.parametrize("eps", [0.5, 30.0, 500.0])
+def test_lengths_of_single_tracks(lens, eps):
+    """Every number of warps a CTA can have and of segments a level can have."""
+    rng = np.random.default_rng(23)
+    check(walks(rng, lens, 20.0, np.array(workloads.FALSE_ORIGIN)), lens, eps)
