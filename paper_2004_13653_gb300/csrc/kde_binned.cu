@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(256)
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   const bool search = off && (!ends || *irregular);
   const int64_t last_end = off ? off[ntraj] : n;  // no fix from here on has a successor
-  int my_added = 0;
+  // a fix adds up to a side of the grid: their sum needs 64 bits
   unsigned long long total = 0;
   for (int64_t b = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32 * rounds;
        b < n; b += warps * 32 * rounds) {
@@ -208,10 +208,8 @@ __global__ void __launch_bounds__(256)
         }
         next = p < off[lo + 1];
       }
-      if (next) my_added += fill_gap(pi, pj, i, j, nx, counts);
+      if (next) total += (unsigned)fill_gap(pi, pj, i, j, nx, counts);
     }
-    total += (unsigned)my_added;
-    my_added = 0;
   }
   for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
   if (lane == 0 && total) atomicAdd(added, total);
