@@ -238,8 +238,9 @@ float2 pair_of(double v) {
 void set_scale(PrepInst& q, double sigma, double cell, const MercParams* m) {
   q.sigma = sigma;
   q.cell_sigma = cell * sigma;
-  // a scale outside the plain range sends every point to prepare_any
-  const bool plain = sigma >= 0x1p-60 && sigma <= 0x1p60;
+  // a scale outside the plain range sends every point to prepare_any: up to 2^27 the
+  // product with a coordinate of the plain range (below 2^100) is an FP32 number
+  const bool plain = sigma >= 0x1p-60 && sigma <= 0x1p27;
   q.usual = plain ? 1 : 0;
   q.sigma2 = plain ? pair_of(sigma) : make_float2(0.f, 0.f);
   q.lonlat = m ? 1 : 0;

@@ -46,7 +46,7 @@ __device__ __forceinline__ bool finite_bits(double v) {
   return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
 }
 // v is zero or between 2^-60 and 2^100: split_bits and products with a scale
-// of 2^-60 .. 2^60 then neither overflow nor lose bits to underflow
+// of 2^-60 .. 2^27 then neither overflow nor lose bits to underflow
 __device__ __forceinline__ bool plain_range(double v) {
   const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
   return (h >> 20) - 963u < 160u || (h | (unsigned)__double2loint(v)) == 0u;

@@ -80,3 +80,20 @@ def test_non_finite_points_are_reported(bad):
         kde.grid(cuda(xy, torch.float64), None, (0.0, 0.0), 10.0, 10, 10, 20.0, "quartic",
                  path="simt", flags=kde.FLAG_SYNC)
     assert e.value.code == kde.KDE_EDATA
+
+
+@pytest.mark.parametrize("h", [1e-6, 3e-9, 1e-12, 1e-17])
+@pytest.mark.parametrize("far", [1e28, -1e30])
+def test_points_too_far_for_fp32_are_only_far(h, far):
+    """A finite coordinate whose offset in bandwidths is past FP32's range: the point
+    is out of every cell's reach, not bad data."""
+    rng = np.random.default_rng(7)
+    xy = rng.uniform(0.0, 40.0 * h, (300, 2))
+    xy[11] = [far, 5.0 * h]
+    xy[12] = [5.0 * h, far]
+    w = np.ones(len(xy), np.float32)
+    args = ((0.0, 0.0), h, 40, 40, 3.0 * h)
+    F = kde.grid(cuda(xy, torch.float64), cuda(w, torch.float32), *args, "quartic",
+                 flags=kde.FLAG_SYNC).cpu().numpy()
+    ref = oracle.kde_grid(xy, w, *args, oracle.QUARTIC)
+    assert rel_linf(F, ref) <= TOL_FP32
