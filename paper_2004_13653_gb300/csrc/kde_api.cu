@@ -975,9 +975,7 @@ int run_small_gauss(const kde_args* a, const kde_opts* o, bool sync) {
   MercParams merc;
   const bool lonlat = o && (o->flags & KDE_FLAG_LONLAT);
   if (lonlat) merc = mercator_params(o->lat0_deg);
-  set_scale(q, kernel_sigma(KDE_GAUSSIAN, a->h), a->cell, lonlat ? &merc : nullptr);
-  q.nx = a->nx;
-  q.ny = a->ny;
+  set_scale(q, a->nx, a->ny, kernel_sigma(KDE_GAUSSIAN, a->h), a->cell, lonlat ? &merc : nullptr);
   CallScalars* scal = nullptr;
   if (sync) {
     void* wsv = nullptr;
@@ -1084,9 +1082,7 @@ int run_batch(const kde_args* A, int count, const kde_opts* o, const kde_tiling*
     q.begin = I.prep_begin;
     q.ox = a->origin_x;
     q.oy = a->origin_y;
-    set_scale(q, kernel_sigma(kid_of(a), a->h), a->cell, lonlat ? &merc : nullptr);
-    q.nx = a->nx;
-    q.ny = a->ny;
+    set_scale(q, a->nx, a->ny, kernel_sigma(kid_of(a), a->h), a->cell, lonlat ? &merc : nullptr);
   }
   auto part_of = [&](int k) {
     return P.in[k].splits > 1 ? reinterpret_cast<float*>(base + P.in[k].off_part) : out_dev[k];
@@ -1589,9 +1585,7 @@ int kde_grid_backward(const kde_args* a, const float* grad_out, float* grad_poin
   q.ox = a->origin_x;
   q.oy = a->origin_y;
   // offsets in bandwidths (window kernel) or in h sqrt(2 ln 2) (contractions)
-  set_scale(q, sigma, a->cell, nullptr);
-  q.nx = a->nx;
-  q.ny = a->ny;
+  set_scale(q, a->nx, a->ny, sigma, a->cell, nullptr);
   double* ht = reinterpret_cast<double*>(base + o.ht);
   double* lt = reinterpret_cast<double*>(base + o.lt);
   double* part = reinterpret_cast<double*>(q.pts);  // done with when the sums run
@@ -1759,9 +1753,7 @@ int kde_lscv_grid(const kde_args* a, const float* F, double* loss, float* grad_F
   q.begin = 0;
   q.ox = a->origin_x;
   q.oy = a->origin_y;
-  set_scale(q, 1.0 / a->h, a->cell, nullptr);
-  q.nx = a->nx;
-  q.ny = a->ny;
+  set_scale(q, a->nx, a->ny, 1.0 / a->h, a->cell, nullptr);
   double* loo = reinterpret_cast<double*>(base + o_loo);
   double* hd = reinterpret_cast<double*>(base + o_hd);
   double* sq = reinterpret_cast<double*>(base + o_sq);

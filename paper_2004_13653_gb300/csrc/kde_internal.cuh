@@ -157,9 +157,9 @@ struct alignas(16) PrepInst {
   float2 sigma2, lat_q;  // pairs of FP32 numbers
   float range_f;
 };
-// Sets q's scale (offsets in units of 1 / sigma) and, with m, the projection of
-// its (lon, lat) points; q's origin is set before.
-void set_scale(PrepInst& q, double sigma, double cell, const MercParams* m);
+// Sets q's grid, its scale (offsets in units of 1 / sigma) and, with m, the
+// projection of its (lon, lat) points; q's origin is set before.
+void set_scale(PrepInst& q, int nx, int ny, double sigma, double cell, const MercParams* m);
 
 struct TcInst {
   const float4* pts;

@@ -166,9 +166,7 @@ extern "C" int kde_grid_noalloc(const double* points, const float* weights, int6
   q.begin = 0;
   q.ox = grid_origin[0];
   q.oy = grid_origin[1];
-  set_scale(q, kernel_sigma(kernel_id, h), cell, nullptr);
-  q.nx = nx;
-  q.ny = ny;
+  set_scale(q, nx, ny, kernel_sigma(kernel_id, h), cell, nullptr);
   const double c1 = kernel_const_1d(kernel_id);
   const float scale = n > 0 ? (float)(c1 * c1 / ((double)n * h * h)) : 0.0f;
 

@@ -235,12 +235,18 @@ float2 pair_of(double v) {
 }
 }  // namespace
 
-void set_scale(PrepInst& q, double sigma, double cell, const MercParams* m) {
+void set_scale(PrepInst& q, int nx, int ny, double sigma, double cell, const MercParams* m) {
+  q.nx = nx;
+  q.ny = ny;
   q.sigma = sigma;
   q.cell_sigma = cell * sigma;
   // a scale outside the plain range sends every point to prepare_any: up to 2^27 the
-  // product with a coordinate of the plain range (below 2^100) is an FP32 number
-  const bool plain = sigma >= 0x1p-60 && sigma <= 0x1p27;
+  // product with a coordinate of the plain range (below 2^100) is an FP32 number.
+  // The pairs' 2^-46 of a position is 2^-30 units or less over a grid of up to
+  // 2^16 of them, far below the 2^-25 that FP32 leaves of an offset of one.  Beyond,
+  // FP64 and its 2^-49 (3e7 cells at h = 0.3 cells, Epanechnikov: 2.7e-6 off with pairs, below 1.1e-6 now).
+  const bool plain = sigma >= 0x1p-60 && sigma <= 0x1p27 &&
+                     (double)std::max(nx, ny) * cell * sigma <= 0x1p16;
   q.usual = plain ? 1 : 0;
   q.sigma2 = plain ? pair_of(sigma) : make_float2(0.f, 0.f);
   q.lonlat = m ? 1 : 0;

@@ -82,7 +82,8 @@ static __device__ __noinline__ float4 prepare_any(double2 v, const PrepInst& I) 
 // FP64's 53 bits (the differences of projected coordinates, and the constant
 // and linear terms of the projection with the centring and scaling in them)
 // stays there, two or three operations a point, and the rest runs on pairs of
-// FP32 numbers, whose 2^-46 is far below the 2^-24 of every use of the result.
+// FP32 numbers, whose 2^-46 is far below the 2^-24 of every use of the result on
+// the grids that set_scale lets in.
 // False: prepare_any decides.
 __device__ __forceinline__ bool prepare_usual(double2 v, const PrepInst& I, float4& r) {
   float2 X, Y;

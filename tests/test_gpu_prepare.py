@@ -97,3 +97,20 @@ def test_points_too_far_for_fp32_are_only_far(h, far):
                  flags=kde.FLAG_SYNC).cpu().numpy()
     ref = oracle.kde_grid(xy, w, *args, oracle.QUARTIC)
     assert rel_linf(F, ref) <= TOL_FP32
+
+
+def test_far_end_of_a_long_axis_in_fp64():
+    """1e8 bandwidths from the origin, points in the last tenth of the cells, each in
+    reach of its own only.  The position and the cell's centre keep 2^-49 of 1e8 each,
+    after two FP64 products each with a rounded factor; the kernel's slope is at most 2."""
+    nx, cell, h = 30_000_000, 1.0, 0.3
+    rng = np.random.default_rng(8)
+    at = rng.choice(nx // 10, 3000, replace=False) + nx - nx // 10
+    u = rng.uniform(-0.9, 0.9, 3000)
+    xy = np.stack([(at + 0.5) * cell - u * h, np.full(3000, 0.5 * cell)], 1)
+    u = ((at + 0.5) * cell - xy[:, 0]) / h  # as the FP64 coordinate has it
+    F = kde.grid(cuda(xy, torch.float64), None, (0.0, 0.0), cell, nx, 1, h, "epanechnikov")
+    got = F[0, torch.as_tensor(at, device="cuda")].cpu().numpy().astype(np.float64)
+    ref = 0.75 ** 2 * (1.0 - u * u) / (3000 * h * h)
+    assert int((F != 0).sum()) == 3000
+    assert rel_linf(got, ref) <= 2 * (nx * cell / h) * (2 * 2.0 ** -49 + 4 * 2.0 ** -53) + 2.0 ** -22
