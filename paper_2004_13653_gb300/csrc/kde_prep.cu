@@ -114,11 +114,13 @@ __global__ void __launch_bounds__(256)
   if ((int)blockIdx.x >= table_block) {
     const int b = (int)blockIdx.x - table_block;
     const PrepInst& I = tab[b / blocks_per_side];
-    const int t = (b % blocks_per_side) * blockDim.x + threadIdx.x;
-    if (t >= max(I.nx, I.ny)) return;
-    const float2 c = split_hi_lo(((double)t + 0.5) * I.cell_sigma);
-    if (t < I.nx) I.gxt[t] = c;
-    if (t < I.ny) I.gyt[t] = c;
+    const int64_t stride = (int64_t)blocks_per_side * blockDim.x;
+    for (int64_t t = (int64_t)(b % blocks_per_side) * blockDim.x + threadIdx.x;
+         t < max(I.nx, I.ny); t += stride) {
+      const float2 c = split_hi_lo(((double)t + 0.5) * I.cell_sigma);
+      if (t < I.nx) I.gxt[t] = c;
+      if (t < I.ny) I.gyt[t] = c;
+    }
     return;
   }
   // A warp takes kPerWarp consecutive points at a time, all of one instance,
@@ -263,7 +265,9 @@ void set_scale(PrepInst& q, int nx, int ny, double sigma, double cell, const Mer
 cudaError_t launch_prepare(const PrepInst* tab, int ninst, int64_t total_pad, int max_side,
                            cudaStream_t s) {
   if (ninst <= 0) return cudaSuccess;
-  const int per_side = (max_side + 255) / 256;
+  // as many table blocks as fill the GPU, at least one an instance: a block for every
+  // 256 cells of the longest side in every instance can be 2^31 of them
+  const int per_side = std::max(1, std::min(blocks_for(max_side, 256), 152 * 32 / ninst));
   const int points = total_pad > 0 ? blocks_for(total_pad, 8 * kPerWarp) : 0;
   k_prepare<<<points + ninst * per_side, 256, 0, s>>>(tab, ninst, total_pad, points, per_side);
   note_launches(1);

@@ -114,3 +114,28 @@ def test_far_end_of_a_long_axis_in_fp64():
     ref = 0.75 ** 2 * (1.0 - u * u) / (3000 * h * h)
     assert int((F != 0).sum()) == 3000
     assert rel_linf(got, ref) <= 2 * (nx * cell / h) * (2 * 2.0 ** -49 + 4 * 2.0 ** -53) + 2.0 ** -22
+
+
+def test_cell_tables_of_long_sides_and_many_instances():
+    """Tables longer than the launch's blocks fill in one go (1.2M cells for one
+    instance, 4864 for each of 256)."""
+    rng = np.random.default_rng(9)
+    nx = 3_000_001
+    xy = np.stack([rng.uniform(0.0, nx, 5000), rng.uniform(0.0, 1.0, 5000)], 1)
+    F = kde.grid(cuda(xy, torch.float64), None, (0.0, 0.0), 1.0, nx, 1, 2.0, "quartic").cpu().numpy()
+    cells = np.unique(np.clip(xy[:, 0].astype(np.int64)[:, None] + [-1, 0, 1], 0, nx - 1))
+    ref = oracle.kde_cells(xy, None, (0.0, 0.0), 1.0, nx, 1, 2.0, oracle.QUARTIC, cells)
+    # an offset of at most one keeps 2^-48 of 1.5e6 and FP32's rounding
+    assert rel_linf(F[0, cells], ref) <= TOL_FP32
+    insts = []
+    for k in range(256):
+        side = 20011 if k == 200 else 16 + k % 5
+        at = rng.uniform(0.0, 1.0, (300, 2)) * [side, 9]
+        insts.append(dict(points=cuda(at, torch.float64), weights=None, origin=(0.0, 0.0), cell=1.0,
+                          nx=side, ny=9, h=2.5, kernel="quartic"))
+    out = kde.grid_batched(insts)
+    for k in (0, 199, 200, 201, 255):
+        q = insts[k]
+        ref = oracle.kde_grid(q["points"].cpu().numpy(), None, q["origin"], 1.0, q["nx"], 9, 2.5,
+                              oracle.QUARTIC)
+        assert rel_linf(out[k].cpu().numpy(), ref) <= TOL_FP32
