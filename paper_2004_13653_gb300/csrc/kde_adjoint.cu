@@ -285,10 +285,10 @@ __global__ void __launch_bounds__(256)
     const double fi = floor(fx), fj = floor(fy);
     const double ax = fx - fi, ay = fy - fj;
     // the cell in 32 bits: far outside either way gives cells outside the grid
-    const int i = (int)fmin(fmax(fi, -2.0), 2147483000.0);
-    const int j = (int)fmin(fmax(fj, -2.0), 2147483000.0);
-    const bool x0 = i >= 0 && i < nx, x1 = i >= -1 && i + 1 < nx;
-    const bool y0 = j >= 0 && j < ny, y1 = j >= -1 && j + 1 < ny;
+    const int i = (int)fmin(fmax(fi, -2.0), (double)nx);
+    const int j = (int)fmin(fmax(fj, -2.0), (double)ny);
+    const bool x0 = i >= 0 && i < nx, x1 = i >= -1 && i < nx - 1;
+    const bool y0 = j >= 0 && j < ny, y1 = j >= -1 && j < ny - 1;
     const int64_t q = (int64_t)j * nx + i;
     const double f00 = x0 && y0 ? F[q] : 0.f, f10 = x1 && y0 ? F[q + 1] : 0.f;
     const double f01 = x0 && y1 ? F[q + nx] : 0.f, f11 = x1 && y1 ? F[q + nx + 1] : 0.f;
