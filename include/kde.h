@@ -251,7 +251,9 @@ int kde_grid_batched_tiled(const kde_args* inst, const kde_tiling* tiles, int co
  * c = 1/(2 pi N h^2), A, B the 1-D Gaussian factors, recomputed on the fly.
  * Two forms: a window kernel that sums each point's +-8h window on the FP32
  * pipes (opts->path KDE_PATH_SIMT_FP32; many points are sorted and share
- * windows in groups), and, for wide bandwidths, two
+ * windows in groups, where there are a dozen or more in a bin of 8 x 8 cells; a
+ * cell of G that is not finite reaches the points within 8h and two cells of it), and,
+ * for wide bandwidths, two
  * tcgen05 contractions U = G B and V = G^T A (split-FP16, three products;
  * KDE_PATH_TC_SPLIT16 or KDE_PATH_TC_FP16) whose epilogues fold U and V
  * into the per-point sums, over the cells within 8h of each tile of sorted

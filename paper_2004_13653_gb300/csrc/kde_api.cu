@@ -318,10 +318,13 @@ int sparse_sort_bin(int nx, int ny, int instances) {
 }
 
 // The adjoint takes the tensor-core contractions when the window kernel's
-// cells per point exceed this fraction of the grid padded to 256-cell tiles
-// (measured on 1M points x 1024^2: the contractions take 6.2 ms at every h,
-// the window 5.7 ms at h = 5.1 cells and 26 ms at h = 8.2 cells, about 1 ns
-// per window cell and point).
+// cells per point exceed this fraction of the grid padded to 256-cell tiles.  The
+// line was drawn when the contractions took the whole grid at every h (6.2 ms for 1M
+// points x 1024^2) and the window one warp per point (5.7 ms at h = 5.1 cells, 26 ms
+// at 8.2).  On sorted points both cost less, the contractions more so: 1M of the
+// mixture x 1024^2, window / contractions 380 / 423 us at h = 1 cell, 687 / 434 at 2,
+// 1919 / 484 at 5; x 2048^2, where the line lies at h = 9.9 cells, 917 / 527 at 3 and
+// 25,767 / 696 at 8.
 constexpr double kAdjointTcRatio = 0.006;
 
 // The contraction form of the adjoint sorts its points into bins of about one
