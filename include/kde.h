@@ -325,8 +325,8 @@ int kde_grid_binned(const double* points, const int64_t* traj_offsets, int64_t n
  * receives the kept points in order; out_offsets: device [ntraj+1] or NULL,
  * the trajectories' bounds in out_points; n_kept, iterations: host, optional.
  * Synchronous: trajectories of up to a few thousand points run their iterations
- * in one launch, a CTA each, and the others all of theirs in one cooperative
- * launch (the loop ends on the device); the call reads the iteration count and
+ * in one launch, a CTA each, and the others (with eps below 1e-8 all of them) all of
+ * theirs in one cooperative launch (the loop ends on the device); the call reads the iteration count and
  * the kept count back once.  Errors: KDE_EINVAL (n,
  * eps, pointers, alignment, offsets that do not rise from 0 to n), KDE_EDATA
  * (non-finite coordinate), KDE_ECUDA (the device cannot hold the cooperative
